@@ -418,7 +418,8 @@ DST_API int dst_testing_fp32_arnoldi(int mode, int64_t n, int nvec, const void *
  * n_unknowns entries (float pairs, the unknown layout), distinct; arithmetic in
  * FP32 (the precision of the inner solve), the layer-solve factors in FP64
  * rounded to FP32.  Takes stream-ordered scratch of about one FP32 vector (plus
- * the factors, 32 NC^2 bytes per x node and frequency, on Dirichlet-x meshes).
+ * the factors, below 32 (6 + 2 log2 n_x) bytes per x node and frequency, on
+ * Dirichlet-x meshes).
  * kind DST_PRECOND_CN_SWEEP, DST_PRECOND_CN_LEARNED (the sweep plus the
  * learned correction below, with the network attached to the mesh by
  * dst_set_learned_precond; two more FP32 vectors of scratch), or

@@ -4,15 +4,21 @@
 // Each CTA loads one plane (n1 x n2 nodes of one layer, or of one x node of a
 // layer) of its component group into shared memory, transforms every line of
 // the inner axis and then every line of the outer axis, and stores the result.
-// The mixed-radix Stockham self-sorting scheme (stages of radix 4, 2, then odd
-// primes; twiddles from a per-axis table w[j] = exp(sign 2 pi i j / n)) runs
+// Mixed-radix Stockham self-sorting stages (16, 8, 4, 2, 3, 5 in registers, other
+// primes by their sums; twiddles from a per-axis table w[j] = exp(sign 2 pi i j / n)) run
 // either over all lines of an axis at once, the CTA's threads sharing every
 // stage's butterflies (when a second plane buffer fits in shared memory), or one
 // line per warp with two scratch lines.
+// What bounds it is shared memory: with the first and last pass a 48 x 48 plane
+// crosses it six times.  Neighbouring lanes take neighbouring lines, whose pitch is
+// odd, so that neither the strided reads nor the scattered writes of a stage meet on a
+// bank, and the stage's index arithmetic is the same for a whole warp.
 // Forward (sign -1): node layout in, frequency layout [b][f][c] out with
 // f = i1 n2 + i2.  Inverse (sign +1): frequency layout in, node layout out,
 // scaled by 1 / (n1 n2).
 #pragma once
+
+#include <algorithm>
 
 #include "sweep.h"
 
@@ -36,122 +42,189 @@ template <typename V> __device__ __forceinline__ V csub(V a, V b) { return mk<V>
 template <typename V> __device__ __forceinline__ V cfma(V a, V b, V acc) {
     return mk<V>(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
 }
+// a times sg i
+template <typename V, typename R> __device__ __forceinline__ V rot(V a, R sg) { return mk<V>(-sg * a.y, sg * a.x); }
 
 __device__ __forceinline__ void sincos_pi(float x, float *s, float *c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincos_pi(double x, double *s, double *c) { sincospi(x, s, c); }
 
+template <typename V> __device__ __forceinline__ void copy_async(V *dst, const V *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"((int)sizeof(V)) : "memory");
+}
+
+// In-place DFTs of R values, X_o = sum_r v_r exp(sg 2 pi i r o / R).
+template <int R> struct Dft;
+template <> struct Dft<2> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S) {
+        const V a = v[0], b = v[1];
+        v[0] = cadd(a, b); v[1] = csub(a, b);
+    }
+};
+template <> struct Dft<3> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S sg) {
+        const S h = (S)0.86602540378443864676;             // sin(pi / 3)
+        const V t = cadd(v[1], v[2]), u = rot(csub(v[1], v[2]), sg * h);
+        const V m = mk<V>(fma((S)-0.5, t.x, v[0].x), fma((S)-0.5, t.y, v[0].y));
+        v[0] = cadd(v[0], t); v[1] = cadd(m, u); v[2] = csub(m, u);
+    }
+};
+template <> struct Dft<4> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S sg) {
+        const V t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]), t2 = cadd(v[1], v[3]), t3 = rot(csub(v[1], v[3]), sg);
+        v[0] = cadd(t0, t2); v[1] = cadd(t1, t3); v[2] = csub(t0, t2); v[3] = csub(t1, t3);
+    }
+};
+template <> struct Dft<5> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S sg) {
+        const S c1 = (S)0.30901699437494742410, c2 = (S)-0.80901699437494742410;     // cos(2 pi / 5), cos(4 pi / 5)
+        const S s1 = (S)0.95105651629515357212, s2 = (S)0.58778525229247312917;      // sin(2 pi / 5), sin(4 pi / 5)
+        const V a = cadd(v[1], v[4]), b = cadd(v[2], v[3]), d = csub(v[1], v[4]), e = csub(v[2], v[3]);
+        const V p = mk<V>(v[0].x + c1 * a.x + c2 * b.x, v[0].y + c1 * a.y + c2 * b.y);
+        const V q = mk<V>(v[0].x + c2 * a.x + c1 * b.x, v[0].y + c2 * a.y + c1 * b.y);
+        const V r = rot(mk<V>(s1 * d.x + s2 * e.x, s1 * d.y + s2 * e.y), sg);
+        const V t = rot(mk<V>(s2 * d.x - s1 * e.x, s2 * d.y - s1 * e.y), sg);
+        v[0] = cadd(v[0], cadd(a, b));
+        v[1] = cadd(p, r); v[4] = csub(p, r); v[2] = cadd(q, t); v[3] = csub(q, t);
+    }
+};
+template <> struct Dft<8> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S sg) {
+        const S c = (S)0.70710678118654752440;
+        V e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        Dft<4>::run(e, sg);
+        Dft<4>::run(o, sg);
+        o[1] = mk<V>(c * (o[1].x - sg * o[1].y), c * (o[1].y + sg * o[1].x));
+        o[2] = rot(o[2], sg);
+        o[3] = mk<V>(-c * (o[3].x + sg * o[3].y), c * (sg * o[3].x - o[3].y));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { v[k] = cadd(e[k], o[k]); v[k + 4] = csub(e[k], o[k]); }
+    }
+};
+template <> struct Dft<16> {
+    template <typename V, typename S> static __device__ __forceinline__ void run(V *v, S sg) {
+        const S co[8] = {(S)1, (S)0.92387953251128675613, (S)0.70710678118654752440, (S)0.38268343236508977173,
+                         (S)0, (S)-0.38268343236508977173, (S)-0.70710678118654752440, (S)-0.92387953251128675613};
+        V e[8], o[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { e[k] = v[2 * k]; o[k] = v[2 * k + 1]; }
+        Dft<8>::run(e, sg);
+        Dft<8>::run(o, sg);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const S sn = k == 0 ? (S)0 : (k <= 4 ? co[4 - k] : co[k - 4]);           // sin(pi k / 8)
+            const V t = k == 0 ? o[0] : (k == 4 ? rot(o[4], sg) : cmul(o[k], mk<V>(co[k], sg * sn)));
+            v[k] = cadd(e[k], t); v[k + 8] = csub(e[k], t);
+        }
+    }
+};
+
+// One butterfly of a stage: elements j + r q of a line (element stride st) times
+// w^(r k step), to (j / Ns) Ns R + k + o Ns of the output line; q = n / R, step = q / Ns.
+template <int R, typename V, typename S>
+__device__ __forceinline__ void butterfly(const V *src, V *dst, int st, int q, int step, int Ns, int j, int k, const V *w, S sg) {
+    V v[R];
+    v[0] = src[j * st];
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(src[(j + r * q) * st], w[r * k * step]);
+    Dft<R>::run(v, sg);
+    const int to = (j - k) * R + k;
+#pragma unroll
+    for (int o = 0; o < R; ++o) dst[(to + o * Ns) * st] = v[o];
+}
+
+// One output of a stage of any radix R: V_o = sum_r v_r w^(r (k step + o q)).
 template <typename V>
-__device__ void warp_fft_line(V *line, int st, int n, const int *rad, int nrad, const V *w, V *a, V *b) {
+__device__ __forceinline__ V general_output(const V *src, int st, int n, int R, int q, int step, int j, int k, int o,
+                                          const V *w) {
+    const int inc = k * step + o * q;                      // < n
+    V acc = src[j * st];
+    int at = inc;
+    for (int r = 1; r < R; ++r) {
+        acc = cfma(w[at], src[(j + r * q) * st], acc);
+        at += inc;
+        if (at >= n) at -= n;
+    }
+    return acc;
+}
+
+// Every butterfly of one stage for threads `id` of `count`; line l starts at line(l),
+// `nl` lines, element stride st; neighbouring threads take neighbouring lines.
+template <typename V, typename S, typename Line>
+__device__ __forceinline__ void stage(const V *d0, V *d1, int n, int st, int nl, Line line, int R, int Ns, const V *w, S sg,
+                                      int id, int count) {
+    const int q = n / R, step = q / Ns;
+    // quotients by nl and Ns by multiplication: the dividends stay below 2^32 / divisor
+    const unsigned rn = nl > 1 ? 0xffffffffu / (unsigned)nl + 1u : 0u, rk = Ns > 1 ? 0xffffffffu / (unsigned)Ns + 1u : 0u;
+    auto by_nl = [&](int i) { return nl > 1 ? (int)__umulhi((unsigned)i, rn) : i; };
+    auto mod_ns = [&](int j) { return Ns > 1 ? j - (int)__umulhi((unsigned)j, rk) * Ns : 0; };
+    const bool direct = R == 2 || R == 3 || R == 4 || R == 5 || R == 8 || R == 16;
+    if (!direct) {
+        for (int i = id; i < nl * n; i += count) {
+            const int jo = by_nl(i), l = i - jo * nl, base = line(l);
+            const int o = jo / q, j = jo - o * q, k = mod_ns(j);
+            d1[base + ((j - k) * R + k + o * Ns) * st] = general_output(d0 + base, st, n, R, q, step, j, k, o, w);
+        }
+        return;
+    }
+    for (int i = id; i < nl * q; i += count) {
+        const int j = by_nl(i), l = i - j * nl, base = line(l), k = mod_ns(j);
+        const V *src = d0 + base;
+        V *dst = d1 + base;
+        switch (R) {
+            case 2: butterfly<2>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+            case 3: butterfly<3>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+            case 4: butterfly<4>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+            case 5: butterfly<5>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+            case 8: butterfly<8>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+            default: butterfly<16>(src, dst, st, q, step, Ns, j, k, w, sg); break;
+        }
+    }
+}
+
+template <typename V, typename S>
+__device__ void warp_fft_line(V *line, int st, int n, const int *rad, int nrad, const V *w, S sg, V *a, V *b) {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < n; i += 32) a[i] = line[i * st];
     __syncwarp();
     V *d0 = a, *d1 = b;
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
-        const int R = rad[s];
-        const int q = n / R;               // butterflies of this stage
-        const int step = n / (Ns * R);     // exp(sign 2 pi i k / (Ns R)) = w[k * step]
-        for (int j = lane; j < q; j += 32) {
-            const int k = j % Ns;
-            const int dst = (j / Ns) * Ns * R + k;
-            if (R == 2) {
-                const V v0 = d0[j], v1 = cmul(d0[j + q], w[k * step]);
-                d1[dst] = cadd(v0, v1);
-                d1[dst + Ns] = csub(v0, v1);
-            } else if (R == 4) {
-                const V v0 = d0[j];
-                const V v1 = cmul(d0[j + q], w[k * step]);
-                const V v2 = cmul(d0[j + 2 * q], w[(2 * k * step) % n]);
-                const V v3 = cmul(d0[j + 3 * q], w[(3 * k * step) % n]);
-                const V om = w[n / 4];                       // exp(sign i pi / 2)
-                const V t0 = cadd(v0, v2), t1 = csub(v0, v2);
-                const V t2 = cadd(v1, v3), t3 = cmul(om, csub(v1, v3));
-                d1[dst] = cadd(t0, t2);
-                d1[dst + Ns] = cadd(t1, t3);
-                d1[dst + 2 * Ns] = csub(t0, t2);
-                d1[dst + 3 * Ns] = csub(t1, t3);
-            } else {
-                // general radix: V_o = sum_r v_r exp(sign 2 pi i r o / R), v_r twiddled
-                for (int o = 0; o < R; ++o) {
-                    V acc = mk<V>(0, 0);
-                    for (int r = 0; r < R; ++r) {
-                        const V vr = cmul(d0[j + r * q], w[(int)(((long long)r * k * step) % n)]);
-                        acc = cfma(w[(int)(((long long)r * o * q) % n)], vr, acc);
-                    }
-                    d1[dst + o * Ns] = acc;
-                }
-            }
-        }
+        stage(d0, d1, n, 1, 1, [](int) { return 0; }, rad[s], Ns, w, sg, lane, 32);
         __syncwarp();
         V *t = d0; d0 = d1; d1 = t;
-        Ns *= R;
+        Ns *= rad[s];
     }
     for (int i = lane; i < n; i += 32) line[i * st] = d0[i];
     __syncwarp();
 }
 
-// All lines of one axis of the plane through the Stockham stages at once: each
-// stage's butterflies of every line are spread over the CTA's threads, with a
-// barrier between stages (ping-pong between the plane and a second buffer).
-// Line l of the axis starts at l_base(l) and has element stride st; `nl` lines.
-// Returns the buffer holding the result (the plane or the second buffer).
-template <typename V>
-__device__ V *cta_fft_axis(V *d0, V *d1, int n, int st, int nl, int lstride_in, int lsplit, int lstride_out,
-                           const int *rad, int nrad, const V *w) {
-    // line l = (la, lb) with la = l / lsplit, lb = l % lsplit; element i of line l at
-    // la * lstride_out + lb * lstride_in + i * st (the same map in both buffers)
+// All lines of one axis of the plane through the stages at once, with a barrier
+// between stages (ping-pong between the two plane buffers).  Returns the buffer that
+// holds the result.
+template <typename V, typename S, typename Line>
+__device__ V *cta_fft_axis(V *d0, V *d1, int n, int st, int nl, Line line, const int *rad, int nrad, const V *w, S sg) {
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
-        const int R = rad[s];
-        const int q = n / R;
-        const int step = n / (Ns * R);
-        for (int idx = threadIdx.x; idx < nl * q; idx += blockDim.x) {
-            const int l = idx / q, j = idx % q;
-            const int base = (l / lsplit) * lstride_out + (l % lsplit) * lstride_in;
-            const V *src = d0 + base;
-            V *dst_ = d1 + base;
-            const int k = j % Ns;
-            const int dst = (j / Ns) * Ns * R + k;
-            if (R == 2) {
-                const V v0 = src[j * st], v1 = cmul(src[(j + q) * st], w[k * step]);
-                dst_[dst * st] = cadd(v0, v1);
-                dst_[(dst + Ns) * st] = csub(v0, v1);
-            } else if (R == 4) {
-                const V v0 = src[j * st];
-                const V v1 = cmul(src[(j + q) * st], w[k * step]);
-                const V v2 = cmul(src[(j + 2 * q) * st], w[(2 * k * step) % n]);
-                const V v3 = cmul(src[(j + 3 * q) * st], w[(3 * k * step) % n]);
-                const V om = w[n / 4];
-                const V t0 = cadd(v0, v2), t1 = csub(v0, v2);
-                const V t2 = cadd(v1, v3), t3 = cmul(om, csub(v1, v3));
-                dst_[dst * st] = cadd(t0, t2);
-                dst_[(dst + Ns) * st] = cadd(t1, t3);
-                dst_[(dst + 2 * Ns) * st] = csub(t0, t2);
-                dst_[(dst + 3 * Ns) * st] = csub(t1, t3);
-            } else {
-                for (int o = 0; o < R; ++o) {
-                    V acc = mk<V>(0, 0);
-                    for (int r = 0; r < R; ++r) {
-                        const V vr = cmul(src[(j + r * q) * st], w[(int)(((long long)r * k * step) % n)]);
-                        acc = cfma(w[(int)(((long long)r * o * q) % n)], vr, acc);
-                    }
-                    dst_[(dst + o * Ns) * st] = acc;
-                }
-            }
-        }
+        stage(d0, d1, n, st, nl, line, rad[s], Ns, w, sg, threadIdx.x, FFT_THREADS);
         __syncthreads();
         V *t = d0; d0 = d1; d1 = t;
-        Ns *= R;
+        Ns *= rad[s];
     }
     return d0;
 }
 
-// Shared memory of one CTA: the plane, two twiddle tables, two scratch lines per warp.
+// Line pitch of a plane in shared memory: odd where two plane buffers are used.
+__host__ __device__ inline int pitch(const SweepFft &a) { return a.pingpong ? a.n2 | 1 : a.n2; }
+
+// Shared memory of one CTA: the plane, two twiddle tables, and a second plane or two
+// scratch lines per warp.
 template <typename V>
 inline size_t fft_smem_bytes(const SweepFft &a) {
     const int nmax = a.n1 > a.n2 ? a.n1 : a.n2;
-    const size_t scratch = a.pingpong ? (size_t)a.ncb * a.n1 * a.n2 : (size_t)FFT_WARPS * 2 * nmax;
-    return sizeof(V) * ((size_t)a.ncb * a.n1 * a.n2 + a.n1 + a.n2 + scratch);
+    const size_t plane = (size_t)a.ncb * a.n1 * pitch(a);
+    const size_t scratch = a.pingpong ? plane : (size_t)FFT_WARPS * 2 * nmax;
+    return sizeof(V) * (plane + a.n1 + a.n2 + scratch);
 }
 
 template <typename V>
@@ -160,10 +233,10 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
     using R = typename Real<V>::type;
     extern __shared__ __align__(16) unsigned char fft_sm_raw[];
     V *sm = reinterpret_cast<V *>(fft_sm_raw);
-    const int n1 = a.n1, n2 = a.n2, nc = a.nc, ncb = a.ncb;
-    const int nf = n1 * n2;
-    V *plane = sm;                                        // [ncb][n1][n2]
-    V *w1 = plane + (size_t)ncb * nf;                     // twiddles of the outer axis (n1)
+    const int n1 = a.n1, n2 = a.n2, nc = a.nc, ncb = a.ncb, pt = pitch(a);
+    const int nf = n1 * n2, pl = n1 * pt;
+    V *plane = sm;                                        // [ncb][n1][pitch]
+    V *w1 = plane + (size_t)ncb * pl;                     // twiddles of the outer axis (n1)
     V *w2 = w1 + n1;                                      // twiddles of the inner axis (n2)
     V *scr = w2 + n2;                                     // second plane, or per warp two lines of nmax
     const int nmax = n1 > n2 ? n1 : n2;
@@ -171,6 +244,16 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
     const int c0 = blockIdx.y * ncb;
     const int64_t base = (b / a.nbx) * a.ns_nodes + (b % a.nbx) * a.sbx;   // node index of (i1, i2) = (0, 0)
     const R sign = inverse ? (R)1 : (R)-1;
+    const int lcb = __ffs(ncb) - 1;                       // components per CTA: 1, 2 or 4
+    const unsigned r2 = n2 > 1 ? 0xffffffffu / (unsigned)n2 + 1u : 0u;
+    auto row = [&](int f) { return n2 > 1 ? (int)__umulhi((unsigned)f, r2) : f; };
+    for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) {
+        const int cc = idx & (ncb - 1), f = idx >> lcb;
+        const int i1 = row(f), i2 = f - i1 * n2;
+        copy_async(plane + cc * pl + i1 * pt + i2,
+                   in + (inverse ? (b * nf + f) * nc : (base + (int64_t)i1 * a.s1 + (int64_t)i2 * a.s2) * nc) + c0 + cc);
+    }
+    // the twiddles while the plane is on its way
     for (int j = threadIdx.x; j < n1; j += FFT_THREADS) {
         R sn, cs;
         sincos_pi((R)2 * (R)j / (R)n1, &sn, &cs);
@@ -181,44 +264,36 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
         sincos_pi((R)2 * (R)j / (R)n2, &sn, &cs);
         w2[j] = mk<V>(cs, sign * sn);
     }
-    for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) {
-        const int cc = idx % ncb, f = idx / ncb;
-        const int i1 = f / n2, i2 = f % n2;
-        V v;
-        if (inverse) v = in[(b * nf + f) * nc + c0 + cc];
-        else v = in[(base + (int64_t)i1 * a.s1 + (int64_t)i2 * a.s2) * nc + c0 + cc];
-        plane[(size_t)cc * nf + f] = v;
-    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
+    V *cur = plane;
     if (a.pingpong) {
-        // CTA-wide stages; scr is a second plane
-        V *cur = plane;
-        if (n2 > 1) cur = cta_fft_axis(cur, cur == plane ? scr : plane, n2, 1, ncb * n1, 0, 1, n2, a.rad2, a.nrad2, w2);
+        // CTA-wide stages; scr is a second plane.  Inner lines start every pitch; outer
+        // line (cc, i2) at cc * pl + i2.
+        if (n2 > 1) cur = cta_fft_axis(cur, scr, n2, 1, ncb * n1, [&](int l) { return l * pt; }, a.rad2, a.nrad2, w2, sign);
         if (n1 > 1)
-            cur = cta_fft_axis(cur, cur == plane ? scr : plane, n1, n2, ncb * n2, 1, n2, nf, a.rad1, a.nrad1, w1);
-        if (cur != plane) {
-            for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) plane[idx] = cur[idx];
-            __syncthreads();
-        }
+            cur = cta_fft_axis(cur, cur == plane ? scr : plane, n1, pt, ncb * n2,
+                               [&](int l) { const int cc = row(l); return cc * pl + (l - cc * n2); }, a.rad1, a.nrad1, w1,
+                               sign);
     } else {
         const int warp = threadIdx.x >> 5;
         V *sa = scr + (size_t)warp * 2 * nmax, *sb = sa + nmax;
         if (n2 > 1)
             for (int line = warp; line < ncb * n1; line += FFT_WARPS)
-                warp_fft_line(plane + (size_t)line * n2, 1, n2, a.rad2, a.nrad2, w2, sa, sb);
+                warp_fft_line(plane + (size_t)line * n2, 1, n2, a.rad2, a.nrad2, w2, sign, sa, sb);
         __syncthreads();
         if (n1 > 1)
             for (int line = warp; line < ncb * n2; line += FFT_WARPS) {
                 const int cc = line / n2, i2 = line % n2;
-                warp_fft_line(plane + (size_t)cc * nf + i2, n2, n1, a.rad1, a.nrad1, w1, sa, sb);
+                warp_fft_line(plane + (size_t)cc * nf + i2, n2, n1, a.rad1, a.nrad1, w1, sign, sa, sb);
             }
         __syncthreads();
     }
     const R scale = inverse ? (R)1 / (R)nf : (R)1;
     for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) {
-        const int cc = idx % ncb, f = idx / ncb;
-        const int i1 = f / n2, i2 = f % n2;
-        V v = plane[(size_t)cc * nf + f];
+        const int cc = idx & (ncb - 1), f = idx >> lcb;
+        const int i1 = row(f), i2 = f - i1 * n2;
+        V v = cur[cc * pl + i1 * pt + i2];
         v.x *= scale;
         v.y *= scale;
         if (inverse) out[(base + (int64_t)i1 * a.s1 + (int64_t)i2 * a.s2) * nc + c0 + cc] = v;
@@ -227,17 +302,18 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
 }
 
 // Pick the components per CTA and the stage layout for planes of a.n1 x a.n2:
-// CTA-wide stages (second plane buffer) when they fit, else one line per warp;
-// fewer components per CTA when the CTAs would not fill the GPU (nb planes per
-// component group).  Returns false if nothing fits in `limit` bytes.
+// CTA-wide stages (second plane buffer) when they fit, else one line per warp.  The
+// components of a node are adjacent in memory, so a CTA takes as many as leave three
+// CTAs per SM and enough CTAs to fill the GPU (nb planes per component group).
+// Returns false if nothing fits in `limit` bytes.
 template <typename V>
 inline bool choose_layout(SweepFft &a, int64_t nb, size_t limit) {
     for (int pp = 1; pp >= 0; --pp) {
         a.pingpong = pp;
-        for (int ncb = a.nc; ncb >= 1; ncb /= 2) {
+        for (int ncb = a.nc; ncb > 1; ncb /= 2) {
             a.ncb = ncb;
-            if (fft_smem_bytes<V>(a) > limit) continue;
-            if (ncb > 1 && nb * (a.nc / ncb) < 304) continue;
+            if (fft_smem_bytes<V>(a) > (pp ? std::min<size_t>(limit, 76 * 1024) : limit)) continue;
+            if (nb * (a.nc / ncb) < 304) continue;
             return true;
         }
         a.ncb = 1;
@@ -246,12 +322,12 @@ inline bool choose_layout(SweepFft &a, int64_t nb, size_t limit) {
     return false;
 }
 
-// Stockham radices of n: fours, a two, then odd primes.
+// Stockham radices of n: the fewest stages of the register butterflies, then other primes.
 inline void radices(int n, int *r, int &nr) {
     nr = 0;
-    while (n % 4 == 0) { r[nr++] = 4; n /= 4; }
-    while (n % 2 == 0) { r[nr++] = 2; n /= 2; }
-    for (int p = 3; n > 1; p += 2)
+    for (int p : {16, 8, 4, 2, 3, 5})
+        while (n % p == 0) { r[nr++] = p; n /= p; }
+    for (int p = 7; n > 1; p += 2)
         while (n % p == 0) { r[nr++] = p; n /= p; }
 }
 

@@ -573,8 +573,8 @@ struct Solver {
         if (precond == DST_PRECOND_BLOCK_JACOBI)       // z = blockdiag(A_nn)^-1 v
             return run(K_PRECOND, 1, (16.0 + 8.0 * mesh->nc) * dn, 8.0 * mesh->nc * dn,
                        [&] { return dst_internal_jacobi_apply(mesh, v, z, s); });
-        const double sweep_bytes = (plan.has_fft ? 48.0 : 40.0) * dn + (double)plan.table_bytes * plan.g.nt;
-        int rc = run(K_PRECOND, plan.has_fft ? 4 : 3, sweep_bytes, 0.0,
+        const double sweep_bytes = plan.bytes_per_entry * dn + (double)plan.table_bytes;
+        int rc = run(K_PRECOND, plan.launches, sweep_bytes, 0.0,
                      [&] { return dst_sweep_apply(plan, n, v, z, s); });
         if (rc || precond == DST_PRECOND_CN_SWEEP) return rc;
         if ((rc = run(K_APPLY32, 1, 16.0 * dn, dst_internal_apply_flops(mesh),
@@ -588,7 +588,7 @@ struct Solver {
             prof.launches[K_PRECOND] += nk;
             return rc;
         }
-        if ((rc = run(K_PRECOND, plan.has_fft ? 4 : 3, sweep_bytes, 0.0,
+        if ((rc = run(K_PRECOND, plan.launches, sweep_bytes, 0.0,
                       [&] { return dst_sweep_apply(plan, n, w.pr, w.pz2, s); })))
             return rc;
         return run(K_MISC, 1, 24.0 * dn, 2.0 * dn, [&] { return dst_k_add_f32(n, w.pz2, z, s); });

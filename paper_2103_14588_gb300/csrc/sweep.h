@@ -27,18 +27,29 @@ struct SweepGeom {
     int ax1, ax2;               // physical axis of each frequency dimension (-1: none)
 };
 
+// One frequency of the banded march: prod of the y, z mass symbols, the transverse term
+// P, cos and sin of half the rotation angle, and the index of its +P (3+1) or own system.
+struct FreqRow {
+    float myz, P, c, s;
+    int sys;
+};
+
 struct SweepPlan {
     SweepGeom g;
     SweepFft fft;
     bool banded, has_fft, vx;
     int64_t nb;                 // FFT planes
     size_t fft_smem;
-    size_t table_bytes;         // banded: block Thomas factors
-    int march_threads;
+    size_t table_bytes;         // banded: reduction factors (sweep_march.cuh)
+    int lanes, steps, systems;  // banded: lanes per system, parallel reduction steps, systems per CTA
     size_t march_smem;
+    int launches;               // kernels of one application
+    double bytes_per_entry;     // algorithmic bytes of one application, factors apart
     // set by dst_sweep_setup inside the caller's scratch
     float2 *work;
-    float2 *table;
+    float *table;
+    FreqRow *freq;
+    float4 *alt_hi, *alt_lo;
     double *dvx;
 };
 

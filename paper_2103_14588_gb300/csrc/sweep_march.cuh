@@ -1,0 +1,451 @@
+// The Crank-Nicolson march of the sweep along a Dirichlet x axis (sweep.cu, banded
+// mode): x_t = Bd^-1 (s_t - Bl x_{t-1}) for every frequency of the periodic axes.
+//
+// Three identities shape the kernels.
+// 1. Bd + Bl = h_t K, so the increment u_t = x_t - x_{t-1} solves
+//    Bd u_t = s_t - h_t K x_{t-1}.  The rounding of the solve is then relative to the
+//    increment, which is small for the modes that the time step resolves.
+// 2. At one (y, z) frequency K contains alpha_y b_y + alpha_z b_z with the same x
+//    mass.  The rotation exp(-i phi / 2 Sigma_x), tan phi = b_z / b_y, commutes with
+//    alpha_x and beta and turns it into alpha_y P, P = |b|, which couples the spinor
+//    components only within the pairs (0, 3) (as sigma_x, P sigma_y, sigma_z) and
+//    (1, 2) (as sigma_x, -P sigma_y, sigma_z).  So a 3+1 frequency is two systems of
+//    2 x 2 blocks, of the 2+1 kind, at a quarter of the block work each; and since
+//    only |sin| enters P, the factors are shared by the frequencies +-k.
+// 3. S^-1 also runs forward: s_0 = 2 sum_t (-1)^t v_t, s_{t+1} = 2 v_t - s_t.  With
+//    s_0 from one reading pass (altsum_kernel) the time scan costs no pass of its own.
+//
+// The layer solve.  The systems are few (2 x 2304 for the 48^3 x 48 Klein mesh) and the
+// time steps are a serial chain, so block Thomas elimination (a chain of 2 n_x small
+// products per layer) leaves the GPU waiting: it took 4.5 ms there.  Here G lanes share a
+// system, two x nodes each: one cyclic-reduction step removes the odd nodes, parallel
+// cyclic reduction over the even ones needs log2(G) exchanges, and the odd nodes follow.
+// Twice the arithmetic of the elimination, a seventh of the chain.  Bd = i M + (h_t/2) K
+// with M positive definite and K Hermitian, so every Schur complement met on the way
+// keeps a positive definite part (no pivoting).  The factors (2 x 2 blocks per lane and
+// step) stay in registers for all layers when G <= 32.
+// Layers stream through a shared-memory ring (cp.async), rows of neighbouring
+// frequencies, so that global memory sees whole sectors although a warp walks along x.
+#pragma once
+
+#include "sweep.h"
+
+namespace dst_march {
+
+constexpr int STAGES = 3;                 // input layers in shared memory
+constexpr int REG_STEPS = 5;              // reduction steps whose factors stay in registers (G <= 32)
+
+struct z2 { double x, y; };
+__device__ __forceinline__ z2 operator+(z2 a, z2 b) { return z2{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ z2 operator-(z2 a, z2 b) { return z2{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ z2 operator*(z2 a, z2 b) { return z2{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+
+struct M22 { z2 a, b, c, d; };            // rows (a b), (c d)
+__device__ __forceinline__ M22 zero22() { const z2 z{0.0, 0.0}; return M22{z, z, z, z}; }
+__device__ __forceinline__ M22 mul(const M22 &p, const M22 &q) {
+    return M22{p.a * q.a + p.b * q.c, p.a * q.b + p.b * q.d, p.c * q.a + p.d * q.c, p.c * q.b + p.d * q.d};
+}
+__device__ __forceinline__ M22 sub(const M22 &p, const M22 &q) { return M22{p.a - q.a, p.b - q.b, p.c - q.c, p.d - q.d}; }
+__device__ __forceinline__ M22 neg(const M22 &p) { return sub(zero22(), p); }
+__device__ __forceinline__ M22 inv(const M22 &p) {
+    const z2 det = p.a * p.d - p.b * p.c;
+    const double r = 1.0 / (det.x * det.x + det.y * det.y);
+    const z2 w{det.x * r, -det.y * r}, m{-w.x, -w.y};
+    return M22{p.d * w, p.b * m, p.c * m, p.a * w};
+}
+
+// Symbols of one frequency: prod of the y, z masses and the two transverse terms.
+__device__ __forceinline__ void symbols(const SweepGeom &g, int i1, int i2, double &myz, double &by, double &bz) {
+    double th[3] = {0.0, 0.0, 0.0};
+    const double PI2 = 6.28318530717958647692;
+    if (g.ax1 >= 0) th[g.ax1] = PI2 * i1 / g.n1;
+    if (g.ax2 >= 0) th[g.ax2] = PI2 * i2 / g.n2;
+    const double my = g.d >= 2 ? g.h[1] * (2.0 + cos(th[1])) / 3.0 : 1.0;
+    const double mz = g.d >= 3 ? g.h[2] * (2.0 + cos(th[2])) / 3.0 : 1.0;
+    myz = my * mz;
+    by = g.d >= 2 ? sin(th[1]) * mz : 0.0;
+    bz = g.d >= 3 ? sin(th[2]) * my : 0.0;
+}
+
+// Distinct frequencies up to sign: classes (k1, k2), k = 0 .. n/2; each has a system for
+// +P and one for -P (index 2 class + (P < 0)).
+__host__ __device__ inline int class_count(int n1, int n2) { return (n1 / 2 + 1) * (n2 / 2 + 1); }
+
+// Block (i, o) of Bd, o in {-1, 0, 1}, on unknown x node i (geometric node i + 1):
+//   i M myz + (h_t/2) [ i C myz sigma_x - M P sigma_y - diag(W+, W-) myz ].
+__device__ __forceinline__ M22 bd_block(const SweepGeom &g, const double *Vx, int i, int o, double myz, double P) {
+    const double h6 = g.h[0] / 6.0, ht2 = 0.5 * g.ht;
+    const double vl = Vx ? Vx[i] : 0.0, vr = Vx ? Vx[i + 1] : 0.0;      // elements left and right of the node
+    const double M = o == 0 ? 4.0 * h6 : h6, C = 0.5 * o;
+    const double v = o == 0 ? 2.0 * (vl + vr) : (o < 0 ? vl : vr), mw = o == 0 ? 4.0 * g.m : g.m;
+    const double im = M * myz, c = ht2 * C * myz, s = ht2 * M * P;
+    return M22{z2{-ht2 * h6 * (mw + v) * myz, im}, z2{0.0, c + s}, z2{0.0, c - s}, z2{-ht2 * h6 * (v - mw) * myz, im}};
+}
+
+// Number of factor blocks per lane: the cyclic step's pair, a pair per parallel step,
+// the even inverse, and the odd nodes' inverse and two couplings.
+__host__ __device__ inline int items(int steps) { return 6 + 2 * steps; }
+
+__device__ __forceinline__ void put(float *tab, int G, int item, int lane, const M22 &m) {
+    float4 *o = reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8);
+    o[0] = make_float4((float)m.a.x, (float)m.a.y, (float)m.b.x, (float)m.b.y);
+    o[1] = make_float4((float)m.c.x, (float)m.c.y, (float)m.d.x, (float)m.d.y);
+}
+
+// The row of one frequency.
+__device__ __forceinline__ FreqRow freq_row(const SweepGeom &g, int f) {
+    const int i1 = f / g.n2, i2 = f % g.n2;
+    double myz, by, bz;
+    symbols(g, i1, i2, myz, by, bz);
+    const int sys = 2 * (min(i1, g.n1 - i1) * (g.n2 / 2 + 1) + min(i2, g.n2 - i2));
+    if (g.nc == 2) return FreqRow{(float)myz, (float)by, 1.f, 0.f, sys + (by < 0.0 ? 1 : 0)};
+    const double phi = atan2(bz, by);
+    return FreqRow{(float)myz, (float)hypot(by, bz), (float)cos(0.5 * phi), (float)sin(0.5 * phi), sys};
+}
+
+// Factors of every distinct system, in FP64, stored in FP32.  G lanes per system; the
+// neighbours' blocks pass through shared memory (three M22 per lane).  The CTAs after the
+// last system's write the rows of the frequencies.
+__global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int steps, const double *__restrict__ Vx,
+                                                     float *__restrict__ table, FreqRow *__restrict__ freq) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    const int fb = (2 * class_count(g.n1, g.n2) + blockDim.x / G - 1) / (blockDim.x / G);
+    if ((int)blockIdx.x >= fb) {
+        const int f = (blockIdx.x - fb) * blockDim.x + threadIdx.x;
+        if (f < g.n1 * g.n2) freq[f] = freq_row(g, f);
+        return;
+    }
+    M22 *xi = reinterpret_cast<M22 *>(fsm), *xl = xi + blockDim.x, *xu = xl + blockDim.x;
+    const int l = threadIdx.x % G, base = threadIdx.x - l;
+    const int nsys = 2 * class_count(g.n1, g.n2);
+    const int sys = blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+    const bool live = sys < nsys;
+    const int cls = (live ? sys : 0) / 2, q2 = g.n2 / 2 + 1;
+    double myz, by, bz;
+    symbols(g, cls / q2, cls % q2, myz, by, bz);
+    const double P = ((sys & 1) ? -1.0 : 1.0) * hypot(by, bz);
+    const int n = g.nx, e = 2 * l, o = e + 1;
+    float *tab = table + (size_t)(live ? sys : 0) * items(steps) * G * 8;
+    const z2 one{1.0, 0.0}, nil{0.0, 0.0};
+    M22 L = zero22(), U = zero22(), D = M22{one, nil, nil, one}, Lo = zero22(), Uo = zero22(), Doi = zero22();
+    if (e < n) {
+        D = bd_block(g, Vx, e, 0, myz, P);
+        if (e > 0) L = bd_block(g, Vx, e, -1, myz, P);
+        if (o < n) {
+            U = bd_block(g, Vx, e, 1, myz, P);
+            Doi = inv(bd_block(g, Vx, o, 0, myz, P));
+            Lo = bd_block(g, Vx, o, -1, myz, P);
+            if (o + 1 < n) Uo = bd_block(g, Vx, o, 1, myz, P);
+        }
+    }
+    auto publish = [&](const M22 &a, const M22 &b, const M22 &c) {
+        __syncthreads();
+        xi[threadIdx.x] = a; xl[threadIdx.x] = b; xu[threadIdx.x] = c;
+        __syncthreads();
+    };
+    publish(Doi, Lo, Uo);
+    {
+        const int left = l > 0 ? threadIdx.x - 1 : threadIdx.x;       // l = 0: L = 0, any block will do
+        const M22 A = mul(L, xi[left]), Bm = mul(U, Doi);
+        D = sub(sub(D, mul(A, xu[left])), mul(Bm, Lo));
+        L = neg(mul(A, xl[left]));
+        U = neg(mul(Bm, Uo));
+        if (live) { put(tab, G, 0, l, A); put(tab, G, 1, l, Bm); }
+    }
+    for (int s = 0; s < steps; ++s) {
+        const int st = 1 << s;
+        publish(inv(D), L, U);
+        const bool hl = l >= st, hr = l + st < G;
+        const int il = hl ? threadIdx.x - st : base, ir = hr ? threadIdx.x + st : base;
+        const M22 al = hl ? mul(L, xi[il]) : zero22(), ga = hr ? mul(U, xi[ir]) : zero22();
+        D = sub(sub(D, mul(al, xu[il])), mul(ga, xl[ir]));
+        L = neg(mul(al, xl[il]));
+        U = neg(mul(ga, xu[ir]));
+        if (live) { put(tab, G, 2 + 2 * s, l, al); put(tab, G, 3 + 2 * s, l, ga); }
+    }
+    if (live) {
+        const int at = 2 + 2 * steps;
+        put(tab, G, at, l, inv(D));
+        put(tab, G, at + 1, l, Doi);
+        put(tab, G, at + 2, l, mul(Doi, Lo));
+        put(tab, G, at + 3, l, mul(Doi, Uo));
+    }
+}
+
+// hi + lo = 2 sum_t (-1)^t v_t per spatial entry (two complex entries per thread;
+// TwoSum keeps the rounding of every addition).
+__device__ __forceinline__ void two_add(float &hi, float &lo, float a) {
+    const float s = hi + a, bb = s - hi;
+    lo += (hi - (s - bb)) + (a - bb);
+    hi = s;
+}
+// s_{t+1} = 2 v_t - s_t
+__device__ __forceinline__ void next_s(float4 &s, float4 &lo, const float4 v) {
+    s = make_float4(-s.x, -s.y, -s.z, -s.w);
+    lo = make_float4(-lo.x, -lo.y, -lo.z, -lo.w);
+    two_add(s.x, lo.x, 2.f * v.x); two_add(s.y, lo.y, 2.f * v.y);
+    two_add(s.z, lo.z, 2.f * v.z); two_add(s.w, lo.w, 2.f * v.w);
+}
+__global__ void __launch_bounds__(256) altsum_kernel(int64_t per2, int64_t nt, const float4 *__restrict__ v,
+                                                     float4 *__restrict__ hi, float4 *__restrict__ lo) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= per2) return;
+    float4 h = make_float4(0.f, 0.f, 0.f, 0.f), r = h;
+    constexpr int PD = 8;
+    for (int64_t t0 = 0; t0 < nt; t0 += PD) {
+        float4 a[PD];
+#pragma unroll
+        for (int q = 0; q < PD; ++q)
+            a[q] = t0 + q < nt ? __ldg(v + (t0 + q) * per2 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < PD; ++q) {
+            const float w = (q & 1) ? -2.f : 2.f;
+            two_add(h.x, r.x, w * a[q].x); two_add(h.y, r.y, w * a[q].y);
+            two_add(h.z, r.z, w * a[q].z); two_add(h.w, r.w, w * a[q].w);
+        }
+    }
+    hi[e] = h;
+    lo[e] = r;
+}
+
+__device__ __forceinline__ float4 add4(const float4 a, const float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+struct Blk { float4 r0, r1; };            // a 2 x 2 complex block by rows
+__device__ __forceinline__ Blk load_blk(const float *tab, int G, int item, int lane) {
+    const float4 *o = reinterpret_cast<const float4 *>(tab + ((size_t)item * G + lane) * 8);
+    return Blk{__ldg(o), __ldg(o + 1)};
+}
+// acc += B v, or acc -= B v; v = (v0.re, v0.im, v1.re, v1.im)
+__device__ __forceinline__ void add_mv(float4 &acc, const Blk &B, const float4 v) {
+    acc.x = fmaf(B.r0.x, v.x, fmaf(-B.r0.y, v.y, fmaf(B.r0.z, v.z, fmaf(-B.r0.w, v.w, acc.x))));
+    acc.y = fmaf(B.r0.x, v.y, fmaf(B.r0.y, v.x, fmaf(B.r0.z, v.w, fmaf(B.r0.w, v.z, acc.y))));
+    acc.z = fmaf(B.r1.x, v.x, fmaf(-B.r1.y, v.y, fmaf(B.r1.z, v.z, fmaf(-B.r1.w, v.w, acc.z))));
+    acc.w = fmaf(B.r1.x, v.y, fmaf(B.r1.y, v.x, fmaf(B.r1.z, v.w, fmaf(B.r1.w, v.z, acc.w))));
+}
+__device__ __forceinline__ void sub_mv(float4 &acc, const Blk &B, const float4 v) {
+    acc.x = fmaf(-B.r0.x, v.x, fmaf(B.r0.y, v.y, fmaf(-B.r0.z, v.z, fmaf(B.r0.w, v.w, acc.x))));
+    acc.y = fmaf(-B.r0.x, v.y, fmaf(-B.r0.y, v.x, fmaf(-B.r0.z, v.w, fmaf(-B.r0.w, v.z, acc.y))));
+    acc.z = fmaf(-B.r1.x, v.x, fmaf(B.r1.y, v.y, fmaf(-B.r1.z, v.z, fmaf(B.r1.w, v.w, acc.z))));
+    acc.w = fmaf(-B.r1.x, v.y, fmaf(-B.r1.y, v.x, fmaf(-B.r1.z, v.w, fmaf(-B.r1.w, v.z, acc.w))));
+}
+
+__device__ __forceinline__ void copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// Shared memory of one CTA of `sys` systems: STAGES input layers, two output layers,
+// two exchange buffers.
+__host__ __device__ inline int row_bytes(int nc, int sys) { return (nc == 4 ? sys / 2 : sys) * nc * 8 + 16; }
+inline size_t march_smem(int nc, int sys, int G, int n) {
+    return (size_t)(STAGES + 2) * ((n + 1) / 2 * 2) * row_bytes(nc, sys) + 2 * sizeof(float4) * (size_t)sys * G;
+}
+
+// LARGE: time steps above half the x spacing.  The reduction then loses digits (K outweighs
+// M: at h_t = 7.5 h an FP32 reduction was ten times further off than the elimination in
+// order), so each solve is refined once, on the form Bd x_t = s_t - Bl x_{t-1}.  Below, the
+// increment form alone is as exact as that elimination or better (relative error against
+// FP64 9.3e-7, was 1.5e-6, on the 48^3 x 48 Klein mesh).
+// blockDim.x = systems per CTA x G.  Layers t of `in` [t][x][f][c] to `out` (in == out allowed).
+template <int NC, int G, bool LARGE>
+__global__ void __launch_bounds__(G > 32 ? 512 : 256)
+march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float *__restrict__ table,
+             const FreqRow *__restrict__ ft, const float4 *__restrict__ alt_hi, const float4 *__restrict__ alt_lo, const float2 *in, float2 *out) {
+    extern __shared__ __align__(16) unsigned char msm[];
+    constexpr bool REG = G <= 32;
+    const int n = g.nx, half = (n + 1) / 2, rows = 2 * half;
+    const int64_t nf = (int64_t)g.n1 * g.n2;
+    const int nsys = blockDim.x / G, fper = NC == 4 ? nsys / 2 : nsys;
+    const int RB = row_bytes(NC, nsys);
+    unsigned char *ring = msm, *otile = ring + (size_t)STAGES * rows * RB;
+    float4 *xch = reinterpret_cast<float4 *>(otile + (size_t)2 * rows * RB);
+    const int l = threadIdx.x % G, sys = threadIdx.x / G;
+    const int slot = NC == 4 ? sys / 2 : sys, pair = NC == 4 ? sys & 1 : 0;
+    const int64_t f0 = (int64_t)blockIdx.x * fper, f = f0 + slot;
+    const FreqRow fq = ft[f < nf ? f : 0];
+    const float *tab = table + (size_t)(fq.sys + pair) * items(steps) * G * 8;
+    // rows past the last frequency stay zero
+    for (int i = threadIdx.x; i < (STAGES + 2) * rows * RB / 16; i += blockDim.x)
+        reinterpret_cast<float4 *>(ring)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    // a row of the ring: the CTA's frequencies of one x node, even nodes first, so that
+    // the lanes of a warp read consecutive rows
+    const int per_row = fper * NC / 2, cl = __ffs(per_row) - 1;
+    const int valid = (int)min((int64_t)per_row, (nf - f0) * (NC / 2));
+    auto pos = [&](int i) { return (i & 1) * half + (i >> 1); };
+    auto issue = [&](int64_t t) {
+        if (t < g.nt) {
+            unsigned char *dst = ring + (size_t)(t % STAGES) * rows * RB;
+            const char *src = reinterpret_cast<const char *>(in + ((t * n) * nf + f0) * NC);
+            for (int k = threadIdx.x; k < n << cl; k += blockDim.x) {
+                const int i = k >> cl, ch = k & (per_row - 1);
+                if (ch < valid) copy16(dst + pos(i) * RB + ch * 16, src + (int64_t)i * nf * NC * 8 + ch * 16);
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    // the rotated pair of one node from its two (2+1) or four (3+1) components
+    const float rc = fq.c, rs = fq.s;
+    auto rotate = [&](const float4 a, const float4 b) {       // a = (v0, v1), b = (v2, v3)
+        if (pair == 0) return make_float4(rc * a.x - rs * a.w, rc * a.y + rs * a.z, rc * b.z - rs * b.y, rc * b.w + rs * b.x);
+        return make_float4(rc * a.z - rs * a.y, rc * a.w + rs * a.x, rc * b.x - rs * b.w, rc * b.y + rs * b.z);
+    };
+    auto node = [&](const unsigned char *tile, int i) {
+        const float4 *q = reinterpret_cast<const float4 *>(tile + pos(i) * RB + slot * NC * 8);
+        return NC == 4 ? rotate(q[0], q[1]) : q[0];
+    };
+    auto alt = [&](const float4 *v, int i) {
+        if (i >= n || f >= nf) return make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 *q = v + (i * nf + f) * (NC / 2);
+        return NC == 4 ? rotate(q[0], q[1]) : q[0];
+    };
+    const int e = 2 * l, o = e + 1;
+    const bool he = e < n, ho = o < n;
+    // K' = h_t K (LARGE: h_t / 2 K) of a node between elements of potential a and b, its neighbours p and r:
+    // component 0 takes i kC (r - p)_1 + i kP (p + 4 c + r)_1 - sum over both elements of
+    // (V + m) kW (neighbour + 2 c)_0, component 1 the same with kP and m negated
+    const double hk = LARGE ? 0.5 * g.ht : g.ht;
+    const float kC = (float)(0.5 * hk) * fq.myz, kW = (float)(hk * g.h[0] / 6.0) * fq.myz;
+    const float kP = (float)(hk * g.h[0] / 6.0) * (pair ? -fq.P : fq.P), km = kW * (float)g.m;
+    const float kM = LARGE ? (float)(g.h[0] / 6.0) * fq.myz : 0.f;
+    float ve[3];                                              // elements e, e + 1, e + 2
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ve[k] = Vx && e + k <= n ? kW * (float)Vx[e + k] : 0.f;
+    Blk A = load_blk(tab, G, 0, l), Bm = load_blk(tab, G, 1, l);
+    Blk al[REG ? REG_STEPS : 1], ga[REG ? REG_STEPS : 1];
+    constexpr int LOGG = G == 8 ? 3 : (G == 16 ? 4 : 5);
+    if (REG) {
+#pragma unroll
+        for (int s = 0; s < LOGG; ++s)
+            if (s < steps) { al[s] = load_blk(tab, G, 2 + 2 * s, l); ga[s] = load_blk(tab, G, 3 + 2 * s, l); }
+    }
+    const int at = 2 + 2 * steps;
+    Blk Di = load_blk(tab, G, at, l), Oi = load_blk(tab, G, at + 1, l), OL = load_blk(tab, G, at + 2, l),
+        OU = load_blk(tab, G, at + 3, l);
+    float4 se = alt(alt_hi, e), so = alt(alt_hi, o), sel = alt(alt_lo, e), sol = alt(alt_lo, o);
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 xe = z4, xo = z4, xn = z4;                          // x_{t-1} at e, o and e + 2
+    int buf = 0;
+    float4 *mine = xch + threadIdx.x;
+    auto sync = [&] { if (G <= 32) __syncwarp(); else __syncthreads(); };
+    auto swap_buf = [&] { buf ^= (int)blockDim.x; };
+    const int left = l > 0 ? -1 : 0, right = l + 1 < G ? 1 : 0;
+    for (int q = 0; q < STAGES - 1; ++q) issue(q);
+
+    // s - K' x + i kM M' x of a node between elements of potential va and vb (M' the [1,4,1]
+    // sum), x at the node and its neighbours p and r
+    auto rhs = [&](const float4 s, const float4 slo, const float4 c, const float4 p, const float4 r, float va, float vb,
+                   float kM) {
+        const float4 S = make_float4(fmaf(4.f, c.x, p.x + r.x), fmaf(4.f, c.y, p.y + r.y), fmaf(4.f, c.z, p.z + r.z),
+                                     fmaf(4.f, c.w, p.w + r.w));
+        const float4 E = make_float4(r.x - p.x, r.y - p.y, r.z - p.z, r.w - p.w);
+        const float4 a = make_float4(fmaf(2.f, c.x, p.x), fmaf(2.f, c.y, p.y), fmaf(2.f, c.z, p.z), fmaf(2.f, c.w, p.w));
+        const float4 b = make_float4(fmaf(2.f, c.x, r.x), fmaf(2.f, c.y, r.y), fmaf(2.f, c.z, r.z), fmaf(2.f, c.w, r.w));
+        const float pa = va + km, pb = vb + km, ma = va - km, mb = vb - km;
+        float4 q = make_float4(s.x + fmaf(kC, E.w, fmaf(kP, S.w, fmaf(pa, a.x, fmaf(pb, b.x, slo.x)))),
+                               s.y + fmaf(-kC, E.z, fmaf(-kP, S.z, fmaf(pa, a.y, fmaf(pb, b.y, slo.y)))),
+                               s.z + fmaf(kC, E.y, fmaf(-kP, S.y, fmaf(ma, a.z, fmaf(mb, b.z, slo.z)))),
+                               s.w + fmaf(-kC, E.x, fmaf(kP, S.x, fmaf(ma, a.w, fmaf(mb, b.w, slo.w)))));
+        if (LARGE) {
+            q.x = fmaf(-kM, S.y, q.x); q.y = fmaf(kM, S.x, q.y); q.z = fmaf(-kM, S.w, q.z); q.w = fmaf(kM, S.z, q.w);
+        }
+        return q;
+    };
+    auto from_left = [&](const float4 v) {                     // the left lane's v (0 at the wall)
+        mine[buf] = v;
+        sync();
+        const float4 w = l > 0 ? mine[buf + left] : z4;
+        swap_buf();
+        return w;
+    };
+    // Bd u = r; un: u at e + 2
+    auto solve = [&](float4 re, const float4 ro, float4 &ue, float4 &uo, float4 &un) {
+        mine[buf] = ro;
+        sync();
+        sub_mv(re, A, mine[buf + left]);
+        sub_mv(re, Bm, ro);
+        swap_buf();
+        auto reduce = [&](int st, const Blk &a, const Blk &b) {
+            mine[buf] = re;
+            sync();
+            const float4 vl = mine[buf + (l >= st ? -st : 0)], vr = mine[buf + (l + st < G ? st : 0)];
+            sub_mv(re, a, vl);
+            sub_mv(re, b, vr);
+            swap_buf();
+        };
+        if (REG) {
+#pragma unroll
+            for (int s = 0; s < LOGG; ++s)
+                if (s < steps) reduce(1 << s, al[s], ga[s]);
+        } else {
+            for (int s = 0; s < steps; ++s) reduce(1 << s, load_blk(tab, G, 2 + 2 * s, l), load_blk(tab, G, 3 + 2 * s, l));
+        }
+        ue = uo = z4;
+        add_mv(ue, Di, re);
+        mine[buf] = ue;
+        sync();
+        un = l + 1 < G ? mine[buf + right] : z4;
+        swap_buf();
+        add_mv(uo, Oi, ro);
+        sub_mv(uo, OL, ue);
+        sub_mv(uo, OU, un);
+    };
+    auto store_layer = [&](int64_t t) {                        // out tile t & 1, rotated back
+        const unsigned char *tile = otile + (size_t)(t & 1) * rows * RB;
+        char *dst = reinterpret_cast<char *>(out + ((t * n) * nf + f0) * NC);
+        for (int k = threadIdx.x; k < n << cl; k += blockDim.x) {
+            const int i = k >> cl, ch = k & (per_row - 1);
+            if (ch >= valid) continue;
+            float4 v = *reinterpret_cast<const float4 *>(tile + pos(i) * RB + ch * 16);
+            if (NC == 4) {
+                const float c = ft[f0 + (ch >> 1)].c, s = ft[f0 + (ch >> 1)].s;
+                v = make_float4(c * v.x + s * v.w, c * v.y - s * v.z, c * v.z + s * v.y, c * v.w - s * v.x);
+            }
+            *reinterpret_cast<float4 *>(dst + (int64_t)i * nf * NC * 8 + ch * 16) = v;
+        }
+    };
+    for (int64_t t = 0; t < g.nt; ++t) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(STAGES - 2) : "memory");
+        __syncthreads();               // layer t staged; layer t - 1 of the output complete; its input slot free
+        issue(t + STAGES - 1);
+        if (t > 0) store_layer(t - 1);
+        // the neighbour's x_{t-1} at o - 2; the odd node needs none beyond e and e + 2
+        float4 re = rhs(se, sel, xe, from_left(xo), xo, ve[0], ve[1], kM);
+        float4 ro = rhs(so, sol, xo, xe, xn, ve[1], ve[2], kM);
+        if (!he) re = z4;
+        if (!ho) ro = z4;
+        float4 ue, uo, un;
+        solve(re, ro, ue, uo, un);
+        if (LARGE) {
+            // one step of refinement: u += Bd^-1 (r - Bd u)
+            re = rhs(re, z4, ue, from_left(uo), uo, ve[0], ve[1], -kM);
+            ro = rhs(ro, z4, uo, ue, un, ve[1], ve[2], -kM);
+            if (!he) re = z4;
+            if (!ho) ro = z4;
+            float4 de, dd, dn;
+            solve(re, ro, de, dd, dn);
+            xe = add4(ue, de); xo = add4(uo, dd); xn = add4(un, dn);
+        } else {
+            xe = add4(ue, xe); xo = add4(uo, xo); xn = add4(un, xn);
+        }
+        unsigned char *ot = otile + (size_t)(t & 1) * rows * RB + slot * NC * 8;
+        auto emit = [&](int i, const float4 x) {
+            unsigned char *d = ot + pos(i) * RB;
+            if (NC == 4) {
+                *reinterpret_cast<float2 *>(d + (pair ? 8 : 0)) = make_float2(x.x, x.y);
+                *reinterpret_cast<float2 *>(d + (pair ? 16 : 24)) = make_float2(x.z, x.w);
+            } else {
+                *reinterpret_cast<float4 *>(d) = x;
+            }
+        };
+        const unsigned char *it = ring + (size_t)(t % STAGES) * rows * RB;
+        if (he) { emit(e, xe); next_s(se, sel, node(it, e)); }
+        if (ho) { emit(o, xo); next_s(so, sol, node(it, o)); }
+    }
+    __syncthreads();
+    store_layer(g.nt - 1);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+}
+
+}  // namespace dst_march
