@@ -41,137 +41,42 @@ enum { E1A, E1B, E2A, E2B, E3A, E3B, U2P, U2C, U1P, U1C, OUT };
 
 struct Layer {
     int ci, co, taps, level;
-    int kpad, co8;          // K padded to 16, output rows padded to 8
+    int kpad;               // K padded to 16
     int64_t woff, boff;     // offsets of weight and bias in the flat parameter vector
 };
 
-__global__ void pool_fwd_kernel(UGrid f, UGrid c, int ch, const float *__restrict__ in, float *__restrict__ out) {
+// Weights of every layer in fragment order (unet_kernels.cuh): wf for the forward pass, B[k][n] =
+// W[n][c][tap] with k = tap * ci + c, and wt for the input gradient, the mirrored
+// transpose B[k][n] = W[o][n][taps - 1 - tap] with k = tap * co + o.  The pair at
+// [chunk][ntile][lane][h] holds k = 16 chunk + 8 h + 2 (lane % 4) and the next, n = 8 ntile + lane / 4.
+struct PackLayer {
+    int ci, co, taps;
+    int nf, nt;                     // n tiles of wf and wt
+    int64_t woff, first, count_f, count_t;   // weight offset; first pair of the layer; pairs of wf, wt
+    uint32_t *wf, *wt;
+};
+struct PackLayers { PackLayer l[NLAYER]; int64_t total; };
+__global__ void pack_weights_kernel(PackLayers P, const float *__restrict__ p) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= c.N * ch) return;
-    const int k = (int)(i % ch);
-    int64_t q = i / ch;
-    int cc[4];
-    coords(c, q, cc);
-    float s = 0.f;
-    const int nb = 1 << f.D;
-    for (int m = 0; m < nb; ++m) {
-        int64_t r = 0;
-        bool ok = true;
-        for (int a = 0; a < f.D; ++a) {
-            const int x = 2 * cc[a] + ((m >> (f.D - 1 - a)) & 1);
-            if (x >= f.n[a]) { ok = false; break; }
-            r = r * f.n[a] + x;
-        }
-        if (ok) s += in[r * ch + k];
+    if (i >= P.total) return;
+    int l = 0;
+    while (l + 1 < NLAYER && i >= P.l[l + 1].first) ++l;
+    const PackLayer &L = P.l[l];
+    int64_t at = i - L.first;
+    const bool back = at >= L.count_f;
+    if (back) at -= L.count_f;
+    const int h = (int)(at & 1), lane = (int)((at >> 1) & 31), nt = back ? L.nt : L.nf;
+    const int tile = (int)((at >> 6) % nt), chunk = (int)((at >> 6) / nt);
+    const int n = tile * 8 + (lane >> 2), in = back ? L.co : L.ci, outs = back ? L.ci : L.co;
+    float v[2];
+    for (int e = 0; e < 2; ++e) {
+        const int k = chunk * 16 + 8 * h + 2 * (lane & 3) + e, tap = k / in, c = k % in;
+        v[e] = 0.f;
+        if (n < outs && tap < L.taps)
+            v[e] = back ? p[L.woff + ((int64_t)c * L.ci + n) * L.taps + (L.taps - 1 - tap)]
+                        : p[L.woff + ((int64_t)n * L.ci + c) * L.taps + tap];
     }
-    out[i] = s / (float)nb;
-}
-
-// d_fine[p] += d_coarse[p / 2] / 2^D
-__global__ void pool_bwd_kernel(UGrid f, UGrid c, int ch, const float *__restrict__ dc, float *__restrict__ df) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= f.N * ch) return;
-    const int k = (int)(i % ch);
-    int cf[4];
-    coords(f, i / ch, cf);
-    int64_t q = 0;
-    for (int a = 0; a < f.D; ++a) q = q * c.n[a] + cf[a] / 2;
-    df[i] += dc[q * ch + k] / (float)(1 << f.D);
-}
-
-// fine[p] = coarse[p / 2]
-__global__ void up_fwd_kernel(UGrid f, UGrid c, int ch, const float *__restrict__ in, float *__restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= f.N * ch) return;
-    const int k = (int)(i % ch);
-    int cf[4];
-    coords(f, i / ch, cf);
-    int64_t q = 0;
-    for (int a = 0; a < f.D; ++a) q = q * c.n[a] + cf[a] / 2;
-    out[i] = in[q * ch + k];
-}
-
-// d_coarse[q] = sum of d_fine over the cells p with p / 2 = q
-__global__ void up_bwd_kernel(UGrid f, UGrid c, int ch, const float *__restrict__ df, float *__restrict__ dc) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= c.N * ch) return;
-    const int k = (int)(i % ch);
-    int cc[4];
-    coords(c, i / ch, cc);
-    float s = 0.f;
-    for (int m = 0; m < (1 << f.D); ++m) {
-        int64_t r = 0;
-        bool ok = true;
-        for (int a = 0; a < f.D; ++a) {
-            const int x = 2 * cc[a] + ((m >> (f.D - 1 - a)) & 1);
-            if (x >= f.n[a]) { ok = false; break; }
-            r = r * f.n[a] + x;
-        }
-        if (ok) s += df[r * ch + k];
-    }
-    dc[i] = s;
-}
-
-// dz = d * (y > 0)
-__global__ void relu_mask_kernel(int64_t n, const float *__restrict__ d, const float *__restrict__ y,
-                                 float *__restrict__ dz) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) dz[i] = y[i] > 0.f ? d[i] : 0.f;
-}
-
-// db[co] += sum_n dz[n][co] (one CTA per channel, fixed order)
-__global__ void bias_grad_kernel(int64_t N, int co, const float *__restrict__ dz, float *__restrict__ db) {
-    __shared__ float red[256];
-    const int c = blockIdx.x;
-    float s = 0.f;
-    for (int64_t n = threadIdx.x; n < N; n += blockDim.x) s += dz[n * co + c];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) db[c] += red[0];
-}
-
-// internal weights: wf[co8][kpad] bf16 (k = tap * ci + c) and the mirrored transpose
-// wt[ci8][kpadT] (k' = tap' * co + o, tap' = taps - 1 - tap) for the input gradient
-__global__ void pack_weights_kernel(Layer L, const float *__restrict__ p, __nv_bfloat16 *__restrict__ wf,
-                                    __nv_bfloat16 *__restrict__ wt, int kpadT) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t nf = (int64_t)L.co8 * L.kpad;
-    if (i < nf) {
-        const int o = (int)(i / L.kpad), k = (int)(i % L.kpad);
-        float v = 0.f;
-        if (o < L.co && k < L.taps * L.ci) {
-            const int tap = k / L.ci, c = k % L.ci;
-            v = p[L.woff + ((int64_t)o * L.ci + c) * L.taps + tap];
-        }
-        wf[i] = __float2bfloat16_rn(v);
-    }
-    if (wt) {
-        const int ci8 = (L.ci + 7) / 8 * 8;
-        if (i < (int64_t)ci8 * kpadT) {
-            const int c = (int)(i / kpadT), k = (int)(i % kpadT);
-            float v = 0.f;
-            if (c < L.ci && k < L.taps * L.co) {
-                const int tapT = k / L.co, o = k % L.co;
-                v = p[L.woff + ((int64_t)o * L.ci + c) * L.taps + (L.taps - 1 - tapT)];
-            }
-            wt[i] = __float2bfloat16_rn(v);
-        }
-    }
-}
-
-// flat gradient (parameter layout) from the internal dW[co][kpad]
-__global__ void unpack_wgrad_kernel(Layer L, const float *__restrict__ dw, float *__restrict__ g) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t n = (int64_t)L.co * L.ci * L.taps;
-    if (i >= n) return;
-    const int tap = (int)(i % L.taps);
-    const int c = (int)((i / L.taps) % L.ci);
-    const int o = (int)(i / ((int64_t)L.taps * L.ci));
-    g[L.woff + i] = dw[(size_t)o * L.kpad + tap * L.ci + c];
+    (back ? L.wt : L.wf)[at] = pack_bf16(v[0], v[1]);
 }
 
 __global__ void adam_kernel(int64_t n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
@@ -185,52 +90,81 @@ __global__ void adam_kernel(int64_t n, float *__restrict__ p, const float *__res
     p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-// sum of squares of a float array into *out (FP64 accumulation, one CTA)
-__global__ void sumsq_kernel(int64_t n, const float *__restrict__ a, double *__restrict__ out) {
+// Sums of squares of one or two float arrays (blockIdx.y), one FP64 partial per CTA.
+constexpr int SUM_CTAS = 152;
+__global__ void __launch_bounds__(256) sumsq_kernel(int64_t n, const float *__restrict__ a, const float *__restrict__ b,
+                                                    double *__restrict__ part) {
     __shared__ double red[256];
+    const float *v = blockIdx.y ? b : a;
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)a[i] * a[i];
+    for (int64_t i = blockIdx.x * 256LL + threadIdx.x; i < n; i += 256LL * gridDim.x) s += (double)v[i] * v[i];
     red[threadIdx.x] = s;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+    for (int w = 128; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = red[0];
+    if (threadIdx.x == 0) part[blockIdx.y * SUM_CTAS + blockIdx.x] = red[0];
 }
 
-// the norm s = sqrt(sum of squares) as a float scalar (the input scale of the network)
-__global__ void sqrt_scalar_kernel(const double *__restrict__ ss, float *__restrict__ s) {
-    if (threadIdx.x == 0) *s = (float)sqrt(*ss);
+// The sum of a sumsq_kernel's partials, the same in every CTA (one warp, fixed order).
+__device__ __forceinline__ double total_of(const double *part, int count) {
+    __shared__ double total;
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        for (int i = threadIdx.x; i < count; i += 32) s += part[i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) total = s;
+    }
+    __syncthreads();
+    const double t = total;
+    __syncthreads();
+    return t;
 }
 
-// loss = ||y - t / s||^2 / ||t / s||^2 into *loss, dy = 2 (y - t / s) / ||t / s||^2
-__global__ void loss_kernel(int64_t n, const float *__restrict__ y, const float *__restrict__ t,
-                            const float *__restrict__ s, const double *__restrict__ tt, float *__restrict__ dy,
-                            double *__restrict__ loss) {
+// The input scale s = ||x|| (a float scalar), and x / s in BF16 (n is even).
+__global__ void __launch_bounds__(256) scale_input_kernel(int64_t n, int parts, const double *__restrict__ part,
+                                                          const float2 *__restrict__ x, float *__restrict__ scale,
+                                                          uint32_t *__restrict__ out) {
+    const float s = (float)sqrt(total_of(part, parts)), inv = 1.0f / s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *scale = s;
+    for (int64_t i = blockIdx.x * 256LL + threadIdx.x; i < n / 2; i += 256LL * gridDim.x) {
+        const float2 v = x[i];
+        out[i] = pack_bf16(v.x * inv, v.y * inv);
+    }
+}
+
+// dy = 2 (y - t / s) / ||t / s||^2 in BF16 with the column sums of its CTAs, and the
+// CTAs' shares of ||y - t / s||^2; lq: log2 of the channels / 4.
+__global__ void __launch_bounds__(256) loss_kernel(int64_t n4, int lq, int parts, const double *__restrict__ tpart,
+                                                   const float4 *__restrict__ y, const float4 *__restrict__ t,
+                                                   const float *__restrict__ s, uint2 *__restrict__ dy,
+                                                   double *__restrict__ lpart, float *__restrict__ colsum) {
     __shared__ double red[256];
     const float inv = 1.0f / *s;
-    const double tn = *tt * (double)inv * inv;
+    const double tn = total_of(tpart, parts) * (double)inv * inv, w = 2.0 / tn;
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const float r = y[i] - t[i] * inv;
-        acc += (double)r * r;
-        dy[i] = (float)(2.0 * r / tn);
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t i = blockIdx.x * 256LL + threadIdx.x; i < n4; i += 256LL * gridDim.x) {
+        const float4 a = y[i], b = t[i];
+        const float4 r = make_float4(a.x - b.x * inv, a.y - b.y * inv, a.z - b.z * inv, a.w - b.w * inv);
+        acc += ((double)r.x * r.x + (double)r.y * r.y) + ((double)r.z * r.z + (double)r.w * r.w);
+        const float4 d = make_float4((float)(w * r.x), (float)(w * r.y), (float)(w * r.z), (float)(w * r.w));
+        dy[i] = pack_bf16x4(d);
+        sum.x += d.x; sum.y += d.y; sum.z += d.z; sum.w += d.w;
     }
     red[threadIdx.x] = acc;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    for (int k = 128; k > 0; k >>= 1) {
+        if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *loss = red[0] / tn;
+    if (threadIdx.x == 0) lpart[blockIdx.x] = red[0] / tn;
+    cta_colsum(sum, lq, colsum);
 }
-
-// z += g s y (the network's output scaled back; y [N][C] is the same floats as a complex vector)
-__global__ void axpy_scaled_kernel(int64_t n, const float *__restrict__ s, const float *__restrict__ g,
-                                   const float *__restrict__ y, float *__restrict__ z) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) z[i] += *g * *s * y[i];
+__global__ void loss_sum_kernel(int parts, const double *__restrict__ lpart, double *__restrict__ loss) {
+    const double t = total_of(lpart, parts);
+    if (threadIdx.x == 0) *loss = t;
 }
 
 // <y, t / s> and ||y||^2 accumulated into acc[0], acc[1] (one CTA, FP64)
@@ -256,7 +190,6 @@ __global__ void dot_kernel(int64_t n, const float *__restrict__ y, const float *
 // Partial sums of <a, r> = sum conj(a_i) r_i (re, im) and ||a||^2 over complex
 // vectors, one triple per CTA (FP64), for the least-squares scale of the correction.
 constexpr int LS_PARTS = 304;
-constexpr int WGRAD_SPLITS = 64;                 // node ranges of the weight-gradient GEMM
 __global__ void __launch_bounds__(256) ls_partials_kernel(int64_t n, const float2 *__restrict__ a,
                                                           const float2 *__restrict__ r, double *__restrict__ part) {
     __shared__ double red[3][256];
@@ -328,19 +261,20 @@ struct dst_unet {
     Layer L[NLAYER];
     int64_t nparams;
     float *params, *grads, *adam_m, *adam_v;     // FP32 [nparams]
-    __nv_bfloat16 *wf[NLAYER], *wt[NLAYER];
-    int kpadT[NLAYER];
-    float *dw;                                   // largest co x kpad
-    float *dw_part;                              // WGRAD_SPLITS partials of dw
-    // activations [N][ch] and their gradients
-    float *x0, *a1, *s1, *p1, *a2, *s2, *p2, *a3, *h3, *u2, *q2, *r2, *u1, *q1, *r1, *y;
-    float *g_big1, *g_big2, *g_big3, *gs1, *gs2, *g_mid;   // gradient scratch
+    PackLayers pack;                             // weight fragments
+    GradLayers sums;                             // partial sums of the weight and bias gradients
+    float *wpart, *bpart;
+    // activations [N][ch]: BF16 where only a convolution (or a ReLU mask) reads them
+    bf16 *x0, *a1, *p1, *a2, *p2, *a3, *h3, *q2, *r2, *q1, *r1;
+    float *s1, *s2, *y;
+    bf16 *z1, *z2;                               // gradients that a convolution reads (the widest layer each)
+    float *gs1, *gs2, *gup;                      // gradients of s1, s2, and before an adjoint
     float *scale;                                          // device scalar s
     float *gamma;                                          // device scalar: output scale of the correction
     double gamma_host;
-    double *dscr;                                          // device doubles: [0] sum sq, [1] loss, [2] target sumsq
+    double *dscr;                                          // device doubles: [1] loss, [2], [3] sums over fresh pairs
+    double *spart;                                         // partial sums of squares and of the loss (3 x SUM_CTAS)
     double *part;                                          // LS_PARTS x 3 partial sums of the correction's scale
-    int64_t act_floats;
     void *mem;
     size_t mem_bytes;
     bool packed;
@@ -357,6 +291,31 @@ static UGrid coarse(const UGrid &f) {
     for (int a = f.D; a < 4; ++a) c.n[a] = 1;
     return c;
 }
+
+// ---- launch shapes ----------------------------------------------------------
+
+// Weight gradients, kernel 3: segments of an x line (up to 64 nodes), and slices so that
+// the CTAs (three or nine warps each) fill the GPU twice while the slices stay within a
+// few million partial sums; kernel 1: 32 nodes at a time, one slice per warp.
+static int wgrad_seg(const UGrid &g) {
+    const int nx = g.n[g.D - 1], segs = (nx + 63) / 64;
+    return (nx + segs - 1) / segs;
+}
+static int wgrad_items(const Layer &L, const UGrid &g) {
+    if (L.taps == 1) return (int)((g.N + 31) / 32);
+    const int nx = g.n[g.D - 1];
+    return (int)(g.N / nx * ((nx + wgrad_seg(g) - 1) / wgrad_seg(g)));
+}
+static int wgrad_slices(const Layer &L, const UGrid &g) {
+    const int items = wgrad_items(L, g);
+    const int64_t dw = (int64_t)L.co * L.kpad, most = std::max<int64_t>(1, (2 << 20) / dw);
+    if (L.taps == 1) return (int)std::min<int64_t>((items + 3) / 4 * 4, 4 * std::min<int64_t>(152, std::max<int64_t>(1, most / 4)));
+    return (int)std::min<int64_t>(items, std::min<int64_t>(std::max(1, 304 * 16 / L.co), most));
+}
+// Rows of column sums a layer's bias gradient may take (one per CTA that produces its dz).
+static int64_t colsum_rows(const UGrid &g) { return std::max<int64_t>((g.N + 16 * CONV_WARPS - 1) / (16 * CONV_WARPS), SUM_CTAS); }
+// CTAs of an element-wise kernel with column sums
+static unsigned sum_ctas(int64_t quads) { return (unsigned)std::min<int64_t>(SUM_CTAS, (quads + 255) / 256); }
 
 static int unet_create(const dst_mesh *mesh, dst_unet **out) {
     dst_unet *u = new (std::nothrow) dst_unet();
@@ -387,40 +346,52 @@ static int unet_create(const dst_mesh *mesh, dst_unet **out) {
         L.taps = spec[l][2] == 3 ? taps3 : 1;
         L.level = spec[l][3];
         L.kpad = (L.taps * L.ci + 15) / 16 * 16;
-        L.co8 = (L.co + 7) / 8 * 8;
         L.woff = off;
         off += (int64_t)L.co * L.ci * L.taps;
         L.boff = off;
         off += L.co;
-        u->kpadT[l] = (L.taps * L.co + 15) / 16 * 16;
     }
     u->nparams = off;
     // one device allocation for everything
     const int64_t N1 = g1.N, N2 = u->grid[1].N, N3 = u->grid[2].N;
-    std::vector<size_t> sizes;
-    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     size_t total = 0;
-    auto take = [&](size_t b) { size_t o = total; total += al(b); return o; };
+    auto take = [&](size_t b) { size_t o = total; total += (b + 255) & ~(size_t)255; return o; };
     const size_t o_par = take(4 * sizeof(float) * u->nparams);
     size_t o_wf[NLAYER], o_wt[NLAYER];
-    size_t maxdw = 0;
+    int64_t pairs = 0, wfloats = 0, bfloats = 0, cells = 0;
     for (int l = 0; l < NLAYER; ++l) {
         const Layer &L = u->L[l];
-        o_wf[l] = take(sizeof(__nv_bfloat16) * (size_t)L.co8 * L.kpad);
-        o_wt[l] = take(sizeof(__nv_bfloat16) * (size_t)((L.ci + 7) / 8 * 8) * u->kpadT[l]);
-        maxdw = std::max(maxdw, (size_t)L.co * L.kpad);
+        PackLayer &P = u->pack.l[l];
+        P.ci = L.ci; P.co = L.co; P.taps = L.taps; P.woff = L.woff;
+        P.nf = (L.co + 7) / 8; P.nt = (L.ci + 7) / 8;
+        P.count_f = (int64_t)(L.kpad / 16) * P.nf * 64;
+        P.count_t = l == E1A ? 0 : (int64_t)((L.taps * L.co + 15) / 16) * P.nt * 64;
+        P.first = pairs;
+        pairs += P.count_f + P.count_t;
+        o_wf[l] = take(sizeof(uint32_t) * P.count_f);
+        o_wt[l] = take(sizeof(uint32_t) * P.count_t);
+        GradLayer &G = u->sums.l[l];
+        G.co = L.co; G.ci = L.ci; G.taps = L.taps; G.kpad = L.kpad; G.woff = L.woff; G.boff = L.boff;
+        G.slices = wgrad_slices(L, u->grid[L.level]);
+        G.wpart = wfloats; G.bpart = bfloats; G.first = cells;
+        wfloats += (int64_t)G.slices * L.co * L.kpad;
+        bfloats += colsum_rows(u->grid[L.level]) * L.co;
+        cells += (int64_t)L.co * L.kpad;
     }
-    const size_t o_dw = take(sizeof(float) * maxdw);
-    const size_t o_dwp = take(sizeof(float) * maxdw * WGRAD_SPLITS);
-    const int64_t acts[] = {N1 * u->C, N1 * 16, N1 * 16, N2 * 16, N2 * 32, N2 * 32, N3 * 32, N3 * 64, N3 * 64,
-                            N2 * 64, N2 * 32, N2 * 32, N1 * 32, N1 * 16, N1 * 16, N1 * u->C};
-    size_t o_act[16];
-    for (int k = 0; k < 16; ++k) o_act[k] = take(sizeof(float) * acts[k]);
-    const int64_t big = std::max(std::max(N1 * 32, N2 * 64), N3 * 64);
-    const size_t o_g1 = take(sizeof(float) * big), o_g2 = take(sizeof(float) * big), o_g3 = take(sizeof(float) * big);
-    const size_t o_gs1 = take(sizeof(float) * N1 * 16), o_gs2 = take(sizeof(float) * N2 * 32);
-    const size_t o_gm = take(sizeof(float) * big);
+    u->pack.total = pairs;
+    u->sums.n = NLAYER;
+    u->sums.total = cells;
+    const size_t o_wp = take(sizeof(float) * wfloats), o_bp = take(sizeof(float) * bfloats);
+    const int64_t half[] = {N1 * u->C, N1 * 16, N2 * 16, N2 * 32, N3 * 32, N3 * 64, N3 * 64, N2 * 32, N2 * 32, N1 * 16, N1 * 16};
+    size_t o_half[11];
+    for (int k = 0; k < 11; ++k) o_half[k] = take(sizeof(bf16) * half[k]);
+    const int64_t wide = std::max(std::max(N1 * 16, N2 * 32), N3 * 64), up = std::max(N1 * 32, N2 * 64);
+    const size_t o_z1 = take(sizeof(bf16) * wide), o_z2 = take(sizeof(bf16) * wide);
+    const size_t o_s1 = take(sizeof(float) * N1 * 16), o_s2 = take(sizeof(float) * N2 * 32);
+    const size_t o_y = take(sizeof(float) * N1 * u->C);
+    const size_t o_gs1 = take(sizeof(float) * N1 * 16), o_gs2 = take(sizeof(float) * N2 * 32), o_gup = take(sizeof(float) * up);
     const size_t o_sc = take(sizeof(float) * 4), o_ds = take(sizeof(double) * 4);
+    const size_t o_sp = take(sizeof(double) * 3 * SUM_CTAS);
     const size_t o_pt = take(sizeof(double) * 3 * LS_PARTS);
     if (cudaMalloc(&u->mem, total) != cudaSuccess) {
         cudaGetLastError();
@@ -434,23 +405,25 @@ static int unet_create(const dst_mesh *mesh, dst_unet **out) {
     u->adam_m = u->grads + u->nparams;
     u->adam_v = u->adam_m + u->nparams;
     for (int l = 0; l < NLAYER; ++l) {
-        u->wf[l] = (__nv_bfloat16 *)(b + o_wf[l]);
-        u->wt[l] = (__nv_bfloat16 *)(b + o_wt[l]);
+        u->pack.l[l].wf = (uint32_t *)(b + o_wf[l]);
+        u->pack.l[l].wt = (uint32_t *)(b + o_wt[l]);
     }
-    u->dw = (float *)(b + o_dw);
-    u->dw_part = (float *)(b + o_dwp);
-    float **acts_p[16] = {&u->x0, &u->a1, &u->s1, &u->p1, &u->a2, &u->s2, &u->p2, &u->a3, &u->h3,
-                          &u->u2, &u->q2, &u->r2, &u->u1, &u->q1, &u->r1, &u->y};
-    for (int k = 0; k < 16; ++k) *acts_p[k] = (float *)(b + o_act[k]);
-    u->g_big1 = (float *)(b + o_g1);
-    u->g_big2 = (float *)(b + o_g2);
-    u->g_big3 = (float *)(b + o_g3);
+    u->wpart = (float *)(b + o_wp);
+    u->bpart = (float *)(b + o_bp);
+    bf16 **half_p[11] = {&u->x0, &u->a1, &u->p1, &u->a2, &u->p2, &u->a3, &u->h3, &u->q2, &u->r2, &u->q1, &u->r1};
+    for (int k = 0; k < 11; ++k) *half_p[k] = (bf16 *)(b + o_half[k]);
+    u->z1 = (bf16 *)(b + o_z1);
+    u->z2 = (bf16 *)(b + o_z2);
+    u->s1 = (float *)(b + o_s1);
+    u->s2 = (float *)(b + o_s2);
+    u->y = (float *)(b + o_y);
     u->gs1 = (float *)(b + o_gs1);
     u->gs2 = (float *)(b + o_gs2);
-    u->g_mid = (float *)(b + o_gm);
+    u->gup = (float *)(b + o_gup);
     u->scale = (float *)(b + o_sc);
     u->gamma = u->scale + 1;
     u->dscr = (double *)(b + o_ds);
+    u->spart = (double *)(b + o_sp);
     u->part = (double *)(b + o_pt);
     cudaError_t e = cudaMemset(u->mem, 0, total);
     const float one = 1.0f;
@@ -466,155 +439,212 @@ static int unet_create(const dst_mesh *mesh, dst_unet **out) {
 }
 
 static int pack(dst_unet *u, cudaStream_t s) {
-    for (int l = 0; l < NLAYER; ++l) {
-        const Layer &L = u->L[l];
-        const int64_t n = std::max((int64_t)L.co8 * L.kpad, (int64_t)((L.ci + 7) / 8 * 8) * u->kpadT[l]);
-        pack_weights_kernel<<<nblk(n), 256, 0, s>>>(L, u->params, u->wf[l], l == E1A ? nullptr : u->wt[l], u->kpadT[l]);
-    }
+    pack_weights_kernel<<<nblk(u->pack.total), 256, 0, s>>>(u->pack, u->params);
     DST_CUDA_TRY(cudaGetLastError());
     u->packed = true;
     return DST_OK;
 }
 
-template <int NT>
-static void launch_conv(const ConvArgs &a, cudaStream_t s) {
-    const int64_t tiles = (a.g.N + 15) / 16;
-    conv_fwd_kernel<NT><<<(unsigned)((tiles + 3) / 4), 128, 0, s>>>(a);
-}
-
-static int conv(dst_unet *u, int l, const float *in, float *out, const float *res, bool relu, const float *in_scale,
-                cudaStream_t s) {
-    const Layer &L = u->L[l];
-    ConvArgs a;
-    a.g = u->grid[L.level];
-    a.ci = L.ci; a.taps = L.taps; a.kpad = L.kpad; a.co = L.co;
-    a.in = in; a.w = u->wf[l]; a.bias = u->params + L.boff; a.res = res; a.in_scale = in_scale;
-    a.relu = relu ? 1 : 0; a.out = out; a.flip = 0;
-    switch (L.co8 / 8) {
-        case 1: launch_conv<1>(a, s); break;
-        case 2: launch_conv<2>(a, s); break;
-        case 4: launch_conv<4>(a, s); break;
-        case 8: launch_conv<8>(a, s); break;
-        default: return DST_ERR_ARG;
+// Channels of output per warp (8 NT) and rows (16 MT): the widest tile that leaves eight
+// warps per SM, because a wide tile loads its operands less often.
+static int launch_conv(const ConvArgs &a, unsigned *ctas, cudaStream_t s) {
+    const int64_t want = 152 * 8, tiles = (a.g.N + 15) / 16;
+    int nt = std::min(a.ntiles, 4), mt = 2;
+    while (mt * nt > 1 && (tiles + mt - 1) / mt * (a.ntiles / nt) < want) {
+        if (mt > 1) mt = 1;
+        else nt /= 2;
     }
+    const dim3 grid((unsigned)((tiles + CONV_WARPS * mt - 1) / (CONV_WARPS * mt)), (unsigned)(a.ntiles / nt));
+    if (ctas) *ctas = grid.x;
+    auto go = [&](auto kern) { kern<<<grid, 32 * CONV_WARPS, 0, s>>>(a); };
+    if (nt == 4) { if (mt == 2) go(conv_kernel<4, 2>); else go(conv_kernel<4, 1>); }
+    else if (nt == 2) { if (mt == 2) go(conv_kernel<2, 2>); else go(conv_kernel<2, 1>); }
+    else { if (mt == 2) go(conv_kernel<1, 2>); else go(conv_kernel<1, 1>); }
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
 
-// input gradient of layer l: dx[n][ci] = sum dz[n - off][co] W[co][ci][tap]
-static int conv_dgrad(dst_unet *u, int l, const float *dz, float *dx, cudaStream_t s) {
-    const Layer &L = u->L[l];
-    ConvArgs a;
-    a.g = u->grid[L.level];
-    a.ci = L.co; a.taps = L.taps; a.kpad = u->kpadT[l]; a.co = L.ci;
-    a.in = dz; a.w = u->wt[l]; a.bias = nullptr; a.res = nullptr; a.in_scale = nullptr;
-    a.relu = 0; a.out = dx; a.flip = 0;
-    // wt holds the mirrored taps already
-    switch ((L.ci + 7) / 8) {
-        case 2: launch_conv<2>(a, s); break;
-        case 4: launch_conv<4>(a, s); break;
-        case 8: launch_conv<8>(a, s); break;
-        default: return DST_ERR_ARG;
-    }
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
+static int log2i(int v) {
+    int l = 0;
+    while ((1 << l) < v) ++l;
+    return l;
 }
 
-static int conv_wgrad(dst_unet *u, int l, const float *in, const float *dz, const float *in_scale, cudaStream_t s) {
+struct ConvOut {
+    float *f32 = nullptr;                   // FP32 and / or BF16 result
+    bf16 *b16 = nullptr;
+    const float *res = nullptr;             // added before the activation
+    bool relu = false;
+    const bf16 *mask = nullptr;             // ReLU mask of a gradient
+    const float *s1 = nullptr, *s2 = nullptr;
+};
+
+// layer l on `in`, read at each node's parent in the next coarser grid if `from_coarse`
+static int conv(dst_unet *u, int l, const bf16 *in, const ConvOut &o, cudaStream_t s, bool from_coarse = false) {
+    const Layer &L = u->L[l];
+    ConvArgs a = {};
+    a.g = u->grid[L.level];
+    a.coarse = from_coarse ? 1 : 0;
+    if (from_coarse) a.up = u->grid[L.level + 1];
+    a.lci = log2i(L.ci); a.taps = L.taps; a.chunks = L.kpad / 16; a.co = L.co; a.ntiles = u->pack.l[l].nf;
+    a.in = in; a.w = u->pack.l[l].wf; a.bias = u->params + L.boff; a.res = o.res; a.relu = o.relu ? 1 : 0;
+    a.s1 = o.s1; a.s2 = o.s2; a.out32 = o.f32; a.out16 = o.b16;
+    return launch_conv(a, nullptr, s);
+}
+
+// input gradient of layer l: dx[n][ci] = sum dz[n - off][co] W[co][ci][tap]; `next`: the
+// layer whose dz the masked result is (its bias gradient takes the column sums), or -1
+static int conv_dgrad(dst_unet *u, int l, const bf16 *dz, const ConvOut &o, int next, cudaStream_t s) {
+    const Layer &L = u->L[l];
+    ConvArgs a = {};
+    a.g = u->grid[L.level];
+    a.lci = log2i(L.co); a.taps = L.taps; a.chunks = (L.taps * L.co + 15) / 16; a.co = L.ci; a.ntiles = u->pack.l[l].nt;
+    a.in = dz; a.w = u->pack.l[l].wt;                   // mirrored taps
+    a.mask = o.mask; a.out32 = o.f32; a.out16 = o.b16;
+    unsigned rows = 0;
+    if (next >= 0) a.colsum = u->bpart + u->sums.l[next].bpart;
+    const int rc = launch_conv(a, &rows, s);
+    if (next >= 0) u->sums.l[next].rows = (int)rows;
+    return rc;
+}
+
+static int conv_wgrad(dst_unet *u, int l, const bf16 *in, const bf16 *dz, cudaStream_t s, bool from_coarse = false) {
     const Layer &L = u->L[l];
     const UGrid &g = u->grid[L.level];
-    WgradArgs a;
+    WgradArgs a = {};
     a.g = g; a.ci = L.ci; a.taps = L.taps; a.kpad = L.kpad; a.co = L.co;
-    a.in = in; a.dz = dz; a.in_scale = in_scale; a.dw = u->dw_part;
-    const int64_t splits = std::min<int64_t>(WGRAD_SPLITS, (g.N + 1023) / 1024);
-    a.nodes_per_cta = ((g.N + splits - 1) / splits + 15) / 16 * 16;
-    const int ktiles = L.kpad / 8;
-    dim3 grid((unsigned)splits, (unsigned)((ktiles + 3) / 4), (unsigned)((L.co + 15) / 16));
-    // every (co < L.co, k < kpad) entry of every split's partial is written by exactly one warp
-    conv_wgrad_kernel<<<grid, 128, 0, s>>>(a);
-    const int64_t ndw = (int64_t)L.co * L.kpad;
-    sum_partials_kernel<<<nblk(ndw), 256, 0, s>>>(ndw, (int)splits, u->dw_part, u->dw);
-    const int64_t nw = (int64_t)L.co * L.ci * L.taps;
-    unpack_wgrad_kernel<<<nblk(nw), 256, 0, s>>>(L, u->dw, u->grads);
-    bias_grad_kernel<<<L.co, 256, 0, s>>>(g.N, L.co, dz, u->grads + L.boff);
+    a.coarse = from_coarse ? 1 : 0;
+    if (from_coarse) a.up = u->grid[L.level + 1];
+    a.in = in; a.dz = dz; a.dw = u->wpart + u->sums.l[l].wpart;
+    a.seg = wgrad_seg(g);
+    a.segs = (g.n[g.D - 1] + a.seg - 1) / a.seg;
+    a.items = wgrad_items(L, g);
+    const int slices = u->sums.l[l].slices;
+    a.per_cta = (a.items + slices - 1) / slices;
+    const unsigned rows16 = (unsigned)((L.co + 15) / 16);
+    if (L.taps == 1) {
+        const dim3 grid((unsigned)(slices / 4), rows16);
+        switch (L.ci) {
+            case 16: wgrad1_kernel<2><<<grid, 128, 0, s>>>(a); break;
+            case 32: wgrad1_kernel<4><<<grid, 128, 0, s>>>(a); break;
+            case 64: wgrad1_kernel<8><<<grid, 128, 0, s>>>(a); break;
+            default: return DST_ERR_ARG;
+        }
+    } else {
+        const int offsets = L.taps / 3, warps = std::min(offsets, 9);
+        const dim3 grid((unsigned)slices, rows16, (unsigned)(offsets / warps));
+        auto go = [&](auto kern, int ci8) -> int {
+            const size_t smem = 2 * wg_buffer(ci8, warps, a.seg);
+            DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            kern<<<grid, 32 * warps, smem, s>>>(a);
+            return DST_OK;
+        };
+        int rc;
+        switch (L.ci) {
+            case 4: case 8: rc = go(wgrad3_kernel<1>, 1); break;
+            case 16: rc = go(wgrad3_kernel<2>, 2); break;
+            case 32: rc = go(wgrad3_kernel<4>, 4); break;
+            case 64: rc = go(wgrad3_kernel<8>, 8); break;
+            default: return DST_ERR_ARG;
+        }
+        if (rc) return rc;
+    }
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
 
-// y = U(x / s) on the node grid (x: the complex unknown vector as [N][C] floats)
-static int forward(dst_unet *u, const float *x, const float *in_scale, cudaStream_t s) {
+// s = ||x|| into u->scale and x / s into u->x0; with a target also the partial sums of its square
+static int set_input(dst_unet *u, const float *x, const float *target, cudaStream_t s) {
+    const int64_t n = u->grid[0].N * u->C;
+    const unsigned parts = sum_ctas(n / 4);
+    sumsq_kernel<<<dim3(parts, target ? 2 : 1), 256, 0, s>>>(n, x, target, u->spart);
+    scale_input_kernel<<<(unsigned)std::min<int64_t>(608, (n / 2 + 255) / 256), 256, 0, s>>>(
+        n, (int)parts, u->spart, (const float2 *)x, u->scale, (uint32_t *)u->x0);
+    DST_CUDA_TRY(cudaGetLastError());
+    return DST_OK;
+}
+
+// U(x0) on the node grid, stored as `out` says
+static int forward(dst_unet *u, const ConvOut &out, cudaStream_t s) {
     int rc;
     if (!u->packed && (rc = pack(u, s))) return rc;
     const UGrid &g1 = u->grid[0], &g2 = u->grid[1], &g3 = u->grid[2];
-    if ((rc = conv(u, E1A, x, u->a1, nullptr, true, in_scale, s))) return rc;
-    if ((rc = conv(u, E1B, u->a1, u->s1, nullptr, true, nullptr, s))) return rc;
-    pool_fwd_kernel<<<nblk(g2.N * 16), 256, 0, s>>>(g1, g2, 16, u->s1, u->p1);
-    if ((rc = conv(u, E2A, u->p1, u->a2, nullptr, true, nullptr, s))) return rc;
-    if ((rc = conv(u, E2B, u->a2, u->s2, nullptr, true, nullptr, s))) return rc;
-    pool_fwd_kernel<<<nblk(g3.N * 32), 256, 0, s>>>(g2, g3, 32, u->s2, u->p2);
-    if ((rc = conv(u, E3A, u->p2, u->a3, nullptr, true, nullptr, s))) return rc;
-    if ((rc = conv(u, E3B, u->a3, u->h3, nullptr, true, nullptr, s))) return rc;
-    up_fwd_kernel<<<nblk(g2.N * 64), 256, 0, s>>>(g2, g3, 64, u->h3, u->u2);
-    if ((rc = conv(u, U2P, u->u2, u->q2, u->s2, false, nullptr, s))) return rc;
-    if ((rc = conv(u, U2C, u->q2, u->r2, nullptr, true, nullptr, s))) return rc;
-    up_fwd_kernel<<<nblk(g1.N * 32), 256, 0, s>>>(g1, g2, 32, u->r2, u->u1);
-    if ((rc = conv(u, U1P, u->u1, u->q1, u->s1, false, nullptr, s))) return rc;
-    if ((rc = conv(u, U1C, u->q1, u->r1, nullptr, true, nullptr, s))) return rc;
-    if ((rc = conv(u, OUT, u->r1, u->y, nullptr, false, nullptr, s))) return rc;
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
+    auto relu16 = [](bf16 *b) { ConvOut o; o.b16 = b; o.relu = true; return o; };
+    auto relu32 = [](float *f) { ConvOut o; o.f32 = f; o.relu = true; return o; };
+    auto plus = [](bf16 *b, const float *res) { ConvOut o; o.b16 = b; o.res = res; return o; };
+    if ((rc = conv(u, E1A, u->x0, relu16(u->a1), s))) return rc;
+    if ((rc = conv(u, E1B, u->a1, relu32(u->s1), s))) return rc;
+    pool_kernel<<<nblk(g2.N * 4), 256, 0, s>>>(g1, g2, 2, (const float4 *)u->s1, (uint2 *)u->p1);
+    if ((rc = conv(u, E2A, u->p1, relu16(u->a2), s))) return rc;
+    if ((rc = conv(u, E2B, u->a2, relu32(u->s2), s))) return rc;
+    pool_kernel<<<nblk(g3.N * 8), 256, 0, s>>>(g2, g3, 3, (const float4 *)u->s2, (uint2 *)u->p2);
+    if ((rc = conv(u, E3A, u->p2, relu16(u->a3), s))) return rc;
+    if ((rc = conv(u, E3B, u->a3, relu16(u->h3), s))) return rc;
+    if ((rc = conv(u, U2P, u->h3, plus(u->q2, u->s2), s, true))) return rc;
+    if ((rc = conv(u, U2C, u->q2, relu16(u->r2), s))) return rc;
+    if ((rc = conv(u, U1P, u->r2, plus(u->q1, u->s1), s, true))) return rc;
+    if ((rc = conv(u, U1C, u->q1, relu16(u->r1), s))) return rc;
+    return conv(u, OUT, u->r1, out, s);
 }
+constexpr int FORWARD_LAUNCHES = 13;
 
-// gradients of every parameter (into u->grads, overwritten) for dy = dL/dy
-static int backward(dst_unet *u, const float *x, const float *in_scale, const float *dy, cudaStream_t s) {
+// gradients of every parameter (into u->grads, overwritten); dL/dy is in u->z1 and its
+// column sums in the partials of OUT
+static int backward(dst_unet *u, cudaStream_t s) {
     const UGrid &g1 = u->grid[0], &g2 = u->grid[1], &g3 = u->grid[2];
-    float *dA = u->g_big1, *dB = u->g_big2, *dZ = u->g_big3;
+    bf16 *z = u->z1, *zn = u->z2;
     int rc;
-    DST_CUDA_TRY(cudaMemsetAsync(u->grads, 0, sizeof(float) * u->nparams, s));
-    // out (conv1 16 -> C): input r1
-    if ((rc = conv_wgrad(u, OUT, u->r1, dy, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, OUT, dy, dA, s))) return rc;                      // d r1
-    relu_mask_kernel<<<nblk(g1.N * 16), 256, 0, s>>>(g1.N * 16, dA, u->r1, dZ);
-    if ((rc = conv_wgrad(u, U1C, u->q1, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, U1C, dZ, dA, s))) return rc;                      // d q1
-    DST_CUDA_TRY(cudaMemcpyAsync(u->gs1, dA, sizeof(float) * g1.N * 16, cudaMemcpyDeviceToDevice, s));   // d s1
-    if ((rc = conv_wgrad(u, U1P, u->u1, dA, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, U1P, dA, dB, s))) return rc;                      // d u1 (g1, 32)
-    up_bwd_kernel<<<nblk(g2.N * 32), 256, 0, s>>>(g1, g2, 32, dB, dA);       // d r2 (g2, 32)
-    relu_mask_kernel<<<nblk(g2.N * 32), 256, 0, s>>>(g2.N * 32, dA, u->r2, dZ);
-    if ((rc = conv_wgrad(u, U2C, u->q2, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, U2C, dZ, dA, s))) return rc;                      // d q2
-    DST_CUDA_TRY(cudaMemcpyAsync(u->gs2, dA, sizeof(float) * g2.N * 32, cudaMemcpyDeviceToDevice, s));   // d s2
-    if ((rc = conv_wgrad(u, U2P, u->u2, dA, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, U2P, dA, dB, s))) return rc;                      // d u2 (g2, 64)
-    up_bwd_kernel<<<nblk(g3.N * 64), 256, 0, s>>>(g2, g3, 64, dB, dA);       // d h3 (g3, 64)
-    relu_mask_kernel<<<nblk(g3.N * 64), 256, 0, s>>>(g3.N * 64, dA, u->h3, dZ);
-    if ((rc = conv_wgrad(u, E3B, u->a3, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, E3B, dZ, dA, s))) return rc;                      // d a3
-    relu_mask_kernel<<<nblk(g3.N * 64), 256, 0, s>>>(g3.N * 64, dA, u->a3, dZ);
-    if ((rc = conv_wgrad(u, E3A, u->p2, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, E3A, dZ, dA, s))) return rc;                      // d p2 (g3, 32)
-    pool_bwd_kernel<<<nblk(g2.N * 32), 256, 0, s>>>(g2, g3, 32, dA, u->gs2);  // d s2 += pool^T d p2
-    relu_mask_kernel<<<nblk(g2.N * 32), 256, 0, s>>>(g2.N * 32, u->gs2, u->s2, dZ);
-    if ((rc = conv_wgrad(u, E2B, u->a2, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, E2B, dZ, dA, s))) return rc;                      // d a2
-    relu_mask_kernel<<<nblk(g2.N * 32), 256, 0, s>>>(g2.N * 32, dA, u->a2, dZ);
-    if ((rc = conv_wgrad(u, E2A, u->p1, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, E2A, dZ, dA, s))) return rc;                      // d p1 (g2, 16)
-    pool_bwd_kernel<<<nblk(g1.N * 16), 256, 0, s>>>(g1, g2, 16, dA, u->gs1);  // d s1 += pool^T d p1
-    relu_mask_kernel<<<nblk(g1.N * 16), 256, 0, s>>>(g1.N * 16, u->gs1, u->s1, dZ);
-    if ((rc = conv_wgrad(u, E1B, u->a1, dZ, nullptr, s))) return rc;
-    if ((rc = conv_dgrad(u, E1B, dZ, dA, s))) return rc;                      // d a1
-    relu_mask_kernel<<<nblk(g1.N * 16), 256, 0, s>>>(g1.N * 16, dA, u->a1, dZ);
-    if ((rc = conv_wgrad(u, E1A, x, dZ, in_scale, s))) return rc;
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
-}
-
-// s = ||v|| of a float array into u->scale
-static int norm_into_scale(dst_unet *u, const float *v, int64_t n, cudaStream_t s) {
-    sumsq_kernel<<<1, 256, 0, s>>>(n, v, u->dscr);
-    sqrt_scalar_kernel<<<1, 32, 0, s>>>(u->dscr, u->scale);
+    // dz of layer l from the gradient at its input's producer: masked by y, BF16
+    auto masked = [](bf16 *b, const bf16 *y) { ConvOut o; o.b16 = b; o.mask = y; return o; };
+    auto both = [](bf16 *b, float *f) { ConvOut o; o.b16 = b; o.f32 = f; return o; };
+    auto plain = [](float *f) { ConvOut o; o.f32 = f; return o; };
+    auto next = [&] { std::swap(z, zn); };
+    auto colsum = [&](int l, unsigned ctas) {
+        u->sums.l[l].rows = (int)ctas;
+        return u->bpart + u->sums.l[l].bpart;
+    };
+    if ((rc = conv_wgrad(u, OUT, u->r1, z, s))) return rc;
+    if ((rc = conv_dgrad(u, OUT, z, masked(zn, u->r1), U1C, s))) return rc;
+    next();
+    if ((rc = conv_wgrad(u, U1C, u->q1, z, s))) return rc;
+    if ((rc = conv_dgrad(u, U1C, z, both(zn, u->gs1), U1P, s))) return rc;         // d q1 = d s1
+    next();
+    if ((rc = conv_wgrad(u, U1P, u->r2, z, s, true))) return rc;
+    if ((rc = conv_dgrad(u, U1P, z, plain(u->gup), -1, s))) return rc;             // d (upsampled r2)
+    unsigned ctas = sum_ctas(g2.N * 8);
+    up_adjoint_kernel<<<ctas, 256, 0, s>>>(g1, g2, 3, (const float4 *)u->gup, (const uint2 *)u->r2, (uint2 *)zn, colsum(U2C, ctas));
+    next();
+    if ((rc = conv_wgrad(u, U2C, u->q2, z, s))) return rc;
+    if ((rc = conv_dgrad(u, U2C, z, both(zn, u->gs2), U2P, s))) return rc;         // d q2 = d s2
+    next();
+    if ((rc = conv_wgrad(u, U2P, u->h3, z, s, true))) return rc;
+    if ((rc = conv_dgrad(u, U2P, z, plain(u->gup), -1, s))) return rc;             // d (upsampled h3)
+    ctas = sum_ctas(g3.N * 16);
+    up_adjoint_kernel<<<ctas, 256, 0, s>>>(g2, g3, 4, (const float4 *)u->gup, (const uint2 *)u->h3, (uint2 *)zn, colsum(E3B, ctas));
+    next();
+    if ((rc = conv_wgrad(u, E3B, u->a3, z, s))) return rc;
+    if ((rc = conv_dgrad(u, E3B, z, masked(zn, u->a3), E3A, s))) return rc;
+    next();
+    if ((rc = conv_wgrad(u, E3A, u->p2, z, s))) return rc;
+    if ((rc = conv_dgrad(u, E3A, z, plain(u->gup), -1, s))) return rc;             // d p2
+    ctas = sum_ctas(g2.N * 8);
+    pool_adjoint_kernel<<<ctas, 256, 0, s>>>(g2, g3, 3, (const float4 *)u->gs2, (const float4 *)u->gup, (const float4 *)u->s2,
+                                             (uint2 *)zn, colsum(E2B, ctas));
+    next();
+    if ((rc = conv_wgrad(u, E2B, u->a2, z, s))) return rc;
+    if ((rc = conv_dgrad(u, E2B, z, masked(zn, u->a2), E2A, s))) return rc;
+    next();
+    if ((rc = conv_wgrad(u, E2A, u->p1, z, s))) return rc;
+    if ((rc = conv_dgrad(u, E2A, z, plain(u->gup), -1, s))) return rc;             // d p1
+    ctas = sum_ctas(g1.N * 4);
+    pool_adjoint_kernel<<<ctas, 256, 0, s>>>(g1, g2, 2, (const float4 *)u->gs1, (const float4 *)u->gup, (const float4 *)u->s1,
+                                             (uint2 *)zn, colsum(E1B, ctas));
+    next();
+    if ((rc = conv_wgrad(u, E1B, u->a1, z, s))) return rc;
+    if ((rc = conv_dgrad(u, E1B, z, masked(zn, u->a1), E1A, s))) return rc;
+    next();
+    if ((rc = conv_wgrad(u, E1A, u->x0, z, s))) return rc;
+    sum_grads_kernel<<<NLAYER + nblk(u->sums.total), 256, 0, s>>>(u->sums, u->wpart, u->bpart, u->grads);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
@@ -623,24 +653,32 @@ static int norm_into_scale(dst_unet *u, const float *v, int64_t n, cudaStream_t 
 static int loss_grad(dst_unet *u, const float *x, const float *t, cudaStream_t s) {
     const int64_t n = u->grid[0].N * u->C;
     int rc;
-    if ((rc = norm_into_scale(u, x, n, s))) return rc;
-    if ((rc = forward(u, x, u->scale, s))) return rc;
-    sumsq_kernel<<<1, 256, 0, s>>>(n, t, u->dscr + 2);
-    loss_kernel<<<1, 256, 0, s>>>(n, u->y, t, u->scale, u->dscr + 2, u->g_mid, u->dscr + 1);
-    return backward(u, x, u->scale, u->g_mid, s);
+    if ((rc = set_input(u, x, t, s))) return rc;
+    ConvOut o;
+    o.f32 = u->y;
+    if ((rc = forward(u, o, s))) return rc;
+    const unsigned parts = sum_ctas(n / 4);
+    u->sums.l[OUT].rows = (int)parts;
+    loss_kernel<<<parts, 256, 0, s>>>(n / 4, log2i(u->C / 4), (int)parts, u->spart + SUM_CTAS, (const float4 *)u->y,
+                                      (const float4 *)t, u->scale, (uint2 *)u->z1, u->spart + 2 * SUM_CTAS,
+                                      u->bpart + u->sums.l[OUT].bpart);
+    loss_sum_kernel<<<1, 32, 0, s>>>((int)parts, u->spart + 2 * SUM_CTAS, u->dscr + 1);
+    return backward(u, s);
 }
 
 // ---- preconditioner hook used by the solver --------------------------------------
 
 int dst_internal_unet_correct(dst_unet *u, const dst_mesh *mesh, const float2 *rho, float2 *z, float2 *tmp,
                               cudaStream_t s, int *launches) {
-    const int64_t n = u->grid[0].N * u->C, nc = n / 2;
+    const int64_t nc = u->grid[0].N * u->C / 2;
     const float *x = reinterpret_cast<const float *>(rho);
     const float2 *y = reinterpret_cast<const float2 *>(u->y);
-    *launches = (u->packed ? 0 : NLAYER) + 2 + 15 + 1 + 2;
+    *launches = (u->packed ? 0 : 1) + 2 + FORWARD_LAUNCHES + 1 + 2;
     int rc;
-    if ((rc = norm_into_scale(u, x, n, s))) return rc;
-    if ((rc = forward(u, x, u->scale, s))) return rc;
+    if ((rc = set_input(u, x, nullptr, s))) return rc;
+    ConvOut o;
+    o.f32 = u->y;
+    if ((rc = forward(u, o, s))) return rc;
     // the correction's scale for this input: alpha minimising ||rho - alpha A y||, so the
     // corrected direction never leaves a larger residual than the sweep alone
     if ((rc = dst_internal_apply(mesh, DST_FP32, y, tmp, s))) return rc;
@@ -697,14 +735,13 @@ extern "C" int dst_unet_get_params(const dst_unet *u, float *host) {
 extern "C" int dst_unet_forward(dst_unet *u, const void *x, void *y, void *stream) {
     if (!u || !x || !y) return DST_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t n = u->grid[0].N * u->C;
-    int rc = norm_into_scale(u, (const float *)x, n, s);
-    if (rc == DST_OK) rc = forward(u, (const float *)x, u->scale, s);
+    const int rc = set_input(u, (const float *)x, nullptr, s);
     if (rc) return rc;
-    DST_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(float) * n, s));
-    axpy_scaled_kernel<<<nblk(n), 256, 0, s>>>(n, u->scale, u->gamma, u->y, (float *)y);
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
+    ConvOut o;                                       // y = gamma s U(x / s)
+    o.f32 = (float *)y;
+    o.s1 = u->gamma;
+    o.s2 = u->scale;
+    return forward(u, o, s);
 }
 
 extern "C" int dst_unet_loss_grad(dst_unet *u, const void *x, const void *target, double *loss, float *grad_host,
@@ -777,9 +814,10 @@ static int train(dst_unet *u, dst_mesh *mesh, int steps, float lr, uint64_t seed
             if ((rc = dst_internal_apply(mesh, DST_FP32, z, az, s))) break;
             if ((rc = dst_k_sub_f32(n, r, az, r, s))) break;
             if ((rc = dst_k_sub_f32(n, e, z, tg, s))) break;
-            const float *x = (const float *)r;
-            if ((rc = norm_into_scale(u, x, 2 * n, s))) break;
-            if ((rc = forward(u, x, u->scale, s))) break;
+            if ((rc = set_input(u, (const float *)r, nullptr, s))) break;
+            ConvOut o;
+            o.f32 = u->y;
+            if ((rc = forward(u, o, s))) break;
             dot_kernel<<<1, 256, 0, s>>>(2 * n, u->y, (const float *)tg, u->scale, acc);
         }
         double hacc[2] = {0.0, 0.0};
