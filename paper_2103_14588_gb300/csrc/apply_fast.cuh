@@ -17,11 +17,6 @@
 
 namespace dst {
 
-template <int D> struct FastTile;
-template <> struct FastTile<1> { static constexpr int TX = 128, TY = 1, TZ = 1, TT = 16; };
-template <> struct FastTile<2> { static constexpr int TX = 32, TY = 4, TZ = 1, TT = 8; };
-template <> struct FastTile<3> { static constexpr int TX = 32, TY = 4, TZ = 1, TT = 8; };
-
 template <int NC, typename T>
 struct NodeV {
     typename C2<T>::type c[NC];
@@ -70,56 +65,6 @@ __device__ __forceinline__ void store_node(typename C2<T>::type *__restrict__ ba
 #pragma unroll
         for (int c = 0; c < NC; ++c) q[c] = make_double2(val[c].x, val[c].y);
     }
-}
-
-// Neighbour offsets of one thread within one time plane, per axis: node index
-// = xo[dx] + yo[dy] + zo[dz]; an absent neighbour (outside a non-periodic
-// axis) carries a large negative offset so that any sum with it is < 0.
-// Planes of up to 2^31 - 1 nodes (checked by the launcher).
-struct Nbr {
-    int xo[3], yo[3], zo[3];
-    __device__ __forceinline__ int at(int dz, int dy, int dx) const { return xo[dx] + yo[dy] + zo[dz]; }
-};
-
-template <int D>
-__device__ __forceinline__ void neighbours(const OpParams &p, int64_t ix, int64_t iy, int64_t iz, Nbr &nb) {
-    const int nx = (int)p.ax[0].n, nxy = (int)(p.ax[0].n * p.ax[1].n);
-    const int ABSENT = -(1 << 30);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int64_t xx = axis_nbr(p.ax[0], ix - 1 + k);
-        nb.xo[k] = xx >= 0 ? (int)xx : ABSENT;
-        if (D >= 2) {
-            const int64_t yy = axis_nbr(p.ax[1], iy - 1 + k);
-            nb.yo[k] = yy >= 0 ? (int)yy * nx : ABSENT;
-        } else {
-            nb.yo[k] = (int)iy * nx;
-        }
-        if (D >= 3) {
-            const int64_t zz = axis_nbr(p.ax[2], iz - 1 + k);
-            nb.zo[k] = zz >= 0 ? (int)zz * nxy : ABSENT;
-        } else {
-            nb.zo[k] = (int)iz * nxy;
-        }
-    }
-}
-
-template <int D, int NC, typename T>
-struct Plane {
-    NodeV<NC, T> v[D == 1 ? 3 : (D == 2 ? 9 : 27)];
-};
-
-template <int D, int NC, typename T>
-__device__ __forceinline__ void load_plane(const typename C2<T>::type *__restrict__ layer, const Nbr &nb,
-                                           bool have, Plane<D, NC, T> &pl) {
-    const int NY = D >= 2 ? 3 : 1;
-#pragma unroll
-    for (int dy = 0; dy < NY; ++dy)
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx) {
-            const int id = nb.at(1, dy, dx);
-            load_node<NC, T>(layer, id, have && id >= 0, pl.v[dy * 3 + dx]);
-        }
 }
 
 // G_C, G_M of one output node from its 3^d neighbourhood; get(r) returns the
@@ -250,102 +195,6 @@ __device__ __forceinline__ void fields_nov(Get get, const NodeCoef<D, T> &k, T m
 #pragma unroll
         for (int c = 0; c < NC; ++c) GM[c] = cadd(GM[c], cmul_i(aS[c]));
     }
-}
-
-template <int D, int NC, typename T>
-__global__ void __launch_bounds__(FastTile<D>::TX * FastTile<D>::TY * FastTile<D>::TZ)
-apply_fast_kernel(OpParams p, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
-                  int64_t tiles_x, int64_t tiles_y) {
-    using V = typename C2<T>::type;
-    using Tile = FastTile<D>;
-    constexpr bool PREFETCH = sizeof(T) == 4 && D <= 2;
-    const int64_t tile = blockIdx.x;
-    const int64_t chunk = blockIdx.y;
-    const int64_t x0 = (tile % tiles_x) * Tile::TX;
-    const int64_t y0 = ((tile / tiles_x) % tiles_y) * Tile::TY;
-    const int64_t z0 = (tile / (tiles_x * tiles_y)) * Tile::TZ;
-    const int tx = threadIdx.x % Tile::TX;
-    const int ty = (threadIdx.x / Tile::TX) % Tile::TY;
-    const int tz = threadIdx.x / (Tile::TX * Tile::TY);
-    const int64_t ix = x0 + tx, iy = y0 + ty, iz = z0 + tz;
-    const int64_t nx = p.ax[0].n, ny = p.ax[1].n, nz = p.ax[2].n;
-    if (ix >= nx || iy >= ny || iz >= nz) return;
-    const int64_t N = p.nt;
-    const int64_t t0 = 1 + chunk * Tile::TT;
-    const int64_t t1 = min(t0 + (int64_t)Tile::TT, N + 1);
-    const int64_t plane_nodes = nx * ny * nz;
-    const int64_t self = (iz * ny + iy) * nx + ix;
-
-    NodeCoef<D, T> k;
-    node_coef<D, T>(p, ix, iy, iz, k);
-    Nbr nb;
-    neighbours<D>(p, ix, iy, iz, nb);
-    const T h6 = (T)(p.ht / 6.0);
-
-    V accP[NC], accC[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) { accP[c] = cz<V>(); accC[c] = cz<V>(); }
-
-    constexpr int K = D == 1 ? 3 : (D == 2 ? 9 : 27);
-    Plane<D, NC, T> cur, nxt;   // used only when prefetching (1+1, 2+1 in FP32)
-    int64_t pl = t0 - 1;
-    if (PREFETCH) load_plane<D, NC, T>(x + (pl - 1) * plane_nodes * NC, nb, pl >= 1 && pl <= N, cur);
-    for (; pl <= t1; ++pl) {
-        const bool have = pl >= 1 && pl <= N;
-        if (PREFETCH && pl + 1 <= t1)
-            load_plane<D, NC, T>(x + pl * plane_nodes * NC, nb, pl + 1 >= 1 && pl + 1 <= N, nxt);
-        V GC[NC], GM[NC];
-        if (have) {
-            if (PREFETCH) {
-                fields<D, NC, T>([&](int r) { return cur.v[r]; }, k, GC, GM);
-            } else {
-                const V *layer = x + (pl - 1) * plane_nodes * NC;
-                fields<D, NC, T>([&](int r) {
-                    NodeV<NC, T> v;
-                    const int NY = D >= 2 ? 3 : 1;
-                    const int id = nb.at(r / (3 * NY), (r / 3) % NY, r % 3);
-                    load_node<NC, T>(layer, id, id >= 0, v);
-                    return v;
-                }, k, GC, GM);
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) { GC[c] = cz<V>(); GM[c] = cz<V>(); }
-        }
-        const T cdiag = pl < N ? (T)0 : (T)0.5;
-        const T mdiag = pl < N ? 4 * h6 : 2 * h6;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            accP[c] = cfma_r((T)0.5, GC[c], cfma_r(h6, GM[c], accP[c]));
-            accC[c] = cfma_r(cdiag, GC[c], cfma_r(mdiag, GM[c], accC[c]));
-        }
-        if (pl - 1 >= t0 && pl - 1 < t1) store_node<NC, T>(y + (pl - 2) * plane_nodes * NC, self, accP);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            accP[c] = accC[c];
-            accC[c] = cfma_r((T)(-0.5), GC[c], cmul_r(h6, GM[c]));
-        }
-        if (PREFETCH) {
-#pragma unroll
-            for (int q = 0; q < K; ++q) cur.v[q] = nxt.v[q];
-        }
-    }
-}
-
-template <int D, int NC, typename T>
-int launch_apply_fast(const OpParams &p, const typename C2<T>::type *x, typename C2<T>::type *y, cudaStream_t s) {
-    using Tile = FastTile<D>;
-    const int64_t tx = (p.ax[0].n + Tile::TX - 1) / Tile::TX;
-    const int64_t ty = (p.ax[1].n + Tile::TY - 1) / Tile::TY;
-    const int64_t tz = (p.ax[2].n + Tile::TZ - 1) / Tile::TZ;
-    const int64_t chunks = (p.nt + Tile::TT - 1) / Tile::TT;
-    const int64_t tiles = tx * ty * tz;
-    if (tiles <= 0 || tiles > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
-    if (p.ax[0].n * p.ax[1].n * p.ax[2].n >= (1LL << 30)) return launch_apply<D, NC, T>(p, x, y, s);
-    dim3 grid((unsigned)tiles, (unsigned)chunks);
-    apply_fast_kernel<D, NC, T><<<grid, Tile::TX * Tile::TY * Tile::TZ, 0, s>>>(p, x, y, tx, ty);
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
 }
 
 }  // namespace dst

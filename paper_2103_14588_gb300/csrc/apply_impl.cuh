@@ -270,78 +270,6 @@ __device__ __forceinline__ void stage_plane(const OpParams &p, const typename C2
     }
 }
 
-// y = A x over one (tile, time chunk) per CTA.
-template <int D, int NC, typename T>
-__global__ void __launch_bounds__(ApplyShape<D, NC, T>::NTHR)
-apply_kernel(OpParams p, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
-             int64_t tiles_x, int64_t tiles_y, int64_t tiles_z) {
-    using V = typename C2<T>::type;
-    using S = ApplyShape<D, NC, T>;
-    using Tile = typename S::Tile;
-    __shared__ V box[S::BOX * NC];
-
-    const int64_t ntiles = tiles_x * tiles_y * tiles_z;
-    const int64_t tile = blockIdx.x % ntiles;
-    const int64_t chunk = blockIdx.x / ntiles;
-    const int64_t x0 = (tile % tiles_x) * Tile::TX;
-    const int64_t y0 = ((tile / tiles_x) % tiles_y) * Tile::TY;
-    const int64_t z0 = (tile / (tiles_x * tiles_y)) * Tile::TZ;
-    const int tx = threadIdx.x % Tile::TX;
-    const int ty = (threadIdx.x / Tile::TX) % Tile::TY;
-    const int tz = threadIdx.x / (Tile::TX * Tile::TY);
-    const int64_t ix = x0 + tx, iy = y0 + ty, iz = z0 + tz;
-    const int64_t nx = p.ax[0].n, ny = p.ax[1].n, nz = p.ax[2].n;
-    const bool valid = ix < nx && iy < ny && iz < nz;
-    const int64_t N = p.nt;
-    const int64_t t0 = 1 + chunk * Tile::TT;                 // first output layer (1-based)
-    const int64_t t1 = min(t0 + (int64_t)Tile::TT, N + 1);   // one past the last
-    const int64_t plane = nx * ny * nz * NC;
-    const int64_t node_off = ((iz * ny + iy) * nx + ix) * NC;
-
-    NodeCoef<D, T> k;
-    if (valid) node_coef<D, T>(p, ix, iy, iz, k);
-    const bool vgen = p.vmode == 1;
-    const T h6 = (T)(p.ht / 6.0);
-
-    V accP[NC], accC[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) { accP[c] = cz<V>(); accC[c] = cz<V>(); }
-
-    for (int64_t pl = t0 - 1; pl <= t1; ++pl) {
-        const bool have = pl >= 1 && pl <= N;
-        V GC[NC], GM[NC];
-        if (have) {
-            __syncthreads();
-            stage_plane<D, NC, T>(p, x + (pl - 1) * plane, box, x0, y0, z0);
-            __syncthreads();
-        }
-        if (have && valid) {
-            spatial_G<D, NC, T, S::BX, S::BY>(box, tx + 1, D >= 2 ? ty + 1 : 0, D >= 3 ? tz + 1 : 0, k, vgen, GC, GM);
-        } else {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) { GC[c] = cz<V>(); GM[c] = cz<V>(); }
-        }
-        // y(pl-1) += C_t[pl-1][pl] G_C + M_t[pl-1][pl] G_M = G_C/2 + h/6 G_M; then complete
-        const T cdiag = pl < N ? (T)0 : (T)0.5;
-        const T mdiag = pl < N ? 4 * h6 : 2 * h6;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            accP[c] = cfma_r((T)0.5, GC[c], cfma_r(h6, GM[c], accP[c]));
-            accC[c] = cfma_r(cdiag, GC[c], cfma_r(mdiag, GM[c], accC[c]));
-        }
-        if (valid && pl - 1 >= t0 && pl - 1 < t1) {
-            V *dst = y + (pl - 2) * plane + node_off;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) dst[c] = accP[c];
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            accP[c] = accC[c];
-            accC[c] = cfma_r((T)(-0.5), GC[c], cmul_r(h6, GM[c]));
-        }
-    }
-}
-
 // b(layer 1) = -( C_t[1][0] G_C(psi0) + M_t[1][0] G_M(psi0) ) = G_C/2 - h/6 G_M.
 template <int D, int NC>
 __global__ void __launch_bounds__(ApplyShape<D, NC, double>::NTHR)
@@ -372,21 +300,6 @@ rhs_kernel(OpParams p, const double2 *__restrict__ psi0, double2 *__restrict__ b
     V *dst = b + ((iz * ny + iy) * nx + ix) * NC;
 #pragma unroll
     for (int c = 0; c < NC; ++c) dst[c] = cfma_r(-h6, GM[c], cmul_r(0.5, GC[c]));
-}
-
-template <int D, int NC, typename T>
-int launch_apply(const OpParams &p, const typename C2<T>::type *x, typename C2<T>::type *y, cudaStream_t s) {
-    using Tile = ApplyTile<D>;
-    using S = ApplyShape<D, NC, T>;
-    const int64_t tx = (p.ax[0].n + Tile::TX - 1) / Tile::TX;
-    const int64_t ty = (p.ax[1].n + Tile::TY - 1) / Tile::TY;
-    const int64_t tz = (p.ax[2].n + Tile::TZ - 1) / Tile::TZ;
-    const int64_t chunks = (p.nt + Tile::TT - 1) / Tile::TT;
-    const int64_t blocks = tx * ty * tz * chunks;
-    if (blocks <= 0 || blocks > 0x7fffffffLL) return DST_ERR_ARG;
-    apply_kernel<D, NC, T><<<(unsigned)blocks, S::NTHR, 0, s>>>(p, x, y, tx, ty, tz);
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
 }
 
 template <int D, int NC>

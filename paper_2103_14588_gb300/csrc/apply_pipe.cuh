@@ -16,6 +16,7 @@
 #pragma once
 
 #include "apply_fast.cuh"
+#include "apply_node.cuh"
 
 #define DST_MAX_DEVICES_APPLY 64
 
@@ -519,13 +520,13 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const typenam
     (void)any_valid;
 }
 
-template <int D, int NC, typename T, bool NOV, bool STD, int TV>
-__global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR,
-                                  sizeof(T) == 8 ? 1 : (D == 3 ? (STD ? 2 : 1) : 3))
+// Meshes without an open axis only (the launches send the others to apply_node.cuh).
+template <int D, int NC, typename T, bool NOV, int TV>
+__global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR, sizeof(T) == 8 ? 1 : (D == 3 ? 2 : 3))
 apply_pipe_kernel(OpParams p, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
                   int64_t tiles_x, int64_t tiles_y) {
     extern __shared__ __align__(16) char ring[];
-    apply_pipe_tile<D, NC, T, NOV, STD, TV>(p, x, y, tiles_x, tiles_y, blockIdx.x, blockIdx.y, ring);
+    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, x, y, tiles_x, tiles_y, blockIdx.x, blockIdx.y, ring);
 }
 
 template <int D, int NC, typename T, int TV>
@@ -539,23 +540,17 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
     const int64_t tiles = tx * ty * tz;
     if (tiles <= 0 || tiles > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
     // byte offsets within one time layer are kept in 32 bits
-    if (p.ax[0].n * p.ax[1].n * p.ax[2].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply<D, NC, T>(p, x, y, s);
+    if (p.ax[0].n * p.ax[1].n * p.ax[2].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<D, NC, T>(p, x, y, s);
     dim3 grid((unsigned)tiles, (unsigned)chunks);
     // the shared-memory opt-in is a per-device function attribute: set it once per device
-    static bool configured[4][DST_MAX_DEVICES_APPLY] = {};
+    static bool configured[2][DST_MAX_DEVICES_APPLY] = {};
     int dev = 0;
     DST_CUDA_TRY(cudaGetDevice(&dev));
     const int nov = p.vmode == 2 ? 1 : 0;
-    bool all_std = true;        // no open axis: every node has the standard stencils
-    for (int k = 0; k < D; ++k) all_std = all_std && p.ax[k].bc != DST_BC_OPEN;
-    const int var = nov + 2 * (all_std ? 1 : 0);
-    auto kern = var == 0   ? apply_pipe_kernel<D, NC, T, false, false, TV>
-                : var == 1 ? apply_pipe_kernel<D, NC, T, true, false, TV>
-                : var == 2 ? apply_pipe_kernel<D, NC, T, false, true, TV>
-                           : apply_pipe_kernel<D, NC, T, true, true, TV>;
-    if (dev < 0 || dev >= DST_MAX_DEVICES_APPLY || !configured[var][dev]) {
+    auto kern = nov ? apply_pipe_kernel<D, NC, T, true, TV> : apply_pipe_kernel<D, NC, T, false, TV>;
+    if (dev < 0 || dev >= DST_MAX_DEVICES_APPLY || !configured[nov][dev]) {
         DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
-        if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[var][dev] = true;
+        if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[nov][dev] = true;
     }
     kern<<<grid, S::NTHR, S::SMEM, s>>>(p, x, y, tx, ty);
     DST_CUDA_TRY(cudaGetLastError());
@@ -574,9 +569,7 @@ template <int D, int NC, typename T>
 int launch_apply_pipe(const OpParams &p, const typename C2<T>::type *x, typename C2<T>::type *y, cudaStream_t s) {
     const int tv = p.tile_variant[sizeof(T) == 4 ? DST_FP32 : DST_FP64];
     if constexpr (D == 3) {
-        bool all_std = true;
-        for (int k = 0; k < 3; ++k) all_std = all_std && p.ax[k].bc != DST_BC_OPEN;
-        if (tv == 1 && all_std && p.vmode != 1) return launch_apply_zblk<T, sizeof(T) == 4 ? 4 : 2>(p, x, y, s);
+        if (tv == 1) return launch_apply_zblk<T, sizeof(T) == 4 ? 4 : 2>(p, x, y, s);
     }
     if (D == 3 || tv <= 0) return launch_apply_pipe_v<D, NC, T, 0>(p, x, y, s);
     if constexpr (D < 3) {

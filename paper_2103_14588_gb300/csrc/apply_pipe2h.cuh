@@ -169,7 +169,7 @@ int launch_apply_pipe2h(const OpParams &p, const float2 *x, float2 *y, cudaStrea
     const int64_t chunks = (p.nt + S::TT - 1) / S::TT;
     const int64_t tiles = tx * ty;
     if (tiles <= 0 || tiles > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
-    if (p.ax[0].n * p.ax[1].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply<2, 2, float>(p, x, y, s);
+    if (p.ax[0].n * p.ax[1].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<2, 2, float>(p, x, y, s);
     static bool configured[2][DST_MAX_DEVICES_APPLY] = {};
     int dev = 0;
     DST_CUDA_TRY(cudaGetDevice(&dev));

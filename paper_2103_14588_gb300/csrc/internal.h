@@ -118,6 +118,7 @@ int dst_internal_update_weights(dst_mesh *mesh);
 int dst_launch_apply_d1(const OpParams &p, int precision, const void *x, void *y, cudaStream_t s);
 int dst_launch_apply_d2(const OpParams &p, int precision, const void *x, void *y, cudaStream_t s);
 int dst_launch_apply_d3(const OpParams &p, int precision, const void *x, void *y, cudaStream_t s);
+bool dst_apply_tiled(const OpParams &p, int d);      // whether the mesh takes a tiled kernel
 int dst_launch_rhs_d1(const OpParams &p, const double2 *psi0, double2 *b, cudaStream_t s);
 int dst_launch_rhs_d2(const OpParams &p, const double2 *psi0, double2 *b, cudaStream_t s);
 int dst_launch_rhs_d3(const OpParams &p, const double2 *psi0, double2 *b, cudaStream_t s);

@@ -103,7 +103,7 @@ int dst_internal_tile_variants(const dst_mesh *mesh) { return mesh->d == 3 ? 2 :
 int dst_internal_tune(dst_mesh *mesh, void *scratch, cudaStream_t s) {
     const int nv = dst_internal_tile_variants(mesh);
     mesh->tuned = true;
-    if (nv <= 1 || mesh->v_general) return DST_OK;     // one shape only / the general-potential kernel
+    if (nv <= 1 || !dst_apply_tiled(dst_internal_params(mesh), mesh->d)) return DST_OK;     // no tiles to choose from
     const int64_t n = mesh->n_unknowns;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     DST_CUDA_TRY(cudaEventCreate(&e0));
@@ -113,6 +113,7 @@ int dst_internal_tune(dst_mesh *mesh, void *scratch, cudaStream_t s) {
     }
     int rc = DST_OK;
     for (int prec = 0; prec < 2 && rc == DST_OK; ++prec) {
+        if (prec == DST_FP64 && mesh->d == 1) continue;     // the FP64 1+1 apply has no tiles
         const size_t esz = prec == DST_FP64 ? 16 : 8;
         char *x = static_cast<char *>(scratch), *y = x + esz * n;
         if (cudaMemsetAsync(x, 0, esz * n, s) != cudaSuccess) { rc = DST_ERR_CUDA; break; }
