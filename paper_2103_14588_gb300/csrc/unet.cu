@@ -91,7 +91,7 @@ __global__ void adam_kernel(int64_t n, float *__restrict__ p, const float *__res
 }
 
 // Sums of squares of one or two float arrays (blockIdx.y), one FP64 partial per CTA.
-constexpr int SUM_CTAS = 152;
+constexpr int SUM_CTAS = 456;
 __global__ void __launch_bounds__(256) sumsq_kernel(int64_t n, const float *__restrict__ a, const float *__restrict__ b,
                                                     double *__restrict__ part) {
     __shared__ double red[256];
@@ -644,7 +644,7 @@ static int backward(dst_unet *u, cudaStream_t s) {
     if ((rc = conv_dgrad(u, E1B, z, masked(zn, u->a1), E1A, s))) return rc;
     next();
     if ((rc = conv_wgrad(u, E1A, u->x0, z, s))) return rc;
-    sum_grads_kernel<<<NLAYER + nblk(u->sums.total), 256, 0, s>>>(u->sums, u->wpart, u->bpart, u->grads);
+    sum_grads_kernel<<<(unsigned)(NLAYER + (u->sums.total + 31) / 32), 256, 0, s>>>(u->sums, u->wpart, u->bpart, u->grads);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }

@@ -150,27 +150,40 @@ __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
         for (int j = 0; j < NT; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
     const uint2 *w = reinterpret_cast<const uint2 *>(a.w) + ((size_t)blockIdx.y * NT) * 32 + lane;
     const size_t wstep = (size_t)a.ntiles * 32;
-#pragma unroll 4
-    for (int kc = 0; kc < a.chunks; ++kc, w += wstep) {
-        uint32_t af[MT][4];
+    // U chunks of both operands in registers before their products: the loads of a group
+    // are in flight together, and with few warps (the coarse levels) that latency is all
+    // there is to a layer
+    constexpr int U = MT * NT >= 8 ? 2 : 4;
+    for (int kc = 0; kc < a.chunks; kc += U) {
+        uint32_t af[U][MT][4];
+        uint2 b[U][NT];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int k = kc * 16 + half * 8 + 2 * tg;
-            const Tap t = tab[min(k >> a.lci, a.taps)];
-            const long long off = t.off + (k & (ci - 1));
+        for (int u = 0; u < U; ++u) {
+            const bool in = kc + u < a.chunks;
 #pragma unroll
-            for (int m = 0; m < MT; ++m)
+            for (int half = 0; half < 2; ++half) {
+                const int k = (kc + u) * 16 + half * 8 + 2 * tg;
+                const Tap t = tab[min(k >> a.lci, a.taps)];
+                const long long off = t.off + (k & (ci - 1));
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    af[m][2 * half + h] =
-                        (ends[m][h] & t.ends) ? 0u : __ldg(reinterpret_cast<const uint32_t *>(row[m][h] + off));
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        af[u][m][2 * half + h] =
+                            (ends[m][h] & t.ends) ? 0u : __ldg(reinterpret_cast<const uint32_t *>(row[m][h] + off));
+            }
+#pragma unroll
+            for (int j = 0; j < NT; ++j) b[u][j] = in ? __ldg(w + u * wstep + j * 32) : make_uint2(0u, 0u);
         }
+        w += U * wstep;
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            const uint2 b = __ldg(w + j * 32);
+        for (int u = 0; u < U; ++u)
+            if (kc + u < a.chunks) {
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma_16816(acc[m][j], af[m], b.x, b.y);
-        }
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_16816(acc[m][j], af[u][m], b[u][j].x, b[u][j].y);
+            }
     }
     const float scale = a.s1 ? *a.s1 * *a.s2 : 1.f;
 #pragma unroll
@@ -482,45 +495,66 @@ __global__ void __launch_bounds__(256) sum_grads_kernel(GradLayers L, const floa
         }
         return;
     }
-    const int64_t i = (int64_t)(blockIdx.x - L.n) * blockDim.x + threadIdx.x;
-    if (i >= L.total) return;
+    // 32 pairs per CTA, their slices over eight warps
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)(blockIdx.x - L.n) * 32 + lane;
     int k = 0;
     while (k + 1 < L.n && i >= L.l[k + 1].first) ++k;
     const GradLayer &l = L.l[k];
     const int at = (int)(i - l.first), o = at / l.kpad, kk = at - o * l.kpad;
-    if (kk >= l.taps * l.ci) return;
-    const float *p = wpart + l.wpart + at;
-    const int64_t step = (int64_t)l.co * l.kpad;
+    const bool live = i < L.total && kk < l.taps * l.ci;
     float t = 0.f;
-#pragma unroll 8
-    for (int s = 0; s < l.slices; ++s) t += p[s * step];
-    grad[l.woff + ((int64_t)o * l.ci + kk % l.ci) * l.taps + kk / l.ci] = t;
+    if (live) {
+        const float *p = wpart + l.wpart + at;
+        const int64_t step = (int64_t)l.co * l.kpad;
+#pragma unroll 4
+        for (int s = warp; s < l.slices; s += 8) t += p[s * step];
+    }
+    part[warp][lane] = t;
+    __syncthreads();
+    if (warp == 0 && live) {
+        for (int w = 1; w < 8; ++w) t += part[w][lane];
+        grad[l.woff + ((int64_t)o * l.ci + kk % l.ci) * l.taps + kk / l.ci] = t;
+    }
 }
 
 // ---- element-wise pieces, four channels per thread ----------------------------
 
-// out[q] = mean of in over the 2^D fine nodes of q (nodes past an odd end count as zero)
+// Sum of four channels over the 2^D fine nodes of a coarse node (nodes past an odd end
+// count as zero), in order; the loads of eight nodes in flight together.
+__device__ __forceinline__ float4 fine_sum(const UGrid &f, const int (&cc)[4], int lq, int k, const float4 *__restrict__ in) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int m0 = 0; m0 < 1 << f.D; m0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int m = m0 + e;
+            int64_t r = 0;
+            bool ok = m < 1 << f.D;
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                if (a < f.D) {
+                    const int x = 2 * cc[a] + ((m >> (f.D - 1 - a)) & 1);
+                    ok = ok && x < f.n[a];
+                    r = r * f.n[a] + x;
+                }
+            v[e] = ok ? __ldg(in + (r << lq) + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { s.x += v[e].x; s.y += v[e].y; s.z += v[e].z; s.w += v[e].w; }
+    }
+    return s;
+}
+
+// out[q] = mean of in over the fine nodes of q
 __global__ void __launch_bounds__(256) pool_kernel(UGrid f, UGrid c, int lq, const float4 *__restrict__ in, uint2 *__restrict__ out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;       // (node, four channels)
     if (i >= c.N << lq) return;
     int cc[4];
     coords(c, (unsigned)(i >> lq), cc);
-    const int k = (int)(i & ((1 << lq) - 1)), nb = 1 << f.D;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int m = 0; m < nb; ++m) {
-        int64_t r = 0;
-        bool ok = true;
-        for (int a = 0; a < f.D; ++a) {
-            const int x = 2 * cc[a] + ((m >> (f.D - 1 - a)) & 1);
-            ok = ok && x < f.n[a];
-            r = r * f.n[a] + x;
-        }
-        if (ok) {
-            const float4 v = __ldg(in + (r << lq) + k);
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
-    }
-    const float w = 1.f / (float)nb;                       // a power of two
+    const float4 s = fine_sum(f, cc, lq, (int)(i & ((1 << lq) - 1)), in);
+    const float w = 1.f / (float)(1 << f.D);               // a power of two
     out[i] = pack_bf16x4(make_float4(s.x * w, s.y * w, s.z * w, s.w * w));
 }
 
@@ -545,21 +579,7 @@ __global__ void __launch_bounds__(256) up_adjoint_kernel(UGrid f, UGrid c, int l
     for (int64_t i = blockIdx.x * 256LL + threadIdx.x; i < c.N << lq; i += (int64_t)gridDim.x * 256) {
         int cc[4];
         coords(c, (unsigned)(i >> lq), cc);
-        const int k = (int)(i & ((1 << lq) - 1));
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int m = 0; m < (1 << f.D); ++m) {
-            int64_t r = 0;
-            bool ok = true;
-            for (int a = 0; a < f.D; ++a) {
-                const int x = 2 * cc[a] + ((m >> (f.D - 1 - a)) & 1);
-                ok = ok && x < f.n[a];
-                r = r * f.n[a] + x;
-            }
-            if (ok) {
-                const float4 v = __ldg(d + (r << lq) + k);
-                s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-            }
-        }
+        float4 s = fine_sum(f, cc, lq, (int)(i & ((1 << lq) - 1)), d);
         const uint2 m = y[i];
         s = make_float4(pos_lo(m.x) ? s.x : 0.f, pos_hi(m.x) ? s.y : 0.f, pos_lo(m.y) ? s.z : 0.f, pos_hi(m.y) ? s.w : 0.f);
         dz[i] = pack_bf16x4(s);
