@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "blas.h"
@@ -264,6 +265,7 @@ struct dst_unet {
     PackLayers pack;                             // weight fragments
     GradLayers sums;                             // partial sums of the weight and bias gradients
     float *wpart, *bpart;
+    bf16 *zeros;                                 // 64 channels of zeros: a node outside the grid
     // activations [N][ch]: BF16 where only a convolution (or a ReLU mask) reads them
     bf16 *x0, *a1, *p1, *a2, *p2, *a3, *h3, *q2, *r2, *q1, *r1;
     float *s1, *s2, *y;
@@ -381,6 +383,7 @@ static int unet_create(const dst_mesh *mesh, dst_unet **out) {
     u->pack.total = pairs;
     u->sums.n = NLAYER;
     u->sums.total = cells;
+    const size_t o_zero = take(sizeof(bf16) * 64);
     const size_t o_wp = take(sizeof(float) * wfloats), o_bp = take(sizeof(float) * bfloats);
     const int64_t half[] = {N1 * u->C, N1 * 16, N2 * 16, N2 * 32, N3 * 32, N3 * 64, N3 * 64, N2 * 32, N2 * 32, N1 * 16, N1 * 16};
     size_t o_half[11];
@@ -408,6 +411,7 @@ static int unet_create(const dst_mesh *mesh, dst_unet **out) {
         u->pack.l[l].wf = (uint32_t *)(b + o_wf[l]);
         u->pack.l[l].wt = (uint32_t *)(b + o_wt[l]);
     }
+    u->zeros = (bf16 *)(b + o_zero);              // (the allocation is cleared below)
     u->wpart = (float *)(b + o_wp);
     u->bpart = (float *)(b + o_bp);
     bf16 **half_p[11] = {&u->x0, &u->a1, &u->p1, &u->a2, &u->p2, &u->a3, &u->h3, &u->q2, &u->r2, &u->q1, &u->r1};
@@ -456,12 +460,35 @@ static int launch_conv(const ConvArgs &a, unsigned *ctas, cudaStream_t s) {
     }
     const dim3 grid((unsigned)((tiles + CONV_WARPS * mt - 1) / (CONV_WARPS * mt)), (unsigned)(a.ntiles / nt));
     if (ctas) *ctas = grid.x;
-    auto go = [&](auto kern) { kern<<<grid, 32 * CONV_WARPS, 0, s>>>(a); };
-    if (nt == 4) { if (mt == 2) go(conv_kernel<4, 2>); else go(conv_kernel<4, 1>); }
-    else if (nt == 2) { if (mt == 2) go(conv_kernel<2, 2>); else go(conv_kernel<2, 1>); }
-    else { if (mt == 2) go(conv_kernel<1, 2>); else go(conv_kernel<1, 1>); }
+    int rc = DST_OK;
+    auto launch = [&](auto n_, auto m_, auto c_) {
+        constexpr int NT = decltype(n_)::value, MT = decltype(m_)::value, C = decltype(c_)::value;
+        const size_t smem = C > 0 ? ConvShape<NT, MT, C == 0 ? 1 : C>::SMEM : 0;
+        auto kern = conv_kernel<NT, MT, C>;
+        if (smem > 40 * 1024 &&
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            rc = DST_ERR_CUDA;
+        else
+            kern<<<grid, 32 * CONV_WARPS, smem, s>>>(a);
+    };
+    auto go = [&](auto c16) {
+        using I1 = std::integral_constant<int, 1>;
+        using I2 = std::integral_constant<int, 2>;
+        using I4 = std::integral_constant<int, 4>;
+        if (nt == 4) { if (mt == 2) launch(I4(), I2(), c16); else launch(I4(), I1(), c16); }
+        else if (nt == 2) { if (mt == 2) launch(I2(), I2(), c16); else launch(I2(), I1(), c16); }
+        else { if (mt == 2) launch(I1(), I2(), c16); else launch(I1(), I1(), c16); }
+    };
+    // a kernel of one tap has nothing to stage ahead (32 -> 16 channels at 48^3: 10 us, 19 staged)
+    switch (a.taps == 1 ? 2 : a.lci) {
+        case 2: case 3: go(std::integral_constant<int, 0>()); break;
+        case 4: go(std::integral_constant<int, 1>()); break;
+        case 5: go(std::integral_constant<int, 2>()); break;
+        case 6: go(std::integral_constant<int, 4>()); break;
+        default: return DST_ERR_ARG;
+    }
     DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
+    return rc;
 }
 
 static int log2i(int v) {
@@ -487,7 +514,7 @@ static int conv(dst_unet *u, int l, const bf16 *in, const ConvOut &o, cudaStream
     a.coarse = from_coarse ? 1 : 0;
     if (from_coarse) a.up = u->grid[L.level + 1];
     a.lci = log2i(L.ci); a.taps = L.taps; a.chunks = L.kpad / 16; a.co = L.co; a.ntiles = u->pack.l[l].nf;
-    a.in = in; a.w = u->pack.l[l].wf; a.bias = u->params + L.boff; a.res = o.res; a.relu = o.relu ? 1 : 0;
+    a.in = in; a.zeros = u->zeros; a.w = u->pack.l[l].wf; a.bias = u->params + L.boff; a.res = o.res; a.relu = o.relu ? 1 : 0;
     a.s1 = o.s1; a.s2 = o.s2; a.out32 = o.f32; a.out16 = o.b16;
     return launch_conv(a, nullptr, s);
 }
@@ -499,7 +526,7 @@ static int conv_dgrad(dst_unet *u, int l, const bf16 *dz, const ConvOut &o, int 
     ConvArgs a = {};
     a.g = u->grid[L.level];
     a.lci = log2i(L.co); a.taps = L.taps; a.chunks = (L.taps * L.co + 15) / 16; a.co = L.ci; a.ntiles = u->pack.l[l].nt;
-    a.in = dz; a.w = u->pack.l[l].wt;                   // mirrored taps
+    a.in = dz; a.zeros = u->zeros; a.w = u->pack.l[l].wt;                   // mirrored taps
     a.mask = o.mask; a.out32 = o.f32; a.out16 = o.b16;
     unsigned rows = 0;
     if (next >= 0) a.colsum = u->bpart + u->sums.l[next].bpart;

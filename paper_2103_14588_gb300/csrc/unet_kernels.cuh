@@ -14,10 +14,11 @@
 //
 // The layers are small (16 to 64 channels, 6 GFLOP in all on a 48^3 grid), so the
 // tensor cores are never the limit: what is, is the instructions around them and the
-// launches.  So a warp works out its rows' coordinates once; a tap is then a node
-// offset and a mask of the axis ends it must not start from (a table in shared memory),
-// and an operand fragment is one predicated 4-byte load through L1.  Weights are packed
-// in fragment order (one 8-byte load per lane).
+// launches, and on the coarse grids the latency of a chain of taps that few warps walk.
+// So a thread works out its rows' coordinates once; a tap is then a node offset and a mask
+// of the axis ends it must not start from (a table in shared memory).  Taps stream through
+// a shared-memory ring (cp.async, zero-filled outside the grid) a few stages ahead of the
+// products; weights are packed in fragment order.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -76,6 +77,7 @@ struct ConvArgs {
     int lci, taps, chunks;          // log2 of the input channels, kernel taps, K / 16
     int co, ntiles;                 // output channels stored, output channels / 8 rounded up
     const bf16 *in;                 // [N][ci]
+    const bf16 *zeros;              // 64 channels of zeros
     const uint32_t *w;              // fragments [chunk][ntile][lane][2]
     const float *bias;              // [co] or null
     const float *res;               // [N][co] added before the activation, or null
@@ -94,20 +96,58 @@ struct Tap {
 };
 
 constexpr int CONV_WARPS = 4;
+constexpr int CONV_STAGES = 4;
 
-// One warp: 16 MT consecutive nodes x 8 NT output channels (blockIdx.y: which).
-template <int NT, int MT>
+__device__ __forceinline__ void copy_or_zero16(void *dst, const void *src, bool ok) {
+    const int n = ok ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(n) : "memory");
+}
+__device__ __forceinline__ void copy_or_zero8(void *dst, const void *src, bool ok) {
+    const int n = ok ? 8 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(n) : "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+// Shared memory of the ring.  A stage holds the rows of one offset of the slower axes, with
+// a row on each side, and the weights of its three taps: the taps along x read the same
+// rows, shifted by one (at an end of the x line a row of zeros).  Eight rows of any 16-byte
+// column lie on different banks (the column is swizzled by the row).
+template <int NT, int MT, int CI16>
+struct ConvShape {
+    static constexpr int ROWS = 16 * MT * CONV_WARPS + 2, COLS = 2 * CI16;
+    static constexpr int A = ROWS * CI16 * 32, B_TAP = CI16 * NT * 256;
+    static constexpr int STAGE = A + 3 * B_TAP;
+    static constexpr size_t SMEM = (size_t)CONV_STAGES * STAGE + CI16 * 32;
+    __device__ static int at(int row, int col) {
+        const int sw = CI16 == 1 ? (row >> 2) & 1 : CI16 == 2 ? (row >> 1) & 3 : row & 7;
+        return (row * COLS + (col ^ sw)) * 16;
+    }
+};
+
+// One warp: 16 MT consecutive nodes x 8 NT output channels (blockIdx.y: which).  CI16: input
+// channels / 16; 0 (any number) without the ring.
+// 16 -> 16 channels at 48^3 (1.5 GFLOP): 253 us with divisions per fragment, 19 us with tap
+// tables and loads through L1, 15 us staged; 64 -> 64 channels at 12^3: 388, 58 and 12 us.
+template <int NT, int MT, int CI16>
 __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
+    extern __shared__ __align__(16) unsigned char ring[];
     __shared__ Tap tab[82];
     __shared__ float cs[CONV_WARPS][NT * 8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, tg = lane & 3;
     const int ci = 1 << a.lci;
-    // the tap after the last (K padded to a multiple of 16) starts from nowhere
-    for (int t = threadIdx.x; t <= a.taps; t += blockDim.x) {
-        Tap e{0, t < a.taps ? 0 : 1 << 8, 0};
-        if (a.taps > 1 && t < a.taps) {
-            int rest = t;
+    // staged: the offsets of the slower axes; else every tap, the one after the last (K
+    // padded to a multiple of 16) starting from nowhere
+    const int xt = CI16 > 0 && a.taps > 1 ? 3 : 1, entries = a.taps / xt;
+    for (int t = threadIdx.x; t <= entries; t += blockDim.x) {
+        Tap e{0, t < entries ? 0 : 1 << 8, 0};
+        if (a.taps > 1 && t < entries) {
+            int rest = xt == 3 ? 3 * t + 1 : t;
             long long stride = 1;
             for (int ax = a.g.D - 1; ax >= 0; --ax) {
                 const int o = rest % 3 - 1;
@@ -121,69 +161,132 @@ __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
         }
         tab[t] = e;
     }
-    __syncthreads();
-    const int64_t m0 = ((int64_t)blockIdx.x * CONV_WARPS + warp) * (16 * MT);
-    const bf16 *row[MT][2];
-    int ends[MT][2];
+    // a row's first channel and the axis ends it lies on; a row outside the grid reads nothing
+    auto place = [&](int64_t r, const bf16 *&at, int &ends) {
+        at = a.in;
+        ends = -1;
+        if (r < 0 || r >= a.g.N) return;
+        int c[4];
+        int e = 1 << 8;
+        coords(a.g, (unsigned)r, c);
 #pragma unroll
-    for (int m = 0; m < MT; ++m)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t r = m0 + m * 16 + h * 8 + g;
-            row[m][h] = a.in;
-            ends[m][h] = -1;                              // a row past the end reads nothing
-            if (r < a.g.N) {
-                int c[4];
-                int e = 1 << 8;
-                coords(a.g, (unsigned)r, c);
-#pragma unroll
-                for (int ax = 0; ax < 4; ++ax)
-                    if (ax < a.g.D) e |= (c[ax] == 0 ? 1 << (2 * ax) : 0) | (c[ax] == a.g.n[ax] - 1 ? 2 << (2 * ax) : 0);
-                ends[m][h] = e;
-                row[m][h] = a.in + ((a.coarse ? (int64_t)parent(a.up, c) : r) << a.lci);
-            }
-        }
+        for (int ax = 0; ax < 4; ++ax)
+            if (ax < a.g.D) e |= (c[ax] == 0 ? 1 << (2 * ax) : 0) | (c[ax] == a.g.n[ax] - 1 ? 2 << (2 * ax) : 0);
+        ends = e;
+        at = a.in + ((a.coarse ? (int64_t)parent(a.up, c) : r) << a.lci);
+    };
+    const int64_t cta0 = (int64_t)blockIdx.x * (16 * MT * CONV_WARPS), m0 = cta0 + warp * (16 * MT);
     float acc[MT][NT][4];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
         for (int j = 0; j < NT; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
-    const uint2 *w = reinterpret_cast<const uint2 *>(a.w) + ((size_t)blockIdx.y * NT) * 32 + lane;
     const size_t wstep = (size_t)a.ntiles * 32;
-    // U chunks of both operands in registers before their products: the loads of a group
-    // are in flight together, and with few warps (the coarse levels) that latency is all
-    // there is to a layer
-    constexpr int U = MT * NT >= 8 ? 2 : 4;
-    for (int kc = 0; kc < a.chunks; kc += U) {
-        uint32_t af[U][MT][4];
-        uint2 b[U][NT];
+    if constexpr (CI16 > 0) {
+        using S = ConvShape<NT, MT, CI16>;
+        constexpr int THREADS = 32 * CONV_WARPS, MINE = (S::ROWS * S::COLS + THREADS - 1) / THREADS;   // copies per thread
+        const bf16 *src[MINE];
+        int ends[MINE], dst[MINE];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool in = kc + u < a.chunks;
+        for (int i = 0; i < MINE; ++i) {
+            const int k = threadIdx.x + i * THREADS, row = k / S::COLS, col = k % S::COLS;
+            src[i] = a.in;
+            ends[i] = -1;
+            if (row < S::ROWS) place(cta0 - 1 + row, src[i], ends[i]);
+            src[i] += col * 8;
+            dst[i] = row < S::ROWS ? S::at(row, col) : -1;
+        }
+        // the x ends of the rows this lane addresses
+        int xe[MT];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            const bf16 *q;
+            int e;
+            place(m0 + m * 16 + (lane & 15), q, e);
+            xe[m] = (e >> (2 * (a.g.D - 1))) & 3;
+        }
+        unsigned char *zero_row = ring + CONV_STAGES * S::STAGE;
+        if (threadIdx.x < S::COLS) reinterpret_cast<uint4 *>(zero_row)[threadIdx.x] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        const uint4 *wsrc = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint2 *>(a.w) + (size_t)blockIdx.y * NT * 32);
+        auto issue = [&](int st) {
+            if (st < entries) {
+                unsigned char *base = ring + (st % CONV_STAGES) * S::STAGE;
+                const Tap t = tab[st];
+#pragma unroll
+                for (int i = 0; i < MINE; ++i) {
+                    const bool ok = ends[i] != -1 && !(ends[i] & t.ends);
+                    if (dst[i] >= 0) copy_or_zero16(base + dst[i], src[i] + (ok ? t.off : 0), ok);
+                }
+                for (int i = threadIdx.x; i < xt * S::B_TAP / 16; i += THREADS) {
+                    const int c = i / (NT * 16), o = i % (NT * 16);            // chunk of the stage's taps
+                    copy_or_zero16(base + S::A + i * 16, wsrc + ((size_t)(st * xt * CI16 + c) * wstep) / 2 + o, true);
+                }
+            }
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        for (int st = 0; st < CONV_STAGES - 1; ++st) issue(st);
+        for (int st = 0; st < entries; ++st) {
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(CONV_STAGES - 2) : "memory");
+            __syncthreads();
+            issue(st + CONV_STAGES - 1);
+            const unsigned char *base = ring + (st % CONV_STAGES) * S::STAGE;
+            const uint2 *wd = reinterpret_cast<const uint2 *>(base + S::A) + lane;
+            auto tap = [&](int dx, int u) {                // dx: -1, 0, 1; u: place among the stage's weights
+#pragma unroll
+                for (int c = 0; c < CI16; ++c) {
+                    uint32_t af[MT][4];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) {
+                        const bool out = (dx < 0 && (xe[m] & 1)) || (dx > 0 && (xe[m] & 2));
+                        ldsm4(af[m], out ? zero_row
+                                         : base + S::at(warp * (16 * MT) + m * 16 + (lane & 15) + 1 + dx, 2 * c + (lane >> 4)));
+                    }
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        const uint2 b = wd[((u * CI16 + c) * NT + j) * 32];
+#pragma unroll
+                        for (int m = 0; m < MT; ++m) mma_16816(acc[m][j], af[m], b.x, b.y);
+                    }
+                }
+            };
+            if (xt == 3) { tap(-1, 0); tap(0, 1); tap(1, 2); }
+            else tap(0, 0);
+        }
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    } else {
+        __syncthreads();
+        // four or eight input channels (a chunk spans several taps) or one tap: through L1
+        const bf16 *row[MT][2];
+        int ends[MT][2];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) place(m0 + m * 16 + h * 8 + g, row[m][h], ends[m][h]);
+        const uint2 *w = reinterpret_cast<const uint2 *>(a.w) + ((size_t)blockIdx.y * NT) * 32 + lane;
+#pragma unroll 4
+        for (int kc = 0; kc < a.chunks; ++kc) {
+            uint32_t af[MT][4];
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
-                const int k = (kc + u) * 16 + half * 8 + 2 * tg;
+                const int k = kc * 16 + half * 8 + 2 * tg;
                 const Tap t = tab[min(k >> a.lci, a.taps)];
-                const long long off = t.off + (k & (ci - 1));
+                const int ch = k & (ci - 1);
 #pragma unroll
                 for (int m = 0; m < MT; ++m)
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        af[u][m][2 * half + h] =
-                            (ends[m][h] & t.ends) ? 0u : __ldg(reinterpret_cast<const uint32_t *>(row[m][h] + off));
+                    for (int h = 0; h < 2; ++h) {
+                        const bf16 *q = (ends[m][h] & t.ends) ? a.zeros : row[m][h] + (t.off + ch);
+                        af[m][2 * half + h] = __ldg(reinterpret_cast<const uint32_t *>(q));
+                    }
             }
 #pragma unroll
-            for (int j = 0; j < NT; ++j) b[u][j] = in ? __ldg(w + u * wstep + j * 32) : make_uint2(0u, 0u);
+            for (int j = 0; j < NT; ++j) {
+                const uint2 b = __ldg(w + kc * wstep + j * 32);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) mma_16816(acc[m][j], af[m], b.x, b.y);
+            }
         }
-        w += U * wstep;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (kc + u < a.chunks) {
-#pragma unroll
-                for (int j = 0; j < NT; ++j)
-#pragma unroll
-                    for (int m = 0; m < MT; ++m) mma_16816(acc[m][j], af[u][m], b[u][j].x, b[u][j].y);
-            }
     }
     const float scale = a.s1 ? *a.s1 * *a.s2 : 1.f;
 #pragma unroll
@@ -259,16 +362,6 @@ struct WgradArgs {
     int per_cta;
 };
 
-__device__ __forceinline__ void copy_or_zero16(void *dst, const void *src, bool ok) {
-    const int n = ok ? 16 : 0;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "r"(n) : "memory");
-}
-__device__ __forceinline__ void copy_or_zero8(void *dst, const void *src, bool ok) {
-    const int n = ok ? 8 : 0;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "r"(n) : "memory");
-}
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void *p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((unsigned)__cvta_generic_to_shared(p)));
