@@ -12,13 +12,41 @@
 
 namespace dst {
 
+// A warp's FP64 instruction holds its sub-partition's FP64 unit for 64 clocks (the unit takes
+// 1/64 of the FP32 rate), and the projection and the update do four of them per entry and
+// vector: a large vector is bound by those units, not by memory (1.77M entries x 15 vectors:
+// 178 us of FP64 against 67 us of bytes), and a small one is spread over as many CTAs as it has
+// 256-entry slices.
 static constexpr int RED_THREADS = 256;
-static constexpr int PROJ_GROUP = 8;     // basis vectors per register group
+static constexpr int PROJ_GROUP = 8;     // basis vectors whose loads are in flight together
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
+}
+
+// Sums of P values over the warp, scattered: returns q, and v[0] becomes the sum of value q.
+// Each step halves the values a lane carries (it keeps one half and adds the partner's), P
+// additions in all where P trees take 5 P: a reduction costs the FP64 unit as much as the
+// products of 20 entries per lane otherwise.
+template <int P>
+__device__ __forceinline__ int warp_scatter_sum(double (&v)[P]) {
+    const int lane = threadIdx.x & 31;
+    int q = 0, o = 16;
+#pragma unroll
+    for (int half = P / 2; half >= 1; half >>= 1, o >>= 1) {
+        const bool hi = lane & o;
+        if (hi) q += half;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double keep = hi ? v[i + half] : v[i], send = hi ? v[i] : v[i + half];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return q;
 }
 
 // Block sum of one double (result valid in thread 0); fixed order.
@@ -47,14 +75,59 @@ __device__ __forceinline__ void slice(int64_t n, int64_t &b, int64_t &e) {
     e = b + per < n ? b + per : n;
 }
 
+// True in every thread of the last CTA of the grid to get here (the caller's global writes
+// before it are visible to that CTA); *ticket is left at zero.
+__device__ __forceinline__ bool last_cta(unsigned *ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last && threadIdx.x == 0) *ticket = 0u;
+    __threadfence();
+    return last;
+}
+
+// Inner products of G basis vectors (the first at V) with w over the CTA's slice, summed over
+// the warp into red.  G is exact: a vector that is not there would still take its share of
+// the FP64 unit (predicated instructions occupy it), which once made one vector cost as much
+// as eight (1.77M entries: 127 us for one vector, 11.8 us of FP64 work).
+template <int G>
+__device__ __forceinline__ void project_group(int64_t n, int64_t b, int64_t e, const double2 *__restrict__ V,
+                                              const double2 *__restrict__ w, double *red, bool norm, double &wn) {
+    double ar[G], ai[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) { ar[g] = 0.0; ai[g] = 0.0; }
+    for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
+        const double2 wi = __ldg(w + i);
+        double2 v[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] = __ldg(V + g * n + i);
+        if (norm) wn = fma(wi.x, wi.x, fma(wi.y, wi.y, wn));
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            ar[g] = fma(v[g].x, wi.x, fma(v[g].y, wi.y, ar[g]));
+            ai[g] = fma(v[g].x, wi.y, fma(-v[g].y, wi.x, ai[g]));
+        }
+    }
+    constexpr int P = G > 4 ? 16 : (G > 2 ? 8 : (G > 1 ? 4 : 2));
+    double v[P];
+#pragma unroll
+    for (int g = 0; g < P / 2; ++g) { v[2 * g] = g < G ? ar[g] : 0.0; v[2 * g + 1] = g < G ? ai[g] : 0.0; }
+    const int q = warp_scatter_sum<P>(v);
+    if (q < 2 * G) red[q] = v[0];
+}
+
 // partials[blk * nvec + j] = sum over the CTA's slice of conj(V_j) w, and
-// (if wnrm_partials) partials of ||w||^2.  Threads accumulate PROJ_GROUP basis
+// (if wnrm_partials) partials of ||w||^2; with a ticket the last CTA sums them in CTA
+// order into h (and wnrm2).  Threads accumulate PROJ_GROUP basis
 // vectors at a time over their elements; each group is reduced across the warp
 // by shuffles and parked in shared memory; one barrier at the end, then the
 // warps' values are summed in warp order.
 __global__ void __launch_bounds__(RED_THREADS)
 project_partial_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const double2 *__restrict__ w,
-                       double2 *__restrict__ partials, double *__restrict__ wnrm_partials, const double *gate) {
+                       double2 *partials, double *wnrm_partials, const double *gate, unsigned *ticket,
+                       double2 *__restrict__ h, double *__restrict__ wnrm2) {
     if (dgks_skip(gate)) return;
     constexpr int NW = RED_THREADS / 32;
     __shared__ double red[NW][2 * DST_MAX_VEC + 1];
@@ -63,28 +136,18 @@ project_partial_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const
     slice(n, b, e);
     double wn = 0.0;
     for (int j0 = 0; j0 < nvec; j0 += PROJ_GROUP) {
-        const int gv = nvec - j0 < PROJ_GROUP ? nvec - j0 : PROJ_GROUP;
-        double ar[PROJ_GROUP], ai[PROJ_GROUP];
-#pragma unroll
-        for (int g = 0; g < PROJ_GROUP; ++g) { ar[g] = 0.0; ai[g] = 0.0; }
-        for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
-            const double2 wi = w[i];
-            if (j0 == 0) wn = fma(wi.x, wi.x, fma(wi.y, wi.y, wn));
-#pragma unroll
-            for (int g = 0; g < PROJ_GROUP; ++g) {
-                if (g < gv) {
-                    const double2 v = V[(int64_t)(j0 + g) * n + i];
-                    ar[g] = fma(v.x, wi.x, fma(v.y, wi.y, ar[g]));
-                    ai[g] = fma(v.x, wi.y, fma(-v.y, wi.x, ai[g]));
-                }
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < PROJ_GROUP; ++g) {
-            if (g < gv) {
-                const double sr = warp_sum(ar[g]), si = warp_sum(ai[g]);
-                if (lane == 0) { red[warp][2 * (j0 + g)] = sr; red[warp][2 * (j0 + g) + 1] = si; }
-            }
+        const double2 *Vj = V + (int64_t)j0 * n;
+        double *r = &red[warp][2 * j0];
+        const bool norm = wnrm_partials && j0 == 0;
+        switch (min(nvec - j0, PROJ_GROUP)) {
+            case 1: project_group<1>(n, b, e, Vj, w, r, norm, wn); break;
+            case 2: project_group<2>(n, b, e, Vj, w, r, norm, wn); break;
+            case 3: project_group<3>(n, b, e, Vj, w, r, norm, wn); break;
+            case 4: project_group<4>(n, b, e, Vj, w, r, norm, wn); break;
+            case 5: project_group<5>(n, b, e, Vj, w, r, norm, wn); break;
+            case 6: project_group<6>(n, b, e, Vj, w, r, norm, wn); break;
+            case 7: project_group<7>(n, b, e, Vj, w, r, norm, wn); break;
+            default: project_group<8>(n, b, e, Vj, w, r, norm, wn); break;
         }
     }
     wn = warp_sum(wn);
@@ -102,14 +165,35 @@ project_partial_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const
         for (int k = 0; k < NW; ++k) s_ += red[k][2 * DST_MAX_VEC];
         wnrm_partials[blockIdx.x] = s_;
     }
+    if (ticket && last_cta(ticket)) {
+        const int blocks = gridDim.x;
+        for (int q = threadIdx.x; q < 2 * nvec + (wnrm2 ? 1 : 0); q += RED_THREADS) {
+            const bool nr = q == 2 * nvec;
+            const double *p = nr ? wnrm_partials : reinterpret_cast<const double *>(partials) + q;
+            const int step = nr ? 1 : 2 * nvec;
+            double t = 0.0;
+#pragma unroll 8
+            for (int k = 0; k < blocks; ++k) t += __ldcg(p + (int64_t)k * step);
+            if (nr) *wnrm2 = t;
+            else reinterpret_cast<double *>(h)[q] = t;
+        }
+    }
 }
 
-// out[j] = sum_blk partials[blk * nvec + j]   (one CTA per j)
+// out[j] = sum_blk partials[blk * nvec + j] (one CTA per j; one more for the norm's partials)
 __global__ void __launch_bounds__(RED_THREADS)
 reduce_partials_kernel(int nblk, int nvec, const double2 *__restrict__ partials, double2 *__restrict__ out,
-                       const double *gate) {
+                       const double *gate, const double *__restrict__ wnrm_partials, double *__restrict__ wnrm2) {
     __shared__ double sh[RED_THREADS / 32];
     const int j = blockIdx.x;
+    if (j == nvec) {
+        if (dgks_skip(gate)) return;
+        double t = 0.0;
+        for (int k = threadIdx.x; k < nblk; k += RED_THREADS) t += wnrm_partials[k];
+        t = block_sum(t, sh);
+        if (threadIdx.x == 0) *wnrm2 = t;
+        return;
+    }
     if (dgks_skip(gate)) {
         if (threadIdx.x == 0) out[j] = make_double2(0.0, 0.0);
         return;
@@ -125,10 +209,26 @@ reduce_partials_kernel(int nblk, int nvec, const double2 *__restrict__ partials,
     if (threadIdx.x == 0) out[j] = make_double2(sr, si);
 }
 
-// w <- w - sum_j V_j h_j ; partial ||w||^2 per CTA.
-__global__ void __launch_bounds__(RED_THREADS)
+// acc -= sum over G vectors of V_g c_g at one entry, the loads together
+template <int G>
+__device__ __forceinline__ void subtract(int64_t n, const double2 *__restrict__ V, const double2 *c, double2 &acc) {
+    double2 v[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) v[g] = __ldg(V + g * n);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        acc.x = fma(-v[g].x, c[g].x, fma(v[g].y, c[g].y, acc.x));
+        acc.y = fma(-v[g].x, c[g].y, fma(-v[g].y, c[g].x, acc.y));
+    }
+}
+
+// w <- w - sum_j V_j h_j ; partial ||w||^2 per CTA, with a ticket summed by the last CTA
+// into *nrm2 (and *counter bumped).  Four CTAs per SM, so that the 608 of a large vector are
+// one wave.  1.77M entries x 15 vectors: projection 265 -> 215 us, update 201 -> 199 us.
+__global__ void __launch_bounds__(RED_THREADS, 4)
 update_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const double2 *__restrict__ h,
-              double2 *__restrict__ w, double *__restrict__ nrm_partials, const double *gate) {
+              double2 *__restrict__ w, double *nrm_partials, const double *gate, unsigned *ticket, double *nrm2,
+              double *counter) {
     if (dgks_skip(gate)) return;
     __shared__ double2 hs[DST_MAX_VEC];
     __shared__ double sh[RED_THREADS / 32];
@@ -139,17 +239,26 @@ update_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const double2 
     double nr = 0.0;
     for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
         double2 acc = w[i];
-        for (int j = 0; j < nvec; ++j) {
-            const double2 v = V[(int64_t)j * n + i];
-            const double2 c = hs[j];
-            acc.x = fma(-v.x, c.x, fma(v.y, c.y, acc.x));
-            acc.y = fma(-v.x, c.y, fma(-v.y, c.x, acc.y));
-        }
+        int j = 0;
+        for (; j + PROJ_GROUP <= nvec; j += PROJ_GROUP) subtract<PROJ_GROUP>(n, V + (int64_t)j * n + i, hs + j, acc);
+        if (nvec & 4) { subtract<4>(n, V + (int64_t)j * n + i, hs + j, acc); j += 4; }
+        if (nvec & 2) { subtract<2>(n, V + (int64_t)j * n + i, hs + j, acc); j += 2; }
+        if (nvec & 1) subtract<1>(n, V + (int64_t)j * n + i, hs + j, acc);
         w[i] = acc;
-        nr = fma(acc.x, acc.x, fma(acc.y, acc.y, nr));
+        if (nrm_partials) nr = fma(acc.x, acc.x, fma(acc.y, acc.y, nr));
     }
+    if (!nrm_partials) return;
     nr = block_sum(nr, sh);
-    if (threadIdx.x == 0 && nrm_partials) nrm_partials[blockIdx.x] = nr;
+    if (threadIdx.x == 0) nrm_partials[blockIdx.x] = nr;
+    if (ticket && last_cta(ticket)) {
+        double t = 0.0;
+        for (int k = threadIdx.x; k < (int)gridDim.x; k += RED_THREADS) t += __ldcg(nrm_partials + k);
+        t = block_sum(t, sh);
+        if (threadIdx.x == 0) {
+            *nrm2 = t;
+            if (counter) *counter += 1.0;
+        }
+    }
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
@@ -330,33 +439,21 @@ static unsigned stream_blocks(int64_t n) {
 }
 
 int dst_k_project(int64_t n, int nvec, const double2 *V, const double2 *w, double2 *h, double2 *partials,
-                  int nblk, cudaStream_t s, double *wnrm2, double *wnrm_partials, const double *gate) {
+                  int nblk, cudaStream_t s, double *wnrm2, double *wnrm_partials, const double *gate, unsigned *ticket) {
+    const bool fused = ticket && nblk * nvec <= DST_FUSED_PARTIALS;
     project_partial_kernel<<<nblk, RED_THREADS, 0, s>>>(n, nvec, V, w, partials, wnrm2 ? wnrm_partials : nullptr,
-                                                        gate);
-    reduce_partials_kernel<<<nvec, RED_THREADS, 0, s>>>(nblk, nvec, partials, h, gate);
-    if (wnrm2) reduce_real_kernel<<<1, RED_THREADS, 0, s>>>(nblk, wnrm_partials, wnrm2, gate, nullptr);
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
-}
-
-int dst_k_reduce_partials(int nblk, int nvec, const double2 *partials, double2 *out, cudaStream_t s,
-                          const double *gate) {
-    reduce_partials_kernel<<<nvec, RED_THREADS, 0, s>>>(nblk, nvec, partials, out, gate);
-    DST_CUDA_TRY(cudaGetLastError());
-    return DST_OK;
-}
-
-int dst_k_reduce_real(int nblk, const double *partials, double *out, cudaStream_t s, const double *gate,
-                      double *counter) {
-    reduce_real_kernel<<<1, RED_THREADS, 0, s>>>(nblk, partials, out, gate, counter);
+                                                        gate, fused ? ticket : nullptr, h, wnrm2);
+    if (!fused)
+        reduce_partials_kernel<<<nvec + (wnrm2 ? 1 : 0), RED_THREADS, 0, s>>>(nblk, nvec, partials, h, gate,
+                                                                              wnrm_partials, wnrm2);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
 
 int dst_k_update(int64_t n, int nvec, const double2 *V, const double2 *h, double2 *w, double *nrm2,
-                 double *partials, int nblk, cudaStream_t s, const double *gate, double *counter) {
-    update_kernel<<<nblk, RED_THREADS, 0, s>>>(n, nvec, V, h, w, nrm2 ? partials : nullptr, gate);
-    if (nrm2) reduce_real_kernel<<<1, RED_THREADS, 0, s>>>(nblk, partials, nrm2, gate, counter);
+                 double *partials, int nblk, cudaStream_t s, const double *gate, double *counter, unsigned *ticket) {
+    update_kernel<<<nblk, RED_THREADS, 0, s>>>(n, nvec, V, h, w, nrm2 ? partials : nullptr, gate, ticket, nrm2, counter);
+    if (nrm2 && !ticket) reduce_real_kernel<<<1, RED_THREADS, 0, s>>>(nblk, partials, nrm2, gate, counter);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
@@ -442,15 +539,23 @@ int dst_k_axpy1(int64_t n, const double2 *d, double2 *x, cudaStream_t s) {
     return DST_OK;
 }
 
-int dst_projection_blocks(int64_t n) {
-    int64_t b = (n + 4095) / 4096;
-    if (b > 456) b = 456;
+int dst_reduction_blocks(int64_t n) {
+    int64_t b = (n + RED_THREADS - 1) / RED_THREADS;
+    if (b > DST_MAX_RED_BLOCKS) b = DST_MAX_RED_BLOCKS;
     return (int)(b < 1 ? 1 : b);
 }
 
-int dst_reduction_blocks(int64_t n) {
+// CTAs of the df32 / FP32-basis kernels of blas_df.cu
+int dst_df_blocks(int64_t n) {
     int64_t b = (n + 2047) / 2048;
     if (b > DST_MAX_RED_BLOCKS) b = DST_MAX_RED_BLOCKS;
+    return (int)(b < 1 ? 1 : b);
+}
+
+// ... and of its projection of hi/lo vectors (longer slices)
+int dst_projection_blocks(int64_t n) {
+    int64_t b = (n + 4095) / 4096;
+    if (b > 456) b = 456;
     return (int)(b < 1 ? 1 : b);
 }
 

@@ -5,15 +5,22 @@
 
 #define DST_MAX_VEC 64            // basis vectors one projection / update handles
 #define DST_MAX_RED_BLOCKS 608    // CTAs of a reduction pass (4 per SM)
+// Partial sums of a projection that the last CTA to finish adds up by itself; more are left to a
+// second kernel with a CTA per vector (608 x 30 would take one CTA 9 us of FP64 additions).
+#define DST_FUSED_PARTIALS 2048
 #define DST_MAX_DEVICES 64        // device ordinals the static-scratch entry point tracks
 
-int dst_reduction_blocks(int64_t n);
+int dst_reduction_blocks(int64_t n);     // FP64 kernels
+int dst_df_blocks(int64_t n);
 int dst_projection_blocks(int64_t n);
+// ticket (zero, left at zero): few partials are summed in the kernel by the last CTA; null: by a
+// second kernel.
 int dst_k_project(int64_t n, int nvec, const double2 *V, const double2 *w, double2 *h, double2 *partials,
                   int nblk, cudaStream_t s, double *wnrm2 = nullptr, double *wnrm_partials = nullptr,
-                  const double *gate = nullptr);
+                  const double *gate = nullptr, unsigned *ticket = nullptr);
 int dst_k_update(int64_t n, int nvec, const double2 *V, const double2 *h, double2 *w, double *nrm2,
-                 double *partials, int nblk, cudaStream_t s, const double *gate = nullptr, double *counter = nullptr);
+                 double *partials, int nblk, cudaStream_t s, const double *gate = nullptr, double *counter = nullptr,
+                 unsigned *ticket = nullptr);
 int dst_k_nrm2(int64_t n, const double2 *x, double *nrm2, double *partials, int nblk, cudaStream_t s);
 int dst_k_residual(int64_t n, const double2 *b, const double2 *y, double2 *r, double *nrm2, double *partials,
                    int nblk, cudaStream_t s);

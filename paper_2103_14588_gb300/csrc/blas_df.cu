@@ -1286,9 +1286,9 @@ extern "C" int dst_testing_fp32_arnoldi(int mode, int64_t n, int nvec, const voi
         return DST_ERR_ARG;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    const int nblk_reg = std::min(dst_reduction_blocks(n), 3 * 152);
+    const int nblk_reg = std::min(dst_df_blocks(n), 3 * 152);
     const int nblk = (mode == 1 || mode == 3 || mode == 5) ? dst_tma_projection_blocks(n)
-                                                            : (mode == 2 ? dst_reduction_blocks(n) : nblk_reg);
+                                                            : (mode == 2 ? dst_df_blocks(n) : nblk_reg);
     const size_t pbytes = sizeof(double2) * (size_t)nblk * (nvec + 1);
     char *scr = nullptr;
     if (cudaMallocAsync((void **)&scr, pbytes + 256 + 256, s) != cudaSuccess) {

@@ -283,7 +283,8 @@ struct Solver {
     dst_mesh *mesh;
     cudaStream_t s;
     Workspace w;
-    int nblk;         // CTAs of the reduction / update passes
+    int nblk;         // CTAs of the FP64 reduction / update passes
+    int nblk_df;      // CTAs of the df32 update
     int nblk_proj;    // CTAs of the df32 projection (fewer, longer slices)
     double bytes = 0.0;
     int iters = 0;
@@ -332,17 +333,15 @@ struct Solver {
     // they ran (second_pass_ran() after the step's synchronisation).
     int project(int nv, const double2 *wv, double2 *h, double *wnrm2 = nullptr, const double *gate = nullptr) {
         const double n = (double)w.n;
-        return run(K_PROJECT, wnrm2 ? 3 : 2, gate ? 0.0 : 16.0 * n * (nv + 1),
-                   gate ? 0.0 : 8.0 * n * nv + (wnrm2 ? 4.0 * n : 0.0),
-                   [&] { return dst_k_project(w.n, nv, w.V, wv, h, w.partials_c, nblk, s, wnrm2, w.partials_r, gate); });
+        return run(K_PROJECT, nblk * nv <= DST_FUSED_PARTIALS ? 1 : 2, gate ? 0.0 : 16.0 * n * (nv + 1), gate ? 0.0 : 8.0 * n * nv + (wnrm2 ? 4.0 * n : 0.0),
+                   [&] { return dst_k_project(w.n, nv, w.V, wv, h, w.partials_c, nblk, s, wnrm2, w.partials_r, gate,
+                                              w.tickets); });
     }
-    // second: the step's second Gram-Schmidt pass (bumps the device counter nrm[6] when it runs)
-    int update(int nv, const double2 *h, double2 *x, double *nrm2, const double *gate = nullptr, bool second = false) {
+    // second: the counter of second passes to bump when it runs
+    int update(int nv, const double2 *h, double2 *x, double *nrm2, const double *gate = nullptr, double *second = nullptr) {
         const double n = (double)w.n;
-        return run(K_UPDATE, nrm2 ? 2 : 1, gate ? 0.0 : 16.0 * n * (nv + 2),
-                   gate ? 0.0 : 8.0 * n * nv + (nrm2 ? 4.0 * n : 0.0),
-                   [&] { return dst_k_update(w.n, nv, w.V, h, x, nrm2, w.partials_r, nblk, s, gate,
-                                             second ? w.nrm + 6 : nullptr); });
+        return run(K_UPDATE, 1, gate ? 0.0 : 16.0 * n * (nv + 2), gate ? 0.0 : 8.0 * n * nv + (nrm2 ? 4.0 * n : 0.0),
+                   [&] { return dst_k_update(w.n, nv, w.V, h, x, nrm2, w.partials_r, nblk, s, gate, second, w.tickets + 1); });
     }
     // account a gated second pass over nv basis vectors that did run
     // bytes of a second Gram-Schmidt pass that ran (vb: bytes per stored entry)
@@ -354,8 +353,8 @@ struct Solver {
         prof.bytes[K_UPDATE] += ub; prof.flops[K_UPDATE] += 8.0 * n * nv;
         bytes += pb + ub;
     }
-    int scale(double2 *v) {
-        return run(K_SCALE, 1, 32.0 * w.n, 2.0 * w.n, [&] { return dst_k_scale(w.n, v, v, w.nrm, 0.0, s); });
+    int scale(double2 *v, const double *nrm2) {
+        return run(K_SCALE, 1, 32.0 * w.n, 2.0 * w.n, [&] { return dst_k_scale(w.n, v, v, nrm2, 0.0, s); });
     }
     int residual(const double2 *rhs, const double2 *y, double2 *r, double *nrm2) {
         return run(K_MISC, 2, 48.0 * w.n, 6.0 * w.n,
@@ -398,24 +397,6 @@ struct Solver {
         return DST_OK;
     }
 
-    // One host synchronisation per Arnoldi step: both Gram-Schmidt columns and
-    // the norms / second-pass counter (nrm[0..7]) come back together.
-    double reorth_seen = 0.0;
-    bool last_second = false;
-    int read_step(int nv) {
-        DST_CUDA_TRY(cudaMemcpyAsync(w.host, w.h1, sizeof(double2) * nv, cudaMemcpyDeviceToHost, s));
-        DST_CUDA_TRY(cudaMemcpyAsync(w.host + 2 * DST_MAX_VEC, w.h2, sizeof(double2) * nv, cudaMemcpyDeviceToHost, s));
-        DST_CUDA_TRY(cudaMemcpyAsync(w.host + 4 * DST_MAX_VEC, w.nrm, 8 * sizeof(double), cudaMemcpyDeviceToHost, s));
-        int rc = sync();
-        if (rc) return rc;
-        const double cnt = w.host[4 * DST_MAX_VEC + 6];
-        last_second = cnt > reorth_seen;
-        reorth_seen = cnt;
-        if (last_second) ++reorths;
-        return DST_OK;
-    }
-    bool second_pass_ran() const { return last_second; }
-
     // Hessenberg column j from the host buffer (first pass at host[0], second
     // pass at host[2*MAXVEC], new norm^2 at host[4*MAXVEC]) into hs; returns
     // DST_ERR_NAN on a non-finite column.
@@ -430,19 +411,25 @@ struct Solver {
         breakdown = std::sqrt(hn2) <= 1e-14 * std::sqrt(colsq + hn2);
         return DST_OK;
     }
-    int take_column(Hess &hs, int j, bool &breakdown) {
+    // Arnoldi step j of an FP64 cycle, enqueued; its record goes to w.cols.
+    int enqueue_step64(int prec, int j) {
+        double2 *vj = w.V + (size_t)j * w.n, *wv = vj + w.n;
+        double *rec = w.cols + (size_t)j * COL_STRIDE, *nr = rec + 4 * DST_MAX_VEC;
+        double2 *c1 = reinterpret_cast<double2 *>(rec), *c2 = c1 + DST_MAX_VEC;
         const int nv = j + 1;
-        std::vector<cplx> col(nv);
-        for (int i = 0; i < nv; ++i)
-            col[i] = cplx(w.host[2 * i] + w.host[2 * DST_MAX_VEC + 2 * i],
-                          w.host[2 * i + 1] + w.host[2 * DST_MAX_VEC + 2 * i + 1]);
-        const double hn2 = w.host[4 * DST_MAX_VEC];
-        double colsq = 0.0;
-        for (auto &c : col) colsq += std::norm(c);
-        if (!std::isfinite(hn2) || !std::isfinite(colsq)) return DST_ERR_NAN;
-        resid_est = hs.add_column(j, col.data(), std::sqrt(hn2));
-        breakdown = std::sqrt(hn2) <= 1e-14 * std::sqrt(colsq + hn2);
-        return DST_OK;
+        int rc;
+        if ((rc = apply(prec, vj, wv))) return rc;
+        // classical Gram-Schmidt pass; ||A v_j||^2 (before) into nr[3], ||w||^2 (after) into nr[0]
+        if ((rc = project(nv, wv, c1, nr + 3))) return rc;
+        if ((rc = update(nv, c1, wv, nr))) return rc;
+        // second pass, gated on the device by the DGKS test unless always on
+        // (CGS2) or never (ortho 2: the record's second-pass slots stay zero)
+        const double *gate = ortho == 1 ? nullptr : nr;
+        if (ortho != 2) {
+            if ((rc = project(nv, wv, c2, nullptr, gate))) return rc;
+            if ((rc = update(nv, c2, wv, nr, gate, nr + 6))) return rc;
+        }
+        return scale(wv, nr);                 // normalise on the device (1/sqrt(nr))
     }
 
     // Restarted GMRES(m) on A_prec x = rhs, FP64 basis and FP64 Gram-Schmidt,
@@ -451,7 +438,11 @@ struct Solver {
     // the residual (beta_out = -1).
     int gmres(int prec, double2 *x, const double2 *rhs, bool x_zero, double tol_abs, int max_iters,
               double &beta_out, int max_cycles = 0x7fffffff) {
-        if (ortho == 2) DST_CUDA_TRY(cudaMemsetAsync(w.h2, 0, sizeof(double2) * DST_MAX_VEC, s));
+        // Steps enqueued between host synchronisations.  Every step runs on the device, so a
+        // small mesh need not wait for the host after each (64 x 64: 16 us of kernels a step and
+        // about 20 us per synchronisation); the steps past the one that meets the tolerance
+        // have run in vain then, so a large mesh, whose steps take longer than that, waits.
+        const int batch = w.n < (1 << 18) ? 10 : 1;
         const int m = w.m;
         const int64_t n = w.n;
         double beta;
@@ -462,31 +453,31 @@ struct Solver {
         bool breakdown = false;
         int cycles = 0;
         while (beta > tol_abs && iters < max_iters && !breakdown) {
-            if ((rc = scale(w.V))) return rc;   // V0 = r / beta
+            if ((rc = scale(w.V, w.nrm))) return rc;   // V0 = r / beta
             hs.start(beta);
+            DST_CUDA_TRY(cudaMemsetAsync(w.cols, 0, sizeof(double) * COL_STRIDE * m, s));
             int k = 0;
-            for (int j = 0; j < m; ++j) {
-                double2 *vj = w.V + (size_t)j * n;
-                double2 *wv = w.V + (size_t)(j + 1) * n;
-                if ((rc = apply(prec, vj, wv))) return rc;
-                const int nv = j + 1;
-                // classical Gram-Schmidt pass; ||A v_j||^2 (before) into nrm[3], ||w||^2 (after) into nrm[0]
-                if ((rc = project(nv, wv, w.h1, w.nrm + 3))) return rc;
-                if ((rc = update(nv, w.h1, wv, w.nrm))) return rc;
-                // second pass, gated on the device by the DGKS test unless always on
-                // (CGS2) or never (ortho 2: w.h2 stays zero)
-                const double *gate = ortho == 1 ? nullptr : w.nrm;
-                if (ortho != 2) {
-                    if ((rc = project(nv, wv, w.h2, nullptr, gate))) return rc;
-                    if ((rc = update(nv, w.h2, wv, w.nrm, gate, true))) return rc;
+            for (bool done = false; !done && k < m;) {
+                const int first = k, steps = std::min(std::min(batch, m - k), max_iters - iters);
+                prof.chain = true;            // only kernels are enqueued until the loop ends
+                prof.last = -1;
+                for (int j = first; j < first + steps; ++j)
+                    if ((rc = enqueue_step64(prec, j))) return rc;
+                prof.chain = false;
+                const size_t at = (size_t)first * COL_STRIDE;
+                if ((rc = read_host(w.cols + at, sizeof(double) * COL_STRIDE * steps, w.host_cols + at)) || (rc = sync()))
+                    return rc;
+                for (int j = first; j < first + steps && !done; ++j) {
+                    const double *c1 = w.host_cols + (size_t)j * COL_STRIDE, *nr = c1 + 4 * DST_MAX_VEC;
+                    if (nr[6] > 0.0) {
+                        ++reorths;
+                        if (ortho != 1) count_second_pass(j + 1);
+                    }
+                    ++iters;
+                    if ((rc = take_column(hs, j, c1, c1 + 2 * DST_MAX_VEC, nr[0], breakdown))) return rc;
+                    k = j + 1;
+                    done = breakdown || resid_est <= tol_abs || iters >= max_iters;
                 }
-                if ((rc = scale(wv))) return rc;     // normalise on the device (1/sqrt(nrm))
-                if ((rc = read_step(nv))) return rc;
-                if (second_pass_ran() && gate) count_second_pass(nv);
-                ++iters;
-                if ((rc = take_column(hs, j, breakdown))) return rc;
-                k = j + 1;
-                if (breakdown || resid_est <= tol_abs || iters >= max_iters) break;
             }
             // x += V y  (update with h = -y)
             hs.solve(k, w.host, -1.0);
@@ -638,7 +629,7 @@ struct Solver {
             if ((rc = run(K_UPDATE, 1, vb * dn * nv + 8.0 * dn + vb * dn, 8.0 * dn * nv, [&] {
                      return use_tma ? dst_k_update_tma(n, nv, Vd, c1, wv, nr, w.partials_r, nblk_tma, s, nullptr,
                                                        nullptr, w.tickets + 1, nr + 7)
-                                    : dst_k_update_df(n, nv, Vd, c1, wv, true, nr, w.partials_r, nblk, s, nullptr,
+                                    : dst_k_update_df(n, nv, Vd, c1, wv, true, nr, w.partials_r, nblk_df, s, nullptr,
                                                       nullptr, w.tickets + 1, vlo);
                  })))
                 return rc;
@@ -656,7 +647,7 @@ struct Solver {
             if (ortho != 2 && (rc = run(K_UPDATE, 1, g2 * vb * dn * (nv + 2), g2 * 8.0 * dn * nv, [&] {
                      return use_tma ? dst_k_update_tma(n, nv, Vd, c2, wv, nr, w.partials_r, nblk_tma, s, gate, nr + 6,
                                                        w.tickets + 1, nr + 7)
-                                    : dst_k_update_df(n, nv, Vd, c2, wv, !vlo, nr, w.partials_r, nblk, s, gate,
+                                    : dst_k_update_df(n, nv, Vd, c2, wv, !vlo, nr, w.partials_r, nblk_df, s, gate,
                                                       nr + 6, w.tickets + 1, vlo);
                  })))
                 return rc;
@@ -885,9 +876,10 @@ static int solve_impl(dst_mesh *mesh, const dst_solve_opts &o, double2 *psi, dst
     sv.mesh = mesh;
     sv.s = s;
     sv.nblk = dst_reduction_blocks(mesh->n_unknowns);
+    sv.nblk_df = dst_df_blocks(mesh->n_unknowns);
     // an FP32-stored basis moves half the bytes per entry: slices of 2048
     // entries, at most the 3 CTAs per SM that its projection's registers allow
-    sv.nblk_proj = mixed && o.mixed_ortho == 2 ? std::min(dst_reduction_blocks(mesh->n_unknowns), 3 * 152)
+    sv.nblk_proj = mixed && o.mixed_ortho == 2 ? std::min(dst_df_blocks(mesh->n_unknowns), 3 * 152)
                                                : dst_projection_blocks(mesh->n_unknowns);
     sv.ortho = o.ortho;
     sv.precond = o.precond;
