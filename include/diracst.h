@@ -300,7 +300,10 @@ DST_API int dst_solve(dst_mesh *mesh, const dst_solve_opts *opts, void *psi, dst
  * dst_set_apply_variant before the first solve).  1+1 and
  * 2+1 meshes have 3 shapes (0 = the default: 1+1 tiles of 256 nodes x 32
  * time layers, then 128 x 16 and 64 x 8; 2+1 tiles of 32 x 8 nodes x 8 layers,
- * then 32 x 8 x 4 and 16 x 8 x 8); 3+1 meshes have one.  dst_solve runs the
+ * then 32 x 8 x 4 and 16 x 8 x 8); 3+1 meshes have 2 (the layers of its tiles shared by as
+ * many CTAs as are resident at once, or by twice as many).  Meshes of fewer than 2^19
+ * unknowns, with an open axis or with a general potential take a kernel without tiles (as
+ * does FP64 in 1+1), which the shape does not change.  dst_solve runs the
  * autotuner on a mesh's first solve (in its own workspace).
  *
  * dst_tune_apply: times every shape of both precisions on the mesh (3 applies

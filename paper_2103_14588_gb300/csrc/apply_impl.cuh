@@ -93,6 +93,17 @@ __device__ __forceinline__ int64_t axis_nbr(const AxisDesc &a, int64_t i) {
     return (i >= 0 && i < a.n) ? i : -1;
 }
 
+// The same in 32 bits, for planes of fewer than 2^31 nodes: a 64-bit remainder costs about a
+// hundred instructions, and a tile's copy table takes three per box node.
+__device__ __forceinline__ int axis_nbr32(const AxisDesc &a, int i) {
+    const int n = (int)a.n;
+    if (a.bc == DST_BC_PERIODIC) {
+        if (i < 0) i += n;
+        return i < n ? i : (int)((unsigned)i % (unsigned)n);
+    }
+    return i >= 0 && i < n ? i : -1;
+}
+
 template <int D> struct Beta;   // beta = gamma^0 signs per component
 template <> struct Beta<1> { __device__ static constexpr int s(int c) { return c == 0 ? 1 : -1; } };
 template <> struct Beta<2> { __device__ static constexpr int s(int c) { return c == 0 ? 1 : -1; } };

@@ -294,8 +294,8 @@ inline int node_chunk(int64_t plane_threads, int64_t nt) {
 // Where the tiled kernels (apply_pipe.cuh and what builds on it) take over: every node with
 // the standard stencils, an x-only or no potential, and enough unknowns for their tiles to
 // fill the GPU.  Measured on both sides of 2^19 unknowns: 1+1 FP32 512^2 4.5 us here, 6.0
-// tiled, 1024^2 11.6 and 10.9; 2+1 FP32 48^3 4.5 and 6.2, 64^3 7.4 and 7.5, 96^3 16.2 and
-// 14.0, FP64 64^3 72 and 68; 3+1 FP32 16^4 10.2 and 25.4, 24^4 32 and 27.  Meshes with an open
+// tiled, 1024^2 11.6 and 7.9; 2+1 FP32 48^3 3.7 and 6.2, 64^3 7.4 and 4.9, 96^3 16.2 and
+// 9.2, FP64 64^3 72 and 66; 3+1 FP32 16^4 8.7 and 25.4, 24^4 27 and 20, FP64 24^4 354 and 331.  Meshes with an open
 // axis stay here at every size (2+1 96^3 FP32 14.5 us, 37.7 tiled).
 template <int D>
 inline bool tiles_pay(const OpParams &p) {

@@ -34,7 +34,6 @@ template <> struct PipeTile<1, 2> { static constexpr int TX = 64, TY = 1, TZ = 1
 template <> struct PipeTile<2, 0> { static constexpr int TX = 32, TY = 8, TZ = 1, TT = 8, RY = 2; };
 template <> struct PipeTile<2, 1> { static constexpr int TX = 32, TY = 8, TZ = 1, TT = 4, RY = 2; };
 template <> struct PipeTile<2, 2> { static constexpr int TX = 16, TY = 8, TZ = 1, TT = 8, RY = 2; };
-template <> struct PipeTile<3, 0> { static constexpr int TX = 16, TY = 4, TZ = 4, TT = 8, RY = 1; };
 
 template <int D, int NC, typename T, int TV = 0>
 struct PipeShape {
@@ -107,11 +106,11 @@ __device__ __forceinline__ void make_copy_plan(const OpParams &p, int64_t x0, in
         if (i >= S::BOX * S::CHUNKS) continue;
         const int node = i / S::CHUNKS, part = i % S::CHUNKS;
         const int bx = node % S::BX, by = (node / S::BX) % S::BY, bz = node / (S::BX * S::BY);
-        const int64_t gx = axis_nbr(p.ax[0], x0 - 1 + bx);
-        const int64_t gy = D >= 2 ? axis_nbr(p.ax[1], y0 - 1 + by) : 0;
-        const int64_t gz = D >= 3 ? axis_nbr(p.ax[2], z0 - 1 + bz) : 0;
+        const int gx = axis_nbr32(p.ax[0], (int)x0 - 1 + bx);
+        const int gy = D >= 2 ? axis_nbr32(p.ax[1], (int)y0 - 1 + by) : 0;
+        const int gz = D >= 3 ? axis_nbr32(p.ax[2], (int)z0 - 1 + bz) : 0;
         cp.dst[j] = node * S::NODE_BYTES + part * 16;
-        if (gx >= 0 && gy >= 0 && gz >= 0) cp.src[j] = (int)(((gz * ny + gy) * nx + gx) * S::NODE_BYTES + part * 16);
+        if (gx >= 0 && gy >= 0 && gz >= 0) cp.src[j] = ((gz * (int)ny + gy) * (int)nx + gx) * S::NODE_BYTES + part * 16;
     }
 }
 
@@ -308,7 +307,8 @@ __device__ __forceinline__ void fields_std_rows(Get get, const StdConst<T> &sc, 
 // Ends with every copy complete; a caller that reuses the ring for another
 // tile synchronises the CTA first.
 template <int D, int NC, typename T, bool NOV, bool STD, int TV = 0>
-__device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const typename C2<T>::type *__restrict__ x,
+__device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdConst<T> &sc,
+                                                const typename C2<T>::type *__restrict__ x,
                                                 typename C2<T>::type *__restrict__ y, int64_t tiles_x,
                                                 int64_t tiles_y, int64_t tile, int64_t chunk, char *ring) {
     using V = typename C2<T>::type;
@@ -357,7 +357,6 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const typenam
         all_std = all_std && (sd || !valid[r]);
     }
     all_std = all_std && valid[0];
-    const StdConst<T> sc = std_const<D, T>(p);
     T wa[2], wb[2];  // mass-plus-potential weights of the standard path (fields_std), h_x / 6 in StdConst
     for (int sb = 0; sb < 2; ++sb) {
         const T wl = valid[0] ? k.wl[sb] : (T)0, wr = valid[0] ? k.wr[sb] : (T)0;
@@ -522,11 +521,11 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const typenam
 
 // Meshes without an open axis only (the launches send the others to apply_node.cuh).
 template <int D, int NC, typename T, bool NOV, int TV>
-__global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR, sizeof(T) == 8 ? 1 : (D == 3 ? 2 : 3))
-apply_pipe_kernel(OpParams p, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
+__global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR, sizeof(T) == 8 ? 1 : 3)
+apply_pipe_kernel(OpParams p, StdConst<T> sc, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
                   int64_t tiles_x, int64_t tiles_y) {
     extern __shared__ __align__(16) char ring[];
-    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, x, y, tiles_x, tiles_y, blockIdx.x, blockIdx.y, ring);
+    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, sc, x, y, tiles_x, tiles_y, blockIdx.x, blockIdx.y, ring);
 }
 
 template <int D, int NC, typename T, int TV>
@@ -552,31 +551,18 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
         DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
         if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[nov][dev] = true;
     }
-    kern<<<grid, S::NTHR, S::SMEM, s>>>(p, x, y, tx, ty);
+    kern<<<grid, S::NTHR, S::SMEM, s>>>(p, std_const<D, T>(p), x, y, tx, ty);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
 
-// Number of tile variants per spatial dimension (3+1: the one-output-per-thread
-// tiles of this file, and the z-columns of apply_zblk.cuh).
-constexpr int pipe_tile_variants(int d) { return d == 3 ? 2 : 3; }
-
-template <typename T, int RZ>
-int launch_apply_zblk(const OpParams &p, const typename C2<T>::type *x, typename C2<T>::type *y, cudaStream_t s);
-
-// Launch with the tile variant the parameters carry for this precision.
+// Launch with the tile variant the parameters carry for this precision (1+1 and 2+1).
 template <int D, int NC, typename T>
 int launch_apply_pipe(const OpParams &p, const typename C2<T>::type *x, typename C2<T>::type *y, cudaStream_t s) {
     const int tv = p.tile_variant[sizeof(T) == 4 ? DST_FP32 : DST_FP64];
-    if constexpr (D == 3) {
-        if (tv == 1) return launch_apply_zblk<T, sizeof(T) == 4 ? 4 : 2>(p, x, y, s);
-    }
-    if (D == 3 || tv <= 0) return launch_apply_pipe_v<D, NC, T, 0>(p, x, y, s);
-    if constexpr (D < 3) {
-        if (tv == 1) return launch_apply_pipe_v<D, NC, T, 1>(p, x, y, s);
-        return launch_apply_pipe_v<D, NC, T, 2>(p, x, y, s);
-    }
-    return DST_ERR_ARG;
+    if (tv <= 0) return launch_apply_pipe_v<D, NC, T, 0>(p, x, y, s);
+    if (tv == 1) return launch_apply_pipe_v<D, NC, T, 1>(p, x, y, s);
+    return launch_apply_pipe_v<D, NC, T, 2>(p, x, y, s);
 }
 
 }  // namespace dst

@@ -36,7 +36,7 @@ struct Pipe2hShape {
 
 template <int TV, bool NOV>
 __global__ void __launch_bounds__(Pipe2hShape<TV>::NTHR, 3)
-apply_pipe2h_kernel(OpParams p, const float2 *__restrict__ x, float2 *__restrict__ y, int64_t tiles_x) {
+apply_pipe2h_kernel(OpParams p, StdConst<float> sc, const float2 *__restrict__ x, float2 *__restrict__ y, int64_t tiles_x) {
     using S = Pipe2hShape<TV>;
     constexpr int RY = S::RY;
     extern __shared__ __align__(16) char ring[];
@@ -66,10 +66,9 @@ apply_pipe2h_kernel(OpParams p, const float2 *__restrict__ x, float2 *__restrict
             dst[j] = -1;
             src[j] = -1;
             if (b >= S::BOX) continue;
-            const int64_t gx = axis_nbr(p.ax[0], x0 - 1 + b % S::BX);
-            const int64_t gy = axis_nbr(p.ax[1], y0 - 1 + b / S::BX);
+            const int gx = axis_nbr32(p.ax[0], (int)x0 - 1 + b % S::BX), gy = axis_nbr32(p.ax[1], (int)y0 - 1 + b / S::BX);
             dst[j] = b * S::NODE_BYTES;
-            if (gx >= 0 && gy >= 0) src[j] = (int)((gy * nx + gx) * S::NODE_BYTES);
+            if (gx >= 0 && gy >= 0) src[j] = (gy * (int)nx + gx) * S::NODE_BYTES;
         }
         const char *layer = reinterpret_cast<const char *>(x) + (pfirst - 1) * (int64_t)plane_bytes;
         for (int i = 0; i < S::PLANES; ++i, layer += plane_bytes) {
@@ -84,14 +83,14 @@ apply_pipe2h_kernel(OpParams p, const float2 *__restrict__ x, float2 *__restrict
     bool valid[RY];
 #pragma unroll
     for (int r = 0; r < RY; ++r) valid[r] = ix < nx && iy + r < ny;
-    const StdConst<float> sc = std_const<2, float>(p);
     // beta = +1 for component 0, -1 for component 1
     const float fm = h == 0 ? -(float)p.m * sc.km : (float)p.m * sc.km;
     float wa = 0.f, wb = 0.f;
     if (!NOV && valid[0]) {
-        NodeCoef<2, float> k;
-        node_coef<2, float>(p, ix, iy, 0, k);
-        const float wl = h ? k.wl[1] : k.wl[0], wr = h ? k.wr[1] : k.wr[0];
+        // weights of the elements left and right of the node (every node has both)
+        const int64_t g = ix + p.ax[0].u0, nel = p.ax[0].nel;
+        const double *w = p.wx + (h ? nel : 0);
+        const float wl = (float)w[g > 0 ? g - 1 : nel - 1], wr = (float)w[g < nel ? g : 0];
         wa = -0.5f * sc.km * (wl + wr);
         wb = -0.5f * sc.km * (wr - wl);
     }
@@ -179,7 +178,7 @@ int launch_apply_pipe2h(const OpParams &p, const float2 *x, float2 *y, cudaStrea
         DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
         if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[nov][dev] = true;
     }
-    kern<<<dim3((unsigned)tiles, (unsigned)chunks), S::NTHR, S::SMEM, s>>>(p, x, y, tx);
+    kern<<<dim3((unsigned)tiles, (unsigned)chunks), S::NTHR, S::SMEM, s>>>(p, std_const<2, float>(p), x, y, tx);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }

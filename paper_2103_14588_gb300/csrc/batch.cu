@@ -128,16 +128,18 @@ batch_solve_kernel(const BatchInst *__restrict__ insts, BatchOpts o) {
     const int m = o.m;
     const int64_t ntc = I.tiles * I.chunks;
 
+    const StdConst<float> sc32 = std_const<D, float>(I.p);
+    const StdConst<double> sc64 = std_const<D, double>(I.p);
     auto apply32 = [&](const float2 *xin, float2 *yout) {
         for (int64_t tc = 0; tc < ntc; ++tc) {
-            apply_pipe_tile<D, 2, float, false, false>(I.p, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
+            apply_pipe_tile<D, 2, float, false, false>(I.p, sc32, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
                                                         tc / I.tiles, ring);
             __syncthreads();
         }
     };
     auto apply64 = [&](const double2 *xin, double2 *yout) {
         for (int64_t tc = 0; tc < ntc; ++tc) {
-            apply_pipe_tile<D, 2, double, false, false>(I.p, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
+            apply_pipe_tile<D, 2, double, false, false>(I.p, sc64, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
                                                          tc / I.tiles, ring);
             __syncthreads();
         }
