@@ -289,9 +289,15 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
     // march reads v and writes z
     const float2 *src = v;
     float2 *dst = z;
+    // (the march wants 16-byte aligned layers: a vector that starts at an odd entry of its
+    // buffer is marched in work too)
+    const bool aside = !p.has_fft && (((uintptr_t)v | (uintptr_t)z) & 15) != 0;
     if (p.has_fft) {
         dst_fft::fft_planes_kernel<float2><<<fgrid, dst_fft::FFT_THREADS, p.fft_smem, s>>>(p.fft, 0, v, p.work);
         DST_CUDA_TRY(cudaGetLastError());
+        src = dst = p.work;
+    } else if (aside) {
+        DST_CUDA_TRY(cudaMemcpyAsync(p.work, v, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
         src = dst = p.work;
     }
     // 2. s_0 and the march
@@ -308,6 +314,8 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
     if (p.has_fft) {
         dst_fft::fft_planes_kernel<float2><<<fgrid, dst_fft::FFT_THREADS, p.fft_smem, s>>>(p.fft, 1, p.work, z);
         DST_CUDA_TRY(cudaGetLastError());
+    } else if (aside) {
+        DST_CUDA_TRY(cudaMemcpyAsync(z, p.work, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
     }
     return DST_OK;
 }
@@ -335,20 +343,25 @@ extern "C" int dst_precond_apply(const dst_mesh *mesh, int kind, const void *v, 
     const int64_t n = mesh->n_unknowns;
     const size_t sweep_bytes = (dst_sweep_scratch_bytes(p, n) + 255) & ~(size_t)255;
     const size_t vec_bytes = ((size_t)n * sizeof(float2) + 255) & ~(size_t)255;
-    const size_t bytes = sweep_bytes + (kind == DST_PRECOND_CN_LEARNED ? 2 * vec_bytes : 0);
+    const bool learned = kind == DST_PRECOND_CN_LEARNED;
+    const bool aside = learned && ((uintptr_t)z & 15) != 0;       // the operator apply wants 16-byte aligned vectors
+    const size_t bytes = sweep_bytes + (learned ? (aside ? 3 : 2) * vec_bytes : 0);
     if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return DST_ERR_OOM;
     }
+    float2 *tmp = reinterpret_cast<float2 *>((char *)scratch + sweep_bytes);
+    float2 *rho = reinterpret_cast<float2 *>((char *)tmp + vec_bytes);
+    float2 *zz = aside ? reinterpret_cast<float2 *>((char *)rho + vec_bytes) : (float2 *)z;
     rc = dst_sweep_setup(mesh, p, scratch, s);
-    if (rc == DST_OK) rc = dst_sweep_apply(p, n, (const float2 *)v, (float2 *)z, s);
-    if (rc == DST_OK && kind == DST_PRECOND_CN_LEARNED) {
-        float2 *tmp = reinterpret_cast<float2 *>((char *)scratch + sweep_bytes);
-        float2 *rho = reinterpret_cast<float2 *>((char *)scratch + sweep_bytes + vec_bytes);
+    if (rc == DST_OK) rc = dst_sweep_apply(p, n, (const float2 *)v, zz, s);
+    if (rc == DST_OK && learned) {
         int nk = 0;
-        rc = dst_internal_apply(mesh, DST_FP32, z, tmp, s);                 // rho = v - A M_CN(v)
+        rc = dst_internal_apply(mesh, DST_FP32, zz, tmp, s);                // rho = v - A M_CN(v)
         if (rc == DST_OK) rc = dst_k_sub_f32(n, (const float2 *)v, tmp, rho, s);
-        if (rc == DST_OK) rc = dst_internal_unet_correct(mesh->unet, mesh, rho, (float2 *)z, tmp, s, &nk);
+        if (rc == DST_OK) rc = dst_internal_unet_correct(mesh->unet, mesh, rho, zz, tmp, s, &nk);
+        if (rc == DST_OK && aside && cudaMemcpyAsync(z, zz, sizeof(float2) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+            rc = DST_ERR_CUDA;
     }
     cudaFreeAsync(scratch, s);
     return rc;
