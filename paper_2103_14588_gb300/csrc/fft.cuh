@@ -19,6 +19,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sweep.h"
 
@@ -48,9 +49,21 @@ template <typename V, typename R> __device__ __forceinline__ V rot(V a, R sg) { 
 __device__ __forceinline__ void sincos_pi(float x, float *s, float *c) { sincospif(x, s, c); }
 __device__ __forceinline__ void sincos_pi(double x, double *s, double *c) { sincospi(x, s, c); }
 
-template <typename V> __device__ __forceinline__ void copy_async(V *dst, const V *src) {
+template <int BYTES> __device__ __forceinline__ void copy_async(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "n"((int)sizeof(V)) : "memory");
+                 "n"(BYTES) : "memory");
+}
+
+// What a thread transforms at a time: W components of a node, which lie side by side in
+// memory and share index arithmetic, twiddles and wide accesses.
+template <typename V, int W> struct alignas(sizeof(V) * W > 16 ? 16 : sizeof(V) * W) Elem { V c[W]; };
+template <typename V, int W> __device__ __forceinline__ void copy_elem(Elem<V, W> *dst, const V *src) {
+    constexpr int B = (int)sizeof(V) * W;
+    if constexpr (B <= 16) copy_async<B>(dst, src);
+    else {
+        copy_async<16>(dst, src);
+        copy_async<16>(reinterpret_cast<char *>(dst) + 16, reinterpret_cast<const char *>(src) + 16);
+    }
 }
 
 // In-place DFTs of R values, X_o = sum_r v_r exp(sg 2 pi i r o / R).
@@ -121,27 +134,41 @@ template <> struct Dft<16> {
 
 // One butterfly of a stage: elements j + r q of a line (element stride st) times
 // w^(r k step), to (j / Ns) Ns R + k + o Ns of the output line; q = n / R, step = q / Ns.
-template <int R, typename V, typename S>
-__device__ __forceinline__ void butterfly(const V *src, V *dst, int st, int q, int step, int Ns, int j, int k, const V *w, S sg) {
-    V v[R];
-    v[0] = src[j * st];
+template <int R, typename V, int W, typename S>
+__device__ __forceinline__ void butterfly(const Elem<V, W> *src, Elem<V, W> *dst, int st, int q, int step, int Ns, int j,
+                                          int k, const V *w, S sg) {
+    V v[W][R];
 #pragma unroll
-    for (int r = 1; r < R; ++r) v[r] = cmul(src[(j + r * q) * st], w[r * k * step]);
-    Dft<R>::run(v, sg);
+    for (int r = 0; r < R; ++r) {
+        const Elem<V, W> e = src[(j + r * q) * st];
+        const V t = r ? w[r * k * step] : V{};
+#pragma unroll
+        for (int c = 0; c < W; ++c) v[c][r] = r ? cmul(e.c[c], t) : e.c[c];
+    }
+#pragma unroll
+    for (int c = 0; c < W; ++c) Dft<R>::run(v[c], sg);
     const int to = (j - k) * R + k;
 #pragma unroll
-    for (int o = 0; o < R; ++o) dst[(to + o * Ns) * st] = v[o];
+    for (int o = 0; o < R; ++o) {
+        Elem<V, W> e;
+#pragma unroll
+        for (int c = 0; c < W; ++c) e.c[c] = v[c][o];
+        dst[(to + o * Ns) * st] = e;
+    }
 }
 
 // One output of a stage of any radix R: V_o = sum_r v_r w^(r (k step + o q)).
-template <typename V>
-__device__ __forceinline__ V general_output(const V *src, int st, int n, int R, int q, int step, int j, int k, int o,
-                                          const V *w) {
+template <typename V, int W>
+__device__ __forceinline__ Elem<V, W> general_output(const Elem<V, W> *src, int st, int n, int R, int q, int step, int j,
+                                                     int k, int o, const V *w) {
     const int inc = k * step + o * q;                      // < n
-    V acc = src[j * st];
+    Elem<V, W> acc = src[j * st];
     int at = inc;
     for (int r = 1; r < R; ++r) {
-        acc = cfma(w[at], src[(j + r * q) * st], acc);
+        const Elem<V, W> e = src[(j + r * q) * st];
+        const V t = w[at];
+#pragma unroll
+        for (int c = 0; c < W; ++c) acc.c[c] = cfma(t, e.c[c], acc.c[c]);
         at += inc;
         if (at >= n) at -= n;
     }
@@ -150,49 +177,49 @@ __device__ __forceinline__ V general_output(const V *src, int st, int n, int R, 
 
 // Every butterfly of one stage for threads `id` of `count`; line l starts at line(l),
 // `nl` lines, element stride st; neighbouring threads take neighbouring lines.
-template <typename V, typename S, typename Line>
-__device__ __forceinline__ void stage(const V *d0, V *d1, int n, int st, int nl, Line line, int R, int Ns, const V *w, S sg,
-                                      int id, int count) {
+template <typename V, int W, typename S, typename Line>
+__device__ __forceinline__ void stage(const Elem<V, W> *d0, Elem<V, W> *d1, int n, int st, int nl, Line line, int R, int Ns,
+                                      const V *w, S sg, int id, int count) {
     const int q = n / R, step = q / Ns;
     // quotients by nl and Ns by multiplication: the dividends stay below 2^32 / divisor
     const unsigned rn = nl > 1 ? 0xffffffffu / (unsigned)nl + 1u : 0u, rk = Ns > 1 ? 0xffffffffu / (unsigned)Ns + 1u : 0u;
     auto by_nl = [&](int i) { return nl > 1 ? (int)__umulhi((unsigned)i, rn) : i; };
     auto mod_ns = [&](int j) { return Ns > 1 ? j - (int)__umulhi((unsigned)j, rk) * Ns : 0; };
-    const bool direct = R == 2 || R == 3 || R == 4 || R == 5 || R == 8 || R == 16;
-    if (!direct) {
-        for (int i = id; i < nl * n; i += count) {
-            const int jo = by_nl(i), l = i - jo * nl, base = line(l);
-            const int o = jo / q, j = jo - o * q, k = mod_ns(j);
-            d1[base + ((j - k) * R + k + o * Ns) * st] = general_output(d0 + base, st, n, R, q, step, j, k, o, w);
+    auto each = [&](auto radix) {
+        constexpr int RR = decltype(radix)::value;
+        for (int i = id; i < nl * q; i += count) {
+            const int j = by_nl(i), l = i - j * nl, base = line(l), k = mod_ns(j);
+            butterfly<RR>(d0 + base, d1 + base, st, q, step, Ns, j, k, w, sg);
         }
-        return;
-    }
-    for (int i = id; i < nl * q; i += count) {
-        const int j = by_nl(i), l = i - j * nl, base = line(l), k = mod_ns(j);
-        const V *src = d0 + base;
-        V *dst = d1 + base;
-        switch (R) {
-            case 2: butterfly<2>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-            case 3: butterfly<3>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-            case 4: butterfly<4>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-            case 5: butterfly<5>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-            case 8: butterfly<8>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-            default: butterfly<16>(src, dst, st, q, step, Ns, j, k, w, sg); break;
-        }
+    };
+    switch (R) {
+        case 2: each(std::integral_constant<int, 2>()); break;
+        case 3: each(std::integral_constant<int, 3>()); break;
+        case 4: each(std::integral_constant<int, 4>()); break;
+        case 5: each(std::integral_constant<int, 5>()); break;
+        case 8: each(std::integral_constant<int, 8>()); break;
+        case 16: each(std::integral_constant<int, 16>()); break;
+        default:
+            for (int i = id; i < nl * n; i += count) {
+                const int jo = by_nl(i), l = i - jo * nl, base = line(l);
+                const int o = jo / q, j = jo - o * q, k = mod_ns(j);
+                d1[base + ((j - k) * R + k + o * Ns) * st] = general_output(d0 + base, st, n, R, q, step, j, k, o, w);
+            }
     }
 }
 
-template <typename V, typename S>
-__device__ void warp_fft_line(V *line, int st, int n, const int *rad, int nrad, const V *w, S sg, V *a, V *b) {
+template <typename V, int W, typename S>
+__device__ void warp_fft_line(Elem<V, W> *line, int st, int n, const int *rad, int nrad, const V *w, S sg, Elem<V, W> *a,
+                              Elem<V, W> *b) {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < n; i += 32) a[i] = line[i * st];
     __syncwarp();
-    V *d0 = a, *d1 = b;
+    Elem<V, W> *d0 = a, *d1 = b;
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
         stage(d0, d1, n, 1, 1, [](int) { return 0; }, rad[s], Ns, w, sg, lane, 32);
         __syncwarp();
-        V *t = d0; d0 = d1; d1 = t;
+        Elem<V, W> *t = d0; d0 = d1; d1 = t;
         Ns *= rad[s];
     }
     for (int i = lane; i < n; i += 32) line[i * st] = d0[i];
@@ -202,13 +229,14 @@ __device__ void warp_fft_line(V *line, int st, int n, const int *rad, int nrad, 
 // All lines of one axis of the plane through the stages at once, with a barrier
 // between stages (ping-pong between the two plane buffers).  Returns the buffer that
 // holds the result.
-template <typename V, typename S, typename Line>
-__device__ V *cta_fft_axis(V *d0, V *d1, int n, int st, int nl, Line line, const int *rad, int nrad, const V *w, S sg) {
+template <typename V, int W, typename S, typename Line>
+__device__ Elem<V, W> *cta_fft_axis(Elem<V, W> *d0, Elem<V, W> *d1, int n, int st, int nl, Line line, const int *rad,
+                                    int nrad, const V *w, S sg) {
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
         stage(d0, d1, n, st, nl, line, rad[s], Ns, w, sg, threadIdx.x, FFT_THREADS);
         __syncthreads();
-        V *t = d0; d0 = d1; d1 = t;
+        Elem<V, W> *t = d0; d0 = d1; d1 = t;
         Ns *= rad[s];
     }
     return d0;
@@ -223,35 +251,37 @@ template <typename V>
 inline size_t fft_smem_bytes(const SweepFft &a) {
     const int nmax = a.n1 > a.n2 ? a.n1 : a.n2;
     const size_t plane = (size_t)a.ncb * a.n1 * pitch(a);
-    const size_t scratch = a.pingpong ? plane : (size_t)FFT_WARPS * 2 * nmax;
+    const size_t scratch = a.pingpong ? plane : (size_t)FFT_WARPS * 2 * nmax * a.ncb;
     return sizeof(V) * (plane + a.n1 + a.n2 + scratch);
 }
 
-template <typename V>
+// W = a.ncb components per CTA.
+template <typename V, int W>
 __global__ void __launch_bounds__(FFT_THREADS)
 fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restrict__ out) {
     using R = typename Real<V>::type;
+    using E = Elem<V, W>;
     extern __shared__ __align__(16) unsigned char fft_sm_raw[];
-    V *sm = reinterpret_cast<V *>(fft_sm_raw);
-    const int n1 = a.n1, n2 = a.n2, nc = a.nc, ncb = a.ncb, pt = pitch(a);
-    const int nf = n1 * n2, pl = n1 * pt;
-    V *plane = sm;                                        // [ncb][n1][pitch]
-    V *w1 = plane + (size_t)ncb * pl;                     // twiddles of the outer axis (n1)
+    const int n1 = a.n1, n2 = a.n2, nc = a.nc, pt = pitch(a);
+    const int nf = n1 * n2, pl = n1 * pt, nmax = n1 > n2 ? n1 : n2;
+    E *plane = reinterpret_cast<E *>(fft_sm_raw);         // [n1][pitch]
+    E *scr = plane + pl;                                  // second plane, or per warp two lines of nmax
+    V *w1 = reinterpret_cast<V *>(scr + (a.pingpong ? pl : FFT_WARPS * 2 * nmax));   // twiddles of the outer axis (n1)
     V *w2 = w1 + n1;                                      // twiddles of the inner axis (n2)
-    V *scr = w2 + n2;                                     // second plane, or per warp two lines of nmax
-    const int nmax = n1 > n2 ? n1 : n2;
-    const int64_t b = blockIdx.x;
-    const int c0 = blockIdx.y * ncb;
+    // the component groups of a plane are neighbours in the grid: together they use the
+    // sectors that each touches half of (apart, DRAM saw three times the plane's bytes)
+    const int groups = nc / W;
+    const int64_t b = blockIdx.x / groups;
+    const int c0 = (int)(blockIdx.x % groups) * W;
     const int64_t base = (b / a.nbx) * a.ns_nodes + (b % a.nbx) * a.sbx;   // node index of (i1, i2) = (0, 0)
     const R sign = inverse ? (R)1 : (R)-1;
-    const int lcb = __ffs(ncb) - 1;                       // components per CTA: 1, 2 or 4
     const unsigned r2 = n2 > 1 ? 0xffffffffu / (unsigned)n2 + 1u : 0u;
     auto row = [&](int f) { return n2 > 1 ? (int)__umulhi((unsigned)f, r2) : f; };
-    for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) {
-        const int cc = idx & (ncb - 1), f = idx >> lcb;
+    const V *src = in + (inverse ? b * nf : base) * nc + c0;
+#pragma unroll 4
+    for (int f = threadIdx.x; f < nf; f += FFT_THREADS) {
         const int i1 = row(f), i2 = f - i1 * n2;
-        copy_async(plane + cc * pl + i1 * pt + i2,
-                   in + (inverse ? (b * nf + f) * nc : (base + (int64_t)i1 * a.s1 + (int64_t)i2 * a.s2) * nc) + c0 + cc);
+        copy_elem<V, W>(plane + i1 * pt + i2, src + (inverse ? (int64_t)f : i1 * a.s1 + i2 * a.s2) * nc);
     }
     // the twiddles while the plane is on its way
     for (int j = threadIdx.x; j < n1; j += FFT_THREADS) {
@@ -266,56 +296,71 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    V *cur = plane;
+    E *cur = plane;
     if (a.pingpong) {
-        // CTA-wide stages; scr is a second plane.  Inner lines start every pitch; outer
-        // line (cc, i2) at cc * pl + i2.
-        if (n2 > 1) cur = cta_fft_axis(cur, scr, n2, 1, ncb * n1, [&](int l) { return l * pt; }, a.rad2, a.nrad2, w2, sign);
+        // CTA-wide stages; scr is a second plane.  Inner lines start every pitch, outer line i2 at i2.
+        if (n2 > 1) cur = cta_fft_axis(cur, scr, n2, 1, n1, [&](int l) { return l * pt; }, a.rad2, a.nrad2, w2, sign);
         if (n1 > 1)
-            cur = cta_fft_axis(cur, cur == plane ? scr : plane, n1, pt, ncb * n2,
-                               [&](int l) { const int cc = row(l); return cc * pl + (l - cc * n2); }, a.rad1, a.nrad1, w1,
-                               sign);
+            cur = cta_fft_axis(cur, cur == plane ? scr : plane, n1, pt, n2, [](int l) { return l; }, a.rad1, a.nrad1, w1, sign);
     } else {
         const int warp = threadIdx.x >> 5;
-        V *sa = scr + (size_t)warp * 2 * nmax, *sb = sa + nmax;
+        E *sa = scr + (size_t)warp * 2 * nmax, *sb = sa + nmax;
         if (n2 > 1)
-            for (int line = warp; line < ncb * n1; line += FFT_WARPS)
+            for (int line = warp; line < n1; line += FFT_WARPS)
                 warp_fft_line(plane + (size_t)line * n2, 1, n2, a.rad2, a.nrad2, w2, sign, sa, sb);
         __syncthreads();
         if (n1 > 1)
-            for (int line = warp; line < ncb * n2; line += FFT_WARPS) {
-                const int cc = line / n2, i2 = line % n2;
-                warp_fft_line(plane + (size_t)cc * nf + i2, n2, n1, a.rad1, a.nrad1, w1, sign, sa, sb);
-            }
+            for (int line = warp; line < n2; line += FFT_WARPS)
+                warp_fft_line(plane + line, n2, n1, a.rad1, a.nrad1, w1, sign, sa, sb);
         __syncthreads();
     }
     const R scale = inverse ? (R)1 / (R)nf : (R)1;
-    for (int idx = threadIdx.x; idx < nf * ncb; idx += FFT_THREADS) {
-        const int cc = idx & (ncb - 1), f = idx >> lcb;
+    V *dst = out + (inverse ? base : b * nf) * nc + c0;
+    for (int f = threadIdx.x; f < nf; f += FFT_THREADS) {
         const int i1 = row(f), i2 = f - i1 * n2;
-        V v = cur[cc * pl + i1 * pt + i2];
-        v.x *= scale;
-        v.y *= scale;
-        if (inverse) out[(base + (int64_t)i1 * a.s1 + (int64_t)i2 * a.s2) * nc + c0 + cc] = v;
-        else out[(b * nf + f) * nc + c0 + cc] = v;
+        E v = cur[i1 * pt + i2];
+#pragma unroll
+        for (int c = 0; c < W; ++c) { v.c[c].x *= scale; v.c[c].y *= scale; }
+        *reinterpret_cast<E *>(dst + (inverse ? i1 * a.s1 + i2 * a.s2 : (int64_t)f) * nc) = v;
     }
 }
 
+// The planes `nb` of every component group.  The kernel's shared-memory limit is a
+// per-device attribute, set once.
+template <typename V>
+inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, int inverse, const V *in, V *out, cudaStream_t s) {
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+        const int limit = 200 * 1024;
+        e = cudaFuncSetAttribute(fft_planes_kernel<V, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fft_planes_kernel<V, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
+    // a caller's FP32 vector may start at any entry (8 bytes): then one component at a time
+    SweepFft b = a;
+    if ((((uintptr_t)in | (uintptr_t)out) & 15) != 0) b.ncb = 1;
+    const unsigned grid = (unsigned)(nb * (b.nc / b.ncb));
+    if (b.ncb == 2) fft_planes_kernel<V, 2><<<grid, FFT_THREADS, fft_smem_bytes<V>(b), s>>>(b, inverse, in, out);
+    else fft_planes_kernel<V, 1><<<grid, FFT_THREADS, fft_smem_bytes<V>(b), s>>>(b, inverse, in, out);
+    return cudaGetLastError();
+}
+
 // Pick the components per CTA and the stage layout for planes of a.n1 x a.n2:
-// CTA-wide stages (second plane buffer) when they fit, else one line per warp.  The
-// components of a node are adjacent in memory, so a CTA takes as many as leave three
-// CTAs per SM and enough CTAs to fill the GPU (nb planes per component group).
+// CTA-wide stages (second plane buffer) when they fit, else one line per warp; two
+// components per CTA where three such CTAs fit an SM and there are enough to fill the GPU
+// (nb planes per component group).
 // Returns false if nothing fits in `limit` bytes.
 template <typename V>
 inline bool choose_layout(SweepFft &a, int64_t nb, size_t limit) {
     for (int pp = 1; pp >= 0; --pp) {
         a.pingpong = pp;
-        for (int ncb = a.nc; ncb > 1; ncb /= 2) {
-            a.ncb = ncb;
-            if (fft_smem_bytes<V>(a) > (pp ? std::min<size_t>(limit, 76 * 1024) : limit)) continue;
-            if (nb * (a.nc / ncb) < 304) continue;
-            return true;
-        }
+        a.ncb = 2;                             // spinors have two or four components
+        if (fft_smem_bytes<V>(a) <= (pp ? std::min<size_t>(limit, 76 * 1024) : limit) && nb * (a.nc / 2) >= 304) return true;
         a.ncb = 1;
         if (fft_smem_bytes<V>(a) <= limit) return true;
     }

@@ -188,26 +188,14 @@ int energy_impl(const dst_mesh *mesh, const double2 *psi, double *out, cudaStrea
         if (b1) cudaFreeAsync(b1, s);
         return DST_ERR_OOM;
     }
-    static bool configured[64] = {};
-    int dev = 0;
     int rc = DST_OK;
-    if (cudaGetDevice(&dev) != cudaSuccess) rc = DST_ERR_CUDA;
-    if (rc == DST_OK && (dev < 0 || dev >= 64 || !configured[dev])) {
-        if (cudaFuncSetAttribute(dst_fft::fft_planes_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)limit) != cudaSuccess)
-            rc = DST_ERR_CUDA;
-        else if (dev >= 0 && dev < 64)
-            configured[dev] = true;
+    cudaError_t fe = dst_fft::fft_launch<double2>(a1, mesh->nt * nz, 0, psi, b1, s);
+    if (fe == cudaSuccess && mesh->d == 3) fe = dst_fft::fft_launch<double2>(a2, mesh->nt * nfyx, 0, b1, b2, s);
+    if (fe != cudaSuccess) {
+        dst_internal_set_cuda_error(fe, "energy FFT", __FILE__, __LINE__);
+        rc = DST_ERR_CUDA;
     }
     if (rc == DST_OK) {
-        const dim3 g1((unsigned)(mesh->nt * nz), (unsigned)(nc / a1.ncb));
-        dst_fft::fft_planes_kernel<double2><<<g1, dst_fft::FFT_THREADS, dst_fft::fft_smem_bytes<double2>(a1), s>>>(
-            a1, 0, psi, b1);
-        if (mesh->d == 3) {
-            const dim3 g2((unsigned)(mesh->nt * nfyx), (unsigned)(nc / a2.ncb));
-            dst_fft::fft_planes_kernel<double2><<<g2, dst_fft::FFT_THREADS, dst_fft::fft_smem_bytes<double2>(a2), s>>>(
-                a2, 0, b1, b2);
-        }
         EGeo g;
         g.d = mesh->d; g.nc = nc; g.n[0] = nx; g.n[1] = ny; g.n[2] = nz;
         for (int k = 0; k < 3; ++k) g.h[k] = mesh->h[k];

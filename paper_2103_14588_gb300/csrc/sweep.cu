@@ -187,7 +187,6 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
         dst_internal_set_error_detail("Crank-Nicolson sweep: a periodic plane too large for shared memory");
         return DST_ERR_ARG;
     }
-    p.fft_smem = dst_fft::fft_smem_bytes<float2>(a);
     // banded march: G lanes per system (two x nodes each), `steps` parallel reduction
     // steps; systems per CTA as many as keep it at 256 threads while the CTAs still
     // cover the GPU (a 2+1 mesh has n_y systems, a 1+1 mesh one)
@@ -276,15 +275,6 @@ static int launch_march(const SweepPlan &p, const float2 *in, float2 *out, cudaS
 int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, float2 *z, cudaStream_t s) {
     const int64_t per2 = n_unknowns / p.g.nt / 2;           // pairs of entries (NC is even)
     const int64_t nf = (int64_t)p.g.n1 * p.g.n2;
-    static bool configured[64] = {};
-    int dev = 0;
-    DST_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !configured[dev]) {
-        DST_CUDA_TRY(cudaFuncSetAttribute(dst_fft::fft_planes_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          200 * 1024));
-        if (dev >= 0 && dev < 64) configured[dev] = true;
-    }
-    const dim3 fgrid((unsigned)p.nb, (unsigned)(p.g.nc / p.fft.ncb));
     // 1. forward FFT of every plane: v -> work (frequency layout); without an FFT the
     // march reads v and writes z
     const float2 *src = v;
@@ -293,8 +283,7 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
     // buffer is marched in work too)
     const bool aside = !p.has_fft && (((uintptr_t)v | (uintptr_t)z) & 15) != 0;
     if (p.has_fft) {
-        dst_fft::fft_planes_kernel<float2><<<fgrid, dst_fft::FFT_THREADS, p.fft_smem, s>>>(p.fft, 0, v, p.work);
-        DST_CUDA_TRY(cudaGetLastError());
+        DST_CUDA_TRY(dst_fft::fft_launch<float2>(p.fft, p.nb, 0, v, p.work, s));
         src = dst = p.work;
     } else if (aside) {
         DST_CUDA_TRY(cudaMemcpyAsync(p.work, v, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
@@ -311,12 +300,8 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
         if (rc) return rc;
     }
     // 3. inverse FFT: work -> z
-    if (p.has_fft) {
-        dst_fft::fft_planes_kernel<float2><<<fgrid, dst_fft::FFT_THREADS, p.fft_smem, s>>>(p.fft, 1, p.work, z);
-        DST_CUDA_TRY(cudaGetLastError());
-    } else if (aside) {
-        DST_CUDA_TRY(cudaMemcpyAsync(z, p.work, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
-    }
+    if (p.has_fft) DST_CUDA_TRY(dst_fft::fft_launch<float2>(p.fft, p.nb, 1, p.work, z, s));
+    else if (aside) DST_CUDA_TRY(cudaMemcpyAsync(z, p.work, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
     return DST_OK;
 }
 

@@ -39,7 +39,6 @@ struct SweepPlan {
     SweepFft fft;
     bool banded, has_fft, vx;
     int64_t nb;                 // FFT planes
-    size_t fft_smem;
     size_t table_bytes;         // banded: reduction factors (sweep_march.cuh)
     int lanes, steps, systems;  // banded: lanes per system, parallel reduction steps, systems per CTA
     size_t march_smem;

@@ -236,10 +236,10 @@ __device__ __forceinline__ void copy16(void *dst, const void *src) {
 }
 
 // Shared memory of one CTA of `sys` systems: STAGES input layers, two output layers,
-// two exchange buffers.
+// two exchange buffers of two values per lane.
 __host__ __device__ inline int row_bytes(int nc, int sys) { return (nc == 4 ? sys / 2 : sys) * nc * 8 + 16; }
 inline size_t march_smem(int nc, int sys, int G, int n) {
-    return (size_t)(STAGES + 2) * ((n + 1) / 2 * 2) * row_bytes(nc, sys) + 2 * sizeof(float4) * (size_t)sys * G;
+    return (size_t)(STAGES + 2) * ((n + 1) / 2 * 2) * row_bytes(nc, sys) + 4 * sizeof(float4) * (size_t)sys * G;
 }
 
 // LARGE: time steps above half the x spacing.  The reduction then loses digits (K outweighs
@@ -270,19 +270,31 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
         reinterpret_cast<float4 *>(ring)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     // a row of the ring: the CTA's frequencies of one x node, even nodes first, so that
-    // the lanes of a warp read consecutive rows
-    const int per_row = fper * NC / 2, cl = __ffs(per_row) - 1;
-    const int valid = (int)min((int64_t)per_row, (nf - f0) * (NC / 2));
+    // the lanes of a warp read consecutive rows.  A thread copies one 16-byte column of
+    // rows i0 and i0 + G (n <= 2 G; G is even, so their places lie G/2 rows apart), the
+    // same ones of every layer: with a division and a comparison per piece instead, a
+    // third of the issue slots went to addresses (386 us against 255 on the 48^3 x 48
+    // Klein mesh).
+    const int per_row = fper * NC / 2, ch = threadIdx.x % per_row, i0 = threadIdx.x / per_row;
+    const bool column = ch < (nf - f0) * (NC / 2);
+    const bool copy0 = column && i0 < n, copy1 = column && i0 + G < n;
     auto pos = [&](int i) { return (i & 1) * half + (i >> 1); };
-    auto issue = [&](int64_t t) {
-        if (t < g.nt) {
-            unsigned char *dst = ring + (size_t)(t % STAGES) * rows * RB;
-            const char *src = reinterpret_cast<const char *>(in + ((t * n) * nf + f0) * NC);
-            for (int k = threadIdx.x; k < n << cl; k += blockDim.x) {
-                const int i = k >> cl, ch = k & (per_row - 1);
-                if (ch < valid) copy16(dst + pos(i) * RB + ch * 16, src + (int64_t)i * nf * NC * 8 + ch * 16);
-            }
+    const int at0 = pos(i0) * RB + ch * 16, at1 = at0 + (G / 2) * RB, tile = rows * RB;
+    const int64_t off0 = (i0 * nf + f0) * NC * 8 + ch * 16, off1 = off0 + (int64_t)G * nf * NC * 8,
+                  layer = (int64_t)n * nf * NC * 8;
+    const char *src = reinterpret_cast<const char *>(in) + off0;
+    char *dst = reinterpret_cast<char *>(out) + off0;
+    const int nt = (int)g.nt;
+    int issued = 0, fill = 0;                                  // layers issued; the ring slot of the next
+    auto issue = [&] {
+        if (issued < nt) {
+            unsigned char *d = ring + fill;
+            if (copy0) copy16(d + at0, src);
+            if (copy1) copy16(d + at1, src + (off1 - off0));
+            src += layer;
         }
+        ++issued;
+        fill = fill == (STAGES - 1) * tile ? 0 : fill + tile;
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     // the rotated pair of one node from its two (2+1) or four (3+1) components
@@ -291,8 +303,8 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
         if (pair == 0) return make_float4(rc * a.x - rs * a.w, rc * a.y + rs * a.z, rc * b.z - rs * b.y, rc * b.w + rs * b.x);
         return make_float4(rc * a.z - rs * a.y, rc * a.w + rs * a.x, rc * b.x - rs * b.w, rc * b.y + rs * b.z);
     };
-    auto node = [&](const unsigned char *tile, int i) {
-        const float4 *q = reinterpret_cast<const float4 *>(tile + pos(i) * RB + slot * NC * 8);
+    auto node = [&](const unsigned char *at) {
+        const float4 *q = reinterpret_cast<const float4 *>(at);
         return NC == 4 ? rotate(q[0], q[1]) : q[0];
     };
     auto alt = [&](const float4 *v, int i) {
@@ -327,11 +339,11 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 xe = z4, xo = z4, xn = z4;                          // x_{t-1} at e, o and e + 2
     int buf = 0;
-    float4 *mine = xch + threadIdx.x;
+    float4 *mine = xch + threadIdx.x, *mine2 = mine + 2 * blockDim.x;
     auto sync = [&] { if (G <= 32) __syncwarp(); else __syncthreads(); };
     auto swap_buf = [&] { buf ^= (int)blockDim.x; };
     const int left = l > 0 ? -1 : 0, right = l + 1 < G ? 1 : 0;
-    for (int q = 0; q < STAGES - 1; ++q) issue(q);
+    for (int q = 0; q < STAGES - 1; ++q) issue();
 
     // s - K' x + i kM M' x of a node between elements of potential va and vb (M' the [1,4,1]
     // sum), x at the node and its neighbours p and r
@@ -352,20 +364,20 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
         }
         return q;
     };
-    auto from_left = [&](const float4 v) {                     // the left lane's v (0 at the wall)
+    // the left lane's v and w (v 0 at the wall, where the factor of w is 0)
+    auto from_left = [&](const float4 v, const float4 w, float4 &vl, float4 &wl) {
         mine[buf] = v;
+        mine2[buf] = w;
         sync();
-        const float4 w = l > 0 ? mine[buf + left] : z4;
+        vl = l > 0 ? mine[buf + left] : z4;
+        wl = mine2[buf + left];
         swap_buf();
-        return w;
     };
     // Bd u = r; un: u at e + 2
-    auto solve = [&](float4 re, const float4 ro, float4 &ue, float4 &uo, float4 &un) {
-        mine[buf] = ro;
-        sync();
-        sub_mv(re, A, mine[buf + left]);
+    // (rl: the left lane's ro)
+    auto solve = [&](float4 re, const float4 ro, const float4 rl, float4 &ue, float4 &uo, float4 &un) {
+        sub_mv(re, A, rl);
         sub_mv(re, Bm, ro);
-        swap_buf();
         auto reduce = [&](int st, const Blk &a, const Blk &b) {
             mine[buf] = re;
             sync();
@@ -391,47 +403,53 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
         sub_mv(uo, OL, ue);
         sub_mv(uo, OU, un);
     };
-    auto store_layer = [&](int64_t t) {                        // out tile t & 1, rotated back
-        const unsigned char *tile = otile + (size_t)(t & 1) * rows * RB;
-        char *dst = reinterpret_cast<char *>(out + ((t * n) * nf + f0) * NC);
-        for (int k = threadIdx.x; k < n << cl; k += blockDim.x) {
-            const int i = k >> cl, ch = k & (per_row - 1);
-            if (ch >= valid) continue;
-            float4 v = *reinterpret_cast<const float4 *>(tile + pos(i) * RB + ch * 16);
-            if (NC == 4) {
-                const float c = ft[f0 + (ch >> 1)].c, s = ft[f0 + (ch >> 1)].s;
-                v = make_float4(c * v.x + s * v.w, c * v.y - s * v.z, c * v.z + s * v.y, c * v.w - s * v.x);
-            }
-            *reinterpret_cast<float4 *>(dst + (int64_t)i * nf * NC * 8 + ch * 16) = v;
-        }
+    // a finished layer from its tile, rotated back
+    float bc = 1.f, bs = 0.f;
+    if (NC == 4 && column) { bc = ft[f0 + (ch >> 1)].c; bs = ft[f0 + (ch >> 1)].s; }
+    auto store_layer = [&](const unsigned char *t) {
+        auto back = [&](const unsigned char *q) {
+            const float4 v = *reinterpret_cast<const float4 *>(q);
+            if (NC == 2) return v;
+            return make_float4(bc * v.x + bs * v.w, bc * v.y - bs * v.z, bc * v.z + bs * v.y, bc * v.w - bs * v.x);
+        };
+        if (copy0) *reinterpret_cast<float4 *>(dst) = back(t + at0);
+        if (copy1) *reinterpret_cast<float4 *>(dst + (off1 - off0)) = back(t + at1);
+        dst += layer;
     };
-    for (int64_t t = 0; t < g.nt; ++t) {
+    // this lane's places in a tile
+    const int ate = (he ? pos(e) : 0) * RB + slot * NC * 8, ato = (ho ? pos(o) : 0) * RB + slot * NC * 8;
+    int used = 0;                                              // the ring slot of layer t
+    for (int t = 0; t < nt; ++t) {
         asm volatile("cp.async.wait_group %0;\n" ::"n"(STAGES - 2) : "memory");
         __syncthreads();               // layer t staged; layer t - 1 of the output complete; its input slot free
-        issue(t + STAGES - 1);
-        if (t > 0) store_layer(t - 1);
-        // the neighbour's x_{t-1} at o - 2; the odd node needs none beyond e and e + 2
-        float4 re = rhs(se, sel, xe, from_left(xo), xo, ve[0], ve[1], kM);
+        issue();
+        if (t > 0) store_layer(otile + (t & 1 ? 0 : tile));
+        // the odd node's right-hand side needs no neighbour beyond e and e + 2, the even one's
+        // the left lane's x_{t-1}, which comes with that lane's odd right-hand side: one exchange
         float4 ro = rhs(so, sol, xo, xe, xn, ve[1], ve[2], kM);
-        if (!he) re = z4;
         if (!ho) ro = z4;
+        float4 xl, rl;
+        from_left(xo, ro, xl, rl);
+        float4 re = rhs(se, sel, xe, xl, xo, ve[0], ve[1], kM);
+        if (!he) re = z4;
         float4 ue, uo, un;
-        solve(re, ro, ue, uo, un);
+        solve(re, ro, rl, ue, uo, un);
         if (LARGE) {
             // one step of refinement: u += Bd^-1 (r - Bd u)
-            re = rhs(re, z4, ue, from_left(uo), uo, ve[0], ve[1], -kM);
             ro = rhs(ro, z4, uo, ue, un, ve[1], ve[2], -kM);
-            if (!he) re = z4;
             if (!ho) ro = z4;
+            from_left(uo, ro, xl, rl);
+            re = rhs(re, z4, ue, xl, uo, ve[0], ve[1], -kM);
+            if (!he) re = z4;
             float4 de, dd, dn;
-            solve(re, ro, de, dd, dn);
+            solve(re, ro, rl, de, dd, dn);
             xe = add4(ue, de); xo = add4(uo, dd); xn = add4(un, dn);
         } else {
             xe = add4(ue, xe); xo = add4(uo, xo); xn = add4(un, xn);
         }
-        unsigned char *ot = otile + (size_t)(t & 1) * rows * RB + slot * NC * 8;
-        auto emit = [&](int i, const float4 x) {
-            unsigned char *d = ot + pos(i) * RB;
+        unsigned char *ot = otile + (t & 1 ? tile : 0);
+        auto emit = [&](int at, const float4 x) {
+            unsigned char *d = ot + at;
             if (NC == 4) {
                 *reinterpret_cast<float2 *>(d + (pair ? 8 : 0)) = make_float2(x.x, x.y);
                 *reinterpret_cast<float2 *>(d + (pair ? 16 : 24)) = make_float2(x.z, x.w);
@@ -439,12 +457,13 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
                 *reinterpret_cast<float4 *>(d) = x;
             }
         };
-        const unsigned char *it = ring + (size_t)(t % STAGES) * rows * RB;
-        if (he) { emit(e, xe); next_s(se, sel, node(it, e)); }
-        if (ho) { emit(o, xo); next_s(so, sol, node(it, o)); }
+        const unsigned char *it = ring + used;
+        used = used == (STAGES - 1) * tile ? 0 : used + tile;
+        if (he) { emit(ate, xe); next_s(se, sel, node(it + ate)); }
+        if (ho) { emit(ato, xo); next_s(so, sol, node(it + ato)); }
     }
     __syncthreads();
-    store_layer(g.nt - 1);
+    store_layer(otile + (nt & 1 ? 0 : tile));
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
