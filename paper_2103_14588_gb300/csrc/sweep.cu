@@ -69,9 +69,12 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
     for (int k = 0; k < g.d; ++k) mk[k] = g.h[k] * (2.0 + cos(th[k])) / 3.0;
     const double pm = mk[0] * mk[1], ht2 = 0.5 * g.ht;
     const double bx = -ht2 * sin(th[0]) * mk[1], by = g.d > 1 ? -ht2 * sin(th[1]) * mk[0] : 0.0;
-    const M22 P = inv(M22{z2{-ht2 * (g.m + g.V0) * pm, pm}, z2{bx, -by}, z2{bx, by}, z2{-ht2 * (g.V0 - g.m) * pm, pm}});
-    const Blk Pf{make_float4((float)P.a.x, (float)P.a.y, (float)P.b.x, (float)P.b.y),
-                 make_float4((float)P.c.x, (float)P.c.y, (float)P.d.x, (float)P.d.y)};
+    // P, the inverse of [a0 + i pm, bx - i by; bx + i by, a1 + i pm]: (wx + i wy) = 1 / det
+    const double a0 = -ht2 * (g.m + g.V0) * pm, a1 = -ht2 * (g.V0 - g.m) * pm;
+    const double dx = a0 * a1 - pm * pm - (bx * bx + by * by), dy = pm * (a0 + a1), r = 1.0 / (dx * dx + dy * dy);
+    const double wx = dx * r, wy = -dy * r;
+    const Blk Pf{make_float4((float)(a1 * wx - pm * wy), (float)(a1 * wy + pm * wx), (float)(-bx * wx - by * wy), (float)(by * wx - bx * wy)),
+                 make_float4((float)(by * wy - bx * wx), (float)(-bx * wy - by * wx), (float)(a0 * wx - pm * wy), (float)(a0 * wy + pm * wx))};
     // h_t K^ = kx sigma_x + ky sigma_y + diag(d0, d1)
     const float kx = (float)(2.0 * bx), ky = (float)(2.0 * by), d0 = (float)(-g.ht * (g.m + g.V0) * pm),
                 d1 = (float)(-g.ht * (g.V0 - g.m) * pm);

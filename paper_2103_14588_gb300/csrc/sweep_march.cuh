@@ -35,51 +35,86 @@ namespace dst_march {
 constexpr int STAGES = 3;                 // input layers in shared memory
 constexpr int REG_STEPS = 5;              // reduction steps whose factors stay in registers (G <= 32)
 
-struct z2 { double x, y; };
+// A pair of floats hi + lo (48 bits): the arithmetic of the factors.  The FP64 unit
+// issues one warp instruction in 64 clocks, a product and a sum of pairs take 12 in FP32.
+// Products are __fmul_rn so that they are not contracted into the sums that follow.
+struct df { float h, l; };
+__device__ __forceinline__ df to_df(double v) { const float h = (float)v; return df{h, (float)(v - (double)h)}; }
+__device__ __forceinline__ df operator*(df a, df b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return df{p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ df operator+(df a, df b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    return df{s, (a.l + b.l) + (__fsub_rn(a.h, __fsub_rn(s, t)) + __fsub_rn(b.h, t))};
+}
+__device__ __forceinline__ df operator-(df a) { return df{-a.h, -a.l}; }
+__device__ __forceinline__ df operator-(df a, df b) { return a + -b; }
+__device__ __forceinline__ df scaled(df a, float power_of_2) { return df{a.h * power_of_2, a.l * power_of_2}; }
+__device__ __forceinline__ df norm(df a) {                 // hi = the sum rounded
+    const float s = __fadd_rn(a.h, a.l);
+    return df{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+
+struct z2 { df x, y; };
 __device__ __forceinline__ z2 operator+(z2 a, z2 b) { return z2{a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ z2 operator-(z2 a, z2 b) { return z2{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ z2 operator-(z2 a) { return z2{-a.x, -a.y}; }
 __device__ __forceinline__ z2 operator*(z2 a, z2 b) { return z2{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+__device__ __forceinline__ z2 norm(z2 a) { return z2{norm(a.x), norm(a.y)}; }
 
 struct M22 { z2 a, b, c, d; };            // rows (a b), (c d)
-__device__ __forceinline__ M22 zero22() { const z2 z{0.0, 0.0}; return M22{z, z, z, z}; }
+__device__ __forceinline__ M22 zero22() { const z2 z{}; return M22{z, z, z, z}; }
+__device__ __forceinline__ M22 norm(const M22 &p) { return M22{norm(p.a), norm(p.b), norm(p.c), norm(p.d)}; }
 __device__ __forceinline__ M22 mul(const M22 &p, const M22 &q) {
-    return M22{p.a * q.a + p.b * q.c, p.a * q.b + p.b * q.d, p.c * q.a + p.d * q.c, p.c * q.b + p.d * q.d};
+    return norm(M22{p.a * q.a + p.b * q.c, p.a * q.b + p.b * q.d, p.c * q.a + p.d * q.c, p.c * q.b + p.d * q.d});
 }
-__device__ __forceinline__ M22 sub(const M22 &p, const M22 &q) { return M22{p.a - q.a, p.b - q.b, p.c - q.c, p.d - q.d}; }
-__device__ __forceinline__ M22 neg(const M22 &p) { return sub(zero22(), p); }
+__device__ __forceinline__ M22 sub(const M22 &p, const M22 &q) {
+    return norm(M22{p.a - q.a, p.b - q.b, p.c - q.c, p.d - q.d});
+}
+__device__ __forceinline__ M22 neg(const M22 &p) { return M22{-p.a, -p.b, -p.c, -p.d}; }
 __device__ __forceinline__ M22 inv(const M22 &p) {
-    const z2 det = p.a * p.d - p.b * p.c;
-    const double r = 1.0 / (det.x * det.x + det.y * det.y);
-    const z2 w{det.x * r, -det.y * r}, m{-w.x, -w.y};
-    return M22{p.d * w, p.b * m, p.c * m, p.a * w};
+    z2 det = norm(p.a * p.d - p.b * p.c);
+    // the determinant scaled to [1, 2) by a power of two: its square stays in range
+    const float big = fmaxf(fabsf(det.x.h), fabsf(det.y.h));
+    const float sc = __int_as_float((254 << 23) - (__float_as_int(big) & 0x7f800000));
+    det = z2{scaled(det.x, sc), scaled(det.y, sc)};
+    const df n = norm(det.x * det.x + det.y * det.y);
+    const float r0 = 1.f / n.h;
+    const df r = norm(df{r0, r0 * fmaf(-n.l, r0, fmaf(-n.h, r0, 1.f))});      // a Newton step for 1 / n
+    const z2 w{scaled(norm(det.x * r), sc), scaled(norm(-(det.y * r)), sc)}, m = -w;
+    return norm(M22{p.d * w, p.b * m, p.c * m, p.a * w});
 }
 
 // Symbols of one frequency: prod of the y, z masses and the two transverse terms.
 __device__ __forceinline__ void symbols(const SweepGeom &g, int i1, int i2, double &myz, double &by, double &bz) {
-    double th[3] = {0.0, 0.0, 0.0};
-    const double PI2 = 6.28318530717958647692;
-    if (g.ax1 >= 0) th[g.ax1] = PI2 * i1 / g.n1;
-    if (g.ax2 >= 0) th[g.ax2] = PI2 * i2 / g.n2;
-    const double my = g.d >= 2 ? g.h[1] * (2.0 + cos(th[1])) / 3.0 : 1.0;
-    const double mz = g.d >= 3 ? g.h[2] * (2.0 + cos(th[2])) / 3.0 : 1.0;
+    // (sine and cosine of an angle come together: the FP64 unit is what these lines wait for)
+    double s1 = 0.0, c1 = 1.0, s2 = 0.0, c2 = 1.0;
+    if (g.ax1 >= 0) sincospi(2.0 * i1 / g.n1, &s1, &c1);
+    if (g.ax2 >= 0) sincospi(2.0 * i2 / g.n2, &s2, &c2);
+    const double sy = g.ax1 == 1 ? s1 : (g.ax2 == 1 ? s2 : 0.0), cy = g.ax1 == 1 ? c1 : (g.ax2 == 1 ? c2 : 1.0);
+    const double sz = g.ax1 == 2 ? s1 : (g.ax2 == 2 ? s2 : 0.0), cz = g.ax1 == 2 ? c1 : (g.ax2 == 2 ? c2 : 1.0);
+    const double my = g.d >= 2 ? g.h[1] * (2.0 + cy) * (1.0 / 3.0) : 1.0;
+    const double mz = g.d >= 3 ? g.h[2] * (2.0 + cz) * (1.0 / 3.0) : 1.0;
     myz = my * mz;
-    by = g.d >= 2 ? sin(th[1]) * mz : 0.0;
-    bz = g.d >= 3 ? sin(th[2]) * my : 0.0;
+    by = g.d >= 2 ? sy * mz : 0.0;
+    bz = g.d >= 3 ? sz * my : 0.0;
 }
 
 // Distinct frequencies up to sign: classes (k1, k2), k = 0 .. n/2; each has a system for
 // +P and one for -P (index 2 class + (P < 0)).
 __host__ __device__ inline int class_count(int n1, int n2) { return (n1 / 2 + 1) * (n2 / 2 + 1); }
 
-// Block (i, o) of Bd, o in {-1, 0, 1}, on unknown x node i (geometric node i + 1):
-//   i M myz + (h_t/2) [ i C myz sigma_x - M P sigma_y - diag(W+, W-) myz ].
-__device__ __forceinline__ M22 bd_block(const SweepGeom &g, const double *Vx, int i, int o, double myz, double P) {
-    const double h6 = g.h[0] / 6.0, ht2 = 0.5 * g.ht;
-    const double vl = Vx ? Vx[i] : 0.0, vr = Vx ? Vx[i + 1] : 0.0;      // elements left and right of the node
-    const double M = o == 0 ? 4.0 * h6 : h6, C = 0.5 * o;
-    const double v = o == 0 ? 2.0 * (vl + vr) : (o < 0 ? vl : vr), mw = o == 0 ? 4.0 * g.m : g.m;
-    const double im = M * myz, c = ht2 * C * myz, s = ht2 * M * P;
-    return M22{z2{-ht2 * h6 * (mw + v) * myz, im}, z2{0.0, c + s}, z2{0.0, c - s}, z2{-ht2 * h6 * (v - mw) * myz, im}};
+// A block of Bd at offset o from its x node, o in {-1, 0, 1}:
+//   i M myz + (h_t/2) [ i C myz sigma_x - M P sigma_y - diag(W+, W-) myz ],
+// from im = h/6 myz, c = h_t/4 myz, s = h_t/2 h/6 P, w = h_t/2 im and v, the potential of
+// the element at that side (o = 0: 2 (left + right)).
+struct BdSymbols { df im, c, s, w, m; };
+__device__ __forceinline__ M22 bd_block(const BdSymbols &q, int o, df v) {
+    const float k = o == 0 ? 4.f : 1.f;
+    const df im = scaled(q.im, k), s = scaled(q.s, k), m = scaled(q.m, k), z{0.f, 0.f};
+    const df c = o == 0 ? z : (o < 0 ? -q.c : q.c);
+    return norm(M22{z2{-(q.w * (v + m)), im}, z2{z, c + s}, z2{z, c - s}, z2{-(q.w * (v - m)), im}});
 }
 
 // Number of factor blocks per lane: the cyclic step's pair, a pair per parallel step,
@@ -88,8 +123,13 @@ __host__ __device__ inline int items(int steps) { return 6 + 2 * steps; }
 
 __device__ __forceinline__ void put(float *tab, int G, int item, int lane, const M22 &m) {
     float4 *o = reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8);
-    o[0] = make_float4((float)m.a.x, (float)m.a.y, (float)m.b.x, (float)m.b.y);
-    o[1] = make_float4((float)m.c.x, (float)m.c.y, (float)m.d.x, (float)m.d.y);
+    o[0] = make_float4(m.a.x.h, m.a.y.h, m.b.x.h, m.b.y.h);
+    o[1] = make_float4(m.c.x.h, m.c.y.h, m.d.x.h, m.d.y.h);
+}
+__device__ __forceinline__ void put_scaled(float *tab, int G, int item, int lane, const M22 &m, int k) {   // 2^k m
+    float4 *o = reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8);
+    o[0] = make_float4(scalbnf(m.a.x.h, k), scalbnf(m.a.y.h, k), scalbnf(m.b.x.h, k), scalbnf(m.b.y.h, k));
+    o[1] = make_float4(scalbnf(m.c.x.h, k), scalbnf(m.c.y.h, k), scalbnf(m.d.x.h, k), scalbnf(m.d.y.h, k));
 }
 
 // The row of one frequency.
@@ -103,9 +143,13 @@ __device__ __forceinline__ FreqRow freq_row(const SweepGeom &g, int f) {
     return FreqRow{(float)myz, (float)hypot(by, bz), (float)cos(0.5 * phi), (float)sin(0.5 * phi), sys};
 }
 
-// Factors of every distinct system, in FP64, stored in FP32.  G lanes per system; the
-// neighbours' blocks pass through shared memory (three M22 per lane).  The CTAs after the
-// last system's write the rows of the frequencies.
+// Factors of every distinct system in 48 bits (pairs of floats), stored in FP32: every
+// block is scaled by one power of two per system, so that the mass is about 1.  G lanes per
+// system; the neighbours' blocks pass through shared memory (three M22 per lane, by
+// quarters of 16 bytes, so that a warp's accesses are contiguous).  The CTAs after the last
+// system's write the rows of the frequencies.
+// In FP64 the 2 x 625 systems of the 48^3 x 48 Klein mesh kept the FP64 unit busy for
+// 215 us.
 __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int steps, const double *__restrict__ Vx,
                                                      float *__restrict__ table, FreqRow *__restrict__ freq) {
     extern __shared__ __align__(16) unsigned char fsm[];
@@ -115,7 +159,7 @@ __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int ste
         if (f < g.n1 * g.n2) freq[f] = freq_row(g, f);
         return;
     }
-    M22 *xi = reinterpret_cast<M22 *>(fsm), *xl = xi + blockDim.x, *xu = xl + blockDim.x;
+    float4 *xch = reinterpret_cast<float4 *>(fsm);
     const int l = threadIdx.x % G, base = threadIdx.x - l;
     const int nsys = 2 * class_count(g.n1, g.n2);
     const int sys = blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
@@ -123,32 +167,55 @@ __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int ste
     const int cls = (live ? sys : 0) / 2, q2 = g.n2 / 2 + 1;
     double myz, by, bz;
     symbols(g, cls / q2, cls % q2, myz, by, bz);
-    const double P = ((sys & 1) ? -1.0 : 1.0) * hypot(by, bz);
+    const int k2 = -ilogb(myz * g.h[0]);
+    myz = scalbn(myz, k2);
+    const double P = scalbn(((sys & 1) ? -1.0 : 1.0) * sqrt(by * by + bz * bz), k2), h6 = g.h[0] * (1.0 / 6.0), ht2 = 0.5 * g.ht;
+    const BdSymbols q{to_df(h6 * myz), to_df(0.5 * ht2 * myz), to_df(ht2 * h6 * P), to_df(ht2 * h6 * myz), to_df(g.m)};
     const int n = g.nx, e = 2 * l, o = e + 1;
     float *tab = table + (size_t)(live ? sys : 0) * items(steps) * G * 8;
-    const z2 one{1.0, 0.0}, nil{0.0, 0.0};
-    M22 L = zero22(), U = zero22(), D = M22{one, nil, nil, one}, Lo = zero22(), Uo = zero22(), Doi = zero22();
+    const df one{1.f, 0.f}, nil{0.f, 0.f};
+    const z2 z1{one, nil}, z0{nil, nil};
+    M22 L = zero22(), U = zero22(), D = M22{z1, z0, z0, z1}, Lo = zero22(), Uo = zero22(), Doi = zero22();
+    df v[3];                                                 // elements e, e + 1, e + 2
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = Vx && e + k <= n ? to_df(Vx[e + k]) : nil;
     if (e < n) {
-        D = bd_block(g, Vx, e, 0, myz, P);
-        if (e > 0) L = bd_block(g, Vx, e, -1, myz, P);
+        D = bd_block(q, 0, scaled(v[0] + v[1], 2.f));
+        if (e > 0) L = bd_block(q, -1, v[0]);
         if (o < n) {
-            U = bd_block(g, Vx, e, 1, myz, P);
-            Doi = inv(bd_block(g, Vx, o, 0, myz, P));
-            Lo = bd_block(g, Vx, o, -1, myz, P);
-            if (o + 1 < n) Uo = bd_block(g, Vx, o, 1, myz, P);
+            U = bd_block(q, 1, v[1]);
+            Doi = inv(bd_block(q, 0, scaled(v[1] + v[2], 2.f)));
+            Lo = bd_block(q, -1, v[1]);
+            if (o + 1 < n) Uo = bd_block(q, 1, v[2]);
         }
     }
+    const int T = blockDim.x;
+    auto put_x = [&](int which, const M22 &m) {
+        const z2 *z = &m.a;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) xch[(4 * which + k) * T + threadIdx.x] = make_float4(z[k].x.h, z[k].x.l, z[k].y.h, z[k].y.l);
+    };
+    auto get_x = [&](int which, int at) {
+        M22 m;
+        z2 *z = &m.a;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float4 w = xch[(4 * which + k) * T + at];
+            z[k] = z2{df{w.x, w.y}, df{w.z, w.w}};
+        }
+        return m;
+    };
     auto publish = [&](const M22 &a, const M22 &b, const M22 &c) {
         __syncthreads();
-        xi[threadIdx.x] = a; xl[threadIdx.x] = b; xu[threadIdx.x] = c;
+        put_x(0, a); put_x(1, b); put_x(2, c);
         __syncthreads();
     };
     publish(Doi, Lo, Uo);
     {
         const int left = l > 0 ? threadIdx.x - 1 : threadIdx.x;       // l = 0: L = 0, any block will do
-        const M22 A = mul(L, xi[left]), Bm = mul(U, Doi);
-        D = sub(sub(D, mul(A, xu[left])), mul(Bm, Lo));
-        L = neg(mul(A, xl[left]));
+        const M22 A = mul(L, get_x(0, left)), Bm = mul(U, Doi);
+        D = sub(sub(D, mul(A, get_x(2, left))), mul(Bm, Lo));
+        L = neg(mul(A, get_x(1, left)));
         U = neg(mul(Bm, Uo));
         if (live) { put(tab, G, 0, l, A); put(tab, G, 1, l, Bm); }
     }
@@ -157,16 +224,16 @@ __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int ste
         publish(inv(D), L, U);
         const bool hl = l >= st, hr = l + st < G;
         const int il = hl ? threadIdx.x - st : base, ir = hr ? threadIdx.x + st : base;
-        const M22 al = hl ? mul(L, xi[il]) : zero22(), ga = hr ? mul(U, xi[ir]) : zero22();
-        D = sub(sub(D, mul(al, xu[il])), mul(ga, xl[ir]));
-        L = neg(mul(al, xl[il]));
-        U = neg(mul(ga, xu[ir]));
+        const M22 al = hl ? mul(L, get_x(0, il)) : zero22(), ga = hr ? mul(U, get_x(0, ir)) : zero22();
+        D = sub(sub(D, mul(al, get_x(2, il))), mul(ga, get_x(1, ir)));
+        L = neg(mul(al, get_x(1, il)));
+        U = neg(mul(ga, get_x(2, ir)));
         if (live) { put(tab, G, 2 + 2 * s, l, al); put(tab, G, 3 + 2 * s, l, ga); }
     }
     if (live) {
         const int at = 2 + 2 * steps;
-        put(tab, G, at, l, inv(D));
-        put(tab, G, at + 1, l, Doi);
+        put_scaled(tab, G, at, l, inv(D), k2);
+        put_scaled(tab, G, at + 1, l, Doi, k2);
         put(tab, G, at + 2, l, mul(Doi, Lo));
         put(tab, G, at + 3, l, mul(Doi, Uo));
     }
