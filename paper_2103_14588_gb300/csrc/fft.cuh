@@ -25,8 +25,7 @@
 
 namespace dst_fft {
 
-constexpr int FFT_THREADS = 256;
-constexpr int FFT_WARPS = FFT_THREADS / 32;
+constexpr int FFT_THREADS = 256;          // at most
 
 template <typename V> struct Real;
 template <> struct Real<float2> { using type = float; };
@@ -134,16 +133,17 @@ template <> struct Dft<16> {
 
 // One butterfly of a stage: elements j + r q of a line (element stride st) times
 // w^(r k step), to (j / Ns) Ns R + k + o Ns of the output line; q = n / R, step = q / Ns.
-template <int R, typename V, int W, typename S>
+// The first stage (Ns = 1) has no factors.
+template <int R, bool FIRST, typename V, int W, typename S>
 __device__ __forceinline__ void butterfly(const Elem<V, W> *src, Elem<V, W> *dst, int st, int q, int step, int Ns, int j,
                                           int k, const V *w, S sg) {
     V v[W][R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const Elem<V, W> e = src[(j + r * q) * st];
-        const V t = r ? w[r * k * step] : V{};
+        const V t = r && !FIRST ? w[r * k * step] : V{};
 #pragma unroll
-        for (int c = 0; c < W; ++c) v[c][r] = r ? cmul(e.c[c], t) : e.c[c];
+        for (int c = 0; c < W; ++c) v[c][r] = r && !FIRST ? cmul(e.c[c], t) : e.c[c];
     }
 #pragma unroll
     for (int c = 0; c < W; ++c) Dft<R>::run(v[c], sg);
@@ -177,19 +177,19 @@ __device__ __forceinline__ Elem<V, W> general_output(const Elem<V, W> *src, int 
 
 // Every butterfly of one stage for threads `id` of `count`; line l starts at line(l),
 // `nl` lines, element stride st; neighbouring threads take neighbouring lines.
-template <typename V, int W, typename S, typename Line>
+template <bool FIRST, typename V, int W, typename S, typename Line>
 __device__ __forceinline__ void stage(const Elem<V, W> *d0, Elem<V, W> *d1, int n, int st, int nl, Line line, int R, int Ns,
                                       const V *w, S sg, int id, int count) {
     const int q = n / R, step = q / Ns;
     // quotients by nl and Ns by multiplication: the dividends stay below 2^32 / divisor
     const unsigned rn = nl > 1 ? 0xffffffffu / (unsigned)nl + 1u : 0u, rk = Ns > 1 ? 0xffffffffu / (unsigned)Ns + 1u : 0u;
     auto by_nl = [&](int i) { return nl > 1 ? (int)__umulhi((unsigned)i, rn) : i; };
-    auto mod_ns = [&](int j) { return Ns > 1 ? j - (int)__umulhi((unsigned)j, rk) * Ns : 0; };
+    auto mod_ns = [&](int j) { return !FIRST && Ns > 1 ? j - (int)__umulhi((unsigned)j, rk) * Ns : 0; };
     auto each = [&](auto radix) {
         constexpr int RR = decltype(radix)::value;
         for (int i = id; i < nl * q; i += count) {
             const int j = by_nl(i), l = i - j * nl, base = line(l), k = mod_ns(j);
-            butterfly<RR>(d0 + base, d1 + base, st, q, step, Ns, j, k, w, sg);
+            butterfly<RR, FIRST>(d0 + base, d1 + base, st, q, step, Ns, j, k, w, sg);
         }
     };
     switch (R) {
@@ -209,7 +209,7 @@ __device__ __forceinline__ void stage(const Elem<V, W> *d0, Elem<V, W> *d1, int 
 }
 
 template <typename V, int W, typename S>
-__device__ void warp_fft_line(Elem<V, W> *line, int st, int n, const int *rad, int nrad, const V *w, S sg, Elem<V, W> *a,
+__device__ __forceinline__ void warp_fft_line(Elem<V, W> *line, int st, int n, const int *rad, int nrad, const V *w, S sg, Elem<V, W> *a,
                               Elem<V, W> *b) {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < n; i += 32) a[i] = line[i * st];
@@ -217,7 +217,8 @@ __device__ void warp_fft_line(Elem<V, W> *line, int st, int n, const int *rad, i
     Elem<V, W> *d0 = a, *d1 = b;
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
-        stage(d0, d1, n, 1, 1, [](int) { return 0; }, rad[s], Ns, w, sg, lane, 32);
+        if (s == 0) stage<true>(d0, d1, n, 1, 1, [](int) { return 0; }, rad[s], 1, w, sg, lane, 32);
+        else stage<false>(d0, d1, n, 1, 1, [](int) { return 0; }, rad[s], Ns, w, sg, lane, 32);
         __syncwarp();
         Elem<V, W> *t = d0; d0 = d1; d1 = t;
         Ns *= rad[s];
@@ -230,11 +231,12 @@ __device__ void warp_fft_line(Elem<V, W> *line, int st, int n, const int *rad, i
 // between stages (ping-pong between the two plane buffers).  Returns the buffer that
 // holds the result.
 template <typename V, int W, typename S, typename Line>
-__device__ Elem<V, W> *cta_fft_axis(Elem<V, W> *d0, Elem<V, W> *d1, int n, int st, int nl, Line line, const int *rad,
+__device__ __forceinline__ Elem<V, W> *cta_fft_axis(Elem<V, W> *d0, Elem<V, W> *d1, int n, int st, int nl, Line line, const int *rad,
                                     int nrad, const V *w, S sg) {
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
-        stage(d0, d1, n, st, nl, line, rad[s], Ns, w, sg, threadIdx.x, FFT_THREADS);
+        if (s == 0) stage<true>(d0, d1, n, st, nl, line, rad[s], 1, w, sg, threadIdx.x, blockDim.x);
+        else stage<false>(d0, d1, n, st, nl, line, rad[s], Ns, w, sg, threadIdx.x, blockDim.x);
         __syncthreads();
         Elem<V, W> *t = d0; d0 = d1; d1 = t;
         Ns *= rad[s];
@@ -247,26 +249,36 @@ __host__ __device__ inline int pitch(const SweepFft &a) { return a.pingpong ? a.
 
 // Shared memory of one CTA: the plane, two twiddle tables, and a second plane or two
 // scratch lines per warp.
+// Threads per plane: a butterfly of four points or more each.  A line of 96 nodes alone
+// in its plane leaves all but one warp of a larger CTA waiting (2+1 sweep of 96 x 96 x 96:
+// 449 us with 256 threads, 302 us with 32); planes of 1024 nodes and more want all 256
+// (48 x 48: 698 us against 780 us with 128).
+inline unsigned fft_threads(const SweepFft &a) {
+    return (unsigned)std::min(FFT_THREADS, std::max(32, (a.n1 * a.n2 / 4 + 31) / 32 * 32));
+}
 template <typename V>
 inline size_t fft_smem_bytes(const SweepFft &a) {
     const int nmax = a.n1 > a.n2 ? a.n1 : a.n2;
     const size_t plane = (size_t)a.ncb * a.n1 * pitch(a);
-    const size_t scratch = a.pingpong ? plane : (size_t)FFT_WARPS * 2 * nmax * a.ncb;
+    const size_t scratch = a.pingpong ? plane : (size_t)(fft_threads(a) / 32) * 2 * nmax * a.ncb;
     return sizeof(V) * (plane + a.n1 + a.n2 + scratch);
 }
 
-// W = a.ncb components per CTA.
-template <typename V, int W>
+// W = a.ncb components per CTA.  The direction is a constant of the kernel: the
+// multiplications by +-i in the butterflies are then signs of their sums.
+template <typename V, int W, bool INVERSE>
 __global__ void __launch_bounds__(FFT_THREADS)
-fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restrict__ out) {
+fft_planes_kernel(SweepFft a, const V *__restrict__ in, V *__restrict__ out) {
     using R = typename Real<V>::type;
+    constexpr bool inverse = INVERSE;
+    constexpr R sign = INVERSE ? (R)1 : (R)-1;
     using E = Elem<V, W>;
     extern __shared__ __align__(16) unsigned char fft_sm_raw[];
     const int n1 = a.n1, n2 = a.n2, nc = a.nc, pt = pitch(a);
     const int nf = n1 * n2, pl = n1 * pt, nmax = n1 > n2 ? n1 : n2;
     E *plane = reinterpret_cast<E *>(fft_sm_raw);         // [n1][pitch]
     E *scr = plane + pl;                                  // second plane, or per warp two lines of nmax
-    V *w1 = reinterpret_cast<V *>(scr + (a.pingpong ? pl : FFT_WARPS * 2 * nmax));   // twiddles of the outer axis (n1)
+    V *w1 = reinterpret_cast<V *>(scr + (a.pingpong ? pl : (int)(blockDim.x >> 5) * 2 * nmax));   // twiddles of the outer axis (n1)
     V *w2 = w1 + n1;                                      // twiddles of the inner axis (n2)
     // the component groups of a plane are neighbours in the grid: together they use the
     // sectors that each touches half of (apart, DRAM saw three times the plane's bytes)
@@ -274,22 +286,21 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
     const int64_t b = blockIdx.x / groups;
     const int c0 = (int)(blockIdx.x % groups) * W;
     const int64_t base = (b / a.nbx) * a.ns_nodes + (b % a.nbx) * a.sbx;   // node index of (i1, i2) = (0, 0)
-    const R sign = inverse ? (R)1 : (R)-1;
     const unsigned r2 = n2 > 1 ? 0xffffffffu / (unsigned)n2 + 1u : 0u;
     auto row = [&](int f) { return n2 > 1 ? (int)__umulhi((unsigned)f, r2) : f; };
     const V *src = in + (inverse ? b * nf : base) * nc + c0;
 #pragma unroll 4
-    for (int f = threadIdx.x; f < nf; f += FFT_THREADS) {
+    for (int f = threadIdx.x; f < nf; f += blockDim.x) {
         const int i1 = row(f), i2 = f - i1 * n2;
         copy_elem<V, W>(plane + i1 * pt + i2, src + (inverse ? (int64_t)f : i1 * a.s1 + i2 * a.s2) * nc);
     }
     // the twiddles while the plane is on its way
-    for (int j = threadIdx.x; j < n1; j += FFT_THREADS) {
+    for (int j = threadIdx.x; j < n1; j += blockDim.x) {
         R sn, cs;
         sincos_pi((R)2 * (R)j / (R)n1, &sn, &cs);
         w1[j] = mk<V>(cs, sign * sn);
     }
-    for (int j = threadIdx.x; j < n2; j += FFT_THREADS) {
+    for (int j = threadIdx.x; j < n2; j += blockDim.x) {
         R sn, cs;
         sincos_pi((R)2 * (R)j / (R)n2, &sn, &cs);
         w2[j] = mk<V>(cs, sign * sn);
@@ -306,17 +317,17 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
         const int warp = threadIdx.x >> 5;
         E *sa = scr + (size_t)warp * 2 * nmax, *sb = sa + nmax;
         if (n2 > 1)
-            for (int line = warp; line < n1; line += FFT_WARPS)
+            for (int line = warp; line < n1; line += blockDim.x >> 5)
                 warp_fft_line(plane + (size_t)line * n2, 1, n2, a.rad2, a.nrad2, w2, sign, sa, sb);
         __syncthreads();
         if (n1 > 1)
-            for (int line = warp; line < n2; line += FFT_WARPS)
+            for (int line = warp; line < n2; line += blockDim.x >> 5)
                 warp_fft_line(plane + line, n2, n1, a.rad1, a.nrad1, w1, sign, sa, sb);
         __syncthreads();
     }
     const R scale = inverse ? (R)1 / (R)nf : (R)1;
     V *dst = out + (inverse ? base : b * nf) * nc + c0;
-    for (int f = threadIdx.x; f < nf; f += FFT_THREADS) {
+    for (int f = threadIdx.x; f < nf; f += blockDim.x) {
         const int i1 = row(f), i2 = f - i1 * n2;
         E v = cur[i1 * pt + i2];
 #pragma unroll
@@ -327,17 +338,17 @@ fft_planes_kernel(SweepFft a, int inverse, const V *__restrict__ in, V *__restri
 
 // The planes `nb` of every component group.  The kernel's shared-memory limit is a
 // per-device attribute, set once.
-template <typename V>
-inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, int inverse, const V *in, V *out, cudaStream_t s) {
+template <typename V, bool INVERSE>
+inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, const V *in, V *out, cudaStream_t s) {
     static bool configured[64] = {};
+    const auto one = fft_planes_kernel<V, 1, INVERSE>, two = fft_planes_kernel<V, 2, INVERSE>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
         const int limit = 200 * 1024;
-        e = cudaFuncSetAttribute(fft_planes_kernel<V, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fft_planes_kernel<V, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+        e = cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(two, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
@@ -345,8 +356,7 @@ inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, int inverse, const 
     SweepFft b = a;
     if ((((uintptr_t)in | (uintptr_t)out) & 15) != 0) b.ncb = 1;
     const unsigned grid = (unsigned)(nb * (b.nc / b.ncb));
-    if (b.ncb == 2) fft_planes_kernel<V, 2><<<grid, FFT_THREADS, fft_smem_bytes<V>(b), s>>>(b, inverse, in, out);
-    else fft_planes_kernel<V, 1><<<grid, FFT_THREADS, fft_smem_bytes<V>(b), s>>>(b, inverse, in, out);
+    (b.ncb == 2 ? two : one)<<<grid, fft_threads(b), fft_smem_bytes<V>(b), s>>>(b, in, out);
     return cudaGetLastError();
 }
 

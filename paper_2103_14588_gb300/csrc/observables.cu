@@ -189,8 +189,8 @@ int energy_impl(const dst_mesh *mesh, const double2 *psi, double *out, cudaStrea
         return DST_ERR_OOM;
     }
     int rc = DST_OK;
-    cudaError_t fe = dst_fft::fft_launch<double2>(a1, mesh->nt * nz, 0, psi, b1, s);
-    if (fe == cudaSuccess && mesh->d == 3) fe = dst_fft::fft_launch<double2>(a2, mesh->nt * nfyx, 0, b1, b2, s);
+    cudaError_t fe = dst_fft::fft_launch<double2, false>(a1, mesh->nt * nz, psi, b1, s);
+    if (fe == cudaSuccess && mesh->d == 3) fe = dst_fft::fft_launch<double2, false>(a2, mesh->nt * nfyx, b1, b2, s);
     if (fe != cudaSuccess) {
         dst_internal_set_cuda_error(fe, "energy FFT", __FILE__, __LINE__);
         rc = DST_ERR_CUDA;

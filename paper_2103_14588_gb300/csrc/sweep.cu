@@ -286,7 +286,7 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
     // buffer is marched in work too)
     const bool aside = !p.has_fft && (((uintptr_t)v | (uintptr_t)z) & 15) != 0;
     if (p.has_fft) {
-        DST_CUDA_TRY(dst_fft::fft_launch<float2>(p.fft, p.nb, 0, v, p.work, s));
+        DST_CUDA_TRY((dst_fft::fft_launch<float2, false>(p.fft, p.nb, v, p.work, s)));
         src = dst = p.work;
     } else if (aside) {
         DST_CUDA_TRY(cudaMemcpyAsync(p.work, v, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
@@ -303,7 +303,7 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
         if (rc) return rc;
     }
     // 3. inverse FFT: work -> z
-    if (p.has_fft) DST_CUDA_TRY(dst_fft::fft_launch<float2>(p.fft, p.nb, 1, p.work, z, s));
+    if (p.has_fft) DST_CUDA_TRY((dst_fft::fft_launch<float2, true>(p.fft, p.nb, p.work, z, s)));
     else if (aside) DST_CUDA_TRY(cudaMemcpyAsync(z, p.work, sizeof(float2) * n_unknowns, cudaMemcpyDeviceToDevice, s));
     return DST_OK;
 }
