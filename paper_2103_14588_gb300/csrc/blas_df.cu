@@ -27,6 +27,7 @@
 // products and updates keep FP64-class accuracy with respect to the stored
 // values; updated vectors are rounded to FP32 once.
 #include <algorithm>
+#include <type_traits>
 
 #include "blas.h"
 #include "df_arith.cuh"
@@ -61,6 +62,50 @@ __device__ __forceinline__ void cdot_acc(float vhr, float vhi, float vlr, float 
     df_prod_t<VL, WL>(vhi, vli, ar, alr, p2, e2);
     im.add(p1, e1);
     im.add(-p2, -e2);
+}
+
+// h[j] = sum of the CTAs' partials [cta][nvec] (and *wnrm2 that of `wparts`, when wanted), by
+// `nw` warps of one CTA: the lanes stride over the CTAs, then a fixed tree.  A warp takes
+// QB sums at a time: their loads are in flight together and the tree adds for all of them
+// at once (one sum at a time, the last CTA kept the projection of 30 vectors of 1.77M
+// entries waiting for 4 us).
+template <int QB>
+__device__ __forceinline__ void sum_columns(const double *pd, const double *wparts, int ctas, int nvec, int nw,
+                                            double2 *h, double *wnrm2) {
+    constexpr int IT = 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q0 = warp * QB; q0 < 2 * nvec + 1; q0 += QB * nw) {
+        double t[QB] = {};
+        for (int k0 = lane; k0 < ctas + lane; k0 += 32 * IT) {
+            double v[QB][IT];
+#pragma unroll
+            for (int c = 0; c < QB; ++c) {
+                const int q = q0 + c;
+                const double *col = q < 2 * nvec ? pd + q : wparts;
+                const size_t step = q < 2 * nvec ? 2 * nvec : 1;
+                const bool want = q < 2 * nvec || (q == 2 * nvec && wnrm2);
+#pragma unroll
+                for (int k = 0; k < IT; ++k)
+                    v[c][k] = want && k0 + 32 * k < ctas ? __ldcg(col + (size_t)(k0 + 32 * k) * step) : 0.0;
+            }
+#pragma unroll
+            for (int c = 0; c < QB; ++c)
+#pragma unroll
+                for (int k = 0; k < IT; ++k)
+                    if (k0 - lane + 32 * k < ctas && q0 + c < 2 * nvec + 1) t[c] += v[c][k];
+        }
+        const double r = dwarp_sums(t);
+        const int q = q0 + lane / (32 / QB);
+        if (lane % (32 / QB) == 0) {
+            if (q < 2 * nvec) reinterpret_cast<double *>(h)[q] = r;
+            else if (q == 2 * nvec && wnrm2) *wnrm2 = r;
+        }
+    }
+}
+__device__ __forceinline__ void sum_partials(const double *pd, const double *wparts, int ctas, int nvec, int nw, double2 *h,
+                                             double *wnrm2) {
+    if (nvec < 8) sum_columns<2>(pd, wparts, ctas, nvec, nw, h, wnrm2);
+    else sum_columns<4>(pd, wparts, ctas, nvec, nw, h, wnrm2);
 }
 
 // h_j partials = sum conj(V_j) w over the CTA's slice; ||w||^2 partials.
@@ -120,13 +165,11 @@ project_df_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const float
                 }
             }
         }
+        DfAcc all[2 * DF_GROUP];
 #pragma unroll
-        for (int g = 0; g < DF_GROUP; ++g) {
-            if (g < gv) {
-                const double sr = dfwarp_sum(re[g]), si = dfwarp_sum(im[g]);
-                if (lane == 0) { red[warp][2 * (j0 + g)] = sr; red[warp][2 * (j0 + g) + 1] = si; }
-            }
-        }
+        for (int g = 0; g < DF_GROUP; ++g) { all[2 * g] = re[g]; all[2 * g + 1] = im[g]; }
+        const double t = dfwarp_sums(all);
+        if (lane % 4 == 0 && lane / 4 < 2 * gv) red[warp][2 * j0 + lane / 4] = t;
     }
     const double wsum = dfwarp_sum(wn);
     if (lane == 0) red[warp][2 * DST_MAX_VEC] = wsum;
@@ -151,21 +194,7 @@ project_df_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const float
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // one warp per value: lanes stride over the CTAs, then a fixed shuffle tree
-    const double *pd = reinterpret_cast<const double *>(partials);
-    for (int q = warp; q < 2 * nvec + 1; q += NW) {
-        double s_ = 0.0;
-        if (q < 2 * nvec) {
-            for (unsigned k = lane; k < gridDim.x; k += 32) s_ += __ldcg(pd + (size_t)k * 2 * nvec + q);
-        } else if (wnrm2) {
-            for (unsigned k = lane; k < gridDim.x; k += 32) s_ += __ldcg(wnrm_partials + k);
-        }
-        s_ = dwarp_sum(s_);
-        if (lane == 0) {
-            if (q < 2 * nvec) reinterpret_cast<double *>(h)[q] = s_;
-            else if (wnrm2) *wnrm2 = s_;
-        }
-    }
+    sum_partials(reinterpret_cast<const double *>(partials), wnrm_partials, (int)gridDim.x, nvec, NW, h, wnrm2);
     __syncthreads();
     if (threadIdx.x == 0) *ticket = 0u;
 }
@@ -318,16 +347,14 @@ project_f32_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
                 }
             }
         }
+        DfAcc all[2 * DF_GROUP];
 #pragma unroll
-        for (int g = 0; g < DF_GROUP; ++g) {
-            if (g < gv) {
-                DfAcc r_, i_;
-                r_.hi = re[g].hi - sigma; r_.lo = re[g].lo;      // exact differences
-                i_.hi = im[g].hi - sigma; i_.lo = im[g].lo;
-                const double sr = dfwarp_sum(r_), si = dfwarp_sum(i_);
-                if (lane == 0) { red[warp][2 * (j0 + g)] = sr; red[warp][2 * (j0 + g) + 1] = si; }
-            }
+        for (int g = 0; g < DF_GROUP; ++g) {                     // exact differences
+            all[2 * g].hi = re[g].hi - sigma; all[2 * g].lo = re[g].lo;
+            all[2 * g + 1].hi = im[g].hi - sigma; all[2 * g + 1].lo = im[g].lo;
         }
+        const double t = dfwarp_sums(all);
+        if (lane % 4 == 0 && lane / 4 < 2 * gv) red[warp][2 * j0 + lane / 4] = t;
     }
     const double wsum = dfwarp_sum(wn);
     if (lane == 0) red[warp][2 * DST_MAX_VEC] = wsum;
@@ -351,20 +378,7 @@ project_f32_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
     __syncthreads();
     if (!last) return;
     __threadfence();
-    const double *pd = reinterpret_cast<const double *>(partials);
-    for (int q = warp; q < 2 * nvec + 1; q += NW) {
-        double s_ = 0.0;
-        if (q < 2 * nvec) {
-            for (unsigned k = lane; k < gridDim.x; k += 32) s_ += __ldcg(pd + (size_t)k * 2 * nvec + q);
-        } else if (wnrm2) {
-            for (unsigned k = lane; k < gridDim.x; k += 32) s_ += __ldcg(wnrm_partials + k);
-        }
-        s_ = dwarp_sum(s_);
-        if (lane == 0) {
-            if (q < 2 * nvec) reinterpret_cast<double *>(h)[q] = s_;
-            else if (wnrm2) *wnrm2 = s_;
-        }
-    }
+    sum_partials(reinterpret_cast<const double *>(partials), wnrm_partials, (int)gridDim.x, nvec, NW, h, wnrm2);
     __syncthreads();
     if (threadIdx.x == 0) *ticket = 0u;
 }
@@ -389,12 +403,13 @@ constexpr int TMA_CHUNK = 2048;                 // entries per copy (16 KB)
 constexpr int TMA_SLOTS = 6;                    // ring: 6 x 16 KB (two CTAs per SM)
 constexpr int TMA_SMEM = TMA_SLOTS * TMA_CHUNK * 8;
 constexpr unsigned TMA_WAIT_LIMIT = 1u << 22;   // try_wait attempts before a wait is declared failed
+constexpr int TMA_CTAS = 2 * 152;              // one wave of two CTAs per SM
 constexpr int TMA_GROUP = 8;                    // basis vectors per projection CTA (at most)
 
 constexpr int TMA_THREADS = DF_THREADS + 32;   // eight consumer warps and one producer warp
 
-// Failure handling.  A consumer warp that meets a failed wait (or sees that
-// another warp failed) stops consuming at once: it neither reads nor releases
+// Failure handling.  A consumer warp that meets a failed wait (or sees, once per
+// chunk, that another warp failed) stops consuming at once: it neither reads nor releases
 // that slot or any later one, and records how many copies it waited for.  A
 // copy is issued into a slot only after every consumer warp has released the
 // copy before it in that slot, and a warp releases only copies it waited for,
@@ -476,14 +491,12 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
             s_issued = k;
         }
     } else {
-        int k = 0;                                   // copies this warp waited for (and released)
-        // warp-uniform: the slot of copy k, or nullptr once a wait failed here or elsewhere
+        int k = 0, slot = 0;                         // copies this warp waited for (and released); the ring slot of copy k
+        unsigned phase = 0;
+        // warp-uniform: the slot of copy k, or nullptr once a wait failed (another warp's failure is
+        // looked for once per chunk)
         auto wait_item = [&]() -> const float4 * {
-            const int slot = k % TMA_SLOTS;
-            bool ok = __shfl_sync(0xffffffffu, *vfailed == 0 ? 1 : 0, 0) != 0;
-            if (ok) ok = mbar_wait_bounded(&full[slot], (unsigned)((k / TMA_SLOTS) & 1), wait_limit);
-            ok = __all_sync(0xffffffffu, ok) != 0;
-            if (!ok) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[slot], phase, wait_limit))) {
                 if (lane == 0) *vfailed = 1;
                 return nullptr;
             }
@@ -491,16 +504,18 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
         };
         auto release_item = [&]() {
             __syncwarp();                            // the warp is done with slot k
-            if (lane == 0) mbar_arrive(&empty[k % TMA_SLOTS]);
+            if (lane == 0) mbar_arrive(&empty[slot]);
             ++k;
+            if (++slot == TMA_SLOTS) { slot = 0; phase ^= 1u; }
         };
         bool stop = false;
         {
             const int g = grp;
-            DfAcc R[TMA_GROUP], I[TMA_GROUP];
+            DfAcc R[TMA_GROUP], I[TMA_GROUP], all[2 * TMA_GROUP];
 #pragma unroll
             for (int q = 0; q < TMA_GROUP; ++q) { R[q].zero(); I[q].zero(); }
             for (int c = 0; c < nch && !stop; ++c) {
+                if (__shfl_sync(0xffffffffu, *vfailed, 0) != 0) break;   // another warp failed
                 const int64_t c0 = b + (int64_t)c * TMA_CHUNK;
                 const int units = (int)(((e - c0 < TMA_CHUNK) ? e - c0 : TMA_CHUNK) >> 1);
                 float4 a[UPT];
@@ -532,14 +547,18 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
                     AnAcc re, im;
                     re.init(sigma);
                     im.init(sigma);
+                    auto add = [&](int i) {
+                        const float4 v = sv[tid + i * DF_THREADS];
+                        cdot_an(v.x, v.y, a[i].x, a[i].y, re, im);
+                        cdot_an(v.z, v.w, a[i].z, a[i].w, re, im);
+                    };
+                    if (units == U) {
 #pragma unroll
-                    for (int i = 0; i < UPT; ++i) {
-                        const int u = tid + i * DF_THREADS;
-                        if (u < units) {
-                            const float4 v = sv[u];
-                            cdot_an(v.x, v.y, a[i].x, a[i].y, re, im);
-                            cdot_an(v.z, v.w, a[i].z, a[i].w, re, im);
-                        }
+                        for (int i = 0; i < UPT; ++i) add(i);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < UPT; ++i)
+                            if (tid + i * DF_THREADS < units) add(i);
                     }
                     df_add(R[q].hi, R[q].lo, re.hi - sigma, re.lo);
                     df_add(I[q].hi, I[q].lo, im.hi - sigma, im.lo);
@@ -547,15 +566,22 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
                 }
             }
 #pragma unroll
-            for (int q = 0; q < TMA_GROUP; ++q) {
-                if (q < gv && !stop) {
-                    const double sr = dfwarp_sum(R[q]), si = dfwarp_sum(I[q]);
-                    if (lane == 0) {
-                        red[warp][2 * q] = sr;
-                        red[warp][2 * q + 1] = si;
-                    }
-                }
-            }
+            for (int q = 0; q < TMA_GROUP; ++q) { all[2 * q] = R[q]; all[2 * q + 1] = I[q]; }
+            // as many sums as the group has vectors, to a power of two: one warp sum after the
+            // other, their conversions to FP64 held the FP64 unit for 6 us per launch (30 vectors of
+            // 1.77M entries: 90 us, 84 us now; of 200,000: 29 us, 22 us now)
+            auto store = [&](auto count) {
+                constexpr int N = decltype(count)::value;
+                DfAcc a[N];
+#pragma unroll
+                for (int q = 0; q < N; ++q) a[q] = all[q];
+                const double t = dfwarp_sums(a);
+                const int q = lane / (32 / N);
+                if (!stop && lane % (32 / N) == 0 && q < 2 * gv) red[warp][q] = t;
+            };
+            if (gv <= 2) store(std::integral_constant<int, 4>());
+            else if (gv <= 4) store(std::integral_constant<int, 8>());
+            else store(std::integral_constant<int, 2 * TMA_GROUP>());
         }
         if (lane == 0) s_done[warp] = k;
     }
@@ -570,8 +596,10 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
     __syncthreads();
     // every issued copy was waited for by the consumers (or the producer stopped
     // issuing after a failed wait); the ring is idle here
-    const double wsum = warp < NW ? dfwarp_sum(wn) : 0.0;
-    if (lane == 0 && warp < NW) red[warp][2 * TMA_GROUP] = wsum;
+    if (grp == 0 && warp < NW) {
+        const double wsum = dfwarp_sum(wn);
+        if (lane == 0) red[warp][2 * TMA_GROUP] = wsum;
+    }
     __syncthreads();
     if (*vfailed && tid == 0 && err) *err = 1.0;
     // partials [slice][nvec]: this CTA's group of coefficients of its slice
@@ -597,19 +625,7 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
     if (!last) return;
     __threadfence();
     const double *pd = reinterpret_cast<const double *>(partials);
-    for (int q = warp; q < 2 * nvec + 1; q += NW) {
-        double s_ = 0.0;
-        if (q < 2 * nvec) {
-            for (int kk = lane; kk < nsl; kk += 32) s_ += __ldcg(pd + (size_t)kk * 2 * nvec + q);
-        } else if (wnrm2) {
-            for (int kk = lane; kk < nsl; kk += 32) s_ += __ldcg(wparts + kk);
-        }
-        s_ = dwarp_sum(s_);
-        if (lane == 0) {
-            if (q < 2 * nvec) reinterpret_cast<double *>(h)[q] = s_;
-            else if (wnrm2) *wnrm2 = s_;
-        }
-    }
+    if (warp < NW) sum_partials(pd, wparts, nsl, nvec, NW, h, wnrm2);
     __syncthreads();
     if (tid == 0) *ticket = 0u;
 }
@@ -689,13 +705,10 @@ update_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const doubl
             s_issued = k;
         }
     } else {
-        int k = 0;
+        int k = 0, slot = 0;
+        unsigned phase = 0;
         auto wait_item = [&]() -> const float4 * {
-            const int slot = k % TMA_SLOTS;
-            bool ok = __shfl_sync(0xffffffffu, *vfailed == 0 ? 1 : 0, 0) != 0;
-            if (ok) ok = mbar_wait_bounded(&full[slot], (unsigned)((k / TMA_SLOTS) & 1), wait_limit);
-            ok = __all_sync(0xffffffffu, ok) != 0;
-            if (!ok) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[slot], phase, wait_limit))) {
                 if (lane == 0) *vfailed = 1;
                 return nullptr;
             }
@@ -703,13 +716,15 @@ update_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const doubl
         };
         auto release_item = [&]() {
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[k % TMA_SLOTS]);
+            if (lane == 0) mbar_arrive(&empty[slot]);
             ++k;
+            if (++slot == TMA_SLOTS) { slot = 0; phase ^= 1u; }
         };
         const float h1 = h1_sh;
         float4 *w4 = reinterpret_cast<float4 *>(w);
         bool stop = false;
         for (int c = 0; c < nch && !stop; ++c) {
+            if (__shfl_sync(0xffffffffu, *vfailed, 0) != 0) break;   // another warp failed
             const int64_t c0 = b + (int64_t)c * TMA_CHUNK;
             const int units = (int)(((e - c0 < TMA_CHUNK) ? e - c0 : TMA_CHUNK) >> 1);
             const int64_t g0 = c0 >> 1;                  // the chunk's first float4 of w
@@ -728,14 +743,18 @@ update_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const doubl
                 const float4 *sv = wait_item();
                 if (!sv) { stop = true; break; }
                 const float4 cj = hs[j];
+                auto add = [&](int i) {
+                    const float4 v = sv[tid + i * DF_THREADS];
+                    caxpy_an(v.x, v.y, cj, acc[i][0], acc[i][1]);
+                    caxpy_an(v.z, v.w, cj, acc[i][2], acc[i][3]);
+                };
+                if (units == U) {
 #pragma unroll
-                for (int i = 0; i < UPT; ++i) {
-                    const int u = tid + i * DF_THREADS;
-                    if (u < units) {
-                        const float4 v = sv[u];
-                        caxpy_an(v.x, v.y, cj, acc[i][0], acc[i][1]);
-                        caxpy_an(v.z, v.w, cj, acc[i][2], acc[i][3]);
-                    }
+                    for (int i = 0; i < UPT; ++i) add(i);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < UPT; ++i)
+                        if (tid + i * DF_THREADS < units) add(i);
                 }
                 release_item();
             }
@@ -852,13 +871,10 @@ combine_tma_kernel(int64_t n, int k, const float2 *__restrict__ V, const double2
             s_issued = kk;
         }
     } else {
-        int q = 0;                                   // copies this warp waited for (and released)
+        int q = 0, slot = 0;                         // copies this warp waited for (and released); the ring slot of copy q
+        unsigned phase = 0;
         auto wait_item = [&]() -> const float4 * {
-            const int slot = q % TMA_SLOTS;
-            bool ok = __shfl_sync(0xffffffffu, *vfailed == 0 ? 1 : 0, 0) != 0;
-            if (ok) ok = mbar_wait_bounded(&full[slot], (unsigned)((q / TMA_SLOTS) & 1), wait_limit);
-            ok = __all_sync(0xffffffffu, ok) != 0;
-            if (!ok) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[slot], phase, wait_limit))) {
                 if (lane == 0) *vfailed = 1;
                 return nullptr;
             }
@@ -866,11 +882,13 @@ combine_tma_kernel(int64_t n, int k, const float2 *__restrict__ V, const double2
         };
         auto release_item = [&]() {
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[q % TMA_SLOTS]);
+            if (lane == 0) mbar_arrive(&empty[slot]);
             ++q;
+            if (++slot == TMA_SLOTS) { slot = 0; phase ^= 1u; }
         };
         bool stop = false;
         for (int c = 0; c < nch && !stop; ++c) {
+            if (__shfl_sync(0xffffffffu, *vfailed, 0) != 0) break;   // another warp failed
             const int64_t c0 = b + (int64_t)c * TMA_CHUNK;
             const int units = (int)(((e - c0 < TMA_CHUNK) ? e - c0 : TMA_CHUNK) >> 1);
             DfAcc ar[UPT][2], ai[UPT][2];
@@ -1171,7 +1189,7 @@ int dst_k_project_df(int64_t n, int nvec, const float2 *V, const float2 *w, bool
 
 int dst_tma_projection_blocks(int64_t n) {
     int64_t b = (n + 2047) / 2048;
-    if (b > 2 * 152) b = 2 * 152;
+    if (b > TMA_CTAS) b = TMA_CTAS;
     return (int)(b < 1 ? 1 : b);
 }
 
@@ -1188,7 +1206,7 @@ int dst_k_project_tma(int64_t n, int nvec, const float2 *V, const float2 *w, dou
     // nblk slices at most (the partials hold nblk x (nvec + 1)), one CTA per slice and group
     // of TMA_GROUP basis vectors, one wave of two CTAs per SM
     const int ngr = (nvec + TMA_GROUP - 1) / TMA_GROUP;
-    int nsl = 2 * 152 / ngr;
+    int nsl = TMA_CTAS / ngr;
     if (nsl > nblk) nsl = nblk;
     if (nsl < 1) nsl = 1;
     project_tma_kernel<<<nsl * ngr, TMA_THREADS, TMA_SMEM, s>>>(n, nvec, V, w, partials, gate, h, wnrm2, ticket, err,

@@ -66,6 +66,51 @@ __device__ __forceinline__ double dwarp_sum(double v) {
     return v;
 }
 
+// N warp sums at once (N a power of two, at most 32): each step halves the number of
+// values that a lane carries, so N values cost N + 5 - log2(N) additions of the warp in
+// place of 5 N, and the conversion to FP64 (three instructions of 64 clocks each, however
+// few lanes want them) is made once.  Lane l returns sum l N / 32, in dfwarp_sum's order.
+template <int N> __device__ __forceinline__ double dfwarp_sums(DfAcc (&a)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int m = N / 2; m >= 1; m /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const DfAcc send = up ? a[i] : a[i + m];
+            if (up) a[i] = a[i + m];
+            const float bh = __shfl_xor_sync(0xffffffffu, send.hi, o), bl = __shfl_xor_sync(0xffffffffu, send.lo, o);
+            df_add(a[i].hi, a[i].lo, bh, bl);
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o /= 2) {
+        const float bh = __shfl_xor_sync(0xffffffffu, a[0].hi, o), bl = __shfl_xor_sync(0xffffffffu, a[0].lo, o);
+        df_add(a[0].hi, a[0].lo, bh, bl);
+    }
+    return a[0].value();
+}
+
+// The same for FP64 values, in dwarp_sum's order.
+template <int N> __device__ __forceinline__ double dwarp_sums(double (&a)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int m = N / 2; m >= 1; m /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const double send = up ? a[i] : a[i + m];
+            if (up) a[i] = a[i + m];
+            a[i] += __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    return a[0];
+}
+
 // (p, e): p + e = a b exactly, plus the lo cross terms that are present
 template <bool AL, bool BL>
 __device__ __forceinline__ void df_prod_t(float ah, float al, float bh, float bl, float &p, float &e) {
