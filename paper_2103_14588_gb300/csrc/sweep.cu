@@ -44,6 +44,7 @@
 namespace {
 
 constexpr double PI2 = 6.28318530717958647692;
+constexpr int SWEEP_SMEM_LIMIT = 200 * 1024;     // dynamic shared memory of a CTA of the FFT and the march
 using namespace dst_march;
 
 // ---- 2a. spectral march: one thread per frequency ---------------------------
@@ -185,7 +186,7 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
         dst_internal_set_error_detail("Crank-Nicolson sweep: a periodic axis longer than 4096 nodes");
         return DST_ERR_ARG;
     }
-    const size_t limit = 200 * 1024;
+    const size_t limit = SWEEP_SMEM_LIMIT;
     if (p.has_fft && !dst_fft::choose_layout<float2>(a, p.nb, limit)) {
         dst_internal_set_error_detail("Crank-Nicolson sweep: a periodic plane too large for shared memory");
         return DST_ERR_ARG;
@@ -258,7 +259,8 @@ static int launch_march(const SweepPlan &p, const float2 *in, float2 *out, cudaS
     const int fper = NC == 4 ? p.systems / 2 : p.systems;
     const unsigned blocks = (unsigned)(((int64_t)p.g.n1 * p.g.n2 + fper - 1) / fper);
     auto go = [&](auto kern) -> int {
-        DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.march_smem));
+        // (the same limit for every plan: another thread may set it between this line and the launch)
+        DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SWEEP_SMEM_LIMIT));
         kern<<<blocks, (unsigned)(p.systems * p.lanes), p.march_smem, s>>>(p.g, p.steps, p.dvx, p.table, p.freq, p.alt_hi,
                                                                           p.alt_lo, in, out);
         DST_CUDA_TRY(cudaGetLastError());

@@ -302,7 +302,7 @@ static UGrid coarse(const UGrid &f) {
 // the CTAs (three or nine warps each) fill the GPU twice while the slices stay within a
 // few million partial sums; kernel 1: 32 nodes at a time, one slice per warp.
 static int wgrad_seg(const UGrid &g) {
-    const int nx = g.n[g.D - 1], segs = (nx + 63) / 64;
+    const int nx = g.n[g.D - 1], segs = (nx + WG_MAX_SEG - 1) / WG_MAX_SEG;
     return (nx + segs - 1) / segs;
 }
 static int wgrad_items(const Layer &L, const UGrid &g) {
@@ -564,7 +564,9 @@ static int conv_wgrad(dst_unet *u, int l, const bf16 *in, const bf16 *dz, cudaSt
         const dim3 grid((unsigned)slices, rows16, (unsigned)(offsets / warps));
         auto go = [&](auto kern, int ci8) -> int {
             const size_t smem = 2 * wg_buffer(ci8, warps, a.seg);
-            DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            // (the kernel's largest: another thread's mesh may set it between this line and the launch)
+            DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)(2 * wg_buffer(ci8, 9, WG_MAX_SEG))));
             kern<<<grid, 32 * warps, smem, s>>>(a);
             return DST_OK;
         };

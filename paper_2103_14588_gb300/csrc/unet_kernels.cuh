@@ -376,6 +376,7 @@ __device__ __forceinline__ void ldsm2t(uint32_t &a, uint32_t &b, const void *p) 
 __host__ __device__ constexpr int wg_pitch(int channels) { return channels * 2 + 16; }
 constexpr int WG_DZ = wg_pitch(16);            // dz: 16 channels of the CTA's row block
 
+constexpr int WG_MAX_SEG = 64;                 // nodes of a segment of an x line, at most
 __host__ __device__ inline int wg_padded(int seg) { return (seg + 15) / 16 * 16; }
 __host__ __device__ inline size_t wg_buffer(int ci8, int warps, int seg) {
     return (size_t)warps * (wg_padded(seg) + 2) * wg_pitch(ci8 * 8) + (size_t)wg_padded(seg) * WG_DZ;
