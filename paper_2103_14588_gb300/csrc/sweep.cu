@@ -246,9 +246,9 @@ int dst_sweep_setup(const dst_mesh *mesh, SweepPlan &p, void *scratch, cudaStrea
         DST_CUDA_TRY(cudaMemcpyAsync(p.dvx, mesh->V.data(), sizeof(double) * mesh->nel[0], cudaMemcpyHostToDevice, s));
     if (p.banded) {
         const int per_cta = p.lanes < 64 ? 64 / p.lanes : 1, nsys = 2 * dst_march::class_count(p.g.n1, p.g.n2);
-        const unsigned threads = (unsigned)(per_cta * p.lanes);
+        const unsigned threads = (unsigned)(2 * per_cta * p.lanes);      // two per lane
         const unsigned blocks = (unsigned)((nsys + per_cta - 1) / per_cta + (nf + (int)threads - 1) / (int)threads);
-        factor_kernel<<<blocks, threads, 3 * sizeof(M22) * threads, s>>>(p.g, p.lanes, p.steps, p.dvx, p.table, p.freq);
+        factor_kernel<<<blocks, threads, 3 * sizeof(M22) * (threads / 2), s>>>(p.g, p.lanes, p.steps, p.dvx, p.table, p.freq);
         DST_CUDA_TRY(cudaGetLastError());
     }
     return DST_OK;

@@ -64,17 +64,20 @@ __device__ __forceinline__ z2 operator*(z2 a, z2 b) { return z2{a.x * b.x - a.y 
 __device__ __forceinline__ z2 norm(z2 a) { return z2{norm(a.x), norm(a.y)}; }
 
 struct M22 { z2 a, b, c, d; };            // rows (a b), (c d)
-__device__ __forceinline__ M22 zero22() { const z2 z{}; return M22{z, z, z, z}; }
-__device__ __forceinline__ M22 norm(const M22 &p) { return M22{norm(p.a), norm(p.b), norm(p.c), norm(p.d)}; }
-__device__ __forceinline__ M22 mul(const M22 &p, const M22 &q) {
-    return norm(M22{p.a * q.a + p.b * q.c, p.a * q.b + p.b * q.d, p.c * q.a + p.d * q.c, p.c * q.b + p.d * q.d});
+struct Row { z2 a, b; };                  // one row of a block
+__device__ __forceinline__ Row norm(const Row &p) { return Row{norm(p.a), norm(p.b)}; }
+__device__ __forceinline__ Row mul(const Row &p, const M22 &q) {
+    return norm(Row{p.a * q.a + p.b * q.c, p.a * q.b + p.b * q.d});
 }
-__device__ __forceinline__ M22 sub(const M22 &p, const M22 &q) {
-    return norm(M22{p.a - q.a, p.b - q.b, p.c - q.c, p.d - q.d});
-}
-__device__ __forceinline__ M22 neg(const M22 &p) { return M22{-p.a, -p.b, -p.c, -p.d}; }
-__device__ __forceinline__ M22 inv(const M22 &p) {
-    z2 det = norm(p.a * p.d - p.b * p.c);
+__device__ __forceinline__ Row sub(const Row &p, const Row &q) { return norm(Row{p.a - q.a, p.b - q.b}); }
+__device__ __forceinline__ Row neg(const Row &p) { return Row{-p.a, -p.b}; }
+__device__ __forceinline__ Row row(const M22 &m, int h) { return h ? Row{m.c, m.d} : Row{m.a, m.b}; }
+// Row h of the inverse of a block of which this lane has row h, the lane beside it the other
+__device__ __forceinline__ Row inv_row(const Row &p, int h) {
+    auto other = [](df v) { return df{__shfl_xor_sync(0xffffffffu, v.h, 1), __shfl_xor_sync(0xffffffffu, v.l, 1)}; };
+    const Row o{z2{other(p.a.x), other(p.a.y)}, z2{other(p.b.x), other(p.b.y)}};
+    // a d - b c, of either row the same
+    z2 det = norm(h ? o.a * p.b - o.b * p.a : p.a * o.b - p.b * o.a);
     // the determinant scaled to [1, 2) by a power of two: its square stays in range
     const float big = fmaxf(fabsf(det.x.h), fabsf(det.y.h));
     const float sc = __int_as_float((254 << 23) - (__float_as_int(big) & 0x7f800000));
@@ -83,7 +86,8 @@ __device__ __forceinline__ M22 inv(const M22 &p) {
     const float r0 = 1.f / n.h;
     const df r = norm(df{r0, r0 * fmaf(-n.l, r0, fmaf(-n.h, r0, 1.f))});      // a Newton step for 1 / n
     const z2 w{scaled(norm(det.x * r), sc), scaled(norm(-(det.y * r)), sc)}, m = -w;
-    return norm(M22{p.d * w, p.b * m, p.c * m, p.a * w});
+    // (d -b; -c a) w
+    return h ? norm(Row{p.a * m, o.a * w}) : norm(Row{o.b * w, p.b * m});
 }
 
 // Symbols of one frequency: prod of the y, z masses and the two transverse terms.
@@ -114,22 +118,20 @@ __device__ __forceinline__ M22 bd_block(const BdSymbols &q, int o, df v) {
     const float k = o == 0 ? 4.f : 1.f;
     const df im = scaled(q.im, k), s = scaled(q.s, k), m = scaled(q.m, k), z{0.f, 0.f};
     const df c = o == 0 ? z : (o < 0 ? -q.c : q.c);
-    return norm(M22{z2{-(q.w * (v + m)), im}, z2{z, c + s}, z2{z, c - s}, z2{-(q.w * (v - m)), im}});
+    return M22{norm(z2{-(q.w * (v + m)), im}), norm(z2{z, c + s}), norm(z2{z, c - s}), norm(z2{-(q.w * (v - m)), im})};
 }
 
 // Number of factor blocks per lane: the cyclic step's pair, a pair per parallel step,
 // the even inverse, and the odd nodes' inverse and two couplings.
 __host__ __device__ inline int items(int steps) { return 6 + 2 * steps; }
 
-__device__ __forceinline__ void put(float *tab, int G, int item, int lane, const M22 &m) {
-    float4 *o = reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8);
-    o[0] = make_float4(m.a.x.h, m.a.y.h, m.b.x.h, m.b.y.h);
-    o[1] = make_float4(m.c.x.h, m.c.y.h, m.d.x.h, m.d.y.h);
+// row h of an item
+__device__ __forceinline__ void put(float *tab, int G, int item, int lane, int h, const Row &m) {
+    reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8)[h] = make_float4(m.a.x.h, m.a.y.h, m.b.x.h, m.b.y.h);
 }
-__device__ __forceinline__ void put_scaled(float *tab, int G, int item, int lane, const M22 &m, int k) {   // 2^k m
-    float4 *o = reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8);
-    o[0] = make_float4(scalbnf(m.a.x.h, k), scalbnf(m.a.y.h, k), scalbnf(m.b.x.h, k), scalbnf(m.b.y.h, k));
-    o[1] = make_float4(scalbnf(m.c.x.h, k), scalbnf(m.c.y.h, k), scalbnf(m.d.x.h, k), scalbnf(m.d.y.h, k));
+__device__ __forceinline__ void put_scaled(float *tab, int G, int item, int lane, int h, const Row &m, int k) {   // 2^k m
+    reinterpret_cast<float4 *>(tab + ((size_t)item * G + lane) * 8)[h] =
+        make_float4(scalbnf(m.a.x.h, k), scalbnf(m.a.y.h, k), scalbnf(m.b.x.h, k), scalbnf(m.b.y.h, k));
 }
 
 // The row of one frequency.
@@ -148,21 +150,25 @@ __device__ __forceinline__ FreqRow freq_row(const SweepGeom &g, int f) {
 // system; the neighbours' blocks pass through shared memory (three M22 per lane, by
 // quarters of 16 bytes, so that a warp's accesses are contiguous).  The CTAs after the last
 // system's write the rows of the frequencies.
-// In FP64 the 2 x 625 systems of the 48^3 x 48 Klein mesh kept the FP64 unit busy for
-// 215 us.
-__global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int steps, const double *__restrict__ Vx,
+// Two threads share a lane, a row of every block each: products by rows need nothing of the
+// other row, an inverse takes it by a shuffle.
+// The 2 x 625 systems of the 48^3 x 48 Klein mesh take 79 us; with whole blocks per thread
+// (a chain twice as long on half the warps) 97 us, and in FP64, which kept that unit busy
+// throughout, 215 us.
+__global__ void __launch_bounds__(512) factor_kernel(SweepGeom g, int G, int steps, const double *__restrict__ Vx,
                                                      float *__restrict__ table, FreqRow *__restrict__ freq) {
     extern __shared__ __align__(16) unsigned char fsm[];
-    const int fb = (2 * class_count(g.n1, g.n2) + blockDim.x / G - 1) / (blockDim.x / G);
+    const int T = blockDim.x / 2, per_cta = T / G;            // nodes and systems of the CTA
+    const int fb = (2 * class_count(g.n1, g.n2) + per_cta - 1) / per_cta;
     if ((int)blockIdx.x >= fb) {
         const int f = (blockIdx.x - fb) * blockDim.x + threadIdx.x;
         if (f < g.n1 * g.n2) freq[f] = freq_row(g, f);
         return;
     }
     float4 *xch = reinterpret_cast<float4 *>(fsm);
-    const int l = threadIdx.x % G, base = threadIdx.x - l;
+    const int h = threadIdx.x & 1, node = threadIdx.x / 2, l = node % G, base = node - l;
     const int nsys = 2 * class_count(g.n1, g.n2);
-    const int sys = blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+    const int sys = blockIdx.x * per_cta + node / G;
     const bool live = sys < nsys;
     const int cls = (live ? sys : 0) / 2, q2 = g.n2 / 2 + 1;
     double myz, by, bz;
@@ -175,25 +181,27 @@ __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int ste
     float *tab = table + (size_t)(live ? sys : 0) * items(steps) * G * 8;
     const df one{1.f, 0.f}, nil{0.f, 0.f};
     const z2 z1{one, nil}, z0{nil, nil};
-    M22 L = zero22(), U = zero22(), D = M22{z1, z0, z0, z1}, Lo = zero22(), Uo = zero22(), Doi = zero22();
+    const Row none{z0, z0}, unit = h ? Row{z0, z1} : Row{z1, z0};
+    Row L = none, U = none, D = unit, Lo = none, Uo = none, Do = unit;
     df v[3];                                                 // elements e, e + 1, e + 2
 #pragma unroll
     for (int k = 0; k < 3; ++k) v[k] = Vx && e + k <= n ? to_df(Vx[e + k]) : nil;
     if (e < n) {
-        D = bd_block(q, 0, scaled(v[0] + v[1], 2.f));
-        if (e > 0) L = bd_block(q, -1, v[0]);
+        D = row(bd_block(q, 0, scaled(v[0] + v[1], 2.f)), h);
+        if (e > 0) L = row(bd_block(q, -1, v[0]), h);
         if (o < n) {
-            U = bd_block(q, 1, v[1]);
-            Doi = inv(bd_block(q, 0, scaled(v[1] + v[2], 2.f)));
-            Lo = bd_block(q, -1, v[1]);
-            if (o + 1 < n) Uo = bd_block(q, 1, v[2]);
+            U = row(bd_block(q, 1, v[1]), h);
+            Do = row(bd_block(q, 0, scaled(v[1] + v[2], 2.f)), h);
+            Lo = row(bd_block(q, -1, v[1]), h);
+            if (o + 1 < n) Uo = row(bd_block(q, 1, v[2]), h);
         }
     }
-    const int T = blockDim.x;
-    auto put_x = [&](int which, const M22 &m) {
-        const z2 *z = &m.a;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) xch[(4 * which + k) * T + threadIdx.x] = make_float4(z[k].x.h, z[k].x.l, z[k].y.h, z[k].y.l);
+    // (both lanes of a node have the same e and o)
+    Row Doi = inv_row(Do, h);
+    if (o >= n) Doi = none;
+    auto put_x = [&](int which, const Row &m) {
+        xch[(4 * which + 2 * h) * T + node] = make_float4(m.a.x.h, m.a.x.l, m.a.y.h, m.a.y.l);
+        xch[(4 * which + 2 * h + 1) * T + node] = make_float4(m.b.x.h, m.b.x.l, m.b.y.h, m.b.y.l);
     };
     auto get_x = [&](int which, int at) {
         M22 m;
@@ -205,38 +213,41 @@ __global__ void __launch_bounds__(256) factor_kernel(SweepGeom g, int G, int ste
         }
         return m;
     };
-    auto publish = [&](const M22 &a, const M22 &b, const M22 &c) {
+    auto publish = [&](const Row &a, const Row &b, const Row &c) {
         __syncthreads();
         put_x(0, a); put_x(1, b); put_x(2, c);
         __syncthreads();
     };
     publish(Doi, Lo, Uo);
     {
-        const int left = l > 0 ? threadIdx.x - 1 : threadIdx.x;       // l = 0: L = 0, any block will do
-        const M22 A = mul(L, get_x(0, left)), Bm = mul(U, Doi);
-        D = sub(sub(D, mul(A, get_x(2, left))), mul(Bm, Lo));
+        const int left = l > 0 ? node - 1 : node;                    // l = 0: L = 0, any block will do
+        const M22 Doi2 = get_x(0, node), Lo2 = get_x(1, node), Uo2 = get_x(2, node);
+        const Row A = mul(L, get_x(0, left)), Bm = mul(U, Doi2);
+        D = sub(sub(D, mul(A, get_x(2, left))), mul(Bm, Lo2));
         L = neg(mul(A, get_x(1, left)));
-        U = neg(mul(Bm, Uo));
-        if (live) { put(tab, G, 0, l, A); put(tab, G, 1, l, Bm); }
+        U = neg(mul(Bm, Uo2));
+        if (live) {
+            const int at = 2 + 2 * steps;
+            put(tab, G, 0, l, h, A);
+            put(tab, G, 1, l, h, Bm);
+            put_scaled(tab, G, at + 1, l, h, Doi, k2);
+            put(tab, G, at + 2, l, h, mul(Doi, Lo2));
+            put(tab, G, at + 3, l, h, mul(Doi, Uo2));
+        }
     }
     for (int s = 0; s < steps; ++s) {
         const int st = 1 << s;
-        publish(inv(D), L, U);
+        publish(inv_row(D, h), L, U);
         const bool hl = l >= st, hr = l + st < G;
-        const int il = hl ? threadIdx.x - st : base, ir = hr ? threadIdx.x + st : base;
-        const M22 al = hl ? mul(L, get_x(0, il)) : zero22(), ga = hr ? mul(U, get_x(0, ir)) : zero22();
+        const int il = hl ? node - st : base, ir = hr ? node + st : base;
+        const Row al = hl ? mul(L, get_x(0, il)) : none, ga = hr ? mul(U, get_x(0, ir)) : none;
         D = sub(sub(D, mul(al, get_x(2, il))), mul(ga, get_x(1, ir)));
         L = neg(mul(al, get_x(1, il)));
         U = neg(mul(ga, get_x(2, ir)));
-        if (live) { put(tab, G, 2 + 2 * s, l, al); put(tab, G, 3 + 2 * s, l, ga); }
+        if (live) { put(tab, G, 2 + 2 * s, l, h, al); put(tab, G, 3 + 2 * s, l, h, ga); }
     }
-    if (live) {
-        const int at = 2 + 2 * steps;
-        put_scaled(tab, G, at, l, inv(D), k2);
-        put_scaled(tab, G, at + 1, l, Doi, k2);
-        put(tab, G, at + 2, l, mul(Doi, Lo));
-        put(tab, G, at + 3, l, mul(Doi, Uo));
-    }
+    const Row Di = inv_row(D, h);
+    if (live) put_scaled(tab, G, 2 + 2 * steps, l, h, Di, k2);
 }
 
 // hi + lo = 2 sum_t (-1)^t v_t per spatial entry (two complex entries per thread;
