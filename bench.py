@@ -320,7 +320,7 @@ def run_ncu_case(case):
     one-pass Gram-Schmidt;
     apply32_zb / apply32_klein / apply64_klein: 12 operator applies on the 96^2 x 96 mesh or
     the 48^3 x 48 3+1 Klein mesh, over rotating buffers (tile variant 0);
-    apply32_klein_zcol / apply64_klein_zcol: the same with the column kernel (variant 1);
+    apply32_klein_zcol / apply64_klein_zcol: the same with tile variant 1;
     sweep_zb: 6 Crank-Nicolson sweeps on the 96^2 x 96 mesh;
     unet_zb48: 4 forward passes of the U-Net on the 48^2 x 48 grid.
     """
