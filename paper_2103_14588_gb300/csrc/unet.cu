@@ -137,9 +137,9 @@ __global__ void __launch_bounds__(256) scale_input_kernel(int64_t n, int parts, 
 
 // dy = 2 (y - t / s) / ||t / s||^2 in BF16 with the column sums of its CTAs, and the
 // CTAs' shares of ||y - t / s||^2; lq: log2 of the channels / 4.  t, a caller's vector, may
-// start at any entry (8 bytes).
+// start at any float.
 __global__ void __launch_bounds__(256) loss_kernel(int64_t n4, int lq, int parts, const double *__restrict__ tpart,
-                                                   const float4 *__restrict__ y, const float2 *__restrict__ t,
+                                                   const float4 *__restrict__ y, const float *__restrict__ t,
                                                    const float *__restrict__ s, uint2 *__restrict__ dy,
                                                    double *__restrict__ lpart, float *__restrict__ colsum) {
     __shared__ double red[256];
@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(256) loss_kernel(int64_t n4, int lq, int parts
     float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t i = blockIdx.x * 256LL + threadIdx.x; i < n4; i += 256LL * gridDim.x) {
         const float4 a = y[i];
-        const float2 b = t[2 * i], c = t[2 * i + 1];
-        const float4 r = make_float4(a.x - b.x * inv, a.y - b.y * inv, a.z - c.x * inv, a.w - c.y * inv);
+        const float4 r = make_float4(a.x - t[4 * i] * inv, a.y - t[4 * i + 1] * inv, a.z - t[4 * i + 2] * inv,
+                                     a.w - t[4 * i + 3] * inv);
         acc += ((double)r.x * r.x + (double)r.y * r.y) + ((double)r.z * r.z + (double)r.w * r.w);
         const float4 d = make_float4((float)(w * r.x), (float)(w * r.y), (float)(w * r.z), (float)(w * r.w));
         dy[i] = pack_bf16x4(d);
@@ -691,7 +691,7 @@ static int loss_grad(dst_unet *u, const float *x, const float *t, cudaStream_t s
     const unsigned parts = sum_ctas(n / 4);
     u->sums.l[OUT].rows = (int)parts;
     loss_kernel<<<parts, 256, 0, s>>>(n / 4, log2i(u->C / 4), (int)parts, u->spart + SUM_CTAS, (const float4 *)u->y,
-                                      (const float2 *)t, u->scale, (uint2 *)u->z1, u->spart + 2 * SUM_CTAS,
+                                      t, u->scale, (uint2 *)u->z1, u->spart + 2 * SUM_CTAS,
                                       u->bpart + u->sums.l[OUT].bpart);
     loss_sum_kernel<<<1, 32, 0, s>>>((int)parts, u->spart + 2 * SUM_CTAS, u->dscr + 1);
     return backward(u, s);
