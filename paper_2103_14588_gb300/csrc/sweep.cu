@@ -49,9 +49,16 @@ using namespace dst_march;
 
 // ---- 2a. spectral march: one thread per frequency ---------------------------
 // Every axis periodic and a constant potential: M_s and K_s are diagonal in
-// frequency with 2 x 2 blocks (1+1 and 2+1 only), so with P = Bd^-1
-//   x_t = x_{t-1} + P (s_t - h_t K^ x_{t-1}),   M^ = prod_k m_k   (sweep_march.cuh),
+// frequency with 2 x 2 blocks (1+1 and 2+1 only), so with P = Bd^-1 and M^ = prod_k m_k
+//   x_t = P s_t - Q x_{t-1},   Q = P Bl = I - 2 i M^ P,
 // Bd = i M^ + (h_t/2) [ sum_k alpha_k (i sin th_k) i prod_{j != k} m_j - (m beta + V0) M^ ].
+// -Q turns the two modes of a frequency by a phase each.  The march takes the nearest c of
+// 1, -1, i, -i and 0 out of it, x_t = c x_{t-1} + P s_t - R x_{t-1} with R = Q + c I formed in
+// FP64: the part that c carries is exact, so the rounding is relative to the small
+// R x, for the modes that the time step resolves (c = 1) as for those that it only turns
+// round (c = -1, h_t K >> M).  Relative error of 48 layers against FP64, at h_t = h / 4, h,
+// 10 h and 40 h (m = 1, V0 = 3, 24 x 24 nodes): 4.5e-7, 5.4e-7, 3.1e-7 and 2.7e-7 (s - h_t K x
+// formed in FP32: 4.7e-7, 1.0e-6, 2.2e-6 and 4.1e-6; the march takes the same time either way).
 // One pass over the layers, the loads of the next PD in flight while one is combined.
 __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ alt_hi,
                                       const float4 *__restrict__ alt_lo, float4 *__restrict__ x) {
@@ -74,11 +81,29 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
     const double a0 = -ht2 * (g.m + g.V0) * pm, a1 = -ht2 * (g.V0 - g.m) * pm;
     const double dx = a0 * a1 - pm * pm - (bx * bx + by * by), dy = pm * (a0 + a1), r = 1.0 / (dx * dx + dy * dy);
     const double wx = dx * r, wy = -dy * r;
-    const Blk Pf{make_float4((float)(a1 * wx - pm * wy), (float)(a1 * wy + pm * wx), (float)(-bx * wx - by * wy), (float)(by * wx - bx * wy)),
-                 make_float4((float)(by * wy - bx * wx), (float)(-bx * wy - by * wx), (float)(a0 * wx - pm * wy), (float)(a0 * wy + pm * wx))};
-    // h_t K^ = kx sigma_x + ky sigma_y + diag(d0, d1)
-    const float kx = (float)(2.0 * bx), ky = (float)(2.0 * by), d0 = (float)(-g.ht * (g.m + g.V0) * pm),
-                d1 = (float)(-g.ht * (g.V0 - g.m) * pm);
+    const double P[8] = {a1 * wx - pm * wy, a1 * wy + pm * wx, -bx * wx - by * wy, by * wx - bx * wy,
+                         by * wy - bx * wx, -bx * wy - by * wx, a0 * wx - pm * wy, a0 * wy + pm * wx};
+    // Q by rows, then the c that leaves the smallest diagonal of R
+    double Q[8];
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) { Q[k] = 2.0 * pm * P[k + 1]; Q[k + 1] = -2.0 * pm * P[k]; }
+    Q[0] += 1.0;
+    Q[6] += 1.0;
+    const float tx = (float)(Q[0] + Q[6]), ty = (float)(Q[1] + Q[7]);
+    // |q0 + c|^2 + |q1 + c|^2 = |q0|^2 + |q1|^2 + 2 (|c|^2 + Re conj(c) (q0 + q1)): below that of c = 0 where the trace
+    // has a part beyond -1 along c
+    float cx = 0.f, cy = 0.f;
+    if (fmaxf(fabsf(tx), fabsf(ty)) > 1.f) {
+        if (fabsf(tx) >= fabsf(ty)) cx = tx > 0.f ? -1.f : 1.f;
+        else cy = ty > 0.f ? -1.f : 1.f;
+    }
+    Q[0] += cx; Q[6] += cx;
+    Q[1] += cy; Q[7] += cy;
+    auto blk = [](const double *v) {
+        return Blk{make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]),
+                   make_float4((float)v[4], (float)v[5], (float)v[6], (float)v[7])};
+    };
+    const Blk Pf = blk(P), Rf = blk(Q);
     float4 s = alt_hi[f], lo = alt_lo[f], xp = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t t0 = 0; t0 < g.nt; t0 += PD) {
 #pragma unroll
@@ -87,14 +112,12 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
             if (t < g.nt) {
                 const float4 v = ring[q];
                 if (t + PD < g.nt) ring[q] = x[(t + PD) * nf + f];
-                const float4 r =
-                    make_float4(s.x - fmaf(kx, xp.z, fmaf(ky, xp.w, fmaf(d0, xp.x, -lo.x))),
-                                s.y - fmaf(kx, xp.w, fmaf(-ky, xp.z, fmaf(d0, xp.y, -lo.y))),
-                                s.z - fmaf(kx, xp.x, fmaf(-ky, xp.y, fmaf(d1, xp.z, -lo.z))),
-                                s.w - fmaf(kx, xp.y, fmaf(ky, xp.x, fmaf(d1, xp.w, -lo.w))));
                 float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                add_mv(u, Pf, r);
-                xp = make_float4(u.x + xp.x, u.y + xp.y, u.z + xp.z, u.w + xp.w);
+                add_mv(u, Pf, lo);
+                add_mv(u, Pf, s);
+                sub_mv(u, Rf, xp);
+                xp = make_float4(fmaf(cx, xp.x, fmaf(-cy, xp.y, u.x)), fmaf(cx, xp.y, fmaf(cy, xp.x, u.y)),
+                                 fmaf(cx, xp.z, fmaf(-cy, xp.w, u.z)), fmaf(cx, xp.w, fmaf(cy, xp.z, u.w)));
                 x[t * nf + f] = xp;
                 next_s(s, lo, v);
             }
