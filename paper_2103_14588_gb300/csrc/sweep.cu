@@ -31,6 +31,7 @@
 // The result is the same linear map as the assembled sweep (up to FP32
 // rounding); meshes of other kinds (open axes, two or more non-periodic axes,
 // a potential varying along a periodic axis) get DST_ERR_ARG.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -237,6 +238,12 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
             dst_internal_set_error_detail("Crank-Nicolson sweep: x axis too long for the banded march");
             return DST_ERR_ARG;
         }
+        // h_t K against M: the x and transverse derivatives, mass and potential (twice, as measured)
+        double vmax = 0.0, k = 2.0 * std::fabs(mesh->m);
+        for (size_t e = 0; e < mesh->V.size() && e < (size_t)mesh->nel[0]; ++e) vmax = std::max(vmax, std::fabs(mesh->V[e]));
+        k += 2.0 * vmax;
+        for (int a_ = 0; a_ < d; ++a_) k += 1.0 / mesh->h[a_];
+        p.refine = g.ht * k > (d == 1 ? 1.0 : 1.5) || g.ht > 0.5 * mesh->h[0];
         p.table_bytes = sizeof(float) * 8 * 2 * (size_t)dst_march::class_count(g.n1, g.n2) * dst_march::items(p.steps) * p.lanes;
     }
     p.launches = 2 + (p.has_fft ? 2 : 0);
@@ -289,8 +296,7 @@ static int launch_march(const SweepPlan &p, const float2 *in, float2 *out, cudaS
         DST_CUDA_TRY(cudaGetLastError());
         return DST_OK;
     };
-    const bool large = p.g.ht > 0.5 * p.g.h[0];
-#define DST_MARCH(G) case G: return large ? go(march_kernel<NC, G, true>) : go(march_kernel<NC, G, false>);
+#define DST_MARCH(G) case G: return p.refine ? go(march_kernel<NC, G, true>) : go(march_kernel<NC, G, false>);
     switch (p.lanes) {
         DST_MARCH(8) DST_MARCH(16) DST_MARCH(32) DST_MARCH(64) DST_MARCH(128) DST_MARCH(256)
         default: return DST_ERR_ARG;
