@@ -19,6 +19,7 @@
 #include "apply_node.cuh"
 
 #define DST_MAX_DEVICES_APPLY 64
+constexpr int64_t MAX_GRID_Y = 65535;      // chunks of time layers in one launch
 
 namespace dst {
 
@@ -523,9 +524,9 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
 template <int D, int NC, typename T, bool NOV, int TV>
 __global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR, sizeof(T) == 8 ? 1 : 3)
 apply_pipe_kernel(OpParams p, StdConst<T> sc, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
-                  int64_t tiles_x, int64_t tiles_y) {
+                  int64_t tiles_x, int64_t tiles_y, int64_t chunk0) {
     extern __shared__ __align__(16) char ring[];
-    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, sc, x, y, tiles_x, tiles_y, blockIdx.x, blockIdx.y, ring);
+    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, sc, x, y, tiles_x, tiles_y, blockIdx.x, chunk0 + blockIdx.y, ring);
 }
 
 template <int D, int NC, typename T, int TV>
@@ -537,10 +538,9 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
     const int64_t tz = (p.ax[2].n + Tile::TZ - 1) / Tile::TZ;
     const int64_t chunks = (p.nt + Tile::TT - 1) / Tile::TT;
     const int64_t tiles = tx * ty * tz;
-    if (tiles <= 0 || tiles > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
+    if (tiles <= 0 || tiles > 0x7fffffffLL) return DST_ERR_ARG;
     // byte offsets within one time layer are kept in 32 bits
     if (p.ax[0].n * p.ax[1].n * p.ax[2].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<D, NC, T>(p, x, y, s);
-    dim3 grid((unsigned)tiles, (unsigned)chunks);
     // the shared-memory opt-in is a per-device function attribute: set it once per device
     static bool configured[2][DST_MAX_DEVICES_APPLY] = {};
     int dev = 0;
@@ -551,7 +551,11 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
         DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
         if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[nov][dev] = true;
     }
-    kern<<<grid, S::NTHR, S::SMEM, s>>>(p, std_const<D, T>(p), x, y, tx, ty);
+    const StdConst<T> sc = std_const<D, T>(p);
+    for (int64_t c = 0; c < chunks; c += MAX_GRID_Y) {
+        const dim3 grid((unsigned)tiles, (unsigned)std::min(MAX_GRID_Y, chunks - c));
+        kern<<<grid, S::NTHR, S::SMEM, s>>>(p, sc, x, y, tx, ty, c);
+    }
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }

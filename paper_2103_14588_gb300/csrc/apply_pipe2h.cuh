@@ -36,11 +36,12 @@ struct Pipe2hShape {
 
 template <int TV, bool NOV>
 __global__ void __launch_bounds__(Pipe2hShape<TV>::NTHR, 3)
-apply_pipe2h_kernel(OpParams p, StdConst<float> sc, const float2 *__restrict__ x, float2 *__restrict__ y, int64_t tiles_x) {
+apply_pipe2h_kernel(OpParams p, StdConst<float> sc, const float2 *__restrict__ x, float2 *__restrict__ y, int64_t tiles_x,
+                    int64_t chunk0) {
     using S = Pipe2hShape<TV>;
     constexpr int RY = S::RY;
     extern __shared__ __align__(16) char ring[];
-    const int64_t tile = blockIdx.x, chunk = blockIdx.y;
+    const int64_t tile = blockIdx.x, chunk = chunk0 + blockIdx.y;
     const int64_t x0 = (tile % tiles_x) * S::TX;
     const int64_t y0 = (tile / tiles_x) * S::TY;
     const int h = threadIdx.x & 1, col = threadIdx.x >> 1;
@@ -167,7 +168,7 @@ int launch_apply_pipe2h(const OpParams &p, const float2 *x, float2 *y, cudaStrea
     const int64_t ty = (p.ax[1].n + S::TY - 1) / S::TY;
     const int64_t chunks = (p.nt + S::TT - 1) / S::TT;
     const int64_t tiles = tx * ty;
-    if (tiles <= 0 || tiles > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
+    if (tiles <= 0 || tiles > 0x7fffffffLL) return DST_ERR_ARG;
     if (p.ax[0].n * p.ax[1].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<2, 2, float>(p, x, y, s);
     static bool configured[2][DST_MAX_DEVICES_APPLY] = {};
     int dev = 0;
@@ -178,7 +179,9 @@ int launch_apply_pipe2h(const OpParams &p, const float2 *x, float2 *y, cudaStrea
         DST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM));
         if (dev >= 0 && dev < DST_MAX_DEVICES_APPLY) configured[nov][dev] = true;
     }
-    kern<<<dim3((unsigned)tiles, (unsigned)chunks), S::NTHR, S::SMEM, s>>>(p, std_const<2, float>(p), x, y, tx);
+    const StdConst<float> sc = std_const<2, float>(p);
+    for (int64_t c = 0; c < chunks; c += MAX_GRID_Y)
+        kern<<<dim3((unsigned)tiles, (unsigned)std::min(MAX_GRID_Y, chunks - c)), S::NTHR, S::SMEM, s>>>(p, sc, x, y, tx, c);
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;
 }
