@@ -269,21 +269,25 @@ apply_node_kernel(OpParams p, NodeConst<T> sc, int tt, const typename LaneOf<T>:
 // Layers per thread.  Each chunk forms the sums of two planes that its neighbours form
 // too, so long chunks save work, but a mesh of few nodes needs its layers spread.
 // FP64: a warp's instruction holds one of the 608 FP64 units for 64 clocks, so the time is
-// the planes of a chunk times the warps that share a unit; the chunk with the least.
+// the planes of a chunk times the warps that share a unit (a CTA's four warps, working or
+// not, sit on four units); the chunk with the least (1+1, 520 x 520: 31 us with 20 layers, 53 with
+// the 58 that a count of the working warps alone would take).
 // FP32: latency; the longest chunk that leaves 12 warps per SM (16 x 16 x 16 x 16 elements
 // 3+1: 17.2 / 11.4 / 10.1 / 11.5 us with 3 / 6 / 12 / 24).
 template <typename T>
 inline int node_chunk(int64_t plane_threads, int64_t nt) {
-    const int64_t warps = (plane_threads + 31) / 32;
     if (sizeof(T) == 4) {
+        const int64_t warps = (plane_threads + 31) / 32;
         int64_t chunks = (152 * 12 + warps - 1) / warps;
         chunks = std::min<int64_t>(std::max<int64_t>(chunks, (nt + 31) / 32), nt);
         return (int)((nt + chunks - 1) / chunks);
     }
-    // a unit's share, rounded up to whole warps while they are few
+    const int64_t warps = (plane_threads + 127) / 128 * 4;
+    // a unit's share, rounded up to whole warps while they are few (the sum then follows the
+    // measured times of 31 meshes to within 7%)
     auto time = [&](int64_t tt) {
         const double share = (double)(warps * ((nt + tt - 1) / tt)) / 608.0;
-        return (double)(tt + 2) * (share > 4.0 ? share + 0.5 : std::ceil(share));
+        return (double)std::min(tt + 2, nt) * (share > 4.0 ? share + 0.5 : std::ceil(share));
     };
     int64_t best = nt;
     for (int64_t tt = 1; tt < std::min<int64_t>(nt, 64); ++tt)
