@@ -222,9 +222,27 @@ __device__ __forceinline__ void subtract(int64_t n, const double2 *__restrict__ 
     }
 }
 
+// w <- w - sum_j V_j c_j over the CTA's slice, j in eights and a rest of R (exact, as in
+// project_group: a rest taken apart by conditions inside the loop over the entries is
+// predicated, so that two vectors cost as much as three); the thread's share of ||w||^2.
+template <int R>
+__device__ __forceinline__ double update_slice(int64_t n, int64_t b, int64_t e, int nvec, const double2 *__restrict__ V,
+                                               const double2 *c, double2 *__restrict__ w) {
+    double nr = 0.0;
+    for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
+        double2 acc = w[i];
+        for (int j = 0; j + PROJ_GROUP <= nvec; j += PROJ_GROUP) subtract<PROJ_GROUP>(n, V + (int64_t)j * n + i, c + j, acc);
+        if constexpr (R > 0) subtract<R>(n, V + (int64_t)(nvec - R) * n + i, c + nvec - R, acc);
+        w[i] = acc;
+        nr = fma(acc.x, acc.x, fma(acc.y, acc.y, nr));
+    }
+    return nr;
+}
+
 // w <- w - sum_j V_j h_j ; partial ||w||^2 per CTA, with a ticket summed by the last CTA
 // into *nrm2 (and *counter bumped).  Four CTAs per SM, so that the 608 of a large vector are
-// one wave.  1.77M entries x 15 vectors: projection 265 -> 215 us, update 201 -> 199 us.
+// one wave.  1.77M entries x 2, 4, 8 and 15 vectors: 70, 95, 141 and 225 us
+// (86, 111, 158 and 226 with the rest taken apart by conditions).
 __global__ void __launch_bounds__(RED_THREADS, 4)
 update_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const double2 *__restrict__ h,
               double2 *__restrict__ w, double *nrm_partials, const double *gate, unsigned *ticket, double *nrm2,
@@ -236,16 +254,16 @@ update_kernel(int64_t n, int nvec, const double2 *__restrict__ V, const double2 
     __syncthreads();
     int64_t b, e;
     slice(n, b, e);
-    double nr = 0.0;
-    for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
-        double2 acc = w[i];
-        int j = 0;
-        for (; j + PROJ_GROUP <= nvec; j += PROJ_GROUP) subtract<PROJ_GROUP>(n, V + (int64_t)j * n + i, hs + j, acc);
-        if (nvec & 4) { subtract<4>(n, V + (int64_t)j * n + i, hs + j, acc); j += 4; }
-        if (nvec & 2) { subtract<2>(n, V + (int64_t)j * n + i, hs + j, acc); j += 2; }
-        if (nvec & 1) subtract<1>(n, V + (int64_t)j * n + i, hs + j, acc);
-        w[i] = acc;
-        if (nrm_partials) nr = fma(acc.x, acc.x, fma(acc.y, acc.y, nr));
+    double nr;
+    switch (nvec % PROJ_GROUP) {
+        case 0: nr = update_slice<0>(n, b, e, nvec, V, hs, w); break;
+        case 1: nr = update_slice<1>(n, b, e, nvec, V, hs, w); break;
+        case 2: nr = update_slice<2>(n, b, e, nvec, V, hs, w); break;
+        case 3: nr = update_slice<3>(n, b, e, nvec, V, hs, w); break;
+        case 4: nr = update_slice<4>(n, b, e, nvec, V, hs, w); break;
+        case 5: nr = update_slice<5>(n, b, e, nvec, V, hs, w); break;
+        case 6: nr = update_slice<6>(n, b, e, nvec, V, hs, w); break;
+        default: nr = update_slice<7>(n, b, e, nvec, V, hs, w); break;
     }
     if (!nrm_partials) return;
     nr = block_sum(nr, sh);
