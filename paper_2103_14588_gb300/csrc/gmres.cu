@@ -439,10 +439,14 @@ struct Solver {
     int gmres(int prec, double2 *x, const double2 *rhs, bool x_zero, double tol_abs, int max_iters,
               double &beta_out, int max_cycles = 0x7fffffff) {
         // Steps enqueued between host synchronisations.  Every step runs on the device, so a
-        // small mesh need not wait for the host after each (64 x 64: 16 us of kernels a step and
-        // about 20 us per synchronisation); the steps past the one that meets the tolerance
-        // have run in vain then, so a large mesh, whose steps take longer than that, waits.
-        const int batch = w.n < (1 << 18) ? 10 : 1;
+        // small mesh need not wait for the host after each; the steps past the one that meets
+        // the tolerance have run in vain then.  So a batch holds as many as the call has
+        // taken already (half as many where a step takes longer than the 100 us that a
+        // synchronisation drains from the pipeline), two or one at first and ten at most: what runs in
+        // vain stays below what the batches have saved, and a long solve waits every ten steps.
+        // 131,072 unknowns, solves of 2, 4, 8 and 28 steps: 0.40, 0.64, 1.10 and 3.75 ms (a
+        // synchronisation per step 0.45, 0.73, 1.32 and 6.1; tens throughout 1.18, 1.18, 1.18 and 3.98).
+        const int first_batch = w.n <= (1 << 17) ? 2 : 1, share = w.n < (1 << 16) ? 1 : 2, start = iters;
         const int m = w.m;
         const int64_t n = w.n;
         double beta;
@@ -458,7 +462,8 @@ struct Solver {
             DST_CUDA_TRY(cudaMemsetAsync(w.cols, 0, sizeof(double) * COL_STRIDE * m, s));
             int k = 0;
             for (bool done = false; !done && k < m;) {
-                const int first = k, steps = std::min(std::min(batch, m - k), max_iters - iters);
+                const int first = k, ahead = std::min(10, std::max(first_batch, (iters - start) / share));
+                const int steps = std::min(std::min(ahead, m - k), max_iters - iters);
                 prof.chain = true;            // only kernels are enqueued until the loop ends
                 prof.last = -1;
                 for (int j = first; j < first + steps; ++j)
