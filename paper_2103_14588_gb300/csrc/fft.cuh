@@ -295,12 +295,12 @@ fft_planes_kernel(SweepFft a, const V *__restrict__ in, V *__restrict__ out) {
         copy_elem<V, W>(plane + i1 * pt + i2, src + (inverse ? (int64_t)f : i1 * a.s1 + i2 * a.s2) * nc);
     }
     // the twiddles while the plane is on its way
-    for (int j = threadIdx.x; j < n1; j += blockDim.x) {
+    for (int j = threadIdx.x; j < n1 && a.nrad1 > 0; j += blockDim.x) {
         R sn, cs;
         sincos_pi((R)2 * (R)j / (R)n1, &sn, &cs);
         w1[j] = mk<V>(cs, sign * sn);
     }
-    for (int j = threadIdx.x; j < n2; j += blockDim.x) {
+    for (int j = threadIdx.x; j < n2 && a.nrad2 > 0; j += blockDim.x) {
         R sn, cs;
         sincos_pi((R)2 * (R)j / (R)n2, &sn, &cs);
         w2[j] = mk<V>(cs, sign * sn);
