@@ -268,7 +268,9 @@ inline size_t fft_smem_bytes(const SweepFft &a) {
 // multiplications by +-i in the butterflies are then signs of their sums.
 template <typename V, int W, bool INVERSE>
 __global__ void __launch_bounds__(FFT_THREADS)
-fft_planes_kernel(SweepFft a, const V *__restrict__ in, V *__restrict__ out) {
+fft_planes_kernel(SweepFft a, int64_t ctas, const V *__restrict__ in, V *__restrict__ out) {
+    const int64_t cta = blockIdx.y * (int64_t)gridDim.x + blockIdx.x;
+    if (cta >= ctas) return;
     using R = typename Real<V>::type;
     constexpr bool inverse = INVERSE;
     constexpr R sign = INVERSE ? (R)1 : (R)-1;
@@ -283,8 +285,8 @@ fft_planes_kernel(SweepFft a, const V *__restrict__ in, V *__restrict__ out) {
     // the component groups of a plane are neighbours in the grid: together they use the
     // sectors that each touches half of (apart, DRAM saw three times the plane's bytes)
     const int groups = nc / W;
-    const int64_t b = blockIdx.x / groups;
-    const int c0 = (int)(blockIdx.x % groups) * W;
+    const int64_t b = cta / groups;
+    const int c0 = (int)(cta - b * groups) * W;
     const int64_t base = (b / a.nbx) * a.ns_nodes + (b % a.nbx) * a.sbx;   // node index of (i1, i2) = (0, 0)
     const unsigned r2 = n2 > 1 ? 0xffffffffu / (unsigned)n2 + 1u : 0u;
     auto row = [&](int f) { return n2 > 1 ? (int)__umulhi((unsigned)f, r2) : f; };
@@ -355,8 +357,10 @@ inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, const V *in, V *out
     // a caller's FP32 vector may start at any entry (8 bytes): then one component at a time
     SweepFft b = a;
     if ((((uintptr_t)in | (uintptr_t)out) & 15) != 0) b.ncb = 1;
-    const unsigned grid = (unsigned)(nb * (b.nc / b.ncb));
-    (b.ncb == 2 ? two : one)<<<grid, fft_threads(b), fft_smem_bytes<V>(b), s>>>(b, in, out);
+    // (more CTAs than a grid's x extent takes go on in y)
+    const int64_t ctas = nb * (b.nc / b.ncb), row = std::min<int64_t>(ctas, 1 << 30);
+    const dim3 grid((unsigned)row, (unsigned)((ctas + row - 1) / row));
+    (b.ncb == 2 ? two : one)<<<grid, fft_threads(b), fft_smem_bytes<V>(b), s>>>(b, ctas, in, out);
     return cudaGetLastError();
 }
 
