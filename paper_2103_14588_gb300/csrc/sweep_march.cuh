@@ -366,8 +366,9 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
                   layer = (int64_t)n * nf * NC * 8;
     const char *src = reinterpret_cast<const char *>(in) + off0;
     char *dst = reinterpret_cast<char *>(out) + off0;
-    const int nt = (int)g.nt;
-    int issued = 0, fill = 0;                                  // layers issued; the ring slot of the next
+    const int64_t nt = g.nt;
+    int64_t issued = 0;
+    int fill = 0;                                              // layers issued; the ring slot of the next
     auto issue = [&] {
         if (issued < nt) {
             unsigned char *d = ring + fill;
@@ -501,7 +502,7 @@ march_kernel(SweepGeom g, int steps, const double *__restrict__ Vx, const float 
     // this lane's places in a tile
     const int ate = (he ? pos(e) : 0) * RB + slot * NC * 8, ato = (ho ? pos(o) : 0) * RB + slot * NC * 8;
     int used = 0;                                              // the ring slot of layer t
-    for (int t = 0; t < nt; ++t) {
+    for (int64_t t = 0; t < nt; ++t) {
         asm volatile("cp.async.wait_group %0;\n" ::"n"(STAGES - 2) : "memory");
         __syncthreads();               // layer t staged; layer t - 1 of the output complete; its input slot free
         issue();
