@@ -405,6 +405,17 @@ DST_API int dst_testing_fp32_arnoldi(int mode, int64_t n, int nvec, const void *
                                      void *stream);
 
 /*
+ * Testing access to the Gram-Schmidt of one FP64 Arnoldi step as dst_solve's cycles enqueue
+ * it (Sec. 2.2's GMRES): h[0..nvec) = V^H w, w <- w - V h, then the second pass into
+ * h[nvec..2 nvec) where the norm fell below a half (else those stay zero).  V holds nvec DEVICE
+ * FP64 complex vectors of length n one after another (1 <= nvec <= 64), w one more; h: DEVICE
+ * 2 nvec complex; rec: DEVICE 8 doubles, [0] ||w||^2 after the last pass, [3] before the
+ * first, [6] 1 where the second pass ran.  The sums of both passes share their counters, as in
+ * a solve.  Takes stream-ordered scratch.  Errors: DST_ERR_ARG, DST_ERR_OOM, DST_ERR_CUDA.
+ */
+DST_API int dst_testing_fp64_step(int64_t n, int nvec, const void *V, void *w, void *h, void *rec, void *stream);
+
+/*
  * Right preconditioners for flexible GMRES (dst_solve_opts.precond).  The paper
  * names none; its conclusion (Sec. 5) asks for one and points at decomposing
  * the time direction.

@@ -32,7 +32,7 @@ EXPORTED = (
     "dst_set_boundary_data", "dst_precond_apply", "dst_energy",
     "dst_unet_create", "dst_unet_destroy", "dst_unet_num_params", "dst_unet_set_params", "dst_unet_get_params",
     "dst_unet_forward", "dst_unet_loss_grad", "dst_unet_train", "dst_set_learned_precond",
-    "dst_testing_fp32_arnoldi", "dst_unet_output_scale",
+    "dst_testing_fp32_arnoldi", "dst_testing_fp64_step", "dst_unet_output_scale",
 )
 
 
@@ -116,6 +116,7 @@ def _load():
         "dst_set_learned_precond": (c_int, [vp, vp]),
         "dst_unet_output_scale": (c_int, [vp, P(c_double)]),
         "dst_testing_fp32_arnoldi": (c_int, [c_int, i64, c_int, vp, vp, vp, vp, vp]),
+        "dst_testing_fp64_step": (c_int, [i64, c_int, vp, vp, vp, vp, vp]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)

@@ -665,3 +665,29 @@ extern "C" int dst_arnoldi_update(int64_t n, int nvec, const void *V, const void
     DST_CUDA_TRY(e);
     return DST_OK;
 }
+
+extern "C" int dst_testing_fp64_step(int64_t n, int nvec, const void *V, void *w, void *h, void *rec, void *stream) {
+    if (n < 1 || nvec < 1 || nvec > DST_MAX_VEC || !V || !w || !h || !rec) return DST_ERR_ARG;
+    cudaStream_t s = (cudaStream_t)stream;
+    const int nblk = dst_reduction_blocks(n);
+    const size_t pc = sizeof(double2) * (size_t)nblk * nvec, pr = sizeof(double) * (size_t)nblk;
+    char *scr = nullptr;
+    if (cudaMallocAsync((void **)&scr, pc + pr + 2 * sizeof(unsigned), s) != cudaSuccess) {
+        cudaGetLastError();
+        return DST_ERR_OOM;
+    }
+    const double2 *v = (const double2 *)V;
+    double2 *wv = (double2 *)w, *h1 = (double2 *)h, *h2 = h1 + nvec, *part = (double2 *)scr;
+    double *nr = (double *)rec, *rpart = (double *)(scr + pc);
+    unsigned *tickets = (unsigned *)(scr + pc + pr);
+    cudaError_t e = cudaMemsetAsync(tickets, 0, 2 * sizeof(unsigned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h, 0, 2 * sizeof(double2) * nvec, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rec, 0, 8 * sizeof(double), s);
+    int rc = e == cudaSuccess ? DST_OK : DST_ERR_CUDA;
+    if (rc == DST_OK) rc = dst_k_project(n, nvec, v, wv, h1, part, nblk, s, nr + 3, rpart, nullptr, tickets);
+    if (rc == DST_OK) rc = dst_k_update(n, nvec, v, h1, wv, nr, rpart, nblk, s, nullptr, nullptr, tickets + 1);
+    if (rc == DST_OK) rc = dst_k_project(n, nvec, v, wv, h2, part, nblk, s, nullptr, rpart, nr, tickets);
+    if (rc == DST_OK) rc = dst_k_update(n, nvec, v, h2, wv, nr, rpart, nblk, s, nr, nr + 6, tickets + 1);
+    cudaFreeAsync(scr, s);
+    return rc;
+}
