@@ -27,28 +27,6 @@
 
 namespace dst {
 
-// Stencil factors of every node (see StdConst in apply_pipe.cuh for the scaling).
-template <typename T>
-struct NodeConst {
-    T kc, km, ka[3];
-};
-template <int D, typename T>
-inline NodeConst<T> node_const(const OpParams &p) {
-    NodeConst<T> c;
-    double pm = 1.0;
-    for (int k = 0; k < D; ++k) pm *= p.ax[k].h / 6.0;
-    const double ht6 = p.ht / 6.0;
-    c.kc = (T)(0.5 * pm);
-    c.km = (T)(ht6 * pm);
-    for (int k = 0; k < 3; ++k) {
-        double q = 0.5 * ht6;
-        for (int j = 0; j < D; ++j)
-            if (j != k) q *= p.ax[j].h / 6.0;
-        c.ka[k] = (T)q;
-    }
-    return c;
-}
-
 // One axis at one node: offsets of the neighbours (of the node itself where there is
 // none), whether they hold a value, and which elements exist.
 template <typename T>
@@ -109,7 +87,7 @@ __device__ __forceinline__ float2 add_i_of(float2 g, float k, float2 v, int m, f
 // every element exists and the selects fall away).
 template <int D, int NC, typename T, int VM, bool OPEN>
 __global__ void __launch_bounds__(128)
-apply_node_kernel(OpParams p, NodeConst<T> sc, int tt, const typename LaneOf<T>::type *__restrict__ x,
+apply_node_kernel(OpParams p, StdConst<T> sc, int tt, const typename LaneOf<T>::type *__restrict__ x,
                   typename LaneOf<T>::type *__restrict__ y) {
     using V = typename LaneOf<T>::type;
     constexpr int NY = D >= 2 ? 3 : 1, NZ = D >= 3 ? 3 : 1, R = LaneOf<T>::PER * NC;   // R: lanes per node
@@ -324,7 +302,7 @@ int launch_apply_node(const OpParams &p, const typename C2<T>::type *xv, typenam
     const int64_t chunks = (p.nt + tt - 1) / tt;
     if (blocks <= 0 || blocks > 0x7fffffffLL || chunks > 65535) return DST_ERR_ARG;
     const dim3 grid((unsigned)blocks, (unsigned)chunks);
-    const NodeConst<T> sc = node_const<D, T>(p);
+    const StdConst<T> sc = std_const<D, T>(p);
     bool open = false;
     for (int k = 0; k < D; ++k) open = open || p.ax[k].bc == DST_BC_OPEN;
     auto go = [&](auto vm) {

@@ -141,35 +141,6 @@ __device__ __forceinline__ NodeV<NC, T> smem_node(const char *slot, int node) {
     return v;
 }
 
-// Per-kernel constants of the standard interior stencils.  With
-// M = h/6 [1,4,1] and C = 1/2 [-1,0,1] on every axis, the spatial fields are
-// unscaled [1,4,1] / [-1,0,1] sums times fixed factors; those factors, the 1/2
-// and h_t/6 of the time stencils and the mass m are folded into these
-// constants, so G_C' = G_C / 2 and G_M' = (h_t/6) G_M come out directly.
-template <typename T>
-struct StdConst {
-    T kc;        // G_C' = i kc PM                      (kc = 1/2 prod h_k/6)
-    T km;        // mass part of G_M': -beta m km PM    (km = (h_t/6) prod h_k/6)
-    T ka[3];     // alpha_k part of G_M': i ka[k] alpha_k PC_k  (ka = (h_t/6) 1/2 prod_{j!=k} h_j/6)
-};
-
-template <int D, typename T>
-__host__ __device__ inline StdConst<T> std_const(const OpParams &p) {
-    StdConst<T> c;
-    double pm = 1.0;
-    for (int k = 0; k < D; ++k) pm *= p.ax[k].h / 6.0;
-    const double ht6 = p.ht / 6.0;
-    c.kc = (T)(0.5 * pm);
-    c.km = (T)(ht6 * pm);
-    for (int k = 0; k < 3; ++k) {
-        double q = 0.5 * ht6;
-        for (int j = 0; j < D; ++j)
-            if (j != k) q *= p.ax[j].h / 6.0;
-        c.ka[k] = (T)q;
-    }
-    return c;
-}
-
 // i s (alpha_k P)[c] accumulated into G (NC = 2: alpha = (sigma_x, sigma_y);
 // NC = 4: alpha_k = [[0, sigma_k], [sigma_k, 0]]).
 template <int NC, typename V, typename T>
