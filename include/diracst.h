@@ -430,13 +430,18 @@ DST_API int dst_testing_fp64_step(int64_t n, int nvec, const void *V, void *w, v
  *     (1+1, 2+1, 3+1).  Other meshes: DST_ERR_ARG.
  * dst_precond_apply: z = M v for DEVICE FP32 complex vectors v, z of
  * n_unknowns entries (float pairs, the unknown layout), distinct; arithmetic in
- * FP32 (the precision of the inner solve), the layer-solve factors in FP64
- * rounded to FP32.  Takes stream-ordered scratch of about one FP32 vector (plus
- * the factors, below 32 (6 + 2 log2 n_x) bytes per x node and frequency, on
- * Dirichlet-x meshes).
+ * FP32 (the precision of the inner solve), on Dirichlet-x meshes with layer-solve factors
+ * formed in pairs of floats (48 bits) and rounded to FP32.  Takes stream-ordered scratch:
+ * one FP32 vector and two of one time layer; on Dirichlet-x meshes also 20 bytes per
+ * frequency of the periodic axes, 8 per x node, and the factors,
+ *     64 (n_1 / 2 + 1) (n_2 / 2 + 1) (6 + 2 s) G bytes,
+ * n_1 and n_2 the periodic lengths (1 for an axis that is not there; halves rounded down),
+ * s = ceil(log2(ceil(n_x / 2))) for n_x unknown x nodes and G = max(8, 2^s) (48^3 Klein mesh:
+ * 20 MB, 2+1 with 95 x 96 nodes: 3.6 MB, 1+1 with 47 nodes: 33 KB).
  * kind DST_PRECOND_CN_SWEEP, DST_PRECOND_CN_LEARNED (the sweep plus the
  * learned correction below, with the network attached to the mesh by
- * dst_set_learned_precond; two more FP32 vectors of scratch), or
+ * dst_set_learned_precond; two more FP32 vectors of scratch, three where z is not
+ * 16-byte aligned), or
  * DST_PRECOND_BLOCK_JACOBI:
  *   DST_PRECOND_BLOCK_JACOBI  z = blockdiag(A_nn)^-1 v, A_nn the NC x NC block of
  *     D_w22 coupling the components of unknown node n with themselves: the

@@ -55,7 +55,8 @@ struct SweepPlan {
 
 // DST_OK or DST_ERR_ARG (with a detail) for meshes the sweep does not cover.
 int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p);
-// Device scratch the sweep needs: one FP32 vector, the factors, the potential.
+// Device scratch the sweep needs: one FP32 vector, the two layers of the alternating sum, and
+// in banded mode the factors, the rows of the frequencies and the potential.
 size_t dst_sweep_scratch_bytes(const SweepPlan &p, int64_t n_unknowns);
 // Carve the scratch and compute the banded factors (enqueued on s).
 int dst_sweep_setup(const dst_mesh *mesh, SweepPlan &p, void *scratch, cudaStream_t s);
