@@ -11,7 +11,7 @@
 // 3-point stencils whose end coefficients drop the missing element.
 //
 // Evaluation order (sum factorisation, spatial first): for every time plane
-// p of x the kernel forms, per spinor component, the spatial fields
+// p of x a kernel forms, per spinor component, the spatial fields
 //     S_M  = (M_z M_y M_x) x_p            (goes with C_t: the i d_t term)
 //     S_Ck = (... C_k ...) x_p             (goes with M_t: the alpha_k terms)
 //     S_w  = (M_z M_y M^w_x) x_p           (goes with M_t: the m beta + V term)
@@ -22,9 +22,10 @@
 // the planes of its time chunk (the t = 0 layer is known: its plane is zero
 // in the apply and is the only input of the right-hand side).
 //
-// One CTA owns a spatial tile (TX x TY x TZ outputs) and a chunk of TT time
-// layers; every plane of the tile plus a one-node halo is staged in shared
-// memory (periodic halos wrap, halos outside a non-periodic axis are zero).
+// Here: the coefficients of a node's stencils, which the applies share (apply_node.cuh,
+// apply_pipe.cuh, apply_col.cuh), and the right-hand side.  One CTA of it owns a spatial tile;
+// the t = 0 plane of the tile plus a one-node halo is staged in shared memory
+// (periodic halos wrap, halos outside a non-periodic axis are zero).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -39,9 +40,9 @@ template <> struct C2<double> { using type = double2; };
 template <> struct C2<float> { using type = float2; };
 
 template <int D> struct ApplyTile;
-template <> struct ApplyTile<1> { static constexpr int TX = 128, TY = 1, TZ = 1, TT = 32; };
-template <> struct ApplyTile<2> { static constexpr int TX = 32, TY = 8, TZ = 1, TT = 16; };
-template <> struct ApplyTile<3> { static constexpr int TX = 16, TY = 4, TZ = 4, TT = 8; };
+template <> struct ApplyTile<1> { static constexpr int TX = 128, TY = 1, TZ = 1; };
+template <> struct ApplyTile<2> { static constexpr int TX = 32, TY = 8, TZ = 1; };
+template <> struct ApplyTile<3> { static constexpr int TX = 16, TY = 4, TZ = 4; };
 
 template <typename V> __device__ __forceinline__ V cz() { V r; r.x = 0; r.y = 0; return r; }
 template <typename V, typename T> __device__ __forceinline__ V cmul_r(T a, V v) { V r; r.x = a * v.x; r.y = a * v.y; return r; }

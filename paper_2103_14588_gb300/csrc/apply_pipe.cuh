@@ -1,4 +1,4 @@
-// Pipelined operator apply: time planes staged through a shared-memory ring
+// Pipelined operator apply in 1+1 and 2+1 (two components): time planes staged through a shared-memory ring
 // by asynchronous copies (cp.async, L2 -> shared, zero-filled outside
 // non-periodic boundaries), several planes in flight per CTA.
 //
@@ -23,29 +23,28 @@ constexpr int64_t MAX_GRID_Y = 65535;      // chunks of time layers in one launc
 
 namespace dst {
 
-// Output tile TX x TY x TZ per CTA and TT time layers; each thread computes RY
+// Output tile TX x TY per CTA and TT time layers; each thread computes RY
 // consecutive y outputs (2+1: the x stencils of the rows they share are
 // computed once).
 // TV selects one of the tile shapes the autotuner chooses from (variant 0 is
 // the default): smaller tiles and time chunks give small meshes more CTAs.
 template <int D, int TV = 0> struct PipeTile;
-template <> struct PipeTile<1, 0> { static constexpr int TX = 256, TY = 1, TZ = 1, TT = 32, RY = 1; };
-template <> struct PipeTile<1, 1> { static constexpr int TX = 128, TY = 1, TZ = 1, TT = 16, RY = 1; };
-template <> struct PipeTile<1, 2> { static constexpr int TX = 64, TY = 1, TZ = 1, TT = 8, RY = 1; };
-template <> struct PipeTile<2, 0> { static constexpr int TX = 32, TY = 8, TZ = 1, TT = 8, RY = 2; };
-template <> struct PipeTile<2, 1> { static constexpr int TX = 32, TY = 8, TZ = 1, TT = 4, RY = 2; };
-template <> struct PipeTile<2, 2> { static constexpr int TX = 16, TY = 8, TZ = 1, TT = 8, RY = 2; };
+template <> struct PipeTile<1, 0> { static constexpr int TX = 256, TY = 1, TT = 32, RY = 1; };
+template <> struct PipeTile<1, 1> { static constexpr int TX = 128, TY = 1, TT = 16, RY = 1; };
+template <> struct PipeTile<1, 2> { static constexpr int TX = 64, TY = 1, TT = 8, RY = 1; };
+template <> struct PipeTile<2, 0> { static constexpr int TX = 32, TY = 8, TT = 8, RY = 2; };
+template <> struct PipeTile<2, 1> { static constexpr int TX = 32, TY = 8, TT = 4, RY = 2; };
+template <> struct PipeTile<2, 2> { static constexpr int TX = 16, TY = 8, TT = 8, RY = 2; };
 
 template <int D, int NC, typename T, int TV = 0>
 struct PipeShape {
     using Tile = PipeTile<D, TV>;
     static constexpr int BX = Tile::TX + 2;
     static constexpr int BY = D >= 2 ? Tile::TY + 2 : 1;
-    static constexpr int BZ = D >= 3 ? Tile::TZ + 2 : 1;
-    static constexpr int BOX = BX * BY * BZ;                          // nodes per staged plane
-    static constexpr int NODE_BYTES = NC * 2 * (int)sizeof(T);        // 16, 32 or 64
+    static constexpr int BOX = BX * BY;                               // nodes per staged plane
+    static constexpr int NODE_BYTES = NC * 2 * (int)sizeof(T);        // 16 or 32
     static constexpr int CHUNKS = NODE_BYTES / 16;                    // 16-byte copies per node
-    static constexpr int NTHR = Tile::TX * (Tile::TY / Tile::RY) * Tile::TZ;
+    static constexpr int NTHR = Tile::TX * (Tile::TY / Tile::RY);
     // two planes per step (twice the independent work per barrier) when one
     // output per thread and an eight-plane ring fits comfortably; otherwise one
     // plane per step, 4 or 3 stages
@@ -95,10 +94,9 @@ struct CopyPlan {
 };
 
 template <int D, int NC, typename T, int TV>
-__device__ __forceinline__ void make_copy_plan(const OpParams &p, int64_t x0, int64_t y0, int64_t z0,
-                                               CopyPlan<D, NC, T, TV> &cp) {
+__device__ __forceinline__ void make_copy_plan(const OpParams &p, int64_t x0, int64_t y0, CopyPlan<D, NC, T, TV> &cp) {
     using S = PipeShape<D, NC, T, TV>;
-    const int64_t nx = p.ax[0].n, ny = p.ax[1].n;
+    const int64_t nx = p.ax[0].n;
 #pragma unroll
     for (int j = 0; j < CopyPlan<D, NC, T, TV>::PER_THREAD; ++j) {
         const int i = threadIdx.x + j * S::NTHR;
@@ -106,12 +104,10 @@ __device__ __forceinline__ void make_copy_plan(const OpParams &p, int64_t x0, in
         cp.src[j] = -1;
         if (i >= S::BOX * S::CHUNKS) continue;
         const int node = i / S::CHUNKS, part = i % S::CHUNKS;
-        const int bx = node % S::BX, by = (node / S::BX) % S::BY, bz = node / (S::BX * S::BY);
-        const int gx = axis_nbr32(p.ax[0], (int)x0 - 1 + bx);
-        const int gy = D >= 2 ? axis_nbr32(p.ax[1], (int)y0 - 1 + by) : 0;
-        const int gz = D >= 3 ? axis_nbr32(p.ax[2], (int)z0 - 1 + bz) : 0;
+        const int gx = axis_nbr32(p.ax[0], (int)x0 - 1 + node % S::BX);
+        const int gy = D >= 2 ? axis_nbr32(p.ax[1], (int)y0 - 1 + node / S::BX) : 0;
         cp.dst[j] = node * S::NODE_BYTES + part * 16;
-        if (gx >= 0 && gy >= 0 && gz >= 0) cp.src[j] = ((gz * (int)ny + gy) * (int)nx + gx) * S::NODE_BYTES + part * 16;
+        if (gx >= 0 && gy >= 0) cp.src[j] = (gy * (int)nx + gx) * S::NODE_BYTES + part * 16;
     }
 }
 
@@ -141,28 +137,15 @@ __device__ __forceinline__ NodeV<NC, T> smem_node(const char *slot, int node) {
     return v;
 }
 
-// i s (alpha_k P)[c] accumulated into G (NC = 2: alpha = (sigma_x, sigma_y);
-// NC = 4: alpha_k = [[0, sigma_k], [sigma_k, 0]]).
-template <int NC, typename V, typename T>
+// i s (alpha_k P)[c] accumulated into G: alpha = (sigma_x, sigma_y).
+template <typename V, typename T>
 __device__ __forceinline__ void add_i_alpha(int k, T s, const V *P, V *G) {
     // i * (a.x + i a.y) * s = (-s a.y, s a.x)
     auto addi = [&](V &g, V a, T f) { g.x = fma(-f, a.y, g.x); g.y = fma(f, a.x, g.y); };
-    if (NC == 2) {
-        if (k == 0) { addi(G[0], P[1], s); addi(G[1], P[0], s); }
-        else {      // sigma_y: (-i b, i a): i*(-i b) = b, i*(i a) = -a
-            G[0].x = fma(s, P[1].x, G[0].x); G[0].y = fma(s, P[1].y, G[0].y);
-            G[1].x = fma(-s, P[0].x, G[1].x); G[1].y = fma(-s, P[0].y, G[1].y);
-        }
-    } else {
-        if (k == 0) { addi(G[0], P[3], s); addi(G[1], P[2], s); addi(G[2], P[1], s); addi(G[3], P[0], s); }
-        else if (k == 1) {
-            G[0].x = fma(s, P[3].x, G[0].x); G[0].y = fma(s, P[3].y, G[0].y);
-            G[1].x = fma(-s, P[2].x, G[1].x); G[1].y = fma(-s, P[2].y, G[1].y);
-            G[2].x = fma(s, P[1].x, G[2].x); G[2].y = fma(s, P[1].y, G[2].y);
-            G[3].x = fma(-s, P[0].x, G[3].x); G[3].y = fma(-s, P[0].y, G[3].y);
-        } else {    // sigma_z: (a, -b)
-            addi(G[0], P[2], s); addi(G[1], P[3], -s); addi(G[2], P[0], s); addi(G[3], P[1], -s);
-        }
+    if (k == 0) { addi(G[0], P[1], s); addi(G[1], P[0], s); }
+    else {      // sigma_y: (-i b, i a): i*(-i b) = b, i*(i a) = -a
+        G[0].x = fma(s, P[1].x, G[0].x); G[0].y = fma(s, P[1].y, G[0].y);
+        G[1].x = fma(-s, P[0].x, G[1].x); G[1].y = fma(-s, P[0].y, G[1].y);
     }
 }
 
@@ -176,43 +159,26 @@ template <int D, int NC, typename T, bool WV, typename Get>
 __device__ __forceinline__ void fields_std(Get get, const StdConst<T> &sc, T m, const T (&wa)[2], const T (&wb)[2],
                                            typename C2<T>::type *GC, typename C2<T>::type *GM) {
     using V = typename C2<T>::type;
-    const int NZ = D >= 3 ? 3 : 1, NY = D >= 2 ? 3 : 1;
-    V QM[NC], QCx[NC], QCy[NC], QCz[NC];   // sums over z of [1,4,1] (and [-1,0,1] for z)
+    const int NY = D >= 2 ? 3 : 1;
+    V QM[NC], QCx[NC], QCy[NC];            // sums over y of [1,4,1] (and [-1,0,1] for y)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) { QM[c] = cz<V>(); QCx[c] = cz<V>(); QCy[c] = cz<V>(); QCz[c] = cz<V>(); }
-#pragma unroll
-    for (int dz = 0; dz < NZ; ++dz) {
-        V PM[NC], PCx[NC], PCy[NC];
-#pragma unroll
-        for (int dy = 0; dy < NY; ++dy) {
-            const int r = (dz * NY + dy) * 3;
-            const NodeV<NC, T> n0 = get(r), n1 = get(r + 1), n2 = get(r + 2);
-            const T wy = (D >= 2 && dy == 1) ? (T)4 : (T)1;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const V x0 = n0.c[c], x1 = n1.c[c], x2 = n2.c[c];
-                V rM, rC;
-                rM.x = fma((T)4, x1.x, x0.x + x2.x); rM.y = fma((T)4, x1.y, x0.y + x2.y);
-                rC.x = x2.x - x0.x; rC.y = x2.y - x0.y;
-                if (dy == 0) {
-                    PM[c] = rM; PCx[c] = rC;
-                    if (D >= 2) { PCy[c].x = -rM.x; PCy[c].y = -rM.y; }
-                } else {
-                    PM[c] = cfma_r(wy, rM, PM[c]);
-                    PCx[c] = cfma_r(wy, rC, PCx[c]);
-                    if (D >= 2 && dy == 2) PCy[c] = cadd(PCy[c], rM);
-                }
-            }
-        }
-        const T wz = (D >= 3 && dz == 1) ? (T)4 : (T)1;
+    for (int dy = 0; dy < NY; ++dy) {
+        const int r = dy * 3;
+        const NodeV<NC, T> n0 = get(r), n1 = get(r + 1), n2 = get(r + 2);
+        const T wy = (D >= 2 && dy == 1) ? (T)4 : (T)1;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            QM[c] = cfma_r(wz, PM[c], QM[c]);
-            QCx[c] = cfma_r(wz, PCx[c], QCx[c]);
-            if (D >= 2) QCy[c] = cfma_r(wz, PCy[c], QCy[c]);
-            if (D >= 3) {
-                if (dz == 0) QCz[c] = cmul_r((T)(-1), PM[c]);
-                else if (dz == 2) QCz[c] = cadd(QCz[c], PM[c]);
+            const V x0 = n0.c[c], x1 = n1.c[c], x2 = n2.c[c];
+            V rM, rC;
+            rM.x = fma((T)4, x1.x, x0.x + x2.x); rM.y = fma((T)4, x1.y, x0.y + x2.y);
+            rC.x = x2.x - x0.x; rC.y = x2.y - x0.y;
+            if (dy == 0) {
+                QM[c] = rM; QCx[c] = rC;
+                if (D >= 2) { QCy[c].x = -rM.x; QCy[c].y = -rM.y; }
+            } else {
+                QM[c] = cfma_r(wy, rM, QM[c]);
+                QCx[c] = cfma_r(wy, rC, QCx[c]);
+                if (D >= 2 && dy == 2) QCy[c] = cadd(QCy[c], rM);
             }
         }
     }
@@ -227,9 +193,8 @@ __device__ __forceinline__ void fields_std(Get get, const StdConst<T> &sc, T m, 
             GM[c] = cmul_r(f, QM[c]);
         }
     }
-    add_i_alpha<NC>(0, sc.ka[0], QCx, GM);
-    if (D >= 2) add_i_alpha<NC>(1, sc.ka[1], QCy, GM);
-    if (D >= 3) add_i_alpha<NC>(2, sc.ka[2], QCz, GM);
+    add_i_alpha(0, sc.ka[0], QCx, GM);
+    if (D >= 2) add_i_alpha(1, sc.ka[1], QCy, GM);
 }
 
 // 2+1, standard interior stencils, RY consecutive y outputs of one thread:
@@ -267,8 +232,8 @@ __device__ __forceinline__ void fields_std_rows(Get get, const StdConst<T> &sc, 
                 GM[r][c] = cmul_r(f, PM[c]);
             }
         }
-        add_i_alpha<NC>(0, sc.ka[0], PCx, GM[r]);
-        add_i_alpha<NC>(1, sc.ka[1], PCy, GM[r]);
+        add_i_alpha(0, sc.ka[0], PCx, GM[r]);
+        add_i_alpha(1, sc.ka[1], PCy, GM[r]);
     }
 }
 
@@ -282,39 +247,32 @@ template <int D, int NC, typename T, bool NOV, bool STD, int TV = 0>
 __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdConst<T> &sc,
                                                 const typename C2<T>::type *__restrict__ x,
                                                 typename C2<T>::type *__restrict__ y, int64_t tiles_x,
-                                                int64_t tiles_y, int64_t tile, int64_t chunk, char *ring) {
+                                                int64_t tile, int64_t chunk, char *ring) {
     using V = typename C2<T>::type;
     using S = PipeShape<D, NC, T, TV>;
     using Tile = typename S::Tile;
     constexpr int RY = Tile::RY;
-    constexpr int TYT = Tile::TY / RY;                  // threads along y
-
     const int64_t x0 = (tile % tiles_x) * Tile::TX;
-    const int64_t y0 = ((tile / tiles_x) % tiles_y) * Tile::TY;
-    const int64_t z0 = (tile / (tiles_x * tiles_y)) * Tile::TZ;
+    const int64_t y0 = tile / tiles_x * Tile::TY;
     const int tx = threadIdx.x % Tile::TX;
-    const int ty = ((threadIdx.x / Tile::TX) % TYT) * RY;     // first of the thread's RY output rows
-    const int tz = threadIdx.x / (Tile::TX * TYT);
-    const int64_t ix = x0 + tx, iy = y0 + ty, iz = z0 + tz;
-    const int64_t nx = p.ax[0].n, ny = p.ax[1].n, nz = p.ax[2].n;
+    const int ty = threadIdx.x / Tile::TX * RY;         // first of the thread's RY output rows
+    const int64_t ix = x0 + tx, iy = y0 + ty;
+    const int64_t nx = p.ax[0].n, ny = p.ax[1].n;
     const int64_t N = p.nt;
     const int64_t t0 = 1 + chunk * Tile::TT;
     const int64_t t1 = min(t0 + (int64_t)Tile::TT, N + 1);
-    const int64_t plane_elems = nx * ny * nz * NC;
-    const int64_t self = (iz * ny + iy) * nx + ix;
+    const int64_t plane_elems = nx * ny * NC;
+    const int64_t self = iy * nx + ix;
     const int nplanes = (int)(t1 - t0 + 2);            // planes t0-1 .. t1
     const int64_t pfirst = t0 - 1;
 
     bool valid[RY];
     bool stdn[RY];
-    bool any_valid = false, all_std = true;
+    bool all_std = true;
 #pragma unroll
-    for (int r = 0; r < RY; ++r) {
-        valid[r] = ix < nx && iy + r < ny && iz < nz;
-        any_valid = any_valid || valid[r];
-    }
-    NodeCoef<D, T> k;      // coefficients of output row 0 (x and z are shared by all rows)
-    if (valid[0]) node_coef<D, T>(p, ix, iy, iz, k);
+    for (int r = 0; r < RY; ++r) valid[r] = ix < nx && iy + r < ny;
+    NodeCoef<D, T> k;      // coefficients of output row 0 (x is shared by all rows)
+    if (valid[0]) node_coef<D, T>(p, ix, iy, 0, k);
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
         // standard interior stencils on every axis (periodic / Dirichlet axes,
@@ -324,7 +282,6 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
             const Coef3<T> cy = r == 0 ? k.cy : axis_coef<T>(p.ax[1], iy + r);
             sd = sd && cy.eL && cy.eR;
         }
-        if (D >= 3) sd = sd && k.cz.eL && k.cz.eR;
         stdn[r] = sd;
         all_std = all_std && (sd || !valid[r]);
     }
@@ -335,10 +292,9 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
         wa[sb] = (T)(-0.5) * sc.km * (wl + wr); wb[sb] = (T)(-0.5) * sc.km * (wr - wl);
     }
     CopyPlan<D, NC, T, TV> cplan;
-    make_copy_plan<D, NC, T, TV>(p, x0, y0, z0, cplan);
+    make_copy_plan<D, NC, T, TV>(p, x0, y0, cplan);
     const T h6 = (T)(p.ht / 6.0);
-    const int NY = D >= 2 ? 3 : 1;
-    const int c0 = (tz * S::BY + ty) * S::BX + tx;      // box index of the (-1,-1,-1) neighbour of row 0
+    const int c0 = ty * S::BX + tx;                     // box index of the (-1, -1) neighbour of row 0
 
     // Plane-loop bookkeeping in 32-bit, relative to the chunk: plane i is time
     // layer pfirst + i; it exists iff i_lo <= i <= i_hi; outputs are stored
@@ -376,10 +332,7 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
                 auto getq = [&](int q, int dx) { return smem_node<NC, T>(slot, c0 + q * S::BX + dx); };
                 fields_std_rows<NC, T, !NOV, RY>(getq, sc, (T)p.m, wa, wb, GC, GM);
             } else {
-                auto get = [&](int q) {
-                    const int dz = q / (3 * NY), dy = (q / 3) % NY, dx = q % 3;
-                    return smem_node<NC, T>(slot, c0 + (dz * S::BY + dy) * S::BX + dx);
-                };
+                auto get = [&](int q) { return smem_node<NC, T>(slot, c0 + q / 3 * S::BX + q % 3); };
                 fields_std<D, NC, T, !NOV>(get, sc, (T)p.m, wa, wb, GC[0], GM[0]);
             }
             return;
@@ -393,18 +346,14 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
         for (int r = 0; r < RY; ++r) {
             if (have && valid[r]) {
                 const int cr = c0 + r * S::BX;
-                auto get = [&](int q) {
-                    const int dz = q / (3 * NY), dy = (q / 3) % NY, dx = q % 3;
-                    return smem_node<NC, T>(slot, cr + (dz * S::BY + dy) * S::BX + dx);
-                };
+                auto get = [&](int q) { return smem_node<NC, T>(slot, cr + q / 3 * S::BX + q % 3); };
                 if (stdn[r]) {
                     fields_std<D, NC, T, !NOV>(get, sc, (T)p.m, wa, wb, GC[r], GM[r]);
                 } else {
                     NodeCoef<D, T> kr;
                     if (r == 0) kr = k;
-                    else node_coef<D, T>(p, ix, iy + r, iz, kr);
-                    if (NOV) fields_nov<D, NC, T>(get, kr, (T)p.m, GC[r], GM[r]);
-                    else fields<D, NC, T>(get, kr, GC[r], GM[r]);
+                    else node_coef<D, T>(p, ix, iy + r, 0, kr);
+                    fields<D, NC, T>(get, kr, GC[r], GM[r]);
 #pragma unroll
                     for (int c = 0; c < NC; ++c) { GC[r][c] = cmul_r((T)0.5, GC[r][c]); GM[r][c] = cmul_r(h6, GM[r][c]); }
                 }
@@ -488,16 +437,15 @@ __device__ __forceinline__ void apply_pipe_tile(const OpParams &p, const StdCons
         }
     }
     cp_async_wait<0>();
-    (void)any_valid;
 }
 
 // Meshes without an open axis only (the launches send the others to apply_node.cuh).
 template <int D, int NC, typename T, bool NOV, int TV>
 __global__ void __launch_bounds__(PipeShape<D, NC, T, TV>::NTHR, sizeof(T) == 8 ? 1 : 3)
 apply_pipe_kernel(OpParams p, StdConst<T> sc, const typename C2<T>::type *__restrict__ x, typename C2<T>::type *__restrict__ y,
-                  int64_t tiles_x, int64_t tiles_y, int64_t chunk0) {
+                  int64_t tiles_x, int64_t chunk0) {
     extern __shared__ __align__(16) char ring[];
-    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, sc, x, y, tiles_x, tiles_y, blockIdx.x, chunk0 + blockIdx.y, ring);
+    apply_pipe_tile<D, NC, T, NOV, true, TV>(p, sc, x, y, tiles_x, blockIdx.x, chunk0 + blockIdx.y, ring);
 }
 
 template <int D, int NC, typename T, int TV>
@@ -506,12 +454,11 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
     using Tile = PipeTile<D, TV>;
     const int64_t tx = (p.ax[0].n + Tile::TX - 1) / Tile::TX;
     const int64_t ty = (p.ax[1].n + Tile::TY - 1) / Tile::TY;
-    const int64_t tz = (p.ax[2].n + Tile::TZ - 1) / Tile::TZ;
     const int64_t chunks = (p.nt + Tile::TT - 1) / Tile::TT;
-    const int64_t tiles = tx * ty * tz;
+    const int64_t tiles = tx * ty;
     if (tiles <= 0 || tiles > 0x7fffffffLL) return DST_ERR_ARG;
     // byte offsets within one time layer are kept in 32 bits
-    if (p.ax[0].n * p.ax[1].n * p.ax[2].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<D, NC, T>(p, x, y, s);
+    if (p.ax[0].n * p.ax[1].n * S::NODE_BYTES >= (1LL << 31)) return launch_apply_node<D, NC, T>(p, x, y, s);
     // the shared-memory opt-in is a per-device function attribute: set it once per device
     static bool configured[2][DST_MAX_DEVICES_APPLY] = {};
     int dev = 0;
@@ -525,7 +472,7 @@ int launch_apply_pipe_v(const OpParams &p, const typename C2<T>::type *x, typena
     const StdConst<T> sc = std_const<D, T>(p);
     for (int64_t c = 0; c < chunks; c += MAX_GRID_Y) {
         const dim3 grid((unsigned)tiles, (unsigned)std::min(MAX_GRID_Y, chunks - c));
-        kern<<<grid, S::NTHR, S::SMEM, s>>>(p, sc, x, y, tx, ty, c);
+        kern<<<grid, S::NTHR, S::SMEM, s>>>(p, sc, x, y, tx, c);
     }
     DST_CUDA_TRY(cudaGetLastError());
     return DST_OK;

@@ -45,7 +45,7 @@ constexpr int BMAXM = 32;              // restart length at most (Hessenberg in 
 struct BatchInst {
     OpParams p;                 // vmode 0: x-only weights (zero potential: weights +-m)
     int64_t n;                  // unknowns
-    int64_t tiles_x, tiles_y, tiles, chunks;
+    int64_t tiles_x, tiles, chunks;
     const double2 *b;           // right-hand side
     double2 *x;                 // solution (the caller's psi)
     double2 *r;                 // FP64 scratch: A x, then the residual
@@ -132,14 +132,14 @@ batch_solve_kernel(const BatchInst *__restrict__ insts, BatchOpts o) {
     const StdConst<double> sc64 = std_const<D, double>(I.p);
     auto apply32 = [&](const float2 *xin, float2 *yout) {
         for (int64_t tc = 0; tc < ntc; ++tc) {
-            apply_pipe_tile<D, 2, float, false, false>(I.p, sc32, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
+            apply_pipe_tile<D, 2, float, false, false>(I.p, sc32, xin, yout, I.tiles_x, tc % I.tiles,
                                                         tc / I.tiles, ring);
             __syncthreads();
         }
     };
     auto apply64 = [&](const double2 *xin, double2 *yout) {
         for (int64_t tc = 0; tc < ntc; ++tc) {
-            apply_pipe_tile<D, 2, double, false, false>(I.p, sc64, xin, yout, I.tiles_x, I.tiles_y, tc % I.tiles,
+            apply_pipe_tile<D, 2, double, false, false>(I.p, sc64, xin, yout, I.tiles_x, tc % I.tiles,
                                                          tc / I.tiles, ring);
             __syncthreads();
         }
@@ -555,14 +555,13 @@ static int solve_batch(int count, dst_mesh *const *meshes, const dst_solve_opts 
             b.n = mh->n_unknowns;
             if (mh->d == 1) {
                 b.tiles_x = (b.p.ax[0].n + PipeTile<1>::TX - 1) / PipeTile<1>::TX;
-                b.tiles_y = 1;
+                b.tiles = b.tiles_x;
                 b.chunks = (b.p.nt + PipeTile<1>::TT - 1) / PipeTile<1>::TT;
             } else {
                 b.tiles_x = (b.p.ax[0].n + PipeTile<2>::TX - 1) / PipeTile<2>::TX;
-                b.tiles_y = (b.p.ax[1].n + PipeTile<2>::TY - 1) / PipeTile<2>::TY;
+                b.tiles = b.tiles_x * ((b.p.ax[1].n + PipeTile<2>::TY - 1) / PipeTile<2>::TY);
                 b.chunks = (b.p.nt + PipeTile<2>::TT - 1) / PipeTile<2>::TT;
             }
-            b.tiles = b.tiles_x * b.tiles_y;
             char *q2 = wsb + off[k];
             b.b = reinterpret_cast<double2 *>(q2);
             b.r = reinterpret_cast<double2 *>(q2 + align256(sizeof(double2) * b.n));

@@ -330,7 +330,7 @@ struct Solver {
     }
     // gate: second-pass kernels that skip themselves on the device when the
     // DGKS test (nrm[0] < nrm[3] / 2) fails; their bytes are counted only if
-    // they ran (second_pass_ran() after the step's synchronisation).
+    // they ran (count_second_pass(), from the step's record).
     int project(int nv, const double2 *wv, double2 *h, double *wnrm2 = nullptr, const double *gate = nullptr) {
         const double n = (double)w.n;
         return run(K_PROJECT, nblk * nv <= DST_FUSED_PARTIALS ? 1 : 2, gate ? 0.0 : 16.0 * n * (nv + 1), gate ? 0.0 : 8.0 * n * nv + (wnrm2 ? 4.0 * n : 0.0),

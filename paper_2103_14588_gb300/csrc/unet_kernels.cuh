@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
     const int ci = 1 << a.lci;
     // staged: the offsets of the slower axes; else every tap, the one after the last (K
     // padded to a multiple of 16) starting from nowhere
-    const int xt = CI16 > 0 && a.taps > 1 ? 3 : 1, entries = a.taps / xt;
+    constexpr int xt = CI16 > 0 ? 3 : 1;                   // (a staged convolution has kernel 3)
+    const int entries = a.taps / xt;
     for (int t = threadIdx.x; t <= entries; t += blockDim.x) {
         Tap e{0, t < entries ? 0 : 1 << 8, 0};
         if (a.taps > 1 && t < entries) {
@@ -250,8 +251,9 @@ __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
                     }
                 }
             };
-            if (xt == 3) { tap(-1, 0); tap(0, 1); tap(1, 2); }
-            else tap(0, 0);
+            tap(-1, 0);
+            tap(0, 1);
+            tap(1, 2);
         }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     } else {
