@@ -58,7 +58,7 @@ using namespace dst_march;
 // FP64: the part that c carries is exact, so the rounding is relative to the small
 // R x, for the modes that the time step resolves (c = 1) as for those that it only turns
 // round (c = -1, h_t K >> M).  Relative error of 48 layers against FP64, at h_t = h / 4, h,
-// 10 h and 40 h (m = 1, V0 = 3, 24 x 24 nodes): 4.5e-7, 5.4e-7, 3.1e-7 and 2.7e-7 (s - h_t K x
+// 10 h and 40 h (m = 1, V0 = 3, 24 x 24 nodes): 4.7e-7, 5.7e-7, 3.1e-7 and 2.8e-7 (s - h_t K x
 // formed in FP32: 4.7e-7, 1.0e-6, 2.2e-6 and 4.1e-6; the march takes the same time either way).
 // One pass over the layers, the loads of the next PD in flight while one is combined.
 __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ alt_hi,
@@ -114,8 +114,7 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
                 const float4 v = ring[q];
                 if (t + PD < g.nt) ring[q] = x[(t + PD) * nf + f];
                 float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                add_mv(u, Pf, lo);
-                add_mv(u, Pf, s);
+                add_mv(u, Pf, add4(s, lo));
                 sub_mv(u, Rf, xp);
                 xp = make_float4(fmaf(cx, xp.x, fmaf(-cy, xp.y, u.x)), fmaf(cx, xp.y, fmaf(cy, xp.x, u.y)),
                                  fmaf(cx, xp.z, fmaf(-cy, xp.w, u.z)), fmaf(cx, xp.w, fmaf(cy, xp.z, u.w)));
