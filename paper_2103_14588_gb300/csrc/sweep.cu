@@ -51,16 +51,18 @@ using namespace dst_march;
 // ---- 2a. spectral march: one thread per frequency ---------------------------
 // Every axis periodic and a constant potential: M_s and K_s are diagonal in
 // frequency with 2 x 2 blocks (1+1 and 2+1 only), so with P = Bd^-1 and M^ = prod_k m_k
-//   x_t = P s_t - Q x_{t-1},   Q = P Bl = I - 2 i M^ P,
+//   x_t = P (s_t - Bl x_{t-1}) = x_{t-1} + P (s_t - h_t K^ x_{t-1})   (sweep_march.cuh),
 // Bd = i M^ + (h_t/2) [ sum_k alpha_k (i sin th_k) i prod_{j != k} m_j - (m beta + V0) M^ ].
-// -Q turns the two modes of a frequency by a phase each.  The march takes the nearest c of
-// 1, -1, i, -i and 0 out of it, x_t = c x_{t-1} + P s_t - R x_{t-1} with R = Q + c I formed in
-// FP64: the part that c carries is exact, so the rounding is relative to the small
-// R x, for the modes that the time step resolves (c = 1) as for those that it only turns
-// round (c = -1, h_t K >> M).  Relative error of 48 layers against FP64, at h_t = h / 4, h,
-// 10 h and 40 h (m = 1, V0 = 3, 24 x 24 nodes): 4.7e-7, 5.7e-7, 3.1e-7 and 2.8e-7 (s - h_t K x
-// formed in FP32: 4.7e-7, 1.0e-6, 2.2e-6 and 4.1e-6; the march takes the same time either way).
+// The second form rounds relative to the increment.  LARGE: h_t K is not small against M
+// (dst_sweep_plan's rule), s and h_t K x cancel, and the march takes
+//   x_t = c x_{t-1} + P s_t - R x_{t-1},   R = Q + c I,   Q = P Bl = I - 2 i M^ P:
+// -Q turns the two modes of a frequency by a phase each; c is the nearest of 1, -1, i, -i and 0 to
+// that, exact, and R is formed in FP64, so the rounding is relative to R x.  Relative error of 48
+// layers against FP64, at h_t = h, 10 h and 40 h (m = 1, V0 = 3, 24 x 24 nodes): 5.7e-7, 3.1e-7 and
+// 2.8e-7 (the increment form 1.0e-6, 2.2e-6 and 4.1e-6); at h / 4 the increment form 4.7e-7, this
+// one the same.  Either takes the same time.
 // One pass over the layers, the loads of the next PD in flight while one is combined.
+template <bool LARGE>
 __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ alt_hi,
                                       const float4 *__restrict__ alt_lo, float4 *__restrict__ x) {
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -84,27 +86,34 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
     const double wx = dx * r, wy = -dy * r;
     const double P[8] = {a1 * wx - pm * wy, a1 * wy + pm * wx, -bx * wx - by * wy, by * wx - bx * wy,
                          by * wy - bx * wx, -bx * wy - by * wx, a0 * wx - pm * wy, a0 * wy + pm * wx};
-    // Q by rows, then the c that leaves the smallest diagonal of R
-    double Q[8];
-#pragma unroll
-    for (int k = 0; k < 8; k += 2) { Q[k] = 2.0 * pm * P[k + 1]; Q[k + 1] = -2.0 * pm * P[k]; }
-    Q[0] += 1.0;
-    Q[6] += 1.0;
-    const float tx = (float)(Q[0] + Q[6]), ty = (float)(Q[1] + Q[7]);
-    // |q0 + c|^2 + |q1 + c|^2 = |q0|^2 + |q1|^2 + 2 (|c|^2 + Re conj(c) (q0 + q1)): below that of c = 0 where the trace
-    // has a part beyond -1 along c
-    float cx = 0.f, cy = 0.f;
-    if (fmaxf(fabsf(tx), fabsf(ty)) > 1.f) {
-        if (fabsf(tx) >= fabsf(ty)) cx = tx > 0.f ? -1.f : 1.f;
-        else cy = ty > 0.f ? -1.f : 1.f;
-    }
-    Q[0] += cx; Q[6] += cx;
-    Q[1] += cy; Q[7] += cy;
     auto blk = [](const double *v) {
         return Blk{make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]),
                    make_float4((float)v[4], (float)v[5], (float)v[6], (float)v[7])};
     };
-    const Blk Pf = blk(P), Rf = blk(Q);
+    const Blk Pf = blk(P);
+    // h_t K^ = kx sigma_x + ky sigma_y + diag(d0, d1)
+    const float kx = (float)(2.0 * bx), ky = (float)(2.0 * by), d0 = (float)(-g.ht * (g.m + g.V0) * pm),
+                d1 = (float)(-g.ht * (g.V0 - g.m) * pm);
+    Blk Rf = {};
+    float cx = 0.f, cy = 0.f;
+    if (LARGE) {
+        // Q by rows, then the c that leaves the smallest diagonal of R
+        double Q[8];
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) { Q[k] = 2.0 * pm * P[k + 1]; Q[k + 1] = -2.0 * pm * P[k]; }
+        Q[0] += 1.0;
+        Q[6] += 1.0;
+        const float tx = (float)(Q[0] + Q[6]), ty = (float)(Q[1] + Q[7]);
+        // |q0 + c|^2 + |q1 + c|^2 = |q0|^2 + |q1|^2 + 2 (|c|^2 + Re conj(c) (q0 + q1)): below that of c = 0 where the
+        // trace has a part beyond -1 along c
+        if (fmaxf(fabsf(tx), fabsf(ty)) > 1.f) {
+            if (fabsf(tx) >= fabsf(ty)) cx = tx > 0.f ? -1.f : 1.f;
+            else cy = ty > 0.f ? -1.f : 1.f;
+        }
+        Q[0] += cx; Q[6] += cx;
+        Q[1] += cy; Q[7] += cy;
+        Rf = blk(Q);
+    }
     float4 s = alt_hi[f], lo = alt_lo[f], xp = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t t0 = 0; t0 < g.nt; t0 += PD) {
 #pragma unroll
@@ -114,10 +123,20 @@ __global__ void march_spectral_kernel(SweepGeom g, const float4 *__restrict__ al
                 const float4 v = ring[q];
                 if (t + PD < g.nt) ring[q] = x[(t + PD) * nf + f];
                 float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                add_mv(u, Pf, add4(s, lo));
-                sub_mv(u, Rf, xp);
-                xp = make_float4(fmaf(cx, xp.x, fmaf(-cy, xp.y, u.x)), fmaf(cx, xp.y, fmaf(cy, xp.x, u.y)),
-                                 fmaf(cx, xp.z, fmaf(-cy, xp.w, u.z)), fmaf(cx, xp.w, fmaf(cy, xp.z, u.w)));
+                if (LARGE) {
+                    add_mv(u, Pf, add4(s, lo));
+                    sub_mv(u, Rf, xp);
+                    xp = make_float4(fmaf(cx, xp.x, fmaf(-cy, xp.y, u.x)), fmaf(cx, xp.y, fmaf(cy, xp.x, u.y)),
+                                     fmaf(cx, xp.z, fmaf(-cy, xp.w, u.z)), fmaf(cx, xp.w, fmaf(cy, xp.z, u.w)));
+                } else {
+                    const float4 r =
+                        make_float4(s.x - fmaf(kx, xp.z, fmaf(ky, xp.w, fmaf(d0, xp.x, -lo.x))),
+                                    s.y - fmaf(kx, xp.w, fmaf(-ky, xp.z, fmaf(d0, xp.y, -lo.y))),
+                                    s.z - fmaf(kx, xp.x, fmaf(-ky, xp.y, fmaf(d1, xp.z, -lo.z))),
+                                    s.w - fmaf(kx, xp.y, fmaf(ky, xp.x, fmaf(d1, xp.w, -lo.w))));
+                    add_mv(u, Pf, r);
+                    xp = add4(u, xp);
+                }
                 x[t * nf + f] = xp;
                 next_s(s, lo, v);
             }
@@ -214,6 +233,13 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
         dst_internal_set_error_detail("Crank-Nicolson sweep: a periodic plane too large for shared memory");
         return DST_ERR_ARG;
     }
+    // h_t K against M: the derivatives, mass and potential (twice, as measured; both marches
+    // give their errors on either side of the limits)
+    double vmax = 0.0, kt = 2.0 * std::fabs(mesh->m);
+    for (size_t e = 0; e < mesh->V.size() && e < (size_t)mesh->nel[0]; ++e) vmax = std::max(vmax, std::fabs(mesh->V[e]));
+    kt += 2.0 * vmax;
+    for (int k = 0; k < d; ++k) kt += 1.0 / mesh->h[k];
+    p.large = g.ht * kt > (d == 1 ? 1.0 : 1.5) || g.ht > 0.5 * mesh->h[0];
     // banded march: G lanes per system (two x nodes each), `steps` parallel reduction
     // steps; systems per CTA as many as keep it at 256 threads while the CTAs still
     // cover the GPU (a 2+1 mesh has n_y systems, a 1+1 mesh one)
@@ -237,12 +263,6 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
             dst_internal_set_error_detail("Crank-Nicolson sweep: x axis too long for the banded march");
             return DST_ERR_ARG;
         }
-        // h_t K against M: the x and transverse derivatives, mass and potential (twice, as measured)
-        double vmax = 0.0, k = 2.0 * std::fabs(mesh->m);
-        for (size_t e = 0; e < mesh->V.size() && e < (size_t)mesh->nel[0]; ++e) vmax = std::max(vmax, std::fabs(mesh->V[e]));
-        k += 2.0 * vmax;
-        for (int a_ = 0; a_ < d; ++a_) k += 1.0 / mesh->h[a_];
-        p.refine = g.ht * k > (d == 1 ? 1.0 : 1.5) || g.ht > 0.5 * mesh->h[0];
         p.table_bytes = sizeof(float) * 8 * 2 * (size_t)dst_march::class_count(g.n1, g.n2) * dst_march::items(p.steps) * p.lanes;
     }
     p.launches = 2 + (p.has_fft ? 2 : 0);
@@ -295,7 +315,7 @@ static int launch_march(const SweepPlan &p, const float2 *in, float2 *out, cudaS
         DST_CUDA_TRY(cudaGetLastError());
         return DST_OK;
     };
-#define DST_MARCH(G) case G: return p.refine ? go(march_kernel<NC, G, true>) : go(march_kernel<NC, G, false>);
+#define DST_MARCH(G) case G: return p.large ? go(march_kernel<NC, G, true>) : go(march_kernel<NC, G, false>);
     switch (p.lanes) {
         DST_MARCH(8) DST_MARCH(16) DST_MARCH(32) DST_MARCH(64) DST_MARCH(128) DST_MARCH(256)
         default: return DST_ERR_ARG;
@@ -326,7 +346,8 @@ int dst_sweep_apply(const SweepPlan &p, int64_t n_unknowns, const float2 *v, flo
     altsum_kernel<<<(unsigned)((per2 + 255) / 256), 256, 0, s>>>(per2, p.g.nt, (const float4 *)src, p.alt_hi, p.alt_lo);
     DST_CUDA_TRY(cudaGetLastError());
     if (!p.banded) {
-        march_spectral_kernel<<<(unsigned)((nf + 63) / 64), 64, 0, s>>>(p.g, p.alt_hi, p.alt_lo, (float4 *)dst);
+        const auto march = p.large ? march_spectral_kernel<true> : march_spectral_kernel<false>;
+        march<<<(unsigned)((nf + 63) / 64), 64, 0, s>>>(p.g, p.alt_hi, p.alt_lo, (float4 *)dst);
         DST_CUDA_TRY(cudaGetLastError());
     } else {
         const int rc = p.g.nc == 2 ? launch_march<2>(p, src, dst, s) : launch_march<4>(p, src, dst, s);

@@ -41,7 +41,7 @@ struct SweepPlan {
     int64_t nb;                 // FFT planes
     size_t table_bytes;         // banded: reduction factors (sweep_march.cuh)
     int lanes, steps, systems;  // banded: lanes per system, parallel reduction steps, systems per CTA
-    bool refine;                // banded: layer solves refined once (sweep_march.cuh)
+    bool large;                 // h_t K not small against M: the marches' other forms
     size_t march_smem;
     int launches;               // kernels of one application
     double bytes_per_entry;     // algorithmic bytes of one application, factors apart
