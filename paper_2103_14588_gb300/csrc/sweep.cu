@@ -239,7 +239,7 @@ int dst_sweep_plan(const dst_mesh *mesh, SweepPlan &p) {
     for (size_t e = 0; e < mesh->V.size() && e < (size_t)mesh->nel[0]; ++e) vmax = std::max(vmax, std::fabs(mesh->V[e]));
     kt += 2.0 * vmax;
     for (int k = 0; k < d; ++k) kt += 1.0 / mesh->h[k];
-    p.large = g.ht * kt > (d == 1 ? 1.0 : 1.5) || g.ht > 0.5 * mesh->h[0];
+    p.large = g.ht * kt > (d == 1 ? 0.6 : 1.5) || g.ht > 0.5 * mesh->h[0];
     // banded march: G lanes per system (two x nodes each), `steps` parallel reduction
     // steps; systems per CTA as many as keep it at 256 threads while the CTAs still
     // cover the GPU (a 2+1 mesh has n_y systems, a 1+1 mesh one)

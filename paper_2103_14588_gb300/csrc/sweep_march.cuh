@@ -325,10 +325,11 @@ inline size_t march_smem(int nc, int sys, int G, int n) {
 // increment form alone is as exact as an elimination along x in order, or better (relative
 // error against FP64 9.3e-7 and 1.5e-6 on the 48^3 x 48 Klein mesh).  With q = h_t (sum of
 // 1 / h_k + 2 (m + max |V|)) the error of 48 layers, as a multiple of that elimination's,
-// is at most 0.8 unrefined up to q = 1.5 (1+1: 0.7 up to q = 1, 1.1 at 1.3), 1.2 at 2.3,
-// 1.6 at 3.5, 2 to 3.7 from 7 on; refined 0.5 on average over 338 meshes from q = 4 on, above
-// 1.1 in eleven of them (high potentials on short transverse spacings, 1.8 at most).  A
-// step's refinement takes about as long as its solve: 48^3 x 12 layers 348 us, 314 without.
+// is at most 0.8 unrefined up to q = 1.5 (1+1: 0.9 up to q = 0.6, 1.2 from 0.65 on), 1.2 at 2.3,
+// 1.6 at 3.5, 2 to 3.7 from 7 on; refined 0.4 to 0.8 there, 0.5 on average over 338 meshes from
+// q = 4 on, above 1.1 in eleven of them (high potentials on short transverse spacings, 1.8
+// at most).  A step's refinement takes about as long as its solve: 48^3 x 12 layers 348 us,
+// 314 without; 1+1 39 nodes x 40 layers 109 us and 95.
 // blockDim.x = systems per CTA x G.  Layers t of `in` [t][x][f][c] to `out` (in == out allowed).
 template <int NC, int G, bool LARGE>
 __global__ void __launch_bounds__(G > 32 ? 512 : 256)
