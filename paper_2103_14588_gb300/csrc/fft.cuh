@@ -53,6 +53,9 @@ template <int BYTES> __device__ __forceinline__ void copy_async(void *dst, const
                  "n"(BYTES) : "memory");
 }
 
+// Components per CTA, at most (choose_layout).
+template <typename V> constexpr int COMPONENTS = sizeof(typename Real<V>::type) == 4 ? 2 : 1;
+
 // What a thread transforms at a time: W components of a node, which lie side by side in
 // memory and share index arithmetic, twiddles and wide accesses.
 template <typename V, int W> struct alignas(sizeof(V) * W > 16 ? 16 : sizeof(V) * W) Elem { V c[W]; };
@@ -343,7 +346,7 @@ fft_planes_kernel(SweepFft a, int64_t ctas, const V *__restrict__ in, V *__restr
 template <typename V, bool INVERSE>
 inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, const V *in, V *out, cudaStream_t s) {
     static bool configured[64] = {};
-    const auto one = fft_planes_kernel<V, 1, INVERSE>, two = fft_planes_kernel<V, 2, INVERSE>;
+    const auto one = fft_planes_kernel<V, 1, INVERSE>, two = fft_planes_kernel<V, COMPONENTS<V>, INVERSE>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -366,15 +369,19 @@ inline cudaError_t fft_launch(const SweepFft &a, int64_t nb, const V *in, V *out
 
 // Pick the components per CTA and the stage layout for planes of a.n1 x a.n2:
 // CTA-wide stages (second plane buffer) when they fit, else one line per warp; two
-// components per CTA where three such CTAs fit an SM and there are enough to fill the GPU
-// (nb planes per component group).
+// components per CTA in FP32, where they share index arithmetic and twiddles, where three
+// such CTAs fit an SM (76 KB; 48 x 48 planes of Klein 48^4: 727 us the sweep, 799 one by
+// one) and there are two for every SM (nb planes per component group; from 1 to 1216 CTAs
+// no mesh below a few microseconds' difference).  FP64 takes one: its stages wait for the FP64 unit,
+// and more lanes with less work each suit it better (energy of 32 x 32 x 400: 157 us, 187 by twos).
 // Returns false if nothing fits in `limit` bytes.
 template <typename V>
 inline bool choose_layout(SweepFft &a, int64_t nb, size_t limit) {
     for (int pp = 1; pp >= 0; --pp) {
         a.pingpong = pp;
-        a.ncb = 2;                             // spinors have two or four components
-        if (fft_smem_bytes<V>(a) <= (pp ? std::min<size_t>(limit, 76 * 1024) : limit) && nb * (a.nc / 2) >= 304) return true;
+        a.ncb = COMPONENTS<V>;                 // spinors have two or four components
+        if (a.ncb > 1 && fft_smem_bytes<V>(a) <= (pp ? std::min<size_t>(limit, 76 * 1024) : limit) && nb * (a.nc / 2) >= 304)
+            return true;
         a.ncb = 1;
         if (fft_smem_bytes<V>(a) <= limit) return true;
     }
@@ -382,10 +389,13 @@ inline bool choose_layout(SweepFft &a, int64_t nb, size_t limit) {
 }
 
 // Stockham radices of n: the fewest stages of the register butterflies, then other primes.
-inline void radices(int n, int *r, int &nr) {
+// `points` (FP64): nodes of the plane; radices of 8 and 16 then want 128 butterflies, four full
+// warps, because an FP64 instruction takes its unit's 64 clocks whatever lanes it serves
+// (energy of 16 x 16 x 16: 49 us, 55 with one stage of 16 per axis; 1+1 512 x 2000 299 us, 323).
+inline void radices(int n, int *r, int &nr, int64_t points = 1 << 30) {
     nr = 0;
     for (int p : {16, 8, 4, 2, 3, 5})
-        while (n % p == 0) { r[nr++] = p; n /= p; }
+        while (n % p == 0 && (p < 8 || points / p >= 128)) { r[nr++] = p; n /= p; }
     for (int p = 7; n > 1; p += 2)
         while (n % p == 0) { r[nr++] = p; n /= p; }
 }

@@ -1,10 +1,10 @@
 """Energy per layer where the FFT's planes change form, against the oracle's numpy FFT.
 
-From 304 CTAs on a CTA takes two spinor components of a plane, below that one; the second pass of a
-3+1 mesh takes as many z lines together as divide a layer's (y, x) plane, up to 32 and 1024
-nodes: meshes whose planes divide by 32, by less, by nothing, z axes of one node and of
-more than 512, odd and prime lengths.  Tolerance as in test_gpu_observables.py: 1e-11 of the
-largest |E|.
+1+1 meshes take x lines of several layers as a plane, as many as divide the layers, and the second
+pass of a 3+1 mesh z lines that divide a layer's (y, x) plane: up to 32 lines and 1024 nodes,
+while 304 CTAs are left.  Meshes on either side of those: lines by 32, by less, alone, z axes of
+one node and of more than 512, odd and prime lengths, planes of few nodes (radices of four
+in place of 16).  Tolerance as in test_gpu_observables.py: 1e-11 of the largest |E|.
 """
 import numpy as np
 import pytest
@@ -15,7 +15,8 @@ from _helpers import oracle_mesh
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,n_el", [(1, [24, 1, 1, 310]), (2, [12, 10, 1, 305]), (2, [7, 5, 1, 304]), (3, [8, 8, 8, 20]),
+@pytest.mark.parametrize("d,n_el", [(1, [24, 1, 1, 310]), (1, [16, 1, 1, 4896]), (1, [512, 1, 1, 305]),
+                                    (1, [512, 1, 1, 306]), (1, [37, 1, 1, 331]), (2, [12, 10, 1, 305]), (2, [7, 5, 1, 304]), (3, [8, 8, 8, 20]),
                                     (3, [12, 10, 9, 16]), (3, [5, 7, 11, 31]), (3, [11, 13, 6, 60]), (3, [4, 4, 1, 40]),
                                     (3, [2, 3, 520, 3]), (3, [32, 3, 32, 7]), (3, [1, 1, 12, 200])])
 def test_energy(d, n_el):
