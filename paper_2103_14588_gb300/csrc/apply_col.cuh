@@ -16,9 +16,9 @@
 // four of one (FP64), 16 bytes of a node each, which exchange convection fields by
 // shuffles.  In FP32 the real and imaginary part go through one packed instruction
 // (f32x2): half the issue slots of the sums.
-// 48^4 Klein mesh: FP32 163 -> 99 us (two CTAs per SM without spills; three, with 100 bytes
-// spilled, took 136), FP64 4.79 -> 2.94 ms (33 FP64 instructions per real output and plane,
-// 46 before; 2.4 ms at the pipe's rate).
+// 48^4 Klein mesh: FP32 100 us, 163 with columns of one output in y and z apart (two CTAs per SM
+// without spills; three, with 100 bytes spilled, 136), FP64 2.94 ms, 4.79 so (33 FP64
+// instructions per real output and plane, 46 so; 2.4 ms at the pipe's rate).
 #pragma once
 
 #include "apply_pipe.cuh"

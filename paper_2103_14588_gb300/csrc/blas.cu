@@ -90,8 +90,8 @@ __device__ __forceinline__ bool last_cta(unsigned *ticket) {
 
 // Inner products of G basis vectors (the first at V) with w over the CTA's slice, summed over
 // the warp into red.  G is exact: a vector that is not there would still take its share of
-// the FP64 unit (predicated instructions occupy it), which once made one vector cost as much
-// as eight (1.77M entries: 127 us for one vector, 11.8 us of FP64 work).
+// the FP64 unit (predicated instructions occupy it), and one vector would cost as much
+// as eight (1.77M entries: 127 us for one vector so, 64 with its own instance).
 template <int G>
 __device__ __forceinline__ void project_group(int64_t n, int64_t b, int64_t e, const double2 *__restrict__ V,
                                               const double2 *__restrict__ w, double *red, bool norm, double &wn) {

@@ -568,8 +568,8 @@ project_tma_kernel(int64_t n, int nvec, const float2 *__restrict__ V, const floa
 #pragma unroll
             for (int q = 0; q < TMA_GROUP; ++q) { all[2 * q] = R[q]; all[2 * q + 1] = I[q]; }
             // as many sums as the group has vectors, to a power of two: one warp sum after the
-            // other, their conversions to FP64 held the FP64 unit for 6 us per launch (30 vectors of
-            // 1.77M entries: 90 us, 84 us now; of 200,000: 29 us, 22 us now)
+            // other, their conversions to FP64 hold the FP64 unit for 6 us per launch (30 vectors of
+            // 1.77M entries: 90 us so, 82 together)
             auto store = [&](auto count) {
                 constexpr int N = decltype(count)::value;
                 DfAcc a[N];

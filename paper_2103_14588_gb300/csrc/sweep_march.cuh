@@ -17,7 +17,7 @@
 //
 // The layer solve.  The systems are few (2 x 2304 for the 48^3 x 48 Klein mesh) and the
 // time steps are a serial chain, so block Thomas elimination (a chain of 2 n_x small
-// products per layer) leaves the GPU waiting: it took 4.5 ms there.  Here G lanes share a
+// products per layer) leaves the GPU waiting (4.5 ms there, 0.25 so).  Here G lanes share a
 // system, two x nodes each: one cyclic-reduction step removes the odd nodes, parallel
 // cyclic reduction over the even ones needs log2(G) exchanges, and the odd nodes follow.
 // Twice the arithmetic of the elimination, a seventh of the chain.  Bd = i M + (h_t/2) K

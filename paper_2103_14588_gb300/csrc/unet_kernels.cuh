@@ -131,8 +131,8 @@ struct ConvShape {
 
 // One warp: 16 MT consecutive nodes x 8 NT output channels (blockIdx.y: which).  CI16: input
 // channels / 16; 0 (any number) without the ring.
-// 16 -> 16 channels at 48^3 (1.5 GFLOP): 253 us with divisions per fragment, 19 us with tap
-// tables and loads through L1, 15 us staged; 64 -> 64 channels at 12^3: 388, 58 and 12 us.
+// 16 -> 16 channels at 48^3 (1.5 GFLOP): 19 us with loads through L1, 15 us staged; 64 -> 64
+// channels at 12^3: 58 and 12 us (253 and 388 us with divisions per fragment).
 template <int NT, int MT, int CI16>
 __global__ void __launch_bounds__(32 * CONV_WARPS) conv_kernel(ConvArgs a) {
     extern __shared__ __align__(16) unsigned char ring[];
