@@ -308,7 +308,7 @@ def time_apply(torch, B, mesh, prec, n, iters=40):
 
 
 NCU_CASES = ("solve60", "solve60_klein32", "solve60_klein", "apply32_zb", "apply32_klein", "apply64_klein",
-             "apply32_klein_zcol", "apply64_klein_zcol", "sweep_zb", "unet_zb48")
+             "apply32_klein_v1", "apply64_klein_v1", "sweep_zb", "unet_zb48")
 
 
 def run_ncu_case(case):
@@ -319,8 +319,8 @@ def run_ncu_case(case):
     32^3 x 32 (4.06M unknowns) or 48^3 x 48 (the bench mesh, seed 1), with the bench's
     one-pass Gram-Schmidt;
     apply32_zb / apply32_klein / apply64_klein: 12 operator applies on the 96^2 x 96 mesh or
-    the 48^3 x 48 3+1 Klein mesh, over rotating buffers (tile variant 0);
-    apply32_klein_zcol / apply64_klein_zcol: the same with tile variant 1;
+    the 48^3 x 48 3+1 Klein mesh (column kernel), over rotating buffers (tile variant 0);
+    apply32_klein_v1 / apply64_klein_v1: the same with tile variant 1;
     sweep_zb: 6 Crank-Nicolson sweeps on the 96^2 x 96 mesh;
     unet_zb48: 4 forward passes of the U-Net on the 48^2 x 48 grid.
     """
@@ -361,7 +361,7 @@ def run_ncu_case(case):
             print("unet_zb48: 4 forward passes")
         else:
             prec = B.DST_FP32 if case.startswith("apply32") else B.DST_FP64
-            if case.endswith("_zcol"):
+            if case.endswith("_v1"):
                 B.dst_set_apply_variant(m.handle, prec, 1)
             ms, gbs = time_apply(torch, B, m.handle, prec, m.n_unknowns, iters=12)
             print("%s: %.1f us per apply" % (case, 1e3 * ms))
