@@ -148,9 +148,9 @@ apply_node_kernel(OpParams p, StdConst<T> sc, int tt, const typename LaneOf<T>::
     const T k1 = c & 1 ? -sc.ka[1] : sc.ka[1], k2 = c & 1 ? -sc.ka[2] : sc.ka[2];
     const int64_t N = p.nt, t0 = 1 + blockIdx.y * (int64_t)tt, t1 = min(t0 + (int64_t)tt, N + 1);
     const int64_t step = plane * R;
-    // planes t0 - 1 .. t1 of x, without the layers 0 and N + 1, which hold nothing: by the bounds
-    // of the loop, or by a branch in it where that takes fewer registers (48^4 elements with an
-    // open axis, FP32: 387 us, 422 by the bounds; a general potential 24^4: 32.5 and 29.7)
+    // planes t0 - 1 .. t1 of x, without the layers 0 and N + 1, which hold nothing, but where
+    // bounds of their own cost the loop registers (48^4 elements with an open axis, FP32:
+    // 390 us as zeros, 422 so)
     constexpr bool TRIM = !(D == 3 && sizeof(T) == 4 && OPEN && VM != 1);
     const int64_t tb = TRIM ? max(t0 - 1, (int64_t)1) : t0 - 1, te = TRIM ? min(t1, N) : t1;
     const V *src = x + (tb - 1) * step + s * R + lane;
@@ -176,70 +176,67 @@ apply_node_kernel(OpParams p, StdConst<T> sc, int tt, const typename LaneOf<T>::
     for (int64_t t = tb; t <= te; ++t, src += step) {
         Rows nxt;
         if (D < 3) load(src + step, t < te, 0, nxt);
-        V GC = zero, GM = zero;
-        if (TRIM || (t >= 1 && t <= N)) {
-            // sums over x and y of each z slice, then over z: mass, convection along x, y, z,
-            // and for a general potential the mass sums of the elements on the eight sides
-            V M, Cx, Cy = zero, Cz = zero, W = zero, Mz[3], Xz[3], Yz[3], Q[3][4];
+        // sums over x and y of each z slice, then over z: mass, convection along x, y, z,
+        // and for a general potential the mass sums of the elements on the eight sides
+        V M, Cx, Cy = zero, Cz = zero, W = zero, Mz[3], Xz[3], Yz[3], Q[3][4];
 #pragma unroll
-            for (int dz = 0; dz < NZ; ++dz) {
-                // (the condition always holds; with it the loads stay predicated: 5 x 40 x 40 x 60 elements with an
-                // open axis, FP64, 581 us, 654 without)
-                if (D == 3) load(src, t >= 1 && t <= N, dz, cur);
-                V rM[NY], rC[NY], L[NY], H[NY];
+        for (int dz = 0; dz < NZ; ++dz) {
+            // (with TRIM the condition always holds; it keeps the loads predicated: 5 x 40 x 40 x 60
+            // elements with an open axis, FP64, 541 us, 654 without)
+            if (D == 3) load(src, t >= 1 && t <= N, dz, cur);
+            V rM[NY], rC[NY], L[NY], H[NY];
 #pragma unroll
-                for (int dy = 0; dy < NY; ++dy) {
-                    const V a = cur.v[dy][0], b = cur.v[dy][1], d = cur.v[dy][2];
-                    rC[dy] = diff(ex.el, a, b, d, ex.er);
-                    if (VM == 1) {
-                        L[dy] = half(ex.el, b, a);
-                        H[dy] = half(ex.er, b, d);
-                        rM[dy] = ladd(L[dy], H[dy]);
-                    } else {
-                        rM[dy] = mass(a, ex.wc, b, d);         // a missing neighbour was loaded as zero
-                    }
-                }
-                if (D == 1) {
-                    Mz[dz] = rM[0]; Xz[dz] = rC[0];
-                    if (VM == 1) { Q[dz][0] = L[0]; Q[dz][1] = H[0]; }
+            for (int dy = 0; dy < NY; ++dy) {
+                const V a = cur.v[dy][0], b = cur.v[dy][1], d = cur.v[dy][2];
+                rC[dy] = diff(ex.el, a, b, d, ex.er);
+                if (VM == 1) {
+                    L[dy] = half(ex.el, b, a);
+                    H[dy] = half(ex.er, b, d);
+                    rM[dy] = ladd(L[dy], H[dy]);
                 } else {
-                    Mz[dz] = mass(rM[0], ey.wc, rM[1], rM[2]);
-                    Xz[dz] = mass(rC[0], ey.wc, rC[1], rC[2]);
-                    Yz[dz] = diff(ey.el, rM[0], rM[1], rM[2], ey.er);
-                    if (VM == 1) {
-                        Q[dz][0] = half(ey.el, L[1], L[0]); Q[dz][1] = half(ey.el, H[1], H[0]);
-                        Q[dz][2] = half(ey.er, L[1], L[2]); Q[dz][3] = half(ey.er, H[1], H[2]);
-                    }
+                    rM[dy] = mass(a, ex.wc, b, d);         // a missing neighbour was loaded as zero
                 }
             }
-            if (D < 3) {
-                M = Mz[0]; Cx = Xz[0];
-                if (D == 2) Cy = Yz[0];
-                if (VM == 1) {
-#pragma unroll
-                    for (int k = 0; k < 1 << D; ++k) W = lfma(vc[k], Q[0][k], W);
-                }
+            if (D == 1) {
+                Mz[dz] = rM[0]; Xz[dz] = rC[0];
+                if (VM == 1) { Q[dz][0] = L[0]; Q[dz][1] = H[0]; }
             } else {
-                M = mass(Mz[0], ez.wc, Mz[1], Mz[2]);
-                Cx = mass(Xz[0], ez.wc, Xz[1], Xz[2]);
-                Cy = mass(Yz[0], ez.wc, Yz[1], Yz[2]);
-                Cz = diff(ez.el, Mz[0], Mz[1], Mz[2], ez.er);
+                Mz[dz] = mass(rM[0], ey.wc, rM[1], rM[2]);
+                Xz[dz] = mass(rC[0], ey.wc, rC[1], rC[2]);
+                Yz[dz] = diff(ey.el, rM[0], rM[1], rM[2], ey.er);
                 if (VM == 1) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        W = lfma(vc[k], half(ez.el, Q[1][k], Q[0][k]), W);
-                        W = lfma(vc[4 + k], half(ez.er, Q[1][k], Q[2][k]), W);
-                    }
+                    Q[dz][0] = half(ey.el, L[1], L[0]); Q[dz][1] = half(ey.el, H[1], H[0]);
+                    Q[dz][2] = half(ey.er, L[1], L[2]); Q[dz][3] = half(ey.er, H[1], H[2]);
                 }
             }
-            GC = add_i_of(zero, sc.kc, M, 0, sg);
-            GM = VM == 1 ? W : VM == 0 ? lfma(wb, Cx, lmul(wm, M)) : lmul(wm, M);
-            // i alpha: x takes component 1 - c (3 - c), y its (-i, i) multiple, z (3+1) the (1, -1) multiple of c ^ 2
-            constexpr int PX = NC == 2 ? 1 : 3;
-            GM = add_i_of(GM, sc.ka[0], Cx, PX, sg);
-            if (D >= 2) GM = add_of(GM, k1, Cy, PX, sg);
-            if (D >= 3) GM = add_i_of(GM, k2, Cz, 2, sg);
         }
+        if (D < 3) {
+            M = Mz[0]; Cx = Xz[0];
+            if (D == 2) Cy = Yz[0];
+            if (VM == 1) {
+#pragma unroll
+                for (int k = 0; k < 1 << D; ++k) W = lfma(vc[k], Q[0][k], W);
+            }
+        } else {
+            M = mass(Mz[0], ez.wc, Mz[1], Mz[2]);
+            Cx = mass(Xz[0], ez.wc, Xz[1], Xz[2]);
+            Cy = mass(Yz[0], ez.wc, Yz[1], Yz[2]);
+            Cz = diff(ez.el, Mz[0], Mz[1], Mz[2], ez.er);
+            if (VM == 1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    W = lfma(vc[k], half(ez.el, Q[1][k], Q[0][k]), W);
+                    W = lfma(vc[4 + k], half(ez.er, Q[1][k], Q[2][k]), W);
+                }
+            }
+        }
+        const V GC = add_i_of(zero, sc.kc, M, 0, sg);
+        V GM = VM == 1 ? W : VM == 0 ? lfma(wb, Cx, lmul(wm, M)) : lmul(wm, M);
+        // i alpha: x takes component 1 - c (3 - c), y its (-i, i) multiple, z (3+1) the (1, -1) multiple of c ^ 2
+        constexpr int PX = NC == 2 ? 1 : 3;
+        GM = add_i_of(GM, sc.ka[0], Cx, PX, sg);
+        if (D >= 2) GM = add_of(GM, k1, Cy, PX, sg);
+        if (D >= 3) GM = add_i_of(GM, k2, Cz, 2, sg);
         // y(t-1) += GC + GM; y(t) += (t < N ? 4 GM : GC + 2 GM); y(t+1) = GM - GC
         accP = ladd(accP, ladd(GC, GM));
         accC = t < N ? lfma((T)4, GM, accC) : ladd(accC, lfma((T)2, GM, GC));
